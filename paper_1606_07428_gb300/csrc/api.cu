@@ -511,11 +511,8 @@ int rbs_get_stats(rbs_ctx* h, rbs_stats* out) {
   if (s.ok()) s = c.harvest();
   if (!s.ok()) return finish(c, s);
   *out = c.stats;
-  for (int k = 0; k < 5; ++k) out->pair_variant[k] = c.tuned[k];
-  for (int k = 0; k < 2; ++k)  // the float32 sums run in the treecode kernel when it is on
-    if (c.tree.active) out->pair_variant[k] = c.tree.nt[k] ? rbs::kPacked + c.tree.nt[k] : 0;
-  for (int k = 0; k < 3; ++k)  // and the double-float ones in the double-float treecode kernel
-    if (c.tree_df.active) out->pair_variant[2 + k] = c.tree_df.nt[k];
+  for (int k = 0; k < 2; ++k) out->pair_variant[k] = c.tree.active ? rbs::kPacked + rbs::tree_variant(c) : c.tuned[k];
+  for (int k = 2; k < 5; ++k) out->pair_variant[k] = rbs::kPacked + 1;
   return RBS_OK;
 }
 

@@ -163,7 +163,6 @@ struct TreeState {
   int degree = 0, npx = 0;   // interpolation degree and (degree + 1)^3 proxy points per cluster
   int n_cells = 0;           // clusters with proxy points
   int tmax = 0;              // largest target count of a work item
-  int nt[3] = {0, 0, 0};     // targets per thread chosen for (traction, Stokeslet, both), 0: not yet
   double theta = 0.0;
   long long n_src = 0;       // sources: N nodes, then n_cells * npx proxy points
   std::vector<TreeItem> items;
@@ -176,12 +175,13 @@ struct TreeState {
   DevBuf<double> d_box;      // per cluster with proxies: box midpoint (3), 1 / half-width (3)
   DevBuf<float> d_cheb;      // Chebyshev points, then barycentric weights (degree + 1 each)
   DevBuf<double> d_cheb64;   // the same in float64 (double-float layout)
-  // sources for the pair kernel: positions as float32 hi + lo (w of hi: particle id bits, -3 for a
-  // proxy point) and float32 weighted density (nodes) or cluster charge (proxy points).  In the
-  // double-float layout: positions as exact three-float splits hi + x3m + lo, weighted densities and
-  // charges as float32 pairs q + wl, and the charges accumulated in float64 (q64, 3 per proxy point)
-  DevBuf<float4> d_hi, d_lo, d_q;
-  DevBuf<float4> d_x3m, d_wl;
+  // proxy coordinates of each cluster's tensor grid, (cluster, axis, k) as exact three-float splits, and its
+  // charges by rows of the last axis (nbp rows of ncp charges per plane, padded with zeros): per row
+  // 3 x ncp floats (float32), or 7 x ncp (double-float: hi, lo and the bound of pairsdf.cuh), split from
+  // charges accumulated in float64 (q64, 3 x ncp per row)
+  int nbp = 0, ncp = 0;
+  DevBuf<float4> d_axis;
+  DevBuf<float> d_pq;
   DevBuf<double> d_q64;
   long long direct_pairs = 0, proxy_pairs = 0, charge_work = 0;
   void release();
@@ -328,7 +328,9 @@ struct Context {
   DevBuf<double4> d_up_x;          // upsampled lab nodes (x, y, z, weight)
   DevBuf<long long> d_up_off;      // per upsampled source particle
   DevBuf<int> d_up_particle, d_up_index;
-  DevBuf<double> d_up_mu;          // upsampled densities, n_up_nodes x 3
+  DevBuf<float4> d_up3h, d_up3m, d_up3l;  // the same positions as exact three-float splits
+  DevBuf<double4> d_up_q;          // upsampled weighted densities in float64 ...
+  DevBuf<float4> d_up_qh, d_up_ql; // ... and in float32 (hi alone) or as float32 pairs
 
   // particle-block work lists: particles whose shape stores every row, as (particle, first node,
   // end node, 0) items of 24 nodes; particles whose shape stores representative rows, one per block
@@ -349,13 +351,14 @@ struct Context {
   DevBuf<const float*> d_upU32;
 
   std::map<const void*, int> resident;  // kernel -> resident blocks per SM
-  // chosen targets per thread: (float32, double-float) x (K, S), then the fused double-float K + S
-  int tuned[5] = {0, 0, 0, 0, 0};
-  float tune_ms[5] = {0, 0, 0, 0, 0};
+  // chosen variants of the direct float32 pair sums (traction, Stokeslet), 0: not yet
+  int tuned[2] = {0, 0};
+  float tune_ms[2] = {0, 0};
 
   // smooth pair-sum work list: (target begin, target end, source begin, source end)
   std::vector<longlong4> work;
   DevBuf<longlong4> d_work;
+  DevBuf<int> d_unit;  // the next work unit of the running pair sum (zeroed before each launch)
 
   // scratch vectors (3N doubles each) and GMRES workspace
   DevBuf<double> d_vec[10];
@@ -465,10 +468,11 @@ struct TreePlan {
 Status plan_treecode(const PlanInput& in, double theta, int degree, TreePlan& plan);
 // Builds (or clears) the treecode of the current geometry; called after the near-pair lists.
 Status build_far_field(Context& c);
-// y += the treecode's float32 smooth pair sum of kind (0 traction, 1 Stokeslet) for density x, with
-// nt targets per thread (1, 2 or 4; 0: the fastest, timed once per geometry).
-Status apply_tree(Context& c, int kind, const double* x, double* y, int nt);
-// The same for the double-float passes: y += kind 0 or 1 sum; kind 2: y += traction, y2 += Stokeslet.
+// y += the treecode's float32 smooth pair sum of kind (0 traction, 1 Stokeslet) for density x, whose weighted
+// values are in d_wmu32.
+Status apply_tree(Context& c, int kind, const double* x, double* y);
+int tree_variant(const Context& c);  // its targets per lane
+// The same for the double-float passes (d_wmuh, d_wmul): y += kind 0 or 1 sum; kind 2: y += traction, y2 += Stokeslet.
 Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y2);
 // Relative error assumed for a float32 operator application: rounding plus, with the treecode,
 // its approximation model C(theta) rho^-n.

@@ -82,4 +82,20 @@ __device__ __forceinline__ dflt df_add_accurate(dflt a, dflt b) {
   return {h2, l - (h2 - h)};
 }
 
+// h + l renormalised (|l| below |h|, or h zero)
+__device__ __forceinline__ dflt df_renorm(dflt a) {
+  const float h = a.h + a.l;
+  return {h, a.l - (h - a.h)};
+}
+// a - (bh + bl), renormalised
+__device__ __forceinline__ dflt df_sub(dflt a, float2 b) {
+  dflt s = df_two_sum(a.h, -b.x);
+  s.l += a.l - b.y;
+  return df_renorm(s);
+}
+__device__ __forceinline__ dflt df_sqr(dflt a) {
+  const float p = a.h * a.h;
+  return {p, fmaf(fmaf(2.0f, a.h, a.l), a.l, fmaf(a.h, a.h, -p))};
+}
+
 }  // namespace rbs

@@ -8,6 +8,7 @@
 //  * near correction: for near particle pairs, the base-grid contribution is replaced by the one
 //    from the source's upsampled grid (Section 3: upsampling for close targets).
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 
 #include <cuda_fp16.h>
@@ -785,81 +786,6 @@ __global__ void __launch_bounds__(128 / NT, NT == 4 ? 12 : (NT == 2 ? 10 : 8)) k
 }
 
 // ------------------------------------------------------------------------------------------
-// Smooth pair sums in double-float arithmetic (dfloat.cuh): about 44 bits per float32-pipe operation;
-// each tile of sources is summed in double-float and the tile sums accumulate in double-float.
-
-// KIND 0: traction into acc; 1: Stokeslet into acc; 2: both for the same density, traction into acc
-// and Stokeslet into acc2, sharing the separation, its inverse powers and r . w rho.
-template <int KIND, bool MASK, int NT>
-__device__ __forceinline__ void pair_tile_df(const float4* __restrict__ sph, const float4* __restrict__ spl,
-                                             const float4* __restrict__ sdh, const float4* __restrict__ sdl, int cnt,
-                                             const dflt (&xt)[NT][3], const dflt (&nt)[NT][3], const int (&pt)[NT],
-                                             dflt (&acc)[NT][3], dflt (&acc2)[NT][3]) {
-  for (int l = 0; l < cnt; ++l) {
-    const float4 yh = sph[l], yl = spl[l], dh = sdh[l], dl = sdl[l];
-    const dflt den[3] = {{dh.x, dl.x}, {dh.y, dl.y}, {dh.z, dl.z}};
-#pragma unroll
-    for (int u = 0; u < NT; ++u) {
-      dflt d[3];
-      d[0] = df_two_sum(xt[u][0].h, -yh.x);
-      d[0].l += xt[u][0].l - yl.x;
-      d[1] = df_two_sum(xt[u][1].h, -yh.y);
-      d[1].l += xt[u][1].l - yl.y;
-      d[2] = df_two_sum(xt[u][2].h, -yh.z);
-      d[2].l += xt[u][2].l - yl.z;
-      // r^2 = sum of d_c^2
-      float p[3], e[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        p[c] = d[c].h * d[c].h;
-        e[c] = fmaf(d[c].h, d[c].h, -p[c]);
-        e[c] = fmaf(d[c].h + d[c].h, d[c].l, e[c]);
-      }
-      const dflt s1 = df_two_sum(p[0], p[1]);
-      const dflt s2 = df_two_sum(s1.h, p[2]);
-      const float r2l = s1.l + s2.l + e[0] + e[1] + e[2];
-      const float r2h = s2.h;
-      // 1 / sqrt(r^2): hardware estimate y0, one Newton step
-      const float y0 = rsqrt_hw(r2h);
-      const float q = y0 * y0;
-      const float qe = fmaf(y0, y0, -q);
-      float t = fmaf(r2h, q, -1.0f);
-      t = fmaf(r2h, qe, t);
-      t = fmaf(r2l, q, t);
-      dflt inv = {y0, -0.5f * t * y0};
-      if (MASK && __float_as_int(yh.w) == pt[u]) inv = {0.0f, 0.0f};
-      const dflt rr = df_dot3(d[0], den[0], d[1], den[1], d[2], den[2]);
-      const dflt inv2 = df_mul(inv, inv);
-      const dflt inv3 = df_mul(inv2, inv);
-      if (KIND == 0) {
-        const dflt inv5 = df_mul(inv3, inv2);
-        const dflt rn = df_dot3(d[0], nt[u][0], d[1], nt[u][1], d[2], nt[u][2]);
-        const dflt cc = df_mul(df_mul(rn, rr), inv5);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) df_acc(acc[u][c], df_mul(cc, d[c]));
-      } else if (KIND == 2) {
-        const dflt inv5 = df_mul(inv3, inv2);
-        const dflt rn = df_dot3(d[0], nt[u][0], d[1], nt[u][1], d[2], nt[u][2]);
-        const dflt ck = df_mul(df_mul(rn, rr), inv5);
-        const dflt cs = df_mul(rr, inv3);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          df_acc(acc[u][c], df_mul(ck, d[c]));
-          df_acc(acc2[u][c], df_mul(den[c], inv));
-          df_acc(acc2[u][c], df_mul(cs, d[c]));
-        }
-      } else {
-        const dflt cc = df_mul(rr, inv3);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          df_acc(acc[u][c], df_mul(den[c], inv));
-          df_acc(acc[u][c], df_mul(cc, d[c]));
-        }
-      }
-    }
-  }
-}
-
 // Weighted density as double-float pairs for the double-float kernels: (w mu) rounded to float32 and
 // the rounded remainder.
 __global__ void k_weight_df(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
@@ -873,450 +799,379 @@ __global__ void k_weight_df(long long N, const double4* __restrict__ x, const do
 }
 
 
-// y += traction sum (KIND 0, 2) or Stokeslet sum (KIND 1); KIND 2 also y2 += Stokeslet sum.  No float64
-// arithmetic runs per pair or per staged source: positions come as exact three-float splits, the
-// weighted density and normals as double-float pairs, and tile sums are accumulated in double-float;
-// the total is converted to float64 once per target.
-template <int KIND, int NT>
-__global__ void __launch_bounds__(128 / NT, 8) k_pairs_df(int nitems, const longlong4* __restrict__ work,
-                                                       const float4* __restrict__ x3h, const float4* __restrict__ x3m,
-                                                       const float4* __restrict__ x3l, const float4* __restrict__ nh,
-                                                       const float4* __restrict__ nl, const float4* __restrict__ wh,
-                                                       const float4* __restrict__ wl, double* __restrict__ y,
-                                                       double* __restrict__ y2) {
-  constexpr int TS = 128, NTH = 128 / NT;
-  __shared__ float4 sph[TS], spl[TS], sdh[TS], sdl[TS];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-  const longlong4 w = work[it];
-  const float4 oh = x3h[w.x], om = x3m[w.x], ol = x3l[w.x];
-  dflt xt[NT][3], nt[NT][3];
-  int pt[NT];
-  bool valid[NT];
-#pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    const long long t = w.x + threadIdx.x + NTH * u;
-    valid[u] = t < w.y;
-    float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
-    pt[u] = -1;
-    if (valid[u]) {
-      ah = x3h[t];
-      am = x3m[t];
-      al = x3l[t];
-      bh = nh[t];
-      bl = nl[t];
-      pt[u] = __float_as_int(ah.w);
+// Direct double-float pair sums: y += traction sum (KIND 0, 2) or Stokeslet sum (KIND 1); KIND 2 also
+// y2 += Stokeslet sum.  A unit is 32 targets of a work item against its sources; warps take units from
+// a counter, stage their own source tiles and never wait for one another (df_tile, shared with the
+// treecode).  No float64 arithmetic runs but the final accumulation per target.
+template <int KIND>
+__global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restrict__ counter,
+                                                      const longlong4* __restrict__ work,
+                                                      const float4* __restrict__ x3h, const float4* __restrict__ x3m,
+                                                      const float4* __restrict__ x3l, const float4* __restrict__ nh,
+                                                      const float4* __restrict__ nl, const float4* __restrict__ wh,
+                                                      const float4* __restrict__ wl, double* __restrict__ y,
+                                                      double* __restrict__ y2) {
+  __shared__ __align__(16) float tiles[4 * kTileDfFloats];
+  float* const wsm = tiles + (threadIdx.x >> 5) * kTileDfFloats;
+  const int lane = threadIdx.x & 31;
+  while (true) {
+    int unit = 0;
+    if (lane == 0) unit = atomicAdd(counter, 1);
+    unit = __shfl_sync(0xffffffffu, unit, 0);
+    if (unit >= nunits) return;
+    const longlong4 w = work[unit >> 2];
+    const int t0 = (int)w.x + 32 * (unit & 3), t1 = (int)w.y;
+    if (t0 >= t1) continue;
+    const bool split = t1 - t0 <= 16;
+    const int half = split ? lane >> 4 : 0;
+    const int t = t0 + (split ? lane & 15 : lane);
+    const bool valid = t < t1;
+    const float4 oh = x3h[t0], om = x3m[t0], ol = x3l[t0];
+    dflt xt[3], nt[3], a[3], a2[3];
+    int pt = -1;
+    {
+      float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
+      if (valid) {
+        ah = x3h[t];
+        am = x3m[t];
+        al = x3l[t];
+        bh = nh[t];
+        bl = nl[t];
+        pt = __float_as_int(ah.w);
+      }
+      xt[0] = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x);
+      xt[1] = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y);
+      xt[2] = df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z);
+      nt[0] = {bh.x, bl.x};
+      nt[1] = {bh.y, bl.y};
+      nt[2] = {bh.z, bl.z};
     }
-    xt[u][0] = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x);
-    xt[u][1] = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y);
-    xt[u][2] = df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z);
-    nt[u][0] = {bh.x, bl.x};
-    nt[u][1] = {bh.y, bl.y};
-    nt[u][2] = {bh.z, bl.z};
-  }
-  const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(x3h[w.y - 1].w);
-  dflt a[NT][3], a2[NT][3];
+    const float xm = warp_max_abs(fmaxf(fabsf(xt[0].h), fmaxf(fabsf(xt[1].h), fabsf(xt[2].h))));
 #pragma unroll
-  for (int u = 0; u < NT; ++u)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a[u][c] = a2[u][c] = dflt{0.0f, 0.0f};
-  for (long long s0 = w.z; s0 < w.w; s0 += TS) {
-    const int cnt = (int)min((long long)TS, w.w - s0);
-    __syncthreads();
-    for (int l = threadIdx.x; l < cnt; l += NTH) {
-      const long long s = s0 + l;
-      const float4 ph = x3h[s], pm = x3m[s], pl = x3l[s];
-      const dflt px = df_diff3(ph.x, pm.x, pl.x, oh.x, om.x, ol.x);
-      const dflt py = df_diff3(ph.y, pm.y, pl.y, oh.y, om.y, ol.y);
-      const dflt pz = df_diff3(ph.z, pm.z, pl.z, oh.z, om.z, ol.z);
-      sph[l] = make_float4(px.h, py.h, pz.h, ph.w);
-      spl[l] = make_float4(px.l, py.l, pz.l, 0.0f);
-      sdh[l] = wh[s];
-      sdl[l] = wl[s];
+    for (int c = 0; c < 3; ++c) a[c] = a2[c] = dflt{0.0f, 0.0f};
+    const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(x3h[min(t0 + 32, t1) - 1].w);
+    for (int s0 = (int)w.z; s0 < (int)w.w; s0 += kTileDf) {
+      const int cnt = min(kTileDf, (int)w.w - s0);
+      const int sidx[2] = {s0 + lane, s0 + lane + 32};
+      const int tlo = __float_as_int(x3h[s0].w), thi = __float_as_int(x3h[s0 + cnt - 1].w);
+      df_tile<KIND>(wsm, sidx, cnt, !(thi < pid_lo || tlo > pid_hi), split, half, x3h, x3m, x3l, wh, wl, oh, om, ol, xt,
+                    nt, xm, pt, a, a2);
     }
-    __syncthreads();
-    const int tlo = __float_as_int(sph[0].w), thi = __float_as_int(sph[cnt - 1].w);
-    dflt acc[NT][3], acc2[NT][3];
-#pragma unroll
-    for (int u = 0; u < NT; ++u)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[u][c] = acc2[u][c] = dflt{0.0f, 0.0f};
-    if (thi < pid_lo || tlo > pid_hi)
-      pair_tile_df<KIND, false, NT>(sph, spl, sdh, sdl, cnt, xt, nt, pt, acc, acc2);
-    else
-      pair_tile_df<KIND, true, NT>(sph, spl, sdh, sdl, cnt, xt, nt, pt, acc, acc2);
-#pragma unroll
-    for (int u = 0; u < NT; ++u)
+    const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
+    if (valid) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        a[u][c] = df_add_accurate(a[u][c], acc[u][c]);
-        if (KIND == 2) a2[u][c] = df_add_accurate(a2[u][c], acc2[u][c]);
-      }
-  }
-  const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
-#pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    if (!valid[u]) continue;
-    const long long t = w.x + threadIdx.x + NTH * u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      atomicAdd(y + 3 * t + c, sc * ((double)a[u][c].h + (double)a[u][c].l));
-      if (KIND == 2) atomicAdd(y2 + 3 * t + c, kStokesletScale * ((double)a2[u][c].h + (double)a2[u][c].l));
-    }
-  }
-  }
-}
-
-// ------------------------------------------------------------------------------------------
-template <int KIND, int NT>
-__global__ void __launch_bounds__(128 / NT, NT == 1 ? 5 : 6) k_pairs_df2(int nitems, const longlong4* __restrict__ work,
-                                                        const float4* __restrict__ x3h, const float4* __restrict__ x3m,
-                                                        const float4* __restrict__ x3l, const float4* __restrict__ nh,
-                                                        const float4* __restrict__ nl, const float4* __restrict__ wh,
-                                                        const float4* __restrict__ wl, double* __restrict__ y,
-                                                        double* __restrict__ y2) {
-  constexpr int TS = 128, NTH = 128 / NT;
-  // structure of arrays: separation parts x, y, z (hi, lo), weighted density (hi, lo), particle id
-  __shared__ __align__(16) float sa[12][TS];
-  __shared__ __align__(16) int spid[TS];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-  const longlong4 w = work[it];
-  const float4 oh = x3h[w.x], om = x3m[w.x], ol = x3l[w.x];
-  df2 xt[NT][3], nt[NT][3];
-  int pt[NT];
-  bool valid[NT];
-#pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    const long long t = w.x + threadIdx.x + NTH * u;
-    valid[u] = t < w.y;
-    float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
-    pt[u] = -1;
-    if (valid[u]) {
-      ah = x3h[t];
-      am = x3m[t];
-      al = x3l[t];
-      bh = nh[t];
-      bl = nl[t];
-      pt[u] = __float_as_int(ah.w);
-    }
-    const dflt dx = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x), dy = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y),
-               dz = df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z);
-    xt[u][0] = {dup2(dx.h), dup2(dx.l)};
-    xt[u][1] = {dup2(dy.h), dup2(dy.l)};
-    xt[u][2] = {dup2(dz.h), dup2(dz.l)};
-    nt[u][0] = {dup2(bh.x), dup2(bl.x)};
-    nt[u][1] = {dup2(bh.y), dup2(bl.y)};
-    nt[u][2] = {dup2(bh.z), dup2(bl.z)};
-  }
-  const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(x3h[w.y - 1].w);
-  dflt a[NT][3], a2[NT][3];
-#pragma unroll
-  for (int u = 0; u < NT; ++u)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a[u][c] = a2[u][c] = dflt{0.0f, 0.0f};
-  for (long long s0 = w.z; s0 < w.w; s0 += TS) {
-    const int cnt = (int)min((long long)TS, w.w - s0);
-    const int cnt2 = (cnt + 1) & ~1;
-    __syncthreads();
-    for (int l = threadIdx.x; l < cnt2; l += NTH) {
-      if (l < cnt) {
-        const long long s = s0 + l;
-        const float4 ph = x3h[s], pm = x3m[s], pl = x3l[s], qh = wh[s], ql = wl[s];
-        const dflt px = df_diff3(ph.x, pm.x, pl.x, oh.x, om.x, ol.x);
-        const dflt py = df_diff3(ph.y, pm.y, pl.y, oh.y, om.y, ol.y);
-        const dflt pz = df_diff3(ph.z, pm.z, pl.z, oh.z, om.z, ol.z);
-        sa[0][l] = px.h;
-        sa[1][l] = px.l;
-        sa[2][l] = py.h;
-        sa[3][l] = py.l;
-        sa[4][l] = pz.h;
-        sa[5][l] = pz.l;
-        sa[6][l] = qh.x;
-        sa[7][l] = ql.x;
-        sa[8][l] = qh.y;
-        sa[9][l] = ql.y;
-        sa[10][l] = qh.z;
-        sa[11][l] = ql.z;
-        spid[l] = __float_as_int(ph.w);
-      } else {
-        sa[0][l] = sa[2][l] = sa[4][l] = 1.0e4f;
-        sa[1][l] = sa[3][l] = sa[5][l] = 0.0f;
-        for (int q = 6; q < 12; ++q) sa[q][l] = 0.0f;
-        spid[l] = -2;
+        atomicAdd(y + 3 * (long long)t + c, sc * ((double)a[c].h + (double)a[c].l));
+        if (KIND == 2) atomicAdd(y2 + 3 * (long long)t + c, kStokesletScale * ((double)a2[c].h + (double)a2[c].l));
       }
     }
-    __syncthreads();
-    const int tlo = spid[0], thi = spid[cnt - 1];
-    const bool masked = !(thi < pid_lo || tlo > pid_hi);
-    df2 acc[NT][3], acc2[NT][3];
-#pragma unroll
-    for (int u = 0; u < NT; ++u)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[u][c] = acc2[u][c] = df2{dup2(0.0f), dup2(0.0f)};
-    for (int l = 0; l < cnt2; l += 2) {
-      df2 ys[3], den[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        ys[c] = {*reinterpret_cast<const float2*>(&sa[2 * c][l]), *reinterpret_cast<const float2*>(&sa[2 * c + 1][l])};
-        den[c] = {*reinterpret_cast<const float2*>(&sa[6 + 2 * c][l]),
-                  *reinterpret_cast<const float2*>(&sa[7 + 2 * c][l])};
-      }
-      const int2 pp = *reinterpret_cast<const int2*>(&spid[l]);
-#pragma unroll
-      for (int u = 0; u < NT; ++u) {
-        if (masked)
-          pair2_df<KIND, true>(ys, den, pp, xt[u], nt[u], pt[u], acc[u], acc2[u]);
-        else
-          pair2_df<KIND, false>(ys, den, pp, xt[u], nt[u], pt[u], acc[u], acc2[u]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < NT; ++u)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        a[u][c] = df_add_accurate(a[u][c], fold2(acc[u][c]));
-        if (KIND == 2) a2[u][c] = df_add_accurate(a2[u][c], fold2(acc2[u][c]));
-      }
-  }
-  const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
-#pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    if (!valid[u]) continue;
-    const long long t = w.x + threadIdx.x + NTH * u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      atomicAdd(y + 3 * t + c, sc * ((double)a[u][c].h + (double)a[u][c].l));
-      if (KIND == 2) atomicAdd(y2 + 3 * t + c, kStokesletScale * ((double)a2[u][c].h + (double)a2[u][c].l));
-    }
-  }
   }
 }
 
 // ------------------------------------------------------------------------------------------
 // Upsampled densities of the near-source particles: mu_up = U mu_j with U stored transposed
 // (N_p x N_up), one thread per upsampled node reading U coalesced and mu_j from shared memory; the
-// arithmetic is that of U's storage type (float32 for the inner solve, float64 otherwise).
-template <typename TU>
+// arithmetic is that of U's storage type (float32 for the inner solve, float64 otherwise).  The near
+// sums take them weighted: FORM 0 w mu as float64 (qd), 1 as float32 (qh), 2 as float32 pairs (qh, ql).
+template <typename TU, int FORM>
 __global__ void __launch_bounds__(128) k_upsample(int n_up, const int* __restrict__ up_particle,
                                                   const long long* __restrict__ up_off,
                                                   const long long* __restrict__ offset, const int* __restrict__ nodes,
                                                   const TU* const* __restrict__ Umats, const double* __restrict__ dens,
-                                                  double* __restrict__ upmu) {
+                                                  const double4* __restrict__ upx, double4* __restrict__ qd,
+                                                  float4* __restrict__ qh, float4* __restrict__ ql) {
   extern __shared__ double mus_raw[];  // 3 N_p values of type TU
   TU* mus = reinterpret_cast<TU*>(mus_raw);
   for (int u = blockIdx.y; u < n_up; u += gridDim.y) {
     const int j = up_particle[u];
     const int np = nodes[j];
     const long long o = offset[j];
+    const long long base = up_off[u];
+    const int nup = (int)(up_off[u + 1] - base);
+    if ((int)(blockIdx.x * blockDim.x) >= nup) continue;
     __syncthreads();
     for (int l = threadIdx.x; l < 3 * np; l += blockDim.x) mus[l] = (TU)dens[3 * o + l];
     __syncthreads();
-    const long long base = up_off[u];
-    const int nup = (int)(up_off[u + 1] - base);
     const TU* Ut = Umats[u];
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nup; r += gridDim.x * blockDim.x) {
       TU a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll 8
       for (int s = 0; s < np; ++s) {
-        const TU uv = Ut[(long long)s * nup + r];
+        const TU uv = __ldg(Ut + (long long)s * nup + r);
         a0 = fma_t(uv, mus[3 * s], a0);
         a1 = fma_t(uv, mus[3 * s + 1], a1);
         a2 = fma_t(uv, mus[3 * s + 2], a2);
       }
-      upmu[3 * (base + r) + 0] = (double)a0;
-      upmu[3 * (base + r) + 1] = (double)a1;
-      upmu[3 * (base + r) + 2] = (double)a2;
+      const double w = upx[base + r].w;
+      const double q0 = w * (double)a0, q1 = w * (double)a1, q2 = w * (double)a2;
+      if (FORM == 0) qd[base + r] = make_double4(q0, q1, q2, 0.0);
+      if (FORM == 1) qh[base + r] = make_float4((float)q0, (float)q1, (float)q2, 0.0f);
+      if (FORM == 2) {
+        const dflt d0 = df_split(q0), d1 = df_split(q1), d2 = df_split(q2);
+        qh[base + r] = make_float4(d0.h, d1.h, d2.h, 0.0f);
+        ql[base + r] = make_float4(d0.l, d1.l, d2.l, 0.0f);
+      }
     }
   }
 }
 
-// Near correction for one near pair (target particle i, source particle j): add the contribution
-// of j's upsampled nodes and subtract that of j's base nodes (already in the smooth sum).  T is the
-// arithmetic type; coordinates are relative to the target particle's centre.
-template <int KIND, typename T>
-__global__ void __launch_bounds__(256) k_near(const int2* __restrict__ near, const long long* __restrict__ offset,
-                                              const int* __restrict__ nodes, const double* __restrict__ centre,
-                                              const int* __restrict__ up_index, const long long* __restrict__ up_off,
-                                              const double4* __restrict__ x, const double4* __restrict__ nrm,
-                                              const double* __restrict__ dens, const double4* __restrict__ upx,
-                                              const double* __restrict__ upmu, double* __restrict__ y) {
-  constexpr int TS = 256;
-  __shared__ T sx[TS][3];
-  __shared__ T sd[TS][3];
-  const int2 pr = near[blockIdx.x];
-  const int i = pr.x, j = pr.y;
-  const double cx = centre[3 * i], cy = centre[3 * i + 1], cz = centre[3 * i + 2];
-  const long long oi = offset[i], oj = offset[j];
-  const int npi = nodes[i], npj = nodes[j];
-  const int u = up_index[j];
-  const long long ub = up_off[u];
-  const int nup = (int)(up_off[u + 1] - ub);
-  const int total = nup + npj;
-  for (int tb = 0; tb < npi; tb += blockDim.x) {
-    const int tl = tb + threadIdx.x;
-    const bool valid = tl < npi;
-    T xx = 0, xy = 0, xz = 0, nx = 0, ny = 0, nz = 0;
-    if (valid) {
-      double4 xt = x[oi + tl], nt = nrm[oi + tl];
-      xx = (T)(xt.x - cx);
-      xy = (T)(xt.y - cy);
-      xz = (T)(xt.z - cz);
-      nx = (T)nt.x;
-      ny = (T)nt.y;
-      nz = (T)nt.z;
+// Near correction.  For a near pair (target particle i, source particle j) the contribution of j's
+// upsampled nodes is added and that of its base nodes (already in the smooth sum) removed.  A unit is
+// (pair, 32 targets of i, one of `parts` equal runs of the N_up + N_j sources), taken by warps from a
+// counter; parts grows until small near lists fill the GPU.  A pair of 144-node particles is 688 sources
+// against five units of targets, so one block per pair left most of the SMs idle on lists of a few hundred
+// pairs and most of its threads idle where orders mix.
+struct NearArgs {
+  int nunits, chunks, parts;
+  int* counter;
+  const int2* near;
+  const long long* offset;
+  const int* nodes;
+  const int* up_index;
+  const long long* up_off;
+};
+struct NearUnit {
+  int t0, t1;           // targets [t0, t1) of particle i that the unit holds, 32 at most (t0 >= t1: none)
+  long long ub, oj;     // first upsampled node and first base node of j
+  int s0, s1, nup;      // sources [s0, s1): below nup upsampled nodes, then base nodes
+};
+__device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
+  int unit = 0;
+  if ((threadIdx.x & 31) == 0) unit = atomicAdd(A.counter, 1);
+  unit = __shfl_sync(0xffffffffu, unit, 0);
+  if (unit >= A.nunits) return false;
+  const int part = unit % A.parts, q = unit / A.parts;
+  const int chunk = q % A.chunks;
+  const int2 pr = A.near[q / A.chunks];
+  const long long oi = A.offset[pr.x];
+  n.t0 = (int)oi + 32 * chunk;
+  n.t1 = min(n.t0 + 32, (int)oi + A.nodes[pr.x]);
+  const int u = A.up_index[pr.y];
+  n.ub = A.up_off[u];
+  n.nup = (int)(A.up_off[u + 1] - n.ub);
+  n.oj = A.offset[pr.y];
+  const int total = n.nup + A.nodes[pr.y];
+  const int step = ((total + A.parts - 1) / A.parts + 3) & ~3;
+  n.s0 = min(total, part * step);
+  n.s1 = min(total, n.s0 + step);
+  return true;
+}
+
+// Float32: the packed tile loop of the smooth sum over per-warp tiles of 128 sources.
+template <int KIND>
+__global__ void __launch_bounds__(128, 6) k_near32(NearArgs A, const float4* __restrict__ xhi,
+                                                   const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
+                                                   const float4* __restrict__ wmu, const float4* __restrict__ uphi,
+                                                   const float4* __restrict__ uplo, const float4* __restrict__ upq,
+                                                   double* __restrict__ y) {
+  constexpr int TW = 128;
+  __shared__ __align__(16) float tiles[4][6 * TW];
+  const int lane = threadIdx.x & 31;
+  float* const ssx = tiles[threadIdx.x >> 5];
+  NearUnit n;
+  while (next_near_unit(A, n)) {
+    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    const bool split = n.t1 - n.t0 <= 16;
+    const int half = split ? lane >> 4 : 0;
+    const int t = n.t0 + (split ? lane & 15 : lane);
+    const bool valid = t < n.t1;
+    const float4 oh = xhi[n.t0], ol = xlo[n.t0];
+    float2 xt[1][3], nt[1][3];
+    const int none[1] = {-1};
+    {
+      const float4 ah = valid ? xhi[t] : oh, al = valid ? xlo[t] : ol;
+      const float4 nn = valid ? nrm32[t] : make_float4(0, 0, 0, 0);
+      const float a0 = (ah.x - oh.x) + (al.x - ol.x), a1 = (ah.y - oh.y) + (al.y - ol.y),
+                  a2 = (ah.z - oh.z) + (al.z - ol.z);
+      xt[0][0] = f2(a0, a0);
+      xt[0][1] = f2(a1, a1);
+      xt[0][2] = f2(a2, a2);
+      nt[0][0] = f2(nn.x, nn.x);
+      nt[0][1] = f2(nn.y, nn.y);
+      nt[0][2] = f2(nn.z, nn.z);
     }
-    T a0 = 0, a1 = 0, a2 = 0;
-    for (int s0 = 0; s0 < total; s0 += TS) {
-      const int cnt = min(TS, total - s0);
-      __syncthreads();
-      for (int l = threadIdx.x; l < cnt; l += blockDim.x) {
-        const int s = s0 + l;
-        double4 ps;
-        double d0, d1, d2, wgt;
-        if (s < nup) {
-          ps = upx[ub + s];
-          wgt = ps.w;
-          d0 = upmu[3 * (ub + s)];
-          d1 = upmu[3 * (ub + s) + 1];
-          d2 = upmu[3 * (ub + s) + 2];
-        } else {
-          ps = x[oj + (s - nup)];
-          wgt = -ps.w;
-          const double* d = dens + 3 * (oj + (s - nup));
-          d0 = d[0];
-          d1 = d[1];
-          d2 = d[2];
-        }
-        sx[l][0] = (T)(ps.x - cx);
-        sx[l][1] = (T)(ps.y - cy);
-        sx[l][2] = (T)(ps.z - cz);
-        sd[l][0] = (T)(wgt * d0);
-        sd[l][1] = (T)(wgt * d1);
-        sd[l][2] = (T)(wgt * d2);
-      }
-      __syncthreads();
-      for (int l = 0; l < cnt; ++l) {
-        const T dx = xx - sx[l][0], dy = xy - sx[l][1], dz = xz - sx[l][2];
-        const T r2 = dx * dx + dy * dy + dz * dz;
-        const T inv = rsq(r2);
-        const T rr = dx * sd[l][0] + dy * sd[l][1] + dz * sd[l][2];
-        if (KIND == 0) {
-          const T inv2 = inv * inv;
-          const T rn = dx * nx + dy * ny + dz * nz;
-          const T c = rn * rr * (inv2 * inv2 * inv);
-          a0 += c * dx;
-          a1 += c * dy;
-          a2 += c * dz;
-        } else {
-          const T c = rr * (inv * inv * inv);
-          a0 += sd[l][0] * inv + c * dx;
-          a1 += sd[l][1] * inv + c * dy;
-          a2 += sd[l][2] * inv + c * dz;
+    float sa[3] = {0, 0, 0}, ea[3] = {0, 0, 0};
+    for (int sb = n.s0; sb < n.s1; sb += TW) {
+      const int cnt = min(TW, n.s1 - sb), cnt8 = (cnt + 7) & ~7;
+      __syncwarp();  // the warp's reads of the previous tile are done
+#pragma unroll
+      for (int l = lane; l < TW; l += 32) {
+        if (l < cnt) {
+          const int s = sb + l;
+          float4 ph, pl, q;
+          if (s < n.nup) {
+            ph = uphi[n.ub + s];
+            pl = uplo[n.ub + s];
+            q = upq[n.ub + s];
+          } else {
+            const long long g = n.oj + (s - n.nup);
+            ph = xhi[g];
+            pl = xlo[g];
+            q = wmu[g];
+            q = make_float4(-q.x, -q.y, -q.z, 0.0f);
+          }
+          ssx[l] = (oh.x - ph.x) + (ol.x - pl.x);
+          ssx[TW + l] = (oh.y - ph.y) + (ol.y - pl.y);
+          ssx[2 * TW + l] = (oh.z - ph.z) + (ol.z - pl.z);
+          ssx[3 * TW + l] = q.x;
+          ssx[4 * TW + l] = q.y;
+          ssx[5 * TW + l] = q.z;
+        } else if (l < cnt8) {
+          ssx[l] = ssx[TW + l] = ssx[2 * TW + l] = 1.0e4f;
+          ssx[3 * TW + l] = ssx[4 * TW + l] = ssx[5 * TW + l] = 0.0f;
         }
       }
+      __syncwarp();
+      float2 p[1][3];
+      p[0][0] = p[0][1] = p[0][2] = f2(0.0f, 0.0f);
+      const int m = split ? cnt8 / 2 : cnt8, l0 = half * m;
+      pair_tile32x2<KIND, false, 1>(ssx + l0, ssx + TW + l0, ssx + 2 * TW + l0, ssx + 3 * TW + l0, ssx + 4 * TW + l0,
+                                    ssx + 5 * TW + l0, nullptr, m, xt, nt, none, p);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) two_sum_acc(sa[c], ea[c], p[0][c].x + p[0][c].y);
     }
     if (valid) {
       const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
-      atomicAdd(y + 3 * (oi + tl) + 0, sc * (double)a0);
-      atomicAdd(y + 3 * (oi + tl) + 1, sc * (double)a1);
-      atomicAdd(y + 3 * (oi + tl) + 2, sc * (double)a2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * (long long)t + c, sc * ((double)sa[c] + (double)ea[c]));
     }
   }
 }
 
-// Near correction in float32 or double-float, sharing the tile loops of the smooth sums.  One
-// block per near pair; the block size covers the largest target particle in one or two passes;
-// sources (upsampled nodes of j with +w, base nodes of j with -w) are staged relative to the target
-// particle's centre.  Tile partials are added in float64.
-template <int KIND, bool DF>
-__global__ void __launch_bounds__(512) k_near_tiled(const int2* __restrict__ near, const long long* __restrict__ offset,
-                                                    const int* __restrict__ nodes, const double* __restrict__ centre,
-                                                    const int* __restrict__ up_index, const long long* __restrict__ up_off,
-                                                    const double4* __restrict__ x, const double4* __restrict__ nrm,
-                                                    const double* __restrict__ dens, const double4* __restrict__ upx,
-                                                    const double* __restrict__ upmu, double* __restrict__ y) {
-  constexpr int TS = 256;
-  __shared__ float4 s0[TS], s1[TS], s2[DF ? TS : 1], s3[DF ? TS : 1];
-  const int2 pr = near[blockIdx.x];
-  const int i = pr.x, j = pr.y;
-  const double ox = centre[3 * i], oy = centre[3 * i + 1], oz = centre[3 * i + 2];
-  const long long oi = offset[i], oj = offset[j];
-  const int npi = nodes[i], npj = nodes[j];
-  const int u = up_index[j];
-  const long long ub = up_off[u];
-  const int nup = (int)(up_off[u + 1] - ub);
-  const int total = nup + npj;
-  for (int tb = 0; tb < npi; tb += blockDim.x) {
-    const int tl = tb + threadIdx.x;
-    const bool valid = tl < npi;
-    double4 xt = make_double4(0, 0, 0, 0), nt = make_double4(0, 0, 0, 0);
-    if (valid) {
-      xt = x[oi + tl];
-      nt = nrm[oi + tl];
+// Double-float: the arithmetic of the smooth sums (df_tile), so that what is removed is what they added;
+// KIND 2 both kernels in one pass.
+template <int KIND>
+__global__ void __launch_bounds__(128, 4) k_near_df(NearArgs A, const float4* __restrict__ x3h,
+                                                    const float4* __restrict__ x3m, const float4* __restrict__ x3l,
+                                                    const float4* __restrict__ nh, const float4* __restrict__ nl,
+                                                    const float4* __restrict__ wh, const float4* __restrict__ wl,
+                                                    const float4* __restrict__ up3h, const float4* __restrict__ up3m,
+                                                    const float4* __restrict__ up3l, const float4* __restrict__ upqh,
+                                                    const float4* __restrict__ upql, double* __restrict__ y,
+                                                    double* __restrict__ y2) {
+  __shared__ __align__(16) float tiles[4 * kTileDfFloats];
+  float* const wsm = tiles + (threadIdx.x >> 5) * kTileDfFloats;
+  const int lane = threadIdx.x & 31;
+  NearUnit n;
+  while (next_near_unit(A, n)) {
+    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    const bool split = n.t1 - n.t0 <= 16;
+    const int half = split ? lane >> 4 : 0;
+    const int t = n.t0 + (split ? lane & 15 : lane);
+    const bool valid = t < n.t1;
+    const float4 oh = x3h[n.t0], om = x3m[n.t0], ol = x3l[n.t0];
+    dflt xt[3], nt[3], a[3], a2[3];
+    {
+      const float4 zero = make_float4(0, 0, 0, 0);
+      const float4 ah = valid ? x3h[t] : oh, am = valid ? x3m[t] : om, al = valid ? x3l[t] : ol;
+      const float4 bh = valid ? nh[t] : zero, bl = valid ? nl[t] : zero;
+      xt[0] = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x);
+      xt[1] = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y);
+      xt[2] = df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z);
+      nt[0] = {bh.x, bl.x};
+      nt[1] = {bh.y, bl.y};
+      nt[2] = {bh.z, bl.z};
     }
+    const float xm = warp_max_abs(fmaxf(fabsf(xt[0].h), fmaxf(fabsf(xt[1].h), fabsf(xt[2].h))));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c] = a2[c] = dflt{0.0f, 0.0f};
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {  // upsampled nodes, then base nodes with the opposite sign
+      const int b = pass == 0 ? n.s0 : max(n.s0, n.nup), e = pass == 0 ? min(n.s1, n.nup) : n.s1;
+      const long long g0 = pass == 0 ? n.ub : n.oj - n.nup;
+      for (int sb = b; sb < e; sb += kTileDf) {
+        const int sidx[2] = {(int)(g0 + sb) + lane, (int)(g0 + sb) + lane + 32};
+        df_tile<KIND>(wsm, sidx, min(kTileDf, e - sb), false, split, half, pass == 0 ? up3h : x3h,
+                      pass == 0 ? up3m : x3m, pass == 0 ? up3l : x3l, pass == 0 ? upqh : wh, pass == 0 ? upql : wl, oh,
+                      om, ol, xt, nt, xm, -1, a, a2, pass == 0 ? 1.0f : -1.0f);
+      }
+    }
+    if (valid) {
+      const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        atomicAdd(y + 3 * (long long)t + c, sc * ((double)a[c].h + (double)a[c].l));
+        if (KIND == 2) atomicAdd(y2 + 3 * (long long)t + c, kStokesletScale * ((double)a2[c].h + (double)a2[c].l));
+      }
+    }
+  }
+}
+
+// Float64: per-warp tiles of 32 sources; coordinates relative to the target particle's centre cancel in the
+// differences, so lab coordinates are used as they are.
+template <int KIND>
+__global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __restrict__ x,
+                                                const double4* __restrict__ nrm, const double* __restrict__ dens,
+                                                const double4* __restrict__ upx, const double4* __restrict__ upq,
+                                                double* __restrict__ y) {
+  __shared__ double4 sp[4][32], sq[4][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  NearUnit n;
+  while (next_near_unit(A, n)) {
+    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    const int t = n.t0 + lane;
+    const bool valid = t < n.t1;
+    const double4 xt = x[valid ? t : n.t0], nt = nrm[valid ? t : n.t0];
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int sb = 0; sb < total; sb += TS) {
-      const int cnt = min(TS, total - sb);
-      __syncthreads();
-      for (int l = threadIdx.x; l < cnt; l += blockDim.x) {
-        const int s = sb + l;
-        double4 ps;
-        double d0, d1, d2, wgt;
-        if (s < nup) {
-          ps = upx[ub + s];
-          wgt = ps.w;
-          d0 = upmu[3 * (ub + s)];
-          d1 = upmu[3 * (ub + s) + 1];
-          d2 = upmu[3 * (ub + s) + 2];
+    for (int sb = n.s0; sb < n.s1; sb += 32) {
+      const int cnt = min(32, n.s1 - sb);
+      __syncwarp();
+      if (lane < cnt) {
+        const int s = sb + lane;
+        if (s < n.nup) {
+          sp[warp][lane] = upx[n.ub + s];
+          sq[warp][lane] = upq[n.ub + s];
         } else {
-          ps = x[oj + (s - nup)];
-          wgt = -ps.w;
-          const double* d = dens + 3 * (oj + (s - nup));
-          d0 = d[0];
-          d1 = d[1];
-          d2 = d[2];
-        }
-        if (DF) {
-          const dflt px = df_split(ps.x - ox), py = df_split(ps.y - oy), pz = df_split(ps.z - oz);
-          const dflt q0 = df_split(wgt * d0), q1 = df_split(wgt * d1), q2 = df_split(wgt * d2);
-          s0[l] = make_float4(px.h, py.h, pz.h, 0.0f);
-          s1[l] = make_float4(px.l, py.l, pz.l, 0.0f);
-          s2[l] = make_float4(q0.h, q1.h, q2.h, 0.0f);
-          s3[l] = make_float4(q0.l, q1.l, q2.l, 0.0f);
-        } else {
-          s0[l] = make_float4((float)(ps.x - ox), (float)(ps.y - oy), (float)(ps.z - oz), 0.0f);
-          s1[l] = make_float4((float)(wgt * d0), (float)(wgt * d1), (float)(wgt * d2), 0.0f);
+          const long long g = n.oj + (s - n.nup);
+          const double4 p = x[g];
+          sp[warp][lane] = p;
+          sq[warp][lane] = make_double4(-p.w * dens[3 * g], -p.w * dens[3 * g + 1], -p.w * dens[3 * g + 2], 0.0);
         }
       }
-      __syncthreads();
-      if (DF) {
-        const dflt xd[1][3] = {{df_split(xt.x - ox), df_split(xt.y - oy), df_split(xt.z - oz)}};
-        const dflt nd[1][3] = {{df_split(nt.x), df_split(nt.y), df_split(nt.z)}};
-        const int none[1] = {-1};
-        dflt acc[1][3] = {{{0, 0}, {0, 0}, {0, 0}}};
-        pair_tile_df<KIND, false, 1>(s0, s1, s2, s3, cnt, xd, nd, none, acc, acc);
-        a0 += (double)acc[0][0].h + (double)acc[0][0].l;
-        a1 += (double)acc[0][1].h + (double)acc[0][1].l;
-        a2 += (double)acc[0][2].h + (double)acc[0][2].l;
-      } else {
-        const float xf[1][3] = {{(float)(xt.x - ox), (float)(xt.y - oy), (float)(xt.z - oz)}};
-        const float nf[1][3] = {{(float)nt.x, (float)nt.y, (float)nt.z}};
-        const int none[1] = {-1};
-        float p[1][3] = {{0, 0, 0}};
-        pair_tile32<KIND, false, 1>(s0, s1, cnt, xf, nf, none, p);
-        a0 += p[0][0];
-        a1 += p[0][1];
-        a2 += p[0][2];
+      __syncwarp();
+#pragma unroll 4
+      for (int l = 0; l < cnt; ++l) {
+        const double4 ps = sp[warp][l], q = sq[warp][l];
+        const double dx = xt.x - ps.x, dy = xt.y - ps.y, dz = xt.z - ps.z;
+        const double inv = rsq(dx * dx + dy * dy + dz * dz);
+        const double rr = dx * q.x + dy * q.y + dz * q.z;
+        if (KIND == 0) {
+          const double inv2 = inv * inv;
+          const double rn = dx * nt.x + dy * nt.y + dz * nt.z;
+          const double c = rn * rr * (inv2 * inv2 * inv);
+          a0 = fma(c, dx, a0);
+          a1 = fma(c, dy, a1);
+          a2 = fma(c, dz, a2);
+        } else {
+          const double c = rr * (inv * inv * inv);
+          a0 = fma(c, dx, fma(q.x, inv, a0));
+          a1 = fma(c, dy, fma(q.y, inv, a1));
+          a2 = fma(c, dz, fma(q.z, inv, a2));
+        }
       }
     }
     if (valid) {
       const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
-      atomicAdd(y + 3 * (oi + tl) + 0, sc * a0);
-      atomicAdd(y + 3 * (oi + tl) + 1, sc * a1);
-      atomicAdd(y + 3 * (oi + tl) + 2, sc * a2);
+      atomicAdd(y + 3 * (long long)t + 0, sc * a0);
+      atomicAdd(y + 3 * (long long)t + 1, sc * a1);
+      atomicAdd(y + 3 * (long long)t + 2, sc * a2);
     }
   }
 }
 
 }  // namespace
+
+// Weighted densities of the float32 and double-float pair sums.
+static Status weight_f32(Context& c, const double* x) {
+  k_weight_f32<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmu32.ptr);
+  RBS_CUDA_TRY(cudaGetLastError());
+  return Status::Ok();
+}
+static Status weight_df(Context& c, const double* x) {
+  k_weight_df<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmuh.ptr, c.d_wmul.ptr);
+  RBS_CUDA_TRY(cudaGetLastError());
+  return Status::Ok();
+}
 
 // Blocks of `kernel` that fit on the GPU at once (occupancy x SMs), capped at the item count: the
 // pair kernels loop over their work items with this persistent grid, so the last wave is not a
@@ -1340,20 +1195,11 @@ template <int KIND>
 static void launch_pairs_kind(Context& c, int prec, int nt, int items, const double* x, double* y, double* y2) {
 #define RBS_PAIR_ARGS items, c.d_work.ptr, c.d_x.ptr, c.d_nrm.ptr, c.d_pid.ptr, x, y
   if (prec == RBS_PREC_DF) {
-#define RBS_DF_ARGS items, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, \
-                    c.d_wmuh.ptr, c.d_wmul.ptr, y, y2
-    k_weight_df<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmuh.ptr, c.d_wmul.ptr);
-    if (nt == 1)
-      k_pairs_df<KIND, 1><<<resident_grid(c, (const void*)k_pairs_df<KIND, 1>, 128, items), 128, 0, c.stream>>>(RBS_DF_ARGS);
-    else if (nt == 2)
-      k_pairs_df<KIND, 2><<<resident_grid(c, (const void*)k_pairs_df<KIND, 2>, 64, items), 64, 0, c.stream>>>(RBS_DF_ARGS);
-    else if (nt == 4)
-      k_pairs_df<KIND, 4><<<resident_grid(c, (const void*)k_pairs_df<KIND, 4>, 32, items), 32, 0, c.stream>>>(RBS_DF_ARGS);
-    else if (nt == kPacked + 1)
-      k_pairs_df2<KIND, 1><<<resident_grid(c, (const void*)k_pairs_df2<KIND, 1>, 128, items), 128, 0, c.stream>>>(RBS_DF_ARGS);
-    else
-      k_pairs_df2<KIND, 2><<<resident_grid(c, (const void*)k_pairs_df2<KIND, 2>, 64, items), 64, 0, c.stream>>>(RBS_DF_ARGS);
-#undef RBS_DF_ARGS
+    cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream);
+    const int units = 4 * items;
+    k_pairs_df2<KIND><<<resident_grid(c, (const void*)k_pairs_df2<KIND>, 128, items), 128, 0, c.stream>>>(
+        units, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
+        c.d_wmuh.ptr, c.d_wmul.ptr, y, y2);
   } else if constexpr (KIND == 2) {
     return;
   } else if (prec == RBS_PREC_FP64) {
@@ -1367,7 +1213,6 @@ static void launch_pairs_kind(Context& c, int prec, int nt, int items, const dou
       k_pairs32<KIND, 4><<<resident_grid(c, (const void*)k_pairs32<KIND, 4>, 32, items), 32, 0, c.stream>>>(RBS_PAIR_ARGS);
     else {
 #define RBS_PACKED_ARGS items, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y
-      k_weight_f32<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmu32.ptr);
       if (nt == kPacked + 1)
         k_pairs32x2<KIND, 1><<<resident_grid(c, (const void*)k_pairs32x2<KIND, 1>, 128, items), 128, 0, c.stream>>>(RBS_PACKED_ARGS);
       else if (nt == kPacked + 2)
@@ -1397,9 +1242,9 @@ static Status launch_pairs(Context& c, int kind, int prec, int nt, int items, co
 // the double-float kernels), otherwise the fastest candidate timed once per (kernel, arithmetic) on a
 // prefix of the work list (the same items for every variant, into a scratch output).
 static int pair_variant(Context& c, int kind, int prec, const double* x) {
-  if (c.opt.pair_variant > 0)
-    return (prec == RBS_PREC_DF && c.opt.pair_variant == kPacked + 4) ? 4 : c.opt.pair_variant;
-  const int key = kind == 2 ? 4 : 2 * (prec == RBS_PREC_DF ? 1 : 0) + kind;
+  if (prec == RBS_PREC_DF) return kPacked + 1;
+  if (c.opt.pair_variant > 0) return c.opt.pair_variant;
+  const int key = kind;
   if (c.tuned[key]) return c.tuned[key];
   int best = 2;
   const int items = std::min<int>((int)c.work.size(), 2 * 32 * std::max(1, c.sm_count));
@@ -1408,10 +1253,7 @@ static int pair_variant(Context& c, int kind, int prec, const double* x) {
   if (cudaMalloc(&scratch, sizeof(double) * 6 * c.N) == cudaSuccess && cudaEventCreate(&a) == cudaSuccess &&
       cudaEventCreate(&b) == cudaSuccess) {
     float best_ms = 1e30f;
-    std::vector<int> cands = {1, 2, 4};
-    if (prec_f32(prec)) cands.insert(cands.end(), {kPacked + 1, kPacked + 2, kPacked + 4});
-    if (prec == RBS_PREC_DF) cands.insert(cands.end(), {kPacked + 1, kPacked + 2});
-    for (int nt : cands) {
+    for (int nt : {1, 2, 4, kPacked + 1, kPacked + 2, kPacked + 4}) {
       launch_pairs(c, kind, prec, nt, items, x, scratch, scratch + 3 * c.N);  // warm (first launch of this variant)
       cudaEventRecord(a, c.stream);
       launch_pairs(c, kind, prec, nt, items, x, scratch, scratch + 3 * c.N);
@@ -1517,52 +1359,84 @@ Status apply_blocks(Context& c, int mode, int prec, const double* x, double* y, 
   return Status::Ok();
 }
 
-// Near correction, step 1: upsampled densities of the near-source particles (float32 interpolation
-// for the inner solve, float64 otherwise).
-static Status near_upsample(Context& c, bool f32, const double* x) {
-  size_t smem = sizeof(double) * 3 * (size_t)c.max_np;
-  if (smem > 48 * 1024) {
-    RBS_CUDA_TRY(cudaFuncSetAttribute(k_upsample<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    RBS_CUDA_TRY(cudaFuncSetAttribute(k_upsample<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  }
+// Near correction, step 1: upsampled weighted densities of the near-source particles (float32
+// interpolation for the inner solve, float64 otherwise), in the form the sums of arithmetic prec read.
+static Status near_upsample(Context& c, int prec, const double* x) {
+  const bool f32 = prec_f32(prec);
+  const size_t smem = (f32 ? sizeof(float) : sizeof(double)) * 3 * (size_t)c.max_np;
   int maxup = 0;
   for (Grid* g : c.grids) maxup = std::max(maxup, g->nup);
   const int nup_p = (int)c.up_particle.size();
   dim3 gu(cdiv(maxup, 128), (unsigned)std::min(nup_p, 65535));
+#define RBS_UPSAMPLE(TU, FORM, U)                                                                                       \
+  do {                                                                                                                  \
+    if (smem > 48 * 1024)                                                                                               \
+      RBS_CUDA_TRY(cudaFuncSetAttribute(k_upsample<TU, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+    k_upsample<TU, FORM><<<gu, 128, smem, c.stream>>>(nup_p, c.d_up_particle.ptr, c.d_up_off.ptr, c.d_offset.ptr,       \
+                                                      c.d_nodes.ptr, U, x, c.d_up_x.ptr, c.d_up_q.ptr, c.d_up_qh.ptr,   \
+                                                      c.d_up_ql.ptr);                                                   \
+  } while (0)
   if (f32)
-    k_upsample<float><<<gu, 128, smem, c.stream>>>(nup_p, c.d_up_particle.ptr, c.d_up_off.ptr, c.d_offset.ptr, c.d_nodes.ptr,
-                                                   c.d_upU32.ptr, x, c.d_up_mu.ptr);
+    RBS_UPSAMPLE(float, 1, c.d_upU32.ptr);
+  else if (prec == RBS_PREC_DF)
+    RBS_UPSAMPLE(double, 2, c.d_upU.ptr);
   else
-    k_upsample<double><<<gu, 128, smem, c.stream>>>(nup_p, c.d_up_particle.ptr, c.d_up_off.ptr, c.d_offset.ptr,
-                                                    c.d_nodes.ptr, c.d_upU.ptr, x, c.d_up_mu.ptr);
+    RBS_UPSAMPLE(double, 0, c.d_upU.ptr);
+#undef RBS_UPSAMPLE
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
 
-// Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one.
-static Status near_sums(Context& c, int kind, int prec, const double* x, double* y) {
-  const int nn = (int)c.near_pairs.size();
-#define RBS_NEAR_ARGS                                                                                            \
-  c.d_near.ptr, c.d_offset.ptr, c.d_nodes.ptr, c.d_centre.ptr, c.d_up_index.ptr, c.d_up_off.ptr, c.d_x.ptr, \
-      c.d_nrm.ptr, x, c.d_up_x.ptr, c.d_up_mu.ptr, y
-  const int nthr = std::min(512, std::max(64, (c.max_np + 31) / 32 * 32));
+// Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one; kind 0
+// traction into y, 1 Stokeslet into y, 2 (double-float only) traction into y and Stokeslet into y2.
+static Status near_sums(Context& c, int kind, int prec, const double* x, double* y, double* y2) {
+  const long long nn = (long long)c.near_pairs.size();
+  NearArgs A;
+  A.chunks = (c.max_np + 31) / 32;
+  // source runs: about 16 units per SM, of at least 128 sources
+  int most = 1;
+  for (Grid* g : c.grids) most = std::max(most, g->nup + g->np);
+  const long long units1 = nn * A.chunks;
+  A.parts = (int)std::max(1LL, std::min<long long>((16LL * c.sm_count + units1 - 1) / units1, most / 128));
+  const long long units = units1 * A.parts;
+  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "near correction: more than 2^31 work units");
+  A.nunits = (int)units;
+  A.counter = c.d_unit.ptr;
+  A.near = c.d_near.ptr;
+  A.offset = c.d_offset.ptr;
+  A.nodes = c.d_nodes.ptr;
+  A.up_index = c.d_up_index.ptr;
+  A.up_off = c.d_up_off.ptr;
+  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
+  const int blocks = (int)std::min<long long>((units + 3) / 4, INT_MAX);
+#define RBS_NEAR_LAUNCH(KERNEL, ...) \
+  KERNEL<<<resident_grid(c, (const void*)KERNEL, 128, blocks), 128, 0, c.stream>>>(A, __VA_ARGS__)
   if (prec == RBS_PREC_DF) {
+#define RBS_NEAR_DF c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, c.d_wmuh.ptr, c.d_wmul.ptr, \
+                    c.d_up3h.ptr, c.d_up3m.ptr, c.d_up3l.ptr, c.d_up_qh.ptr, c.d_up_ql.ptr, y, y2
     if (kind == 0)
-      k_near_tiled<0, true><<<nn, nthr, 0, c.stream>>>(RBS_NEAR_ARGS);
+      RBS_NEAR_LAUNCH(k_near_df<0>, RBS_NEAR_DF);
+    else if (kind == 1)
+      RBS_NEAR_LAUNCH(k_near_df<1>, RBS_NEAR_DF);
     else
-      k_near_tiled<1, true><<<nn, nthr, 0, c.stream>>>(RBS_NEAR_ARGS);
+      RBS_NEAR_LAUNCH(k_near_df<2>, RBS_NEAR_DF);
+#undef RBS_NEAR_DF
   } else if (prec_f32(prec)) {
+#define RBS_NEAR_32 c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, c.d_up3h.ptr, c.d_up3m.ptr, c.d_up_qh.ptr, y
     if (kind == 0)
-      k_near_tiled<0, false><<<nn, nthr, 0, c.stream>>>(RBS_NEAR_ARGS);
+      RBS_NEAR_LAUNCH(k_near32<0>, RBS_NEAR_32);
     else
-      k_near_tiled<1, false><<<nn, nthr, 0, c.stream>>>(RBS_NEAR_ARGS);
+      RBS_NEAR_LAUNCH(k_near32<1>, RBS_NEAR_32);
+#undef RBS_NEAR_32
   } else {
+#define RBS_NEAR_64 c.d_x.ptr, c.d_nrm.ptr, x, c.d_up_x.ptr, c.d_up_q.ptr, y
     if (kind == 0)
-      k_near<0, double><<<nn, 256, 0, c.stream>>>(RBS_NEAR_ARGS);
+      RBS_NEAR_LAUNCH(k_near64<0>, RBS_NEAR_64);
     else
-      k_near<1, double><<<nn, 256, 0, c.stream>>>(RBS_NEAR_ARGS);
+      RBS_NEAR_LAUNCH(k_near64<1>, RBS_NEAR_64);
+#undef RBS_NEAR_64
   }
-#undef RBS_NEAR_ARGS
+#undef RBS_NEAR_LAUNCH
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
@@ -1570,8 +1444,16 @@ static Status near_sums(Context& c, int kind, int prec, const double* x, double*
 Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
   const int nw = (int)c.work.size();
   const bool f32 = prec_f32(prec);
+  // the weighted densities that the smooth sums and the near correction read
+  if (f32) {
+    c.stats.launches++;
+    RBS_TRY(weight_f32(c, x));
+  } else if (prec == RBS_PREC_DF) {
+    c.stats.launches++;
+    RBS_TRY(weight_df(c, x));
+  }
   if (f32 && c.tree.active) {
-    RBS_TRY(apply_tree(c, kind, x, y, 0));  // treecode in place of the direct float32 sum
+    RBS_TRY(apply_tree(c, kind, x, y));  // treecode in place of the direct float32 sum
   } else if (prec == RBS_PREC_DF && c.tree_df.active) {
     RBS_TRY(apply_tree_df(c, kind, x, y, nullptr));  // and of the direct double-float sum
   } else if (nw > 0) {
@@ -1585,8 +1467,8 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
   }
   if (!c.near_pairs.empty()) {
     KernelTimer timer(c, RBS_KC_NEAR);
-    RBS_TRY(near_upsample(c, f32, x));
-    RBS_TRY(near_sums(c, kind, prec, x, y));
+    RBS_TRY(near_upsample(c, prec, x));
+    RBS_TRY(near_sums(c, kind, prec, x, y, nullptr));
     timer.done((double)c.near_pair_nodes, 2);
   }
   return Status::Ok();
@@ -1598,6 +1480,10 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
     return apply_pairs(c, 1, prec, x, yS);
   }
   const int nw = (int)c.work.size();
+  if (prec == RBS_PREC_DF) {
+    c.stats.launches++;
+    RBS_TRY(weight_df(c, x));
+  }
   if (prec == RBS_PREC_DF && c.tree_df.active) {
     RBS_TRY(apply_tree_df(c, 2, x, yK, yS));
   } else if (nw > 0) {
@@ -1619,10 +1505,15 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
   }
   if (!c.near_pairs.empty()) {
     KernelTimer timer(c, RBS_KC_NEAR);
-    RBS_TRY(near_upsample(c, false, x));
-    RBS_TRY(near_sums(c, 0, prec, x, yK));
-    RBS_TRY(near_sums(c, 1, prec, x, yS));
-    timer.done(2.0 * c.near_pair_nodes, 3);
+    RBS_TRY(near_upsample(c, prec, x));
+    if (prec == RBS_PREC_DF) {
+      RBS_TRY(near_sums(c, 2, prec, x, yK, yS));
+      timer.done(2.0 * c.near_pair_nodes, 2);
+    } else {
+      RBS_TRY(near_sums(c, 0, prec, x, yK, nullptr));
+      RBS_TRY(near_sums(c, 1, prec, x, yS, nullptr));
+      timer.done(2.0 * c.near_pair_nodes, 3);
+    }
   }
   return Status::Ok();
 }

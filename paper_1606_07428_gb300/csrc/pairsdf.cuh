@@ -7,10 +7,8 @@
 
 namespace rbs {
 
-// Double-float pair sums with two sources per instruction: the operations of pair_tile_df on float2
-// pairs (__fadd2_rn, __fmul2_rn, __ffma2_rn, each two round-to-nearest float32 operations, so the
-// error-free transformations stay exact per source), sources staged structure-of-arrays and padded
-// to an even count with zero-density sources far away (they add exactly zero).
+// Double-float pair sums with two sources per instruction (__fadd2_rn, __fmul2_rn, __ffma2_rn, each two
+// round-to-nearest float32 operations, so the error-free transformations stay exact per source).
 struct df2 {
   float2 h, l;
 };
@@ -29,12 +27,6 @@ __device__ __forceinline__ df2 mul2(df2 a, df2 b) {
   e = __ffma2_rn(a.l, b.h, e);
   return {p, e};
 }
-__device__ __forceinline__ df2 dot3_2(df2 a0, df2 b0, df2 a1, df2 b1, df2 a2, df2 b2) {
-  const df2 p0 = mul2(a0, b0), p1 = mul2(a1, b1), p2 = mul2(a2, b2);
-  const df2 s1 = two_sum2(p0.h, p1.h);
-  const df2 s2 = two_sum2(s1.h, p2.h);
-  return {s2.h, __fadd2_rn(__fadd2_rn(__fadd2_rn(s1.l, s2.l), __fadd2_rn(p0.l, p1.l)), p2.l)};
-}
 __device__ __forceinline__ void acc2_add(df2& acc, df2 v) {
   const df2 s = two_sum2(acc.h, v.h);
   acc.h = s.h;
@@ -46,55 +38,245 @@ __device__ __forceinline__ dflt fold2(const df2& a) {
   return {s.h, s.l + (a.l.x + a.l.y)};
 }
 
-template <int KIND, bool MASK>
-__device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], int2 spid, const df2 (&xt)[3],
-                                         const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
+// Bias of a sum of products whose terms are bounded: partial sums of d . q never exceed |d| |q|, so with
+// B >= 2 |d| |q| added first every partial sum stays within [B / 2, 2 B], where the difference of
+// successive partial sums is exact (Sterbenz) and one multiply-add gives what a step rounded off:
+//   s' = fl(s + a b),  e = a b - (s' - s).
+// A product and its addition then take three operations where a two-product and a two-sum take eight.
+// kBiasFactor is 2 with a margin for the rounded norms.
+constexpr float kBiasFactor = 2.002f;
+
+__device__ __forceinline__ df2 norm2(float2 h, float2 l) {  // h + l, renormalised
+  const float2 s = __fadd2_rn(h, l);
+  return {s, __fadd2_rn(l, ng2(__fadd2_rn(s, ng2(h))))};
+}
+// a0 b0 + a1 b1 + a2 b2 by biased accumulation (B as above); renormalised.
+__device__ __forceinline__ df2 bdot2(df2 a0, df2 b0, df2 a1, df2 b1, df2 a2, df2 b2, float2 B) {
+  const float2 s0 = __ffma2_rn(a0.h, b0.h, B), s1 = __ffma2_rn(a1.h, b1.h, s0), s2 = __ffma2_rn(a2.h, b2.h, s1);
+  float2 e0 = __ffma2_rn(a0.h, b0.h, __fadd2_rn(B, ng2(s0)));
+  float2 e1 = __ffma2_rn(a1.h, b1.h, __fadd2_rn(s0, ng2(s1)));
+  float2 e2 = __ffma2_rn(a2.h, b2.h, __fadd2_rn(s1, ng2(s2)));
+  e0 = __ffma2_rn(a0.l, b0.h, __ffma2_rn(a0.h, b0.l, e0));
+  e1 = __ffma2_rn(a1.l, b1.h, __ffma2_rn(a1.h, b1.l, e1));
+  e2 = __ffma2_rn(a2.l, b2.h, __ffma2_rn(a2.h, b2.l, e2));
+  return norm2(__fadd2_rn(s2, ng2(B)), __fadd2_rn(__fadd2_rn(e0, e1), e2));
+}
+
+// Odd powers of 1 / r from r^2 = h + l and the hardware estimate y0 = (1 / r)(1 + O(2^-22)): with
+// t = r^2 y0^2 - 1, (1 / r)^k = y0^k (1 - k t / 2 + k (k + 2) t^2 / 8) to 2^-64.  The powers of y0 are
+// exact to a float32 pair, and the series multiplies a product once, at its end.
+struct inv_powers {
+  float2 y0, q, qe, t;  // q + qe = y0^2
+  __device__ __forceinline__ inv_powers(float2 r2h, float2 r2l, float2 y) : y0(y) {
+    q = __fmul2_rn(y, y);
+    qe = __ffma2_rn(y, y, ng2(q));
+    t = __ffma2_rn(r2l, q, __ffma2_rn(r2h, qe, __ffma2_rn(r2h, q, dup2(-1.0f))));
+  }
+  __device__ __forceinline__ float2 series(float lin, float quad) const {
+    return __fmul2_rn(t, __ffma2_rn(t, dup2(quad), dup2(lin)));
+  }
+  __device__ __forceinline__ float2 w3() const { return series(-1.5f, 1.875f); }
+  __device__ __forceinline__ float2 w5() const { return series(-2.5f, 4.375f); }
+  __device__ __forceinline__ df2 y3() const {
+    const float2 h = __fmul2_rn(q, y0);
+    return {h, __ffma2_rn(qe, y0, __ffma2_rn(q, y0, ng2(h)))};
+  }
+  __device__ __forceinline__ df2 inv() const { return {y0, __fmul2_rn(y0, series(-0.5f, 0.375f))}; }
+};
+
+// How a tile forms separations: by two-sums, the same with the target's own particle masked by its id,
+// or on a common grid (df_tile).
+enum DfMode { kDfPlain = 0, kDfMask = 1, kDfGrid = 2 };
+
+// One target against two sources, KIND 0 traction into acc, 1 Stokeslet into acc, 2 traction into acc and
+// Stokeslet into acc2; fb = kBiasFactor |density| of the sources.  With two-sums 221 float32 operations
+// for both kernels, 154 for the traction alone and 139 for the Stokeslet alone; 9 fewer on the grid.
+template <int KIND, int MODE>
+__device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], float2 fb, int2 spid,
+                                         const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
   df2 d[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    d[c] = two_sum2(xt[c].h, ng2(y[c].h));
-    d[c].l = __fadd2_rn(d[c].l, __fadd2_rn(xt[c].l, ng2(y[c].l)));
+    if (MODE == kDfGrid) {
+      d[c] = norm2(__fadd2_rn(xt[c].h, y[c].h), __fadd2_rn(xt[c].l, y[c].l));
+    } else {
+      d[c] = two_sum2(xt[c].h, y[c].h);
+      d[c].l = __fadd2_rn(d[c].l, __fadd2_rn(xt[c].l, y[c].l));
+    }
   }
-  float2 p[3], e[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    p[c] = __fmul2_rn(d[c].h, d[c].h);
-    e[c] = __ffma2_rn(d[c].h, d[c].h, ng2(p[c]));
-    e[c] = __ffma2_rn(__fadd2_rn(d[c].h, d[c].h), d[c].l, e[c]);
+  // r^2 by biased accumulation over 5/4 of its own float32 value R (over R itself the sum can round to
+  // just above 2 R, where the difference from R is inexact)
+  const float2 R = __ffma2_rn(d[2].h, d[2].h, __ffma2_rn(d[1].h, d[1].h, __fmul2_rn(d[0].h, d[0].h)));
+  float2 y0 = make_float2(rsqrt_hw(R.x), rsqrt_hw(R.y));
+  if (MODE == kDfMask) {  // the target's own particle: every power of 1 / r becomes zero
+    if (spid.x == pt) y0.x = 0.0f;
+    if (spid.y == pt) y0.y = 0.0f;
   }
-  const df2 s1 = two_sum2(p[0], p[1]);
-  const df2 s2 = two_sum2(s1.h, p[2]);
-  const float2 r2l = __fadd2_rn(__fadd2_rn(__fadd2_rn(__fadd2_rn(s1.l, s2.l), e[0]), e[1]), e[2]);
-  const float2 r2h = s2.h;
-  const float2 y0 = make_float2(rsqrt_hw(r2h.x), rsqrt_hw(r2h.y));
-  const float2 q = __fmul2_rn(y0, y0);
-  const float2 qe = __ffma2_rn(y0, y0, ng2(q));
-  float2 t = __ffma2_rn(r2h, q, dup2(-1.0f));
-  t = __ffma2_rn(r2h, qe, t);
-  t = __ffma2_rn(r2l, q, t);
-  df2 inv = {y0, __fmul2_rn(__fmul2_rn(dup2(-0.5f), t), y0)};
-  if (MASK) {
-    if (spid.x == pt) inv.h.x = inv.l.x = 0.0f;
-    if (spid.y == pt) inv.h.y = inv.l.y = 0.0f;
-  }
-  const df2 rr = dot3_2(d[0], den[0], d[1], den[1], d[2], den[2]);
-  const df2 inv2 = mul2(inv, inv);
-  const df2 inv3 = mul2(inv2, inv);
+  const float2 Rb = __fmul2_rn(dup2(1.25f), R);
+  const float2 s0 = __ffma2_rn(d[0].h, d[0].h, Rb), s1 = __ffma2_rn(d[1].h, d[1].h, s0), s2 = __ffma2_rn(d[2].h, d[2].h, s1);
+  float2 e0 = __ffma2_rn(d[0].h, d[0].h, __fadd2_rn(Rb, ng2(s0)));
+  float2 e1 = __ffma2_rn(d[1].h, d[1].h, __fadd2_rn(s0, ng2(s1)));
+  float2 e2 = __ffma2_rn(d[2].h, d[2].h, __fadd2_rn(s1, ng2(s2)));
+  e0 = __ffma2_rn(__ffma2_rn(dup2(2.0f), d[0].h, d[0].l), d[0].l, e0);
+  e1 = __ffma2_rn(__ffma2_rn(dup2(2.0f), d[1].h, d[1].l), d[1].l, e1);
+  e2 = __ffma2_rn(__ffma2_rn(dup2(2.0f), d[2].h, d[2].l), d[2].l, e2);
+  const inv_powers p(__fadd2_rn(s2, ng2(Rb)), __fadd2_rn(__fadd2_rn(e0, e1), e2), y0);
+  const float2 r = __fmul2_rn(R, y0);
+  const df2 rr = bdot2(d[0], den[0], d[1], den[1], d[2], den[2], __fmul2_rn(r, fb));
+  const df2 a = mul2(rr, p.y3());  // r . q / r^3 but for the series
   if (KIND == 0 || KIND == 2) {
-    const df2 inv5 = mul2(inv3, inv2);
-    const df2 rn = dot3_2(d[0], nt[0], d[1], nt[1], d[2], nt[2]);
-    const df2 ck = mul2(mul2(rn, rr), inv5);
+    const df2 rn = bdot2(d[0], nt[0], d[1], nt[1], d[2], nt[2], __fmul2_rn(r, dup2(kBiasFactor)));
+    df2 ck = mul2(a, mul2(rn, df2{p.q, p.qe}));
+    ck.l = __ffma2_rn(p.w5(), ck.h, ck.l);
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc2_add(acc[c], mul2(ck, d[c]));
   }
   if (KIND == 1 || KIND == 2) {
-    const df2 cs = mul2(rr, inv3);
+    // q / r + (r . q) r / r^3, each component bounded by 2 |q| / r: biased by twice that
+    const df2 cs = {a.h, __ffma2_rn(p.w3(), a.h, a.l)};
+    const df2 inv = p.inv();
+    const float2 B = __fmul2_rn(__fmul2_rn(dup2(2.0f), y0), fb);
     df2(&as)[3] = KIND == 2 ? acc2 : acc;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      acc2_add(as[c], mul2(den[c], inv));
-      acc2_add(as[c], mul2(cs, d[c]));
+      const float2 u = __ffma2_rn(cs.h, d[c].h, B), v = __ffma2_rn(den[c].h, inv.h, u);
+      float2 f = __ffma2_rn(cs.h, d[c].h, __fadd2_rn(B, ng2(u)));
+      float2 g = __ffma2_rn(den[c].h, inv.h, __fadd2_rn(u, ng2(v)));
+      f = __ffma2_rn(cs.l, d[c].h, __ffma2_rn(cs.h, d[c].l, f));
+      g = __ffma2_rn(den[c].l, inv.h, __ffma2_rn(den[c].h, inv.l, g));
+      acc2_add(as[c], df2{__fadd2_rn(v, ng2(B)), __fadd2_rn(f, g)});
     }
+  }
+}
+
+constexpr int kTileDf = 64;
+constexpr int kTileDfFloats = 14 * kTileDf;
+
+// ------------------------------------------------------------------------------------------
+// A warp's tile of up to kTileDf sources against its 32 targets (one a lane): the double-float sums of
+// both the direct and the treecode kernels.  Lane l stages sources sidx[0] (tile slot l) and sidx[1]
+// (slot 32 + l), filled in all, into the warp's kTileDfFloats floats of shared memory.
+//
+// Where every source is at least a quarter of the tile's extent away from the targets, coordinates are
+// split so that every hi part of the tile, sources and targets, is a multiple of g = 2^-24 times the power of
+// two above the largest separation: differences of hi parts are exact without a two-sum, and the lo parts
+// (at most g / 2) keep the separation within a few times 2^-50 of itself.  Closer tiles take two-sums.
+// split: each half-warp holds the same 16 targets and takes its half of the tile.  xm = the
+// warp's largest target coordinate; sign (1 or -1) multiplies the densities; totals go to tot (and tot2
+// for KIND 2).
+
+__device__ __forceinline__ float warp_max_abs(float v) {  // of non-negative values
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+
+__device__ __forceinline__ float warp_min_abs(float v) {
+  return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(v)));
+}
+
+template <int KIND, int MODE>
+__device__ __forceinline__ void df_tile_pairs(const float (*sa)[kTileDf], const int* spid, int l0, int l1, const df2 (&xt)[3],
+                                              const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
+#pragma unroll 1
+  for (int l = l0; l < l1; l += 2) {
+    df2 ys[3], den[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ys[c] = {*reinterpret_cast<const float2*>(&sa[2 * c][l]), *reinterpret_cast<const float2*>(&sa[2 * c + 1][l])};
+      den[c] = {*reinterpret_cast<const float2*>(&sa[6 + 2 * c][l]), *reinterpret_cast<const float2*>(&sa[7 + 2 * c][l])};
+    }
+    const float2 fb = *reinterpret_cast<const float2*>(&sa[12][l]);
+    int2 pp = make_int2(0, 0);
+    if (MODE == kDfMask) pp = *reinterpret_cast<const int2*>(&spid[l]);
+    pair2_df<KIND, MODE>(ys, den, fb, pp, xt, nt, pt, acc, acc2);
+  }
+}
+
+template <int KIND>
+__device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int filled, bool masked, bool split, int half,
+                                        const float4* __restrict__ x3h, const float4* __restrict__ x3m,
+                                        const float4* __restrict__ x3l, const float4* __restrict__ qh_,
+                                        const float4* __restrict__ ql_, const float4& oh, const float4& om,
+                                        const float4& ol, const dflt (&x0)[3], const dflt (&n0)[3], float xm, int pt,
+                                        dflt (&tot)[3], dflt (&tot2)[3], float sign = 1.0f) {
+  const int lane = threadIdx.x & 31;
+  float(*sa)[kTileDf] = reinterpret_cast<float(*)[kTileDf]>(wsm);
+  int* const spid = reinterpret_cast<int*>(&sa[13][0]);
+  dflt p[2][3];
+  float m = 0.0f, mn = 3.0e38f;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    p[k][0] = p[k][1] = p[k][2] = dflt{0.0f, 0.0f};
+    if (lane + 32 * k < filled) {
+      const float4 ph = x3h[sidx[k]], pm = x3m[sidx[k]], pl = x3l[sidx[k]];
+      p[k][0] = df_diff3(oh.x, om.x, ol.x, ph.x, pm.x, pl.x);
+      p[k][1] = df_diff3(oh.y, om.y, ol.y, ph.y, pm.y, pl.y);
+      p[k][2] = df_diff3(oh.z, om.z, ol.z, ph.z, pm.z, pl.z);
+      const float far = fmaxf(fabsf(p[k][0].h), fmaxf(fabsf(p[k][1].h), fabsf(p[k][2].h)));
+      m = fmaxf(m, far);
+      mn = fminf(mn, far);
+    }
+  }
+  m = warp_max_abs(m) + xm;
+  // in the largest coordinate alone a source is at least mn - xm away
+  const bool grid = !masked && warp_min_abs(mn) - xm >= 0.25f * m;
+  // g = 2^(e - 24), 2^e > m; its exponent field is that of m less 23
+  const int ge = max(1, (int)(__float_as_uint(m) >> 23) - 23);
+  const float g = __uint_as_float((unsigned)ge << 23), ginv = __uint_as_float((unsigned)(254 - ge) << 23);
+  auto on_grid = [&](dflt v) -> dflt {
+    if (!grid) return v;
+    const float h = rintf(v.h * ginv) * g;
+    return {h, (v.h - h) + v.l};
+  };
+  const int cnt4 = (filled + 3) & ~3;
+  __syncwarp();  // the warp's reads of the previous tile are done
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int l = lane + 32 * k;
+    if (l < filled) {
+      const float4 qh = qh_[sidx[k]], ql = ql_[sidx[k]];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const dflt v = on_grid(p[k][c]);
+        sa[2 * c][l] = v.h;
+        sa[2 * c + 1][l] = v.l;
+      }
+      sa[6][l] = sign * qh.x;
+      sa[7][l] = sign * ql.x;
+      sa[8][l] = sign * qh.y;
+      sa[9][l] = sign * ql.y;
+      sa[10][l] = sign * qh.z;
+      sa[11][l] = sign * ql.z;
+      sa[12][l] = kBiasFactor * sqrtf(fmaf(qh.x, qh.x, fmaf(qh.y, qh.y, qh.z * qh.z)));
+      spid[l] = __float_as_int(x3h[sidx[k]].w);
+    } else if (l < cnt4) {  // zero-density sources away from every target: they add exactly zero
+      sa[0][l] = sa[2][l] = sa[4][l] = 8.0f * m;
+      sa[1][l] = sa[3][l] = sa[5][l] = 0.0f;
+      for (int q = 6; q < 13; ++q) sa[q][l] = 0.0f;
+      spid[l] = -2;
+    }
+  }
+  df2 xt[3], nt[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const dflt v = on_grid(x0[c]);
+    xt[c] = {dup2(v.h), dup2(v.l)};
+    nt[c] = {dup2(n0[c].h), dup2(n0[c].l)};
+  }
+  __syncwarp();
+  df2 acc[3], acc2[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) acc[c] = acc2[c] = df2{dup2(0.0f), dup2(0.0f)};
+  const int cnt = split ? cnt4 / 2 : cnt4, l0 = half * cnt;
+  if (masked)
+    df_tile_pairs<KIND, kDfMask>(sa, spid, l0, l0 + cnt, xt, nt, pt, acc, acc2);
+  else if (grid)
+    df_tile_pairs<KIND, kDfGrid>(sa, spid, l0, l0 + cnt, xt, nt, pt, acc, acc2);
+  else
+    df_tile_pairs<KIND, kDfPlain>(sa, spid, l0, l0 + cnt, xt, nt, pt, acc, acc2);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    tot[c] = df_add_accurate(tot[c], fold2(acc[c]));
+    if (KIND == 2) tot2[c] = df_add_accurate(tot2[c], fold2(acc2[c]));
   }
 }
 

@@ -494,7 +494,8 @@ __global__ void k_to_16bit(const double* in, uint16_t* out, long long n, int bf1
 // (pup + 1) x nphi_up grid.
 __global__ void k_up_nodes(int nu, const int* up_particle, const long long* up_off, const int* pvec, const int* nphivec,
                            const int* pupvec, const int* shape_of, RBS_SHAPE_ARGS, const double* centre,
-                           const double* rot, const long long* gtab_up_off, const double* gtab, double4* out) {
+                           const double* rot, const long long* gtab_up_off, const double* gtab, double4* out, float4* u3h,
+                           float4* u3m, float4* u3l) {
   for (int u = blockIdx.y; u < nu; u += gridDim.y) {
     const int i = up_particle[u];
     const int pup = pupvec[i];
@@ -511,10 +512,18 @@ __global__ void k_up_nodes(int nu, const int* up_particle, const long long* up_o
       sincospi(2.0 * k / nphi_up, &sp, &cp);
       double xb[3], J, nb[3];
       eval_surface(S, st * cp, st * sp, ct, xb, &J, nb);
-      out[up_off[u] + l] = make_double4(R[0] * xb[0] + R[1] * xb[1] + R[2] * xb[2] + centre[3 * i],
-                                        R[3] * xb[0] + R[4] * xb[1] + R[5] * xb[2] + centre[3 * i + 1],
-                                        R[6] * xb[0] + R[7] * xb[1] + R[8] * xb[2] + centre[3 * i + 2],
-                                        2.0 * kPi / nphi_up * lam[j] * J);
+      const double4 v = make_double4(R[0] * xb[0] + R[1] * xb[1] + R[2] * xb[2] + centre[3 * i],
+                                     R[3] * xb[0] + R[4] * xb[1] + R[5] * xb[2] + centre[3 * i + 1],
+                                     R[6] * xb[0] + R[7] * xb[1] + R[8] * xb[2] + centre[3 * i + 2],
+                                     2.0 * kPi / nphi_up * lam[j] * J);
+      const long long g = up_off[u] + l;
+      out[g] = v;
+      const float hx = (float)v.x, hy = (float)v.y, hz = (float)v.z;
+      const double rx = v.x - (double)hx, ry = v.y - (double)hy, rz = v.z - (double)hz;
+      const float mx = (float)rx, my = (float)ry, mz = (float)rz;
+      u3h[g] = make_float4(hx, hy, hz, 0.0f);
+      u3m[g] = make_float4(mx, my, mz, 0.0f);
+      u3l[g] = make_float4((float)(rx - (double)mx), (float)(ry - (double)my), (float)(rz - (double)mz), 0.0f);
     }
   }
 }
@@ -913,14 +922,16 @@ Status build_near(Context& c) {
   RBS_TRY(upload(c.d_up_off, c.up_offset, s));
   RBS_TRY(upload(c.d_up_index, c.up_index, s));
   RBS_TRY(c.d_up_x.alloc(c.n_up_nodes));
-  RBS_TRY(c.d_up_mu.alloc(3 * c.n_up_nodes));
+  RBS_TRY(c.d_up_q.alloc(c.n_up_nodes));
+  for (DevBuf<float4>* b : {&c.d_up3h, &c.d_up3m, &c.d_up3l, &c.d_up_qh, &c.d_up_ql}) RBS_TRY(b->alloc(c.n_up_nodes));
   if (!c.up_particle.empty()) {
     int maxnup = 0;
     for (Grid* g : c.grids) maxnup = std::max(maxnup, g->nup);
     dim3 grd(cdiv(maxnup, 128), (unsigned)std::min<size_t>(c.up_particle.size(), 65535));
     k_up_nodes<<<grd, 128, 0, s>>>((int)c.up_particle.size(), c.d_up_particle.ptr, c.d_up_off.ptr, c.d_p.ptr, c.d_nphi.ptr,
                                    c.d_pup.ptr, c.d_shape.ptr, RBS_SHAPE_PASS, c.d_centre.ptr, c.d_rot.ptr,
-                                   c.d_gtab_up_off.ptr, c.d_gtab.ptr, c.d_up_x.ptr);
+                                   c.d_gtab_up_off.ptr, c.d_gtab.ptr, c.d_up_x.ptr, c.d_up3h.ptr, c.d_up3m.ptr,
+                                   c.d_up3l.ptr);
     RBS_CUDA_TRY(cudaGetLastError());
   }
 
@@ -1236,7 +1247,9 @@ Status build_geometry(Context& c) {
     int splits = (int)std::max(1LL, (want + tiles - 1) / std::max(1LL, tiles));
     for (auto& sp : susp) {
       long long ns = sp.second - sp.first;
-      int sc = (int)std::min<long long>(splits, std::max(1LL, ns / 2048));
+      // small systems: as many chunks as give every SM eight items, of 128 sources at least
+      const long long few = std::min((8LL * c.sm_count + tiles - 1) / tiles, ns / 128);
+      int sc = (int)std::max(few, std::min<long long>(splits, std::max(1LL, ns / 2048)));
       long long chunk = (ns + sc - 1) / sc;
       for (long long tb = sp.first; tb < sp.second; tb += TT)
         for (long long sb = sp.first; sb < sp.second; sb += chunk) {
@@ -1250,6 +1263,7 @@ Status build_geometry(Context& c) {
     }
   }
   RBS_TRY(upload(c.d_work, c.work, s));
+  RBS_TRY(c.d_unit.alloc(1));
 
   // particle-block work list
   c.bwork.clear();

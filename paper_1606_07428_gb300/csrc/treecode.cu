@@ -36,8 +36,10 @@ namespace {
 constexpr int kTreeMaxQ = 11;        // degree <= 10
 constexpr int kTreeMaxTargets = 512; // targets per work item at most
 constexpr int kTreeTile32 = 128;     // sources per warp tile of the float32 treecode sum
-constexpr int kTreeTileDf = 64;      // and of the double-float one
-constexpr int kProxyPid = -3;        // particle id carried by proxy points (never a target's)
+constexpr int kTreeMaxQ64 = 13;      // degree <= 12 (double-float passes)
+
+__device__ __forceinline__ float fma_any(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_any(double a, double b, double c) { return fma(a, b, c); }
 
 // Bounding box of each particle's nodes: lo (3) then hi (3) per particle.
 __global__ void __launch_bounds__(128) k_particle_boxes(int n, const long long* __restrict__ offset,
@@ -75,27 +77,19 @@ __global__ void __launch_bounds__(128) k_particle_boxes(int n, const long long* 
   }
 }
 
-// Float32 weighted density of the nodes, the sources' charges: q[t] = (w_t mu_t, 0).
-__global__ void k_tree_node_charges(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
-                                    float4* __restrict__ q) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= N) return;
-  const double w = x[t].w;
-  q[t] = make_float4((float)(w * dens[3 * t]), (float)(w * dens[3 * t + 1]), (float)(w * dens[3 * t + 2]), 0.0f);
-}
-
 // Barycentric Lagrange basis of the nq Chebyshev points s (weights bw) at u in [-1, 1]; a point on a
 // node gets that node's unit vector.
-__device__ __forceinline__ void lagrange_row(float u, const float* s, const float* bw, int nq, float* L) {
-  float t[kTreeMaxQ];
-  float sum = 0.0f;
+template <typename T, int MAXQ>
+__device__ __forceinline__ void lagrange_row(T u, const T* s, const T* bw, int nq, T* L) {
+  T t[MAXQ];
+  T sum = 0;
   int hit = -1;
 #pragma unroll
-  for (int k = 0; k < kTreeMaxQ; ++k) {
-    t[k] = 0.0f;
+  for (int k = 0; k < MAXQ; ++k) {
+    t[k] = 0;
     if (k < nq) {
-      const float d = u - s[k];
-      if (d == 0.0f)
+      const T d = u - s[k];
+      if (d == (T)0)
         hit = k;
       else
         t[k] = bw[k] / d;
@@ -103,126 +97,226 @@ __device__ __forceinline__ void lagrange_row(float u, const float* s, const floa
     }
   }
 #pragma unroll
-  for (int k = 0; k < kTreeMaxQ; ++k)
-    if (k < nq) L[k] = hit >= 0 ? (k == hit ? 1.0f : 0.0f) : t[k] / sum;
+  for (int k = 0; k < MAXQ; ++k)
+    if (k < nq) L[k] = hit >= 0 ? (k == hit ? (T)1 : (T)0) : t[k] / sum;
 }
 
-// Cluster charges: one block per (cluster, run of its particles); each thread owns up to
-// kProxyPerThread proxy points and sums L_a L_b L_c q over the run's nodes, staged 256 at a time with
-// their Lagrange rows; the partial charges are added atomically (the charges are zeroed first).
+// Cluster charges, one block per (cluster, run of its particles); T = float or double.  Nodes are staged
+// kChargeTile at a time with their Lagrange rows in x and y and the products L_c(z) q_k (k = 0, 1, 2); a
+// thread owns NB values of b for one a of the proxy grid and every c, so a node costs it NB products
+// L_a L_b and 3 multiply-adds per proxy.  The threads form groups of one (a, b) plane each that take the
+// staged nodes in turn; in float32 the groups add up in shared memory first, then one group's worth of
+// partial charges is added atomically to the cluster's (zeroed before).  Charges are stored by rows of the
+// grid's last axis, the layout that the pair kernels read: q[(((cluster nq + a) nbp + b) 3 + k) ncp + c],
+// rows padded to ncp and planes to nbp rows with zeros.
 constexpr int kChargeThreads = 256;
-constexpr int kProxyPerThread = (kTreeMaxQ * kTreeMaxQ * kTreeMaxQ + kChargeThreads - 1) / kChargeThreads;
+constexpr int kChargeTile = 64;
 
+template <typename T, int MAXQ, int NB>
 __global__ void __launch_bounds__(kChargeThreads) k_tree_charges(const int4* __restrict__ items,
                                                                  const int* __restrict__ order,
                                                                  const long long* __restrict__ offset,
                                                                  const double4* __restrict__ x,
-                                                                 const float4* __restrict__ qnode,
+                                                                 const double* __restrict__ dens,
                                                                  const double* __restrict__ box,
-                                                                 const float* __restrict__ cheb, int nq,
-                                                                 float4* __restrict__ qproxy) {
-  constexpr int TS = kChargeThreads;
-  __shared__ float sL[3][TS][kTreeMaxQ];
-  __shared__ float4 sq[TS];
-  __shared__ float s_pts[kTreeMaxQ], s_bw[kTreeMaxQ];
-  const int npx = nq * nq * nq;
-  if (threadIdx.x < nq) {
+                                                                 const T* __restrict__ cheb, int nq, int nbp, int ncp,
+                                                                 T* __restrict__ qproxy) {
+  constexpr int TS = kChargeTile;
+  constexpr int MC = (MAXQ + 3) & ~3, MB = (MAXQ + NB - 1) / NB * NB;
+  constexpr bool kReduce = sizeof(T) == 4;
+  __shared__ T sLx[TS][MAXQ];
+  __shared__ __align__(16) T sLy[TS][MB];
+  __shared__ __align__(16) T sq[TS][3][MC];
+  __shared__ T s_sum[kReduce ? 3 * MAXQ * MAXQ * MAXQ : 1];
+  __shared__ T s_pts[MAXQ], s_bw[MAXQ];
+  if ((int)threadIdx.x < nq) {
     s_pts[threadIdx.x] = cheb[threadIdx.x];
     s_bw[threadIdx.x] = cheb[nq + threadIdx.x];
   }
+  if (kReduce)
+    for (int k = threadIdx.x; k < 3 * nq * nq * nq; k += kChargeThreads) s_sum[k] = 0;
   const int4 it = items[blockIdx.x];
   const int u = it.x;
-  const double m0 = box[6 * (size_t)u], m1 = box[6 * (size_t)u + 1], m2 = box[6 * (size_t)u + 2];
-  const double h0 = box[6 * (size_t)u + 3], h1 = box[6 * (size_t)u + 4], h2 = box[6 * (size_t)u + 5];
-  int ka[kProxyPerThread], kb[kProxyPerThread], kc[kProxyPerThread];
-  float acc[kProxyPerThread][3];
+  const int nbt = (nq + NB - 1) / NB, plane = nq * nbt;
+  const int groups = kChargeThreads / plane;  // at least one: plane <= 169
+  const int g = threadIdx.x / plane;
+  const int ab = threadIdx.x - g * plane, a = ab / nbt, b = NB * (ab - a * nbt);
+  T acc[NB][3][MAXQ];
 #pragma unroll
-  for (int m = 0; m < kProxyPerThread; ++m) {
-    const int k = threadIdx.x + kChargeThreads * m;
-    ka[m] = k / (nq * nq);
-    kb[m] = (k / nq) % nq;
-    kc[m] = k % nq;
-    acc[m][0] = acc[m][1] = acc[m][2] = 0.0f;
-  }
+  for (int h = 0; h < NB; ++h)
+#pragma unroll
+    for (int c = 0; c < MAXQ; ++c) acc[h][0][c] = acc[h][1][c] = acc[h][2][c] = 0;
   for (int pi = it.y; pi < it.z; ++pi) {
     const int j = order[pi];
     const long long o = offset[j], e = offset[j + 1];
     for (long long s0 = o; s0 < e; s0 += TS) {
       const int cnt = (int)min((long long)TS, e - s0);
       __syncthreads();
-      if ((int)threadIdx.x < cnt) {
-        const double4 p = x[s0 + threadIdx.x];
-        lagrange_row((float)((p.x - m0) * h0), s_pts, s_bw, nq, sL[0][threadIdx.x]);
-        lagrange_row((float)((p.y - m1) * h1), s_pts, s_bw, nq, sL[1][threadIdx.x]);
-        lagrange_row((float)((p.z - m2) * h2), s_pts, s_bw, nq, sL[2][threadIdx.x]);
-        sq[threadIdx.x] = qnode[s0 + threadIdx.x];
+      // one thread per (node, axis)
+      const int ax = threadIdx.x / TS, l = threadIdx.x - TS * ax;
+      if (ax < 3 && l < cnt) {
+        const double4 p = x[s0 + l];
+        const double v = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
+        const double m = box[6 * (size_t)u + ax], h = box[6 * (size_t)u + 3 + ax];
+        T L[MAXQ];
+        lagrange_row<T, MAXQ>((T)((v - m) * h), s_pts, s_bw, nq, L);
+        if (ax == 0) {
+#pragma unroll
+          for (int k = 0; k < MAXQ; ++k)
+            if (k < nq) sLx[l][k] = L[k];
+        } else if (ax == 1) {
+#pragma unroll
+          for (int k = 0; k < MB; ++k) sLy[l][k] = k < nq && k < MAXQ ? L[k < MAXQ ? k : 0] : (T)0;
+        } else {
+          const double* d = dens + 3 * (s0 + l);
+          const T q0 = (T)(p.w * d[0]), q1 = (T)(p.w * d[1]), q2 = (T)(p.w * d[2]);
+#pragma unroll
+          for (int k = 0; k < MAXQ; ++k)
+            if (k < nq) {
+              sq[l][0][k] = L[k] * q0;
+              sq[l][1][k] = L[k] * q1;
+              sq[l][2][k] = L[k] * q2;
+            }
+        }
       }
       __syncthreads();
-      for (int l = 0; l < cnt; ++l) {
-        const float4 q = sq[l];
+      if (g < groups) {
+        for (int l2 = g; l2 < cnt; l2 += groups) {
+          T w[NB];
 #pragma unroll
-        for (int m = 0; m < kProxyPerThread; ++m) {
-          if (threadIdx.x + kChargeThreads * m < npx) {
-            const float f = sL[0][l][ka[m]] * sL[1][l][kb[m]] * sL[2][l][kc[m]];
-            acc[m][0] = fmaf(f, q.x, acc[m][0]);
-            acc[m][1] = fmaf(f, q.y, acc[m][1]);
-            acc[m][2] = fmaf(f, q.z, acc[m][2]);
-          }
+          for (int h = 0; h < NB; ++h) w[h] = sLx[l2][a] * sLy[l2][b + h];
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int c = 0; c < MAXQ; ++c)
+              if (c < nq) {
+                const T v = sq[l2][k][c];
+#pragma unroll
+                for (int h = 0; h < NB; ++h) acc[h][k][c] = fma_any(w[h], v, acc[h][k][c]);
+              }
         }
       }
     }
   }
+  // the groups add their sums in turn
+  for (int gg = 0; gg < (kReduce ? groups : 1); ++gg) {
+    if (kReduce) __syncthreads();
+    if (kReduce ? g == gg : g < groups) {
 #pragma unroll
-  for (int m = 0; m < kProxyPerThread; ++m) {
-    const int k = threadIdx.x + kChargeThreads * m;
-    if (k < npx) {
-      float4* dst = qproxy + (size_t)u * npx + k;
-      atomicAdd(&dst->x, acc[m][0]);
-      atomicAdd(&dst->y, acc[m][1]);
-      atomicAdd(&dst->z, acc[m][2]);
+      for (int h = 0; h < NB; ++h) {
+        if (b + h >= nq) continue;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+          for (int c = 0; c < MAXQ; ++c)
+            if (c < nq) {
+              if (kReduce)
+                s_sum[((a * nq + b + h) * 3 + k) * nq + c] += acc[h][k][c];
+              else
+                atomicAdd(qproxy + (((size_t)(u * nq + a) * nbp + b + h) * 3 + k) * ncp + c, acc[h][k][c]);
+            }
+      }
+    }
+  }
+  if (kReduce) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < 3 * nq * nq * nq; e += kChargeThreads) {
+      const int row = e / nq, c = e - row * nq, r3 = row / 3, k = row - 3 * r3, aa = r3 / nq, bb = r3 - aa * nq;
+      atomicAdd(qproxy + (((size_t)(u * nq + aa) * nbp + bb) * 3 + k) * ncp + c, s_sum[e]);
     }
   }
 }
 
-// The float32 treecode pair sum: the packed tile loop of the direct kernel (pairs32.cuh) over source
-// tiles filled from the item's segments.  Coordinates are relative to the item's first target; tiles
-// that may hold nodes of the targets' own particle (the first nmask sources) mask them by particle id.
-// The block size is chosen at launch so that blockDim.x * NT covers the largest item (a whole particle
-// where it fits).  Each warp stages its own tiles of 128 sources and never waits for the other warps
-// of its block: a block of an odd warp count (five warps for a 144-node particle) spreads unevenly over
-// the SM's four schedulers, so block-wide tiles left the warps of the lighter schedulers waiting at
-// every tile barrier.  Registers are capped (64 at one target per thread: six 160-thread blocks per SM).
-template <int KIND, int NT>
-__global__ void __maxnreg__(NT == 1 ? 64 : (NT == 2 ? 128 : 168))
-    k_tree32x2(int nitems, const TreeItem* __restrict__ items, const int2* __restrict__ segs,
+// Float64 cluster charges to the rows the double-float kernel reads, per row of the last proxy axis:
+// (x, y, z hi, x, y, z lo, bound) x ncp, bound = 2 |q| rounded up (the bias of the biased sums).
+__global__ void k_tree_q64_split(long long rows, int ncp, const double* __restrict__ q64, float* __restrict__ q) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (k >= rows * ncp) return;
+  const long long r = k / ncp;
+  const int c = (int)(k - r * ncp);
+  float* dst = q + r * 7 * ncp + c;
+  float s = 0.0f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const dflt v = df_split(q64[(r * 3 + d) * ncp + c]);
+    dst[d * ncp] = v.h;
+    dst[(3 + d) * ncp] = v.l;
+    s = fmaf(v.h, v.h, s);
+  }
+  dst[6 * ncp] = kBiasFactor * sqrtf(s);
+}
+
+// Next unit of a warp: units are (work item, run of 32 NT of its targets) in item order, taken from a
+// counter that the launch starts at zero.  Warps never wait for one another, and no warp is tied to a
+// fixed share: with whole-particle blocks striding over the items, the warp that held a particle's
+// last few targets finished early and blocks of an odd warp count loaded the SM's four schedulers
+// unevenly (10 of 15 resident warps active on average).
+__device__ __forceinline__ int next_unit(int* counter) {
+  int u = 0;
+  if ((threadIdx.x & 31) == 0) u = atomicAdd(counter, 1);
+  return __shfl_sync(0xffffffffu, u, 0);
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// ---- float32 treecode pair sum
+//
+// A unit walks its item's segments: runs of nodes (direct particles), then clusters.
+//
+// Nodes: the packed tile loop of the direct kernel (pairs32.cuh) over per-warp tiles of 128 sources;
+// tiles that may hold nodes of the targets' own particle (the first nmask sources) mask them by id.
+//
+// Clusters: the proxy points form a tensor grid, so a target's separations from all (n + 1)^3 of them
+// come from n + 1 differences per axis.  Per row (a, b) the parts d_x^2 + d_y^2 and d_x n_x + d_y n_y are
+// formed once; a proxy then takes one multiply-add for r^2, one for r . n, three for r . q, five for the
+// kernel's factor c, and two for the sums: sum c and sum c d_z, the x and y components following
+// per row as d_x sum c and d_y sum c.  That is 12 float32 operations per proxy pair (Stokeslet: 12)
+// in place of the 20 (18) of a node pair.  Two proxies of the last axis share each packed instruction;
+// NQ2 = ceil((n + 1) / 2).  Charges come in slabs (one a) through a per-warp ring of asynchronous
+// copies.
+//
+// A unit with at most 16 targets gives its two half-warps alternate halves of the sources.
+constexpr int kRing32 = 4;
+
+template <int KIND, int NT, int NQ2>
+__global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
+    k_tree32x2(int nunits, int per_item, int* __restrict__ counter, const TreeItem* __restrict__ items,
+               const int2* __restrict__ segs, long long N, int npx, int nq, int nbp, int ncp,
                const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
-               const float4* __restrict__ shi, const float4* __restrict__ slo, const float4* __restrict__ sq,
-               double* __restrict__ y) {
+               const float4* __restrict__ sq, const float4* __restrict__ axis, const float* __restrict__ pq,
+               int warp_floats, double* __restrict__ y) {
   constexpr int TW = kTreeTile32, SL = TW / 32;
   const int lane = threadIdx.x & 31;
-  const int wbase = (threadIdx.x >> 5) * 32 * NT;  // the warp's targets: wbase + 32 u + lane of the item
   extern __shared__ __align__(16) float tree_smem32[];
-  float* const ssx = tree_smem32 + (threadIdx.x >> 5) * (7 * TW);
+  float* const wsm = tree_smem32 + (threadIdx.x >> 5) * warp_floats;
+  float* const ssx = wsm;
   float* const ssy = ssx + TW;
   float* const ssz = ssx + 2 * TW;
   float* const srx = ssx + 3 * TW;
   float* const sry = ssx + 4 * TW;
   float* const srz = ssx + 5 * TW;
   int* const spid = reinterpret_cast<int*>(ssx + 6 * TW);
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const TreeItem w = items[it];
-    // target slots of this warp that hold a target: u < nu (a warp owns 32 NT consecutive targets, so
-    // only the item's last warp has empty slots; they are skipped, and a warp without targets skips
-    // the item)
-    const int nu = min(NT, max(0, (w.t1 - w.t0 - wbase + 31) / 32));
-    if (nu == 0) continue;
+  const int slab = 3 * nbp * ncp;            // floats of one a-slab
+  float* const ring = wsm;                   // kRing32 slabs
+  float* const sax = wsm + kRing32 * slab;   // 3 nq (+ 3 pad) origin-relative proxy coordinates, negated
+  const uint32_t ring_s = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
+  for (int unit = next_unit(counter); unit < nunits; unit = next_unit(counter)) {
+    const int item = unit / per_item;
+    const TreeItem w = items[item];
+    const int tb = w.t0 + (unit - item * per_item) * 32 * NT;
+    if (tb >= w.t1) continue;
+    const int nu = min(NT, (w.t1 - tb + 31) / 32);      // target slots that hold a target
+    const bool split = w.t1 - tb <= 16;
+    const int half = split ? lane >> 4 : 0;
     const float4 oh = xhi[w.t0], ol = xlo[w.t0];
     float2 xt[NT][3], nt[NT][3];
     int pt[NT];
     bool valid[NT];
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
-      const int t = w.t0 + wbase + 32 * u + lane;
+      const int t = tb + 32 * u + (split ? lane & 15 : lane);
       valid[u] = t < w.t1;
       float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, n0 = 0.0f, n1 = 0.0f, n2 = 0.0f;
       pt[u] = -1;
@@ -247,15 +341,16 @@ __global__ void __maxnreg__(NT == 1 ? 64 : (NT == 2 ? 128 : 168))
 #pragma unroll
     for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
     int seg = w.s0, off = 0, done = 0;
-    while (seg < w.s1) {
+    int2 sg = segs[seg];
+    // nodes
+    while (seg < w.s1 && sg.x < N) {
       // the source of each of this lane's slots (lane + 32 k) from a walk over consecutive segments
       // that every lane of the warp takes in step, then all of its loads at once
       int sidx[SL];
 #pragma unroll
       for (int k = 0; k < SL; ++k) sidx[k] = 0;
       int filled = 0;
-      while (filled < TW && seg < w.s1) {
-        const int2 sg = segs[seg];
+      while (filled < TW && seg < w.s1 && sg.x < N) {
         const int take = min(sg.y - off, TW - filled);
 #pragma unroll
         for (int k = 0; k < SL; ++k) {
@@ -267,16 +362,17 @@ __global__ void __maxnreg__(NT == 1 ? 64 : (NT == 2 ? 128 : 168))
         if (off >= sg.y) {
           ++seg;
           off = 0;
+          if (seg < w.s1) sg = segs[seg];
         }
       }
-      const int cnt4 = (filled + 3) & ~3;
+      const int cnt8 = (filled + 7) & ~7;
       __syncwarp();  // the warp's reads of the previous tile are done
 #pragma unroll 2
       for (int k = 0; k < SL; ++k) {
         const int l = lane + 32 * k;
         if (l < filled) {
           const int s = sidx[k];
-          const float4 ph = shi[s], pl = slo[s], q = sq[s];
+          const float4 ph = xhi[s], pl = xlo[s], q = sq[s];
           ssx[l] = (oh.x - ph.x) + (ol.x - pl.x);
           ssy[l] = (oh.y - ph.y) + (ol.y - pl.y);
           ssz[l] = (oh.z - ph.z) + (ol.z - pl.z);
@@ -284,7 +380,7 @@ __global__ void __maxnreg__(NT == 1 ? 64 : (NT == 2 ? 128 : 168))
           sry[l] = q.y;
           srz[l] = q.z;
           spid[l] = __float_as_int(ph.w);
-        } else if (l < cnt4) {
+        } else if (l < cnt8) {
           ssx[l] = ssy[l] = ssz[l] = 1.0e4f;
           srx[l] = sry[l] = srz[l] = 0.0f;
           spid[l] = -2;
@@ -294,21 +390,20 @@ __global__ void __maxnreg__(NT == 1 ? 64 : (NT == 2 ? 128 : 168))
       float2 p[NT][3];
 #pragma unroll
       for (int u = 0; u < NT; ++u) p[u][0] = p[u][1] = p[u][2] = f2(0.0f, 0.0f);
-#define RBS_TILE(NUV)                                                                              \
-  do {                                                                                             \
-    if (done < w.nmask)                                                                            \
-      pair_tile32x2<KIND, true, NT, NUV>(ssx, ssy, ssz, srx, sry, srz, spid, cnt4, xt, nt, pt, p);  \
-    else                                                                                           \
-      pair_tile32x2<KIND, false, NT, NUV>(ssx, ssy, ssz, srx, sry, srz, spid, cnt4, xt, nt, pt, p); \
+      const int cnt = split ? cnt8 / 2 : cnt8, l0 = half * cnt;
+#define RBS_TILE(NUV)                                                                                        \
+  do {                                                                                                       \
+    if (done < w.nmask)                                                                                      \
+      pair_tile32x2<KIND, true, NT, NUV>(ssx + l0, ssy + l0, ssz + l0, srx + l0, sry + l0, srz + l0, spid + l0, \
+                                         cnt, xt, nt, pt, p);                                                \
+    else                                                                                                     \
+      pair_tile32x2<KIND, false, NT, NUV>(ssx + l0, ssy + l0, ssz + l0, srx + l0, sry + l0, srz + l0, spid + l0, \
+                                          cnt, xt, nt, pt, p);                                               \
   } while (0)
       if (nu == NT) {
         RBS_TILE(NT);
       } else if constexpr (NT > 1) {
-        if (nu == 1) RBS_TILE(1);
-        if constexpr (NT > 2) {
-          if (nu == 2) RBS_TILE(2);
-          if (nu == 3) RBS_TILE(3);
-        }
+        RBS_TILE(1);
       }
 #undef RBS_TILE
       done += filled;
@@ -317,218 +412,193 @@ __global__ void __maxnreg__(NT == 1 ? 64 : (NT == 2 ? 128 : 168))
 #pragma unroll
         for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c].x + p[u][c].y);
     }
+    // clusters
+    if (seg < w.s1) {
+      __syncwarp();  // the tile's reads are done: the ring takes its place
+      int iss_seg = seg, iss_a = 0, iss_slot = 0, iss_left = (w.s1 - seg) * nq;
+      const float* iss_src = pq + (size_t)((sg.x - N) / npx) * nq * slab;
+      auto issue = [&]() {
+        if (iss_left > 0) {
+          const uint32_t dst = ring_s + iss_slot * slab * 4;
+          for (int k = lane; k < slab / 4; k += 32) cp_async16(dst + 16 * k, iss_src + 4 * k);
+          --iss_left;
+          iss_slot = iss_slot + 1 == kRing32 ? 0 : iss_slot + 1;
+          iss_src += slab;
+          if (++iss_a == nq) {
+            iss_a = 0;
+            ++iss_seg;
+            if (iss_left > 0) iss_src = pq + (size_t)((segs[iss_seg].x - N) / npx) * nq * slab;
+          }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+#pragma unroll
+      for (int k = 0; k < kRing32 - 1; ++k) issue();
+      int slot = 0;
+      for (; seg < w.s1; ++seg) {
+        const long long cell = (segs[seg].x - N) / npx;
+        __syncwarp();  // the previous cluster's coordinates are read
+        for (int k = lane; k < 3 * nq; k += 32) {
+          const float4 c4 = axis[cell * 3 * nq + k];  // hi, lo of coordinate k of its axis
+          const int ax = k / nq;
+          const float h = ax == 0 ? oh.x : (ax == 1 ? oh.y : oh.z), l = ax == 0 ? ol.x : (ax == 1 ? ol.y : ol.z);
+          sax[k] = (h - c4.x) + (l - c4.y);
+        }
+        __syncwarp();
+        float2 dz[NT][NQ2];
+#pragma unroll
+        for (int i = 0; i < NQ2; ++i) {
+          const float2 s = f2(sax[2 * nq + 2 * i], sax[2 * nq + min(2 * i + 1, nq - 1)]);
+#pragma unroll
+          for (int u = 0; u < NT; ++u) dz[u][i] = __fadd2_rn(xt[u][2], s);
+        }
+        for (int a = 0; a < nq; ++a) {
+          issue();
+          asm volatile("cp.async.wait_group %0;" ::"n"(kRing32 - 1) : "memory");
+          __syncwarp();
+          const float* row = ring + slot * slab + half * 3 * ncp;
+          float2 dx[NT], dx2[NT], rnx[NT], p[NT][3], s0x[NT], s0y[NT];
+          const float sxa = sax[a];
+#pragma unroll
+          for (int u = 0; u < NT; ++u) {
+            dx[u] = __fadd2_rn(xt[u][0], f2(sxa, sxa));
+            dx2[u] = __fmul2_rn(dx[u], dx[u]);
+            rnx[u] = __fmul2_rn(dx[u], nt[u][0]);
+            p[u][0] = p[u][1] = p[u][2] = s0x[u] = s0y[u] = f2(0.0f, 0.0f);
+          }
+          for (int b = half; b < nbp; b += split ? 2 : 1, row += (split ? 2 : 1) * 3 * ncp) {
+            const float syb = sax[nq + min(b, nq - 1)];
+            float4 q[3][(NQ2 + 1) / 2];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+              for (int i = 0; i < (NQ2 + 1) / 2; ++i) q[k][i] = *reinterpret_cast<const float4*>(row + k * ncp + 4 * i);
+#pragma unroll
+            for (int u = 0; u < NT; ++u) {
+              if (u >= nu) continue;
+              const float2 dy = __fadd2_rn(xt[u][1], f2(syb, syb));
+              const float2 sab = __ffma2_rn(dy, dy, dx2[u]);
+              const float2 rnab = __ffma2_rn(dy, nt[u][1], rnx[u]);
+              float2 s0 = f2(0.0f, 0.0f);
+#pragma unroll
+              for (int i = 0; i < NQ2; ++i) {
+                const float2 qx = (i & 1) ? f2(q[0][i / 2].z, q[0][i / 2].w) : f2(q[0][i / 2].x, q[0][i / 2].y);
+                const float2 qy = (i & 1) ? f2(q[1][i / 2].z, q[1][i / 2].w) : f2(q[1][i / 2].x, q[1][i / 2].y);
+                const float2 qz = (i & 1) ? f2(q[2][i / 2].z, q[2][i / 2].w) : f2(q[2][i / 2].x, q[2][i / 2].y);
+                const float2 d = dz[u][i];
+                const float2 r2 = __ffma2_rn(d, d, sab);
+                const float2 inv = f2(rsqrt_hw(r2.x), rsqrt_hw(r2.y));
+                const float2 rr = __ffma2_rn(d, qz, __ffma2_rn(dy, qy, __fmul2_rn(dx[u], qx)));
+                const float2 inv2 = __fmul2_rn(inv, inv);
+                const float2 inv3 = __fmul2_rn(inv2, inv);
+                float2 c;
+                if (KIND == 0) {
+                  const float2 rn = __ffma2_rn(d, nt[u][2], rnab);
+                  c = __fmul2_rn(__fmul2_rn(__fmul2_rn(rn, rr), inv2), inv3);
+                } else {
+                  c = __fmul2_rn(rr, inv3);
+                  p[u][0] = __ffma2_rn(qx, inv, p[u][0]);
+                  p[u][1] = __ffma2_rn(qy, inv, p[u][1]);
+                  p[u][2] = __ffma2_rn(qz, inv, p[u][2]);
+                }
+                s0 = __fadd2_rn(s0, c);
+                p[u][2] = __ffma2_rn(c, d, p[u][2]);
+              }
+              s0x[u] = __fadd2_rn(s0x[u], s0);
+              s0y[u] = __ffma2_rn(dy, s0, s0y[u]);
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < NT; ++u) {
+            p[u][0] = __ffma2_rn(dx[u], s0x[u], p[u][0]);
+            p[u][1] = __fadd2_rn(p[u][1], s0y[u]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c].x + p[u][c].y);
+          }
+          __syncwarp();  // every lane has read the slab before its slot is refilled
+          slot = slot + 1 == kRing32 ? 0 : slot + 1;
+        }
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
     const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
       if (!valid[u]) continue;
-      const long long t = w.t0 + wbase + 32 * u + lane;
+      const long long t = tb + 32 * u + (split ? lane & 15 : lane);
 #pragma unroll
       for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
     }
   }
 }
 
-// ---- double-float layout (the treecode of the double-float passes)
-
-constexpr int kTreeMaxQ64 = 13;  // degree <= 12
-constexpr int kChargeTile64 = 128;
-constexpr int kProxyPerThread64 = (kTreeMaxQ64 * kTreeMaxQ64 * kTreeMaxQ64 + kChargeThreads - 1) / kChargeThreads;
-
-// Weighted density of the nodes as float32 pairs: (qh, ql)[t] = split(w_t mu_t).
-__global__ void k_tree_df_node_charges(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
-                                       float4* __restrict__ qh, float4* __restrict__ ql) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= N) return;
-  const double w = x[t].w;
-  const dflt a = df_split(w * dens[3 * t]), b = df_split(w * dens[3 * t + 1]), e = df_split(w * dens[3 * t + 2]);
-  qh[t] = make_float4(a.h, b.h, e.h, 0.0f);
-  ql[t] = make_float4(a.l, b.l, e.l, 0.0f);
-}
-
-// Barycentric Lagrange basis in float64 (as lagrange_row).
-__device__ __forceinline__ void lagrange_row64(double u, const double* s, const double* bw, int nq, double* L) {
-  double t[kTreeMaxQ64];
-  double sum = 0.0;
-  int hit = -1;
-#pragma unroll
-  for (int k = 0; k < kTreeMaxQ64; ++k) {
-    t[k] = 0.0;
-    if (k < nq) {
-      const double d = u - s[k];
-      if (d == 0.0)
-        hit = k;
-      else
-        t[k] = bw[k] / d;
-      sum += t[k];
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < kTreeMaxQ64; ++k)
-    if (k < nq) L[k] = hit >= 0 ? (k == hit ? 1.0 : 0.0) : t[k] / sum;
-}
-
-// Cluster charges in float64 (as k_tree_charges, from the float64 density): q64[3 (u npx + k) + c].
-__global__ void __launch_bounds__(kChargeThreads) k_tree_charges64(const int4* __restrict__ items,
-                                                                   const int* __restrict__ order,
-                                                                   const long long* __restrict__ offset,
-                                                                   const double4* __restrict__ x,
-                                                                   const double* __restrict__ dens,
-                                                                   const double* __restrict__ box,
-                                                                   const double* __restrict__ cheb, int nq,
-                                                                   double* __restrict__ q64) {
-  constexpr int TS = kChargeTile64;
-  __shared__ double sL[3][TS][kTreeMaxQ64];
-  __shared__ double sq[TS][3];
-  __shared__ double s_pts[kTreeMaxQ64], s_bw[kTreeMaxQ64];
-  const int npx = nq * nq * nq;
-  if (threadIdx.x < nq) {
-    s_pts[threadIdx.x] = cheb[threadIdx.x];
-    s_bw[threadIdx.x] = cheb[nq + threadIdx.x];
-  }
-  const int4 it = items[blockIdx.x];
-  const int u = it.x;
-  const double m0 = box[6 * (size_t)u], m1 = box[6 * (size_t)u + 1], m2 = box[6 * (size_t)u + 2];
-  const double h0 = box[6 * (size_t)u + 3], h1 = box[6 * (size_t)u + 4], h2 = box[6 * (size_t)u + 5];
-  int ka[kProxyPerThread64], kb[kProxyPerThread64], kc[kProxyPerThread64];
-  double acc[kProxyPerThread64][3];
-#pragma unroll
-  for (int m = 0; m < kProxyPerThread64; ++m) {
-    const int k = threadIdx.x + kChargeThreads * m;
-    ka[m] = k / (nq * nq);
-    kb[m] = (k / nq) % nq;
-    kc[m] = k % nq;
-    acc[m][0] = acc[m][1] = acc[m][2] = 0.0;
-  }
-  for (int pi = it.y; pi < it.z; ++pi) {
-    const int j = order[pi];
-    const long long o = offset[j], e = offset[j + 1];
-    for (long long s0 = o; s0 < e; s0 += TS) {
-      const int cnt = (int)min((long long)TS, e - s0);
-      __syncthreads();
-      if ((int)threadIdx.x < cnt) {
-        const long long t = s0 + threadIdx.x;
-        const double4 p = x[t];
-        lagrange_row64((p.x - m0) * h0, s_pts, s_bw, nq, sL[0][threadIdx.x]);
-        lagrange_row64((p.y - m1) * h1, s_pts, s_bw, nq, sL[1][threadIdx.x]);
-        lagrange_row64((p.z - m2) * h2, s_pts, s_bw, nq, sL[2][threadIdx.x]);
-        sq[threadIdx.x][0] = p.w * dens[3 * t];
-        sq[threadIdx.x][1] = p.w * dens[3 * t + 1];
-        sq[threadIdx.x][2] = p.w * dens[3 * t + 2];
-      }
-      __syncthreads();
-      for (int l = 0; l < cnt; ++l) {
-        const double q0 = sq[l][0], q1 = sq[l][1], q2 = sq[l][2];
-#pragma unroll
-        for (int m = 0; m < kProxyPerThread64; ++m) {
-          if (threadIdx.x + kChargeThreads * m < npx) {
-            const double f = sL[0][l][ka[m]] * sL[1][l][kb[m]] * sL[2][l][kc[m]];
-            acc[m][0] = fma(f, q0, acc[m][0]);
-            acc[m][1] = fma(f, q1, acc[m][1]);
-            acc[m][2] = fma(f, q2, acc[m][2]);
-          }
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < kProxyPerThread64; ++m) {
-    const int k = threadIdx.x + kChargeThreads * m;
-    if (k < npx)
-      for (int c = 0; c < 3; ++c) atomicAdd(q64 + 3 * ((size_t)u * npx + k) + c, acc[m][c]);
-  }
-}
-
-// Float64 cluster charges to the float32 pairs the double-float kernel reads.
-__global__ void k_tree_q64_split(long long count, const double* __restrict__ q64, float4* __restrict__ qh,
-                                 float4* __restrict__ ql) {
-  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (k >= count) return;
-  const dflt a = df_split(q64[3 * k]), b = df_split(q64[3 * k + 1]), e = df_split(q64[3 * k + 2]);
-  qh[k] = make_float4(a.h, b.h, e.h, 0.0f);
-  ql[k] = make_float4(a.l, b.l, e.l, 0.0f);
-}
-
-// The double-float treecode pair sum: the packed double-float pair of the direct kernel (pairsdf.cuh)
-// over source tiles filled from the item's segments (as k_tree32x2).  KIND 0 traction into y, 1
-// Stokeslet into y, 2 traction into y and Stokeslet into y2.
-// The double-float treecode pair sum: the packed double-float pair of the direct kernel (pairsdf.cuh)
-// over source tiles filled from the item's segments (as k_tree32x2: each warp stages its own tiles, of
-// 64 sources here, and never waits for the rest of its block).  KIND 0 traction into y, 1 Stokeslet
-// into y, 2 traction into y and Stokeslet into y2.  Registers are capped (96 for one target per
-// thread) so that four 160-thread blocks, the size a p = 8 particle's targets take, are resident per
-// SM: the double-float pair is a long dependent chain, and with the uncapped 126 registers only three
-// blocks (or, at two targets per thread, 238 registers and two 96-thread blocks: under five warps per
-// SM) hid its latency.
-template <int KIND, int NT>
-__global__ void __maxnreg__(NT == 1 ? 96 : 168)
-    k_tree_df2(int nitems, const TreeItem* __restrict__ items, const int2* __restrict__ segs,
+// ---- double-float treecode pair sum: KIND 0 traction into y, 1 Stokeslet into y, 2 traction into y and
+// Stokeslet into y2.
+//
+// The same walk, one target per lane.  Nodes: the packed double-float pair of pairsdf.cuh over per-warp
+// tiles of 64 sources.  Clusters: the tensor-grid form of the float32 kernel with every product and sum
+// in double-float.  The z differences, their squares and products with n_z are kept per lane in shared
+// memory for the whole cluster, the row sums d_x^2 + d_y^2 and d_x n_x + d_y n_y in registers, so a proxy
+// pair takes 144 float32 operations (traction and Stokeslet) where the node pair takes pairsdf.cuh's.
+// Charge rows are read through L1: a warp spends thousands of cycles on each 128-byte line.
+template <int KIND>
+__global__ void __launch_bounds__(128, 4)
+    k_tree_df2(int nunits, int per_item, int* __restrict__ counter, const TreeItem* __restrict__ items,
+               const int2* __restrict__ segs, long long N, int npx, int nq, int nbp, int ncp,
                const float4* __restrict__ x3h, const float4* __restrict__ x3m, const float4* __restrict__ x3l,
-               const float4* __restrict__ nh, const float4* __restrict__ nl, const float4* __restrict__ shi,
-               const float4* __restrict__ smid, const float4* __restrict__ slo, const float4* __restrict__ sqh,
-               const float4* __restrict__ sql, double* __restrict__ y, double* __restrict__ y2) {
-  constexpr int TW = kTreeTileDf, SL = TW / 32;
+               const float4* __restrict__ nh, const float4* __restrict__ nl, const float4* __restrict__ sqh,
+               const float4* __restrict__ sql, const float4* __restrict__ axis, const float* __restrict__ pq,
+               int warp_floats, double* __restrict__ y, double* __restrict__ y2) {
   const int lane = threadIdx.x & 31;
-  const int wbase = (threadIdx.x >> 5) * 32 * NT;  // the warp's targets: wbase + 32 u + lane of the item
   extern __shared__ __align__(16) float tree_smem_df[];
-  // per warp: the tile (12 float rows and the particle ids), then the item's origin (three float4)
-  float(*sa)[TW] = reinterpret_cast<float(*)[TW]>(tree_smem_df + (threadIdx.x >> 5) * (13 * TW + 12));
-  int* const spid = reinterpret_cast<int*>(&sa[12][0]);
-  float4* const org = reinterpret_cast<float4*>(&sa[13][0]);
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const TreeItem w = items[it];
-    // target slots of this warp that hold a target (as k_tree32x2); a warp without targets skips
-    const int nu = min(NT, max(0, (w.t1 - w.t0 - wbase + 31) / 32));
-    if (nu == 0) continue;
-    __syncwarp();  // the warp's reads of the previous item's origin are done
-    if (lane == 0) {
-      org[0] = x3h[w.t0];
-      org[1] = x3m[w.t0];
-      org[2] = x3l[w.t0];
-    }
-    __syncwarp();
-    df2 xt[NT][3], nt[NT][3];
-    int pt[NT];
-    bool valid[NT];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) {
-      const int t = w.t0 + wbase + 32 * u + lane;
-      valid[u] = t < w.t1;
-      const float4 oh = org[0], om = org[1], ol = org[2];
+  float* const wsm = tree_smem_df + (threadIdx.x >> 5) * warp_floats;
+  const int nq2 = (nq + 1) / 2;
+  // clusters: per lane and pair of the last axis, (d_z, d_z^2, d_z n_z) hi and lo; then the
+  // origin-relative proxy coordinates
+  float2* const sz = reinterpret_cast<float2*>(wsm) + lane;
+  float2* const sax = reinterpret_cast<float2*>(wsm + nq2 * 6 * 64);
+  for (int unit = next_unit(counter); unit < nunits; unit = next_unit(counter)) {
+    const int item = unit / per_item;
+    const TreeItem w = items[item];
+    const int tb = w.t0 + (unit - item * per_item) * 32;
+    if (tb >= w.t1) continue;
+    const bool split = w.t1 - tb <= 16;
+    const int half = split ? lane >> 4 : 0;
+    const int t = tb + (split ? lane & 15 : lane);
+    const float4 oh = x3h[w.t0], om = x3m[w.t0], ol = x3l[w.t0];
+    const bool valid = t < w.t1;
+    dflt xt[3], nt[3], a[3], a2[3];
+    int pt = -1;
+    {
       float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
-      pt[u] = -1;
-      if (valid[u]) {
+      if (valid) {
         ah = x3h[t];
         am = x3m[t];
         al = x3l[t];
         bh = nh[t];
         bl = nl[t];
-        pt[u] = __float_as_int(ah.w);
+        pt = __float_as_int(ah.w);
       }
-      const dflt dx = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x), dy = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y),
-                 dz = df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z);
-      xt[u][0] = {dup2(dx.h), dup2(dx.l)};
-      xt[u][1] = {dup2(dy.h), dup2(dy.l)};
-      xt[u][2] = {dup2(dz.h), dup2(dz.l)};
-      nt[u][0] = {dup2(bh.x), dup2(bl.x)};
-      nt[u][1] = {dup2(bh.y), dup2(bl.y)};
-      nt[u][2] = {dup2(bh.z), dup2(bl.z)};
+      xt[0] = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x);
+      xt[1] = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y);
+      xt[2] = df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z);
+      nt[0] = {bh.x, bl.x};
+      nt[1] = {bh.y, bl.y};
+      nt[2] = {bh.z, bl.z};
     }
-    dflt a[NT][3], a2[NT][3];
+    const float xm = warp_max_abs(fmaxf(fabsf(xt[0].h), fmaxf(fabsf(xt[1].h), fabsf(xt[2].h))));
 #pragma unroll
-    for (int u = 0; u < NT; ++u)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) a[u][c] = a2[u][c] = dflt{0.0f, 0.0f};
+    for (int c = 0; c < 3; ++c) a[c] = a2[c] = dflt{0.0f, 0.0f};
     int seg = w.s0, off = 0, done = 0;
-    while (seg < w.s1) {
-      int sidx[SL];
-#pragma unroll
-      for (int k = 0; k < SL; ++k) sidx[k] = 0;
+    int2 sg = segs[seg];
+    // nodes
+    while (seg < w.s1 && sg.x < N) {
+      int sidx[2] = {0, 0};
       int filled = 0;
-      while (filled < TW && seg < w.s1) {
-        const int2 sg = segs[seg];
-        const int take = min(sg.y - off, TW - filled);
+      while (filled < kTileDf && seg < w.s1 && sg.x < N) {
+        const int take = min(sg.y - off, kTileDf - filled);
 #pragma unroll
-        for (int k = 0; k < SL; ++k) {
+        for (int k = 0; k < 2; ++k) {
           const int l = lane + 32 * k;
           if (l >= filled && l < filled + take) sidx[k] = sg.x + off + (l - filled);
         }
@@ -537,86 +607,128 @@ __global__ void __maxnreg__(NT == 1 ? 96 : 168)
         if (off >= sg.y) {
           ++seg;
           off = 0;
+          if (seg < w.s1) sg = segs[seg];
         }
       }
-      const int cnt2 = (filled + 1) & ~1;
-      __syncwarp();  // the warp's reads of the previous tile are done
-#pragma unroll 1
-      for (int k = 0; k < SL; ++k) {
-        const int l = lane + 32 * k;
-        if (l < filled) {
-          const int s = sidx[k];
-          const float4 ph = shi[s], pm = smid[s], pl = slo[s], qh = sqh[s], ql = sql[s];
-          const float4 oh = org[0], om = org[1], ol = org[2];
-          const dflt px = df_diff3(ph.x, pm.x, pl.x, oh.x, om.x, ol.x);
-          const dflt py = df_diff3(ph.y, pm.y, pl.y, oh.y, om.y, ol.y);
-          const dflt pz = df_diff3(ph.z, pm.z, pl.z, oh.z, om.z, ol.z);
-          sa[0][l] = px.h;
-          sa[1][l] = px.l;
-          sa[2][l] = py.h;
-          sa[3][l] = py.l;
-          sa[4][l] = pz.h;
-          sa[5][l] = pz.l;
-          sa[6][l] = qh.x;
-          sa[7][l] = ql.x;
-          sa[8][l] = qh.y;
-          sa[9][l] = ql.y;
-          sa[10][l] = qh.z;
-          sa[11][l] = ql.z;
-          spid[l] = __float_as_int(ph.w);
-        } else if (l < cnt2) {
-          sa[0][l] = sa[2][l] = sa[4][l] = 1.0e4f;
-          sa[1][l] = sa[3][l] = sa[5][l] = 0.0f;
-          for (int q = 6; q < 12; ++q) sa[q][l] = 0.0f;
-          spid[l] = -2;
-        }
+      df_tile<KIND>(wsm, sidx, filled, done < w.nmask, split, half, x3h, x3m, x3l, sqh, sql, oh, om, ol, xt, nt, xm,
+                    pt, a, a2);
+      done += filled;
+    }
+    // clusters
+    for (; seg < w.s1; ++seg) {
+      const long long cell = (segs[seg].x - N) / npx;
+      __syncwarp();  // the reads of the tile or of the previous cluster are done
+      for (int k = lane; k < 3 * nq; k += 32) {
+        const float4 c4 = axis[cell * 3 * nq + k];
+        const int ax = k / nq;
+        const float h = ax == 0 ? oh.x : (ax == 1 ? oh.y : oh.z), m = ax == 0 ? om.x : (ax == 1 ? om.y : om.z),
+                    l = ax == 0 ? ol.x : (ax == 1 ? ol.y : ol.z);
+        const dflt v = df_diff3(c4.x, c4.y, c4.z, h, m, l);
+        sax[k] = make_float2(v.h, v.l);
       }
       __syncwarp();
-      const bool masked = done < w.nmask;
-      df2 acc[NT][3], acc2[NT][3];
+      for (int c = 0; c < 2 * nq2; ++c) {
+        const dflt d = df_sub(xt[2], sax[2 * nq + min(c, nq - 1)]);
+        const dflt z2 = df_sqr(d), zn = df_renorm(df_mul(d, nt[2]));
+        float* dst = reinterpret_cast<float*>(sz + (c / 2) * 6 * 32) + (c & 1);
+        dst[0] = d.h;
+        dst[64] = d.l;
+        dst[128] = z2.h;
+        dst[192] = z2.l;
+        dst[256] = zn.h;
+        dst[320] = zn.l;
+      }
+      const float* row0 = pq + (size_t)cell * nq * nbp * 7 * ncp;
+      df2 accf[3], acckz, accsz;
 #pragma unroll
-      for (int u = 0; u < NT; ++u)
+      for (int c = 0; c < 3; ++c) accf[c] = df2{dup2(0.0f), dup2(0.0f)};
+      acckz = accsz = df2{dup2(0.0f), dup2(0.0f)};
+      int since = 0;
+      for (int ia = 0; ia < nq; ++ia) {
+        const dflt dx = df_sub(xt[0], sax[ia]);
+        const dflt x2 = df_sqr(dx), xn = df_mul(dx, nt[0]);
+        for (int b = half; b < nbp; b += split ? 2 : 1) {
+          const dflt dy = df_sub(xt[1], sax[nq + min(b, nq - 1)]);
+          const dflt sab = df_add(x2, df_sqr(dy));
+          const dflt rnab = df_add(xn, df_mul(dy, nt[1]));
+          const float2 sh = dup2(sab.h), sl = dup2(sab.l), rh = dup2(rnab.h), rl = dup2(rnab.l);
+          const df2 dx2 = {dup2(dx.h), dup2(dx.l)}, dy2 = {dup2(dy.h), dup2(dy.l)};
+          const float* row = row0 + (size_t)(ia * nbp + b) * 7 * ncp;
+          df2 s0k = {dup2(0.0f), dup2(0.0f)}, s0s = {dup2(0.0f), dup2(0.0f)};
+#pragma unroll 1
+          for (int i = 0; i < nq2; ++i) {
+            const float2* z = sz + i * 6 * 32;
+            const df2 d = {z[0], z[32]};
+            df2 den[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) acc[u][c] = acc2[u][c] = df2{dup2(0.0f), dup2(0.0f)};
-      for (int l = 0; l < cnt2; l += 2) {
-        df2 ys[3], den[3];
+            for (int c = 0; c < 3; ++c)
+              den[c] = {__ldg(reinterpret_cast<const float2*>(row + c * ncp) + i),
+                        __ldg(reinterpret_cast<const float2*>(row + (3 + c) * ncp) + i)};
+            const float2 fb = __ldg(reinterpret_cast<const float2*>(row + 6 * ncp) + i);
+            df2 r2 = two_sum2(sh, z[64]);
+            r2.l = __fadd2_rn(r2.l, __fadd2_rn(sl, z[96]));
+            const float2 y0 = make_float2(rsqrt_hw(r2.h.x), rsqrt_hw(r2.h.y));
+            const inv_powers p(r2.h, r2.l, y0);
+            const df2 rr = bdot2(dx2, den[0], dy2, den[1], d, den[2], __fmul2_rn(__fmul2_rn(r2.h, y0), fb));
+            const df2 am = mul2(rr, p.y3());  // r . q / r^3 but for the series
+            if (KIND != 1) {
+              df2 rn = two_sum2(rh, z[128]);
+              rn.l = __fadd2_rn(rn.l, __fadd2_rn(rl, z[160]));
+              df2 ck = mul2(am, mul2(rn, df2{p.q, p.qe}));
+              ck.l = __ffma2_rn(p.w5(), ck.h, ck.l);
+              acc2_add(s0k, ck);
+              acc2_add(acckz, mul2(ck, d));
+            }
+            if (KIND != 0) {
+              const df2 cs = {am.h, __ffma2_rn(p.w3(), am.h, am.l)};
+              const df2 inv = p.inv();
+              acc2_add(s0s, cs);
+              acc2_add(accsz, mul2(cs, d));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          ys[c] = {*reinterpret_cast<const float2*>(&sa[2 * c][l]), *reinterpret_cast<const float2*>(&sa[2 * c + 1][l])};
-          den[c] = {*reinterpret_cast<const float2*>(&sa[6 + 2 * c][l]),
-                    *reinterpret_cast<const float2*>(&sa[7 + 2 * c][l])};
-        }
-        const int2 pp = *reinterpret_cast<const int2*>(&spid[l]);
+              for (int c = 0; c < 3; ++c) acc2_add(accf[c], mul2(den[c], inv));
+            }
+          }
+          if (KIND != 1) {
+            const dflt s = fold2(s0k);
+            df_acc(a[0], df_mul(s, dx));
+            df_acc(a[1], df_mul(s, dy));
+          }
+          if (KIND != 0) {
+            dflt(&as)[3] = KIND == 2 ? a2 : a;
+            const dflt s = fold2(s0s);
+            df_acc(as[0], df_mul(s, dx));
+            df_acc(as[1], df_mul(s, dy));
+          }
+          // the packed sums go to the totals every few rows, about 64 sources as for node tiles
+          if (++since == 5 || (ia == nq - 1 && b + (split ? 2 : 1) >= nbp)) {
+            since = 0;
+            if (KIND != 1) {
+              a[2] = df_add_accurate(a[2], fold2(acckz));
+              a[0] = df_renorm(a[0]);
+              a[1] = df_renorm(a[1]);
+              acckz = df2{dup2(0.0f), dup2(0.0f)};
+            }
+            if (KIND != 0) {
+              dflt(&as)[3] = KIND == 2 ? a2 : a;
+              as[2] = df_add_accurate(as[2], fold2(accsz));
+              accsz = df2{dup2(0.0f), dup2(0.0f)};
 #pragma unroll
-        for (int u = 0; u < NT; ++u) {
-          if (u < nu) {
-            if (masked)
-              pair2_df<KIND, true>(ys, den, pp, xt[u], nt[u], pt[u], acc[u], acc2[u]);
-            else
-              pair2_df<KIND, false>(ys, den, pp, xt[u], nt[u], pt[u], acc[u], acc2[u]);
+              for (int c = 0; c < 3; ++c) {
+                as[c] = df_add_accurate(df_renorm(as[c]), fold2(accf[c]));
+                accf[c] = df2{dup2(0.0f), dup2(0.0f)};
+              }
+            }
           }
         }
       }
-      done += filled;
-#pragma unroll
-      for (int u = 0; u < NT; ++u)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          a[u][c] = df_add_accurate(a[u][c], fold2(acc[u][c]));
-          if (KIND == 2) a2[u][c] = df_add_accurate(a2[u][c], fold2(acc2[u][c]));
-        }
     }
     const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
-#pragma unroll
-    for (int u = 0; u < NT; ++u) {
-      if (!valid[u]) continue;
-      const long long t = w.t0 + wbase + 32 * u + lane;
+    if (valid)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        atomicAdd(y + 3 * t + c, sc * ((double)a[u][c].h + (double)a[u][c].l));
-        if (KIND == 2) atomicAdd(y2 + 3 * t + c, kStokesletScale * ((double)a2[u][c].h + (double)a2[u][c].l));
+        atomicAdd(y + 3 * (long long)t + c, sc * ((double)a[c].h + (double)a[c].l));
+        if (KIND == 2) atomicAdd(y2 + 3 * (long long)t + c, kStokesletScale * ((double)a2[c].h + (double)a2[c].l));
       }
-    }
   }
 }
 
@@ -722,13 +834,13 @@ struct TreeBuilder {
 void TreeState::release() {
   active = false;
   tmax = 0;
-  nt[0] = nt[1] = nt[2] = 0;
   n_cells = 0;
   n_src = 0;
   items.clear();
   segs.clear();
   charge_items.clear();
-  for (DevBuf<float4>* b : {&d_hi, &d_lo, &d_q, &d_x3m, &d_wl}) b->release();
+  d_axis.release();
+  d_pq.release();
   d_items.release();
   d_segs.release();
   d_charge_items.release();
@@ -902,6 +1014,11 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
   T.corder.clear();
   T.charge_items.clear();
   T.charge_work = 0;
+  // nodes per charge block: about eight blocks per SM over all clusters, between 256 nodes (below,
+  // the atomic additions of a block's (n + 1)^3 partial charges outweigh its work) and 4,096
+  long long cell_nodes = 0;
+  for (int u = 0; u < n_used; ++u) cell_nodes += cells[used_cells[u]].nodes;
+  const long long run = std::min(4096LL, std::max(256LL, cell_nodes / (8LL * std::max(1, c.sm_count))));
   for (int u = 0; u < n_used; ++u) {
     const HCell& C = cells[used_cells[u]];
     double mid[3], half[3];
@@ -919,12 +1036,12 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
           T.proxy[3 * k + 1] = mid[1] + half[1] * std::cos(b * kPi / degree);
           T.proxy[3 * k + 2] = mid[2] + half[2] * std::cos(e * kPi / degree);
         }
-    // charge blocks over the cell's particles, about 4,096 nodes each
+    // charge blocks over the cell's particles
     int q = C.pb;
     while (q < C.pe) {
       const int first = (int)T.corder.size();
       long long nodes = 0;
-      while (q < C.pe && (nodes == 0 || nodes + (c.offset[order[q] + 1] - c.offset[order[q]]) <= 4096)) {
+      while (q < C.pe && (nodes == 0 || nodes + (c.offset[order[q] + 1] - c.offset[order[q]]) <= run)) {
         nodes += c.offset[order[q] + 1] - c.offset[order[q]];
         T.corder.push_back(order[q]);
         ++q;
@@ -943,7 +1060,6 @@ static Status build_lists(Context& c, TreeState& T, const std::vector<double>& p
                           bool df) {
   cudaStream_t s = c.stream;
   const int nq = degree + 1, npx = nq * nq * nq;
-  const long long N = c.N;
   std::vector<double> radius(c.n);
   for (int i = 0; i < c.n; ++i) radius[i] = c.shapes[c.shape_of[i]].radius;
   const PlanInput in{c.n, c.offset.data(), c.centres.data(), radius.data(), c.sid.data(), pbox.data(),
@@ -954,7 +1070,6 @@ static Status build_lists(Context& c, TreeState& T, const std::vector<double>& p
   T.npx = npx;
   T.theta = theta;
   T.df = df;
-  if (P.tmax != T.tmax) T.nt[0] = T.nt[1] = T.nt[2] = 0;  // the block shape changed: time the variants again
   T.tmax = P.tmax;
   T.n_cells = P.n_cells;
   T.n_src = P.n_src;
@@ -967,35 +1082,24 @@ static Status build_lists(Context& c, TreeState& T, const std::vector<double>& p
   const int n_used = P.n_cells;
   std::vector<double>& box = P.box;
   std::vector<int>& corder = P.corder;
-  std::vector<float4> phi((size_t)n_used * npx), plo((size_t)n_used * npx), pm(df ? (size_t)n_used * npx : 0);
   std::vector<double> cheb(2 * (size_t)nq);
   for (int k = 0; k < nq; ++k) {
     cheb[k] = std::cos(k * kPi / degree);
     cheb[nq + k] = ((k & 1) ? -1.0 : 1.0) * ((k == 0 || k == degree) ? 0.5 : 1.0);
   }
-  // proxy points carry kProxyPid in the w bits of their hi position, like a node's particle id
-  float proxy_w;
-  {
-    const int v = kProxyPid;
-    std::memcpy(&proxy_w, &v, sizeof(float));
-  }
-  for (size_t k = 0; k < (size_t)n_used * npx; ++k) {
-    float h[3], m[3], l[3];
+  // the proxy grid's coordinates per cluster and axis, as exact three-float splits
+  std::vector<float4> axis(3 * (size_t)n_used * nq);
+  for (int u = 0; u < n_used; ++u)
     for (int d = 0; d < 3; ++d) {
-      const double v = P.proxy[3 * k + d];
-      h[d] = (float)v;
-      const double r = v - (double)h[d];
-      m[d] = (float)r;
-      l[d] = df ? (float)(r - (double)m[d]) : 0.0f;
+      const size_t stride = d == 0 ? (size_t)nq * nq : (d == 1 ? (size_t)nq : 1);
+      for (int k = 0; k < nq; ++k) {
+        const double v = P.proxy[3 * ((size_t)u * npx + k * stride) + d];
+        const float h = (float)v;
+        const double r = v - (double)h;
+        const float m = (float)r;
+        axis[((size_t)u * 3 + d) * nq + k] = make_float4(h, m, (float)(r - (double)m), 0.0f);
+      }
     }
-    phi[k] = make_float4(h[0], h[1], h[2], proxy_w);
-    if (df) {  // exact three-float split, as the nodes' x3h / x3m / x3l
-      pm[k] = make_float4(m[0], m[1], m[2], 0.0f);
-      plo[k] = make_float4(l[0], l[1], l[2], 0.0f);
-    } else {   // float32 hi + lo, as the nodes' xhi / xlo
-      plo[k] = make_float4(m[0], m[1], m[2], 0.0f);
-    }
-  }
 
   // 6. device copies
   RBS_TRY(upload_vec(T.d_items, T.items, s));
@@ -1009,25 +1113,13 @@ static Status build_lists(Context& c, TreeState& T, const std::vector<double>& p
       RBS_TRY(upload_vec(T.d_cheb64, cheb, s));
     else
       RBS_TRY(upload_vec(T.d_cheb, cheb32, s));
-    RBS_TRY(T.d_hi.alloc(T.n_src));
-    RBS_TRY(T.d_lo.alloc(T.n_src));
-    RBS_TRY(T.d_q.alloc(T.n_src));  // float32 charges, or the hi parts of the double-float ones
-    const float4* node_hi = df ? c.d_x3h.ptr : c.d_xhi.ptr;
-    const float4* node_lo = df ? c.d_x3l.ptr : c.d_xlo.ptr;
-    RBS_CUDA_TRY(cudaMemcpyAsync(T.d_hi.ptr, node_hi, sizeof(float4) * N, cudaMemcpyDeviceToDevice, s));
-    RBS_CUDA_TRY(cudaMemcpyAsync(T.d_lo.ptr, node_lo, sizeof(float4) * N, cudaMemcpyDeviceToDevice, s));
-    if (df) {
-      RBS_TRY(T.d_x3m.alloc(T.n_src));
-      RBS_TRY(T.d_wl.alloc(T.n_src));
-      RBS_TRY(T.d_q64.alloc(std::max<size_t>(1, 3 * (size_t)n_used * npx)));
-      RBS_CUDA_TRY(cudaMemcpyAsync(T.d_x3m.ptr, c.d_x3m.ptr, sizeof(float4) * N, cudaMemcpyDeviceToDevice, s));
-    }
-    if (n_used > 0) {
-      RBS_CUDA_TRY(cudaMemcpyAsync(T.d_hi.ptr + N, phi.data(), sizeof(float4) * phi.size(), cudaMemcpyHostToDevice, s));
-      RBS_CUDA_TRY(cudaMemcpyAsync(T.d_lo.ptr + N, plo.data(), sizeof(float4) * plo.size(), cudaMemcpyHostToDevice, s));
-      if (df)
-        RBS_CUDA_TRY(cudaMemcpyAsync(T.d_x3m.ptr + N, pm.data(), sizeof(float4) * pm.size(), cudaMemcpyHostToDevice, s));
-    }
+    RBS_TRY(upload_vec(T.d_axis, axis, s));
+    // rows of the last proxy axis padded to a multiple of four charges, planes to an even row count
+    T.nbp = (nq + 1) & ~1;
+    T.ncp = (nq + 3) & ~3;
+    const size_t rows = (size_t)n_used * nq * T.nbp;
+    RBS_TRY(T.d_pq.alloc(std::max<size_t>(1, rows * (df ? 7 : 3) * T.ncp)));
+    if (df) RBS_TRY(T.d_q64.alloc(std::max<size_t>(1, rows * 3 * T.ncp)));
     // the host vectors above must outlive their copies
     RBS_CUDA_TRY(cudaStreamSynchronize(s));
   }
@@ -1070,199 +1162,125 @@ Status build_far_field(Context& c) {
   return Status::Ok();
 }
 
-// Launch of the treecode pair sum over the first `items` work items with nt targets per thread,
-// blocks just large enough for the largest item.
-static Status launch_tree(Context& c, int kind, int nt, int items, double* y) {
+// Blocks of the persistent grid: what the SMs hold at once.
+static int tree_grid(Context& c, const void* kernel, size_t smem, long long units) {
+  if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 128, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+  return (int)std::max(1LL, std::min<long long>((units + 3) / 4, (long long)per_sm * std::max(1, c.sm_count)));
+}
+
+template <int KIND, int NT, int NQ2>
+static Status launch_tree(Context& c, double* y) {
   TreeState& T = c.tree;
-  const int threads = ((T.tmax + nt - 1) / nt + 31) / 32 * 32;
-  const size_t smem = (size_t)(threads / 32) * 7 * kTreeTile32 * sizeof(float);  // one tile per warp
-#define RBS_TREE_ARGS items, T.d_items.ptr, T.d_segs.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, T.d_hi.ptr, T.d_lo.ptr, \
-                      T.d_q.ptr, y
-  auto grid = [&](const void* k) {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
-    return std::max(1, std::min(items, per_sm * std::max(1, c.sm_count)));
-  };
-  if (kind == 0) {
-    if (nt == 1)
-      k_tree32x2<0, 1><<<grid((const void*)k_tree32x2<0, 1>), threads, smem, c.stream>>>(RBS_TREE_ARGS);
-    else if (nt == 4)
-      k_tree32x2<0, 4><<<grid((const void*)k_tree32x2<0, 4>), threads, smem, c.stream>>>(RBS_TREE_ARGS);
-    else
-      k_tree32x2<0, 2><<<grid((const void*)k_tree32x2<0, 2>), threads, smem, c.stream>>>(RBS_TREE_ARGS);
-  } else {
-    if (nt == 1)
-      k_tree32x2<1, 1><<<grid((const void*)k_tree32x2<1, 1>), threads, smem, c.stream>>>(RBS_TREE_ARGS);
-    else if (nt == 4)
-      k_tree32x2<1, 4><<<grid((const void*)k_tree32x2<1, 4>), threads, smem, c.stream>>>(RBS_TREE_ARGS);
-    else
-      k_tree32x2<1, 2><<<grid((const void*)k_tree32x2<1, 2>), threads, smem, c.stream>>>(RBS_TREE_ARGS);
-  }
-#undef RBS_TREE_ARGS
+  const int nq = T.degree + 1;
+  const int slab = 3 * T.nbp * T.ncp;
+  const int warp_floats = std::max(7 * kTreeTile32, (kRing32 * slab + 3 * nq + 3) & ~3);
+  const size_t smem = 4 * (size_t)warp_floats * sizeof(float);
+  const int per_item = (T.tmax + 32 * NT - 1) / (32 * NT);
+  const long long units = (long long)T.items.size() * per_item;
+  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "treecode: more than 2^31 work units");
+  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
+  const auto kernel = k_tree32x2<KIND, NT, NQ2>;
+  kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
+      (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_xhi.ptr,
+      c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, T.d_axis.ptr, T.d_pq.ptr, warp_floats, y);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
 
-// Targets per thread of the treecode pair sum: rbs_options.pair_variant when set (its targets per
-// thread), otherwise the fastest of 1, 2 and 4 timed once per geometry and kind on a prefix of the
-// work items (the charges of the current apply as sources, into a scratch output).
-static int tree_variant(Context& c, int kind) {
-  TreeState& T = c.tree;
-  if (c.opt.pair_variant > 0) {
-    const int v = c.opt.pair_variant > kPacked ? c.opt.pair_variant - kPacked : c.opt.pair_variant;
-    return (v == 1 || v == 4) ? v : 2;
+template <int KIND>
+static Status launch_tree(Context& c, double* y) {
+  const int nq2 = (c.tree.degree + 2) / 2;  // pairs of the last proxy axis; degree 2 to 10
+  if (tree_variant(c) == 2) {
+    if (nq2 == 2) return launch_tree<KIND, 2, 2>(c, y);
+    return nq2 == 3 ? launch_tree<KIND, 2, 3>(c, y) : launch_tree<KIND, 2, 4>(c, y);
   }
-  if (T.nt[kind]) return T.nt[kind];
-  int best = 2;
-  const int items = std::min<int>((int)T.items.size(), 8 * std::max(1, c.sm_count));
-  double* scratch = nullptr;
-  cudaEvent_t a = nullptr, b = nullptr;
-  if (cudaMalloc(&scratch, sizeof(double) * 3 * c.N) == cudaSuccess && cudaEventCreate(&a) == cudaSuccess &&
-      cudaEventCreate(&b) == cudaSuccess) {
-    float best_ms = 1e30f;
-    for (int nt : {1, 2, 4}) {
-      if (((T.tmax + nt - 1) / nt + 31) / 32 * 32 > kTreeMaxTargets / nt) continue;  // block too large
-      if (!launch_tree(c, kind, nt, items, scratch).ok()) continue;  // warm
-      cudaEventRecord(a, c.stream);
-      if (!launch_tree(c, kind, nt, items, scratch).ok()) continue;
-      cudaEventRecord(b, c.stream);
-      float ms = 0.0f;
-      if (cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&ms, a, b) == cudaSuccess && ms < best_ms) {
-        best_ms = ms;
-        best = nt;
-      }
-      c.stats.launches += 2;
-    }
+  switch (nq2) {
+    case 2: return launch_tree<KIND, 1, 2>(c, y);
+    case 3: return launch_tree<KIND, 1, 3>(c, y);
+    case 4: return launch_tree<KIND, 1, 4>(c, y);
+    case 5: return launch_tree<KIND, 1, 5>(c, y);
+    default: return launch_tree<KIND, 1, 6>(c, y);
   }
-  if (a) cudaEventDestroy(a);
-  if (b) cudaEventDestroy(b);
-  if (scratch) cudaFree(scratch);
-  cudaGetLastError();
-  T.nt[kind] = best;
-  return best;
 }
 
-Status apply_tree(Context& c, int kind, const double* x, double* y, int nt) {
+// Targets per lane of the float32 treecode sum: two, which share the loads of each charge row and tile
+// (1,740 against 1,620 Gpair/s on 1,500 particles of 144 nodes, 1,810 against 1,640 on 700 of 312), unless
+// rbs_options.pair_variant asks for one; one above degree 7, where the z differences of two targets no
+// longer fit in registers.
+int tree_variant(const Context& c) {
+  return c.tree.degree > 7 || c.opt.pair_variant == 1 || c.opt.pair_variant == kPacked + 1 ? 1 : 2;
+}
+
+Status apply_tree(Context& c, int kind, const double* x, double* y) {
   TreeState& T = c.tree;
-  const long long N = c.N;
   {
     KernelTimer timer(c, RBS_KC_TREE);
-    k_tree_node_charges<<<cdiv(N, 256), 256, 0, c.stream>>>(N, c.d_x.ptr, x, T.d_q.ptr);
-    int launches = 1;
+    int launches = 0;
     if (T.n_cells > 0) {
-      RBS_CUDA_TRY(cudaMemsetAsync(T.d_q.ptr + N, 0, sizeof(float4) * (size_t)T.n_cells * T.npx, c.stream));
-      k_tree_charges<<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
-          T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, T.d_q.ptr, T.d_box.ptr, T.d_cheb.ptr,
-          T.degree + 1, T.d_q.ptr + N);
+      RBS_CUDA_TRY(cudaMemsetAsync(T.d_pq.ptr, 0, sizeof(float) * T.d_pq.n, c.stream));
+      const int nq = T.degree + 1;
+      if (nq <= 8)
+        k_tree_charges<float, 8, 2><<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
+            T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb.ptr, nq, T.nbp,
+            T.ncp, T.d_pq.ptr);
+      else
+        k_tree_charges<float, kTreeMaxQ, 2><<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
+            T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb.ptr, nq, T.nbp,
+            T.ncp, T.d_pq.ptr);
+      launches = 1;
+    }
+    RBS_CUDA_TRY(cudaGetLastError());
+    timer.done((double)T.charge_work, launches);
+  }
+  if (T.items.empty()) return Status::Ok();
+  KernelTimer timer(c, kind == 0 ? RBS_KC_PAIR_K32 : RBS_KC_PAIR_S32);
+  RBS_TRY(kind == 0 ? launch_tree<0>(c, y) : launch_tree<1>(c, y));
+  timer.done((double)(T.direct_pairs + T.proxy_pairs));
+  return Status::Ok();
+}
+
+template <int KIND>
+static Status launch_tree_df(Context& c, double* y, double* y2) {
+  TreeState& T = c.tree_df;
+  const int nq = T.degree + 1;
+  const int warp_floats = std::max(kTileDfFloats, ((nq + 1) / 2 * 6 * 64 + 6 * nq + 3) & ~3);
+  const size_t smem = 4 * (size_t)warp_floats * sizeof(float);
+  const int per_item = (T.tmax + 31) / 32;
+  const long long units = (long long)T.items.size() * per_item;
+  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "treecode: more than 2^31 work units");
+  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
+  const auto kernel = k_tree_df2<KIND>;
+  kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
+      (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_x3h.ptr,
+      c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, c.d_wmuh.ptr, c.d_wmul.ptr, T.d_axis.ptr, T.d_pq.ptr,
+      warp_floats, y, y2);
+  RBS_CUDA_TRY(cudaGetLastError());
+  return Status::Ok();
+}
+
+Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y2) {
+  TreeState& T = c.tree_df;
+  {
+    KernelTimer timer(c, RBS_KC_TREE);
+    int launches = 0;
+    if (T.n_cells > 0) {
+      const int nq = T.degree + 1;
+      const long long rows = (long long)T.n_cells * nq * T.nbp;
+      RBS_CUDA_TRY(cudaMemsetAsync(T.d_q64.ptr, 0, sizeof(double) * T.d_q64.n, c.stream));
+      k_tree_charges<double, kTreeMaxQ64, 1><<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
+          T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb64.ptr, nq, T.nbp,
+          T.ncp, T.d_q64.ptr);
+      k_tree_q64_split<<<cdiv(rows * T.ncp, 256), 256, 0, c.stream>>>(rows, T.ncp, T.d_q64.ptr, T.d_pq.ptr);
       launches = 2;
     }
     RBS_CUDA_TRY(cudaGetLastError());
     timer.done((double)T.charge_work, launches);
   }
-  const int items = (int)T.items.size();
-  if (items == 0) return Status::Ok();
-  if (nt <= 0) nt = tree_variant(c, kind);
-  KernelTimer timer(c, kind == 0 ? RBS_KC_PAIR_K32 : RBS_KC_PAIR_S32);
-  RBS_TRY(launch_tree(c, kind, nt, items, y));
-  RBS_CUDA_TRY(cudaGetLastError());
-  timer.done((double)(T.direct_pairs + T.proxy_pairs));
-  return Status::Ok();
-}
-
-// Launch of the double-float treecode pair sum over the first `items` work items.
-static Status launch_tree_df(Context& c, int kind, int nt, int items, double* y, double* y2) {
-  TreeState& T = c.tree_df;
-  const int threads = ((T.tmax + nt - 1) / nt + 31) / 32 * 32;
-  const size_t smem = (size_t)(threads / 32) * (13 * kTreeTileDf + 12) * sizeof(float);  // one tile per warp
-#define RBS_TREE_DF_ARGS items, T.d_items.ptr, T.d_segs.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, \
-                         c.d_nrml.ptr, T.d_hi.ptr, T.d_x3m.ptr, T.d_lo.ptr, T.d_q.ptr, T.d_wl.ptr, y, y2
-  auto grid = [&](const void* k) {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
-    return std::max(1, std::min(items, per_sm * std::max(1, c.sm_count)));
-  };
-  if (kind == 0) {
-    if (nt == 1)
-      k_tree_df2<0, 1><<<grid((const void*)k_tree_df2<0, 1>), threads, smem, c.stream>>>(RBS_TREE_DF_ARGS);
-    else
-      k_tree_df2<0, 2><<<grid((const void*)k_tree_df2<0, 2>), threads, smem, c.stream>>>(RBS_TREE_DF_ARGS);
-  } else if (kind == 1) {
-    if (nt == 1)
-      k_tree_df2<1, 1><<<grid((const void*)k_tree_df2<1, 1>), threads, smem, c.stream>>>(RBS_TREE_DF_ARGS);
-    else
-      k_tree_df2<1, 2><<<grid((const void*)k_tree_df2<1, 2>), threads, smem, c.stream>>>(RBS_TREE_DF_ARGS);
-  } else {
-    if (nt == 1)
-      k_tree_df2<2, 1><<<grid((const void*)k_tree_df2<2, 1>), threads, smem, c.stream>>>(RBS_TREE_DF_ARGS);
-    else
-      k_tree_df2<2, 2><<<grid((const void*)k_tree_df2<2, 2>), threads, smem, c.stream>>>(RBS_TREE_DF_ARGS);
-  }
-#undef RBS_TREE_DF_ARGS
-  RBS_CUDA_TRY(cudaGetLastError());
-  return Status::Ok();
-}
-
-// Targets per thread of the double-float treecode pair sum: 1 or 2, timed once per configuration and
-// kind on a prefix of the work items (the current charges as sources, into scratch outputs).
-static int tree_df_variant(Context& c, int kind) {
-  TreeState& T = c.tree_df;
-  if (c.opt.pair_variant > 0) return (c.opt.pair_variant == 2 || c.opt.pair_variant == kPacked + 2) ? 2 : 1;
-  if (T.nt[kind]) return T.nt[kind];
-  int best = 1;
-  // a prefix of eight items per SM: whole rounds of the persistent grid for either variant
-  const int items = std::min<int>((int)T.items.size(), 8 * std::max(1, c.sm_count));
-  double* scratch = nullptr;
-  cudaEvent_t a = nullptr, b = nullptr;
-  if (cudaMalloc(&scratch, sizeof(double) * 6 * c.N) == cudaSuccess && cudaEventCreate(&a) == cudaSuccess &&
-      cudaEventCreate(&b) == cudaSuccess) {
-    float best_ms = 1e30f;
-    for (int nt : {1, 2}) {
-      if (!launch_tree_df(c, kind, nt, items, scratch, scratch + 3 * c.N).ok()) continue;  // warm
-      cudaEventRecord(a, c.stream);
-      if (!launch_tree_df(c, kind, nt, items, scratch, scratch + 3 * c.N).ok()) continue;
-      cudaEventRecord(b, c.stream);
-      float ms = 0.0f;
-      if (cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&ms, a, b) == cudaSuccess && ms < best_ms) {
-        best_ms = ms;
-        best = nt;
-      }
-      c.stats.launches += 2;
-    }
-  }
-  if (a) cudaEventDestroy(a);
-  if (b) cudaEventDestroy(b);
-  if (scratch) cudaFree(scratch);
-  cudaGetLastError();
-  T.nt[kind] = best;
-  return best;
-}
-
-Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y2) {
-  TreeState& T = c.tree_df;
-  const long long N = c.N;
-  {
-    KernelTimer timer(c, RBS_KC_TREE);
-    k_tree_df_node_charges<<<cdiv(N, 256), 256, 0, c.stream>>>(N, c.d_x.ptr, x, T.d_q.ptr, T.d_wl.ptr);
-    int launches = 1;
-    if (T.n_cells > 0) {
-      const long long np = (long long)T.n_cells * T.npx;
-      RBS_CUDA_TRY(cudaMemsetAsync(T.d_q64.ptr, 0, sizeof(double) * 3 * (size_t)np, c.stream));
-      k_tree_charges64<<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
-          T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb64.ptr,
-          T.degree + 1, T.d_q64.ptr);
-      k_tree_q64_split<<<cdiv(np, 256), 256, 0, c.stream>>>(np, T.d_q64.ptr, T.d_q.ptr + N, T.d_wl.ptr + N);
-      launches = 3;
-    }
-    RBS_CUDA_TRY(cudaGetLastError());
-    timer.done((double)T.charge_work, launches);
-  }
-  const int items = (int)T.items.size();
-  if (items == 0) return Status::Ok();
-  const int nt = tree_df_variant(c, kind);
+  if (T.items.empty()) return Status::Ok();
   KernelTimer timer(c, kind == 0 ? RBS_KC_PAIR_KDF : (kind == 1 ? RBS_KC_PAIR_SDF : RBS_KC_PAIR_KSDF));
-  RBS_TRY(launch_tree_df(c, kind, nt, items, y, y2));
+  RBS_TRY(kind == 0 ? launch_tree_df<0>(c, y, y2) : (kind == 1 ? launch_tree_df<1>(c, y, y2) : launch_tree_df<2>(c, y, y2)));
   timer.done((double)(T.direct_pairs + T.proxy_pairs));
   return Status::Ok();
 }
