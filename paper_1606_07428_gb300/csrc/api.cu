@@ -511,7 +511,7 @@ int rbs_get_stats(rbs_ctx* h, rbs_stats* out) {
   if (s.ok()) s = c.harvest();
   if (!s.ok()) return finish(c, s);
   *out = c.stats;
-  for (int k = 0; k < 2; ++k) out->pair_variant[k] = c.tree.active ? rbs::kPacked + rbs::tree_variant(c) : c.tuned[k];
+  for (int k = 0; k < 2; ++k) out->pair_variant[k] = c.tree.active ? rbs::kPacked + rbs::tree_variant(c) : rbs::direct_variant(c);
   for (int k = 2; k < 5; ++k) out->pair_variant[k] = rbs::kPacked + 1;
   return RBS_OK;
 }

@@ -140,8 +140,8 @@ struct MagState {
   std::vector<DevBuf<double>*> d_Dt, d_Dp;
   DevBuf<const double*> d_Dt_ptr, d_Dp_ptr, d_upU;
   DevBuf<int> d_grid_of;
-  DevBuf<double> d_q, d_b, d_phi, d_hn, d_f, d_qup, d_FT;
-  DevBuf<float2> d_wq;
+  DevBuf<double> d_q, d_b, d_phi, d_hn, d_f, d_FT;
+  DevBuf<float2> d_wq, d_qup;  // weighted densities of the nodes and of the upsampled nodes
   void release();
   MagState() = default;
   ~MagState();
@@ -188,7 +188,7 @@ struct TreeState {
 };
 
 // Contiguous segments of a vector (the suspensions of a batch) for the segmented GMRES (gmres.cu):
-// element offsets, and chunks of at most 4,096 elements that never straddle a segment.
+// element offsets, and chunks of at most 1,024 elements that never straddle a segment.
 struct SegChunk {
   long long b, e;
   int seg, pad;
@@ -320,6 +320,7 @@ struct Context {
 
   // near-field data
   std::vector<int2> near_pairs;   // (target particle, source particle)
+  bool near_multi = false;        // some target particle has several near sources
   DevBuf<int2> d_near;
   std::vector<int> up_index;      // per particle: index into upsampled-source list or -1
   std::vector<long long> up_offset;  // per upsampled source particle: first upsampled node
@@ -349,11 +350,10 @@ struct Context {
   // per upsampled-source particle: interpolation matrix of its grid (float64 and float32)
   DevBuf<const double*> d_upU;
   DevBuf<const float*> d_upU32;
+  std::vector<int4> up_groups;  // upsampled-source particles of one grid, four at a time (indices, -1: none)
+  DevBuf<int4> d_up_groups;
 
   std::map<const void*, int> resident;  // kernel -> resident blocks per SM
-  // chosen variants of the direct float32 pair sums (traction, Stokeslet), 0: not yet
-  int tuned[2] = {0, 0};
-  float tune_ms[2] = {0, 0};
 
   // smooth pair-sum work list: (target begin, target end, source begin, source end)
   std::vector<longlong4> work;
@@ -468,9 +468,9 @@ struct TreePlan {
 Status plan_treecode(const PlanInput& in, double theta, int degree, TreePlan& plan);
 // Builds (or clears) the treecode of the current geometry; called after the near-pair lists.
 Status build_far_field(Context& c);
-// y += the treecode's float32 smooth pair sum of kind (0 traction, 1 Stokeslet) for density x, whose weighted
-// values are in d_wmu32.
-Status apply_tree(Context& c, int kind, const double* x, double* y);
+// y += the treecode's float32 smooth pair sum of kind (0 traction, 1 Stokeslet) of the weighted densities in
+// d_wmu32.
+Status apply_tree(Context& c, int kind, double* y);
 int tree_variant(const Context& c);  // its targets per lane
 // The same for the double-float passes (d_wmuh, d_wmul): y += kind 0 or 1 sum; kind 2: y += traction, y2 += Stokeslet.
 Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y2);
@@ -504,8 +504,9 @@ Status invert_batched(Context& c, double* mats, int n, int count);
 
 // ---- operator pieces (operators.cu)
 // Particle-block kernel modes.
-// Pair-kernel variant code: targets per thread, plus kPacked for the packed-float32 kernels.
+// Pair-kernel variant code: targets per lane, plus kPacked for the packed-float32 kernels.
 constexpr int kPacked = 8;
+int direct_variant(const Context& c);  // the direct float32 sums' variant
 
 enum BlockMode {
   kModeSelfK = 0,      // y = 1/2 x + R K0 R^T x + L x      (system operator, self part)

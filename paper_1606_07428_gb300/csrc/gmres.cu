@@ -9,7 +9,7 @@
 // operator maps zero to zero), so small suspensions converge on their own norm instead of on the
 // union's.
 //
-// One Arnoldi step (basis gather, operator, two-pass classical Gram-Schmidt, norm, Givens, scaling)
+// One Arnoldi step (operator, two-pass classical Gram-Schmidt, norm, Givens, scaling)
 // is a fixed sequence of kernels whose step index lives in device memory.  For the mobility operator
 // the steps of a restart cycle run as one CUDA graph: a conditional WHILE node whose body is the
 // captured step, re-entered by the device as long as some segment is active, so a cycle costs one
@@ -26,8 +26,11 @@ namespace rbs {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr long long kChunk = 4096;  // elements per chunk; chunks never straddle a segment
-constexpr int kDotBlocksX = 2048;
+// Elements per chunk; chunks never straddle a segment.  Four per thread: small systems (a few thousand
+// unknowns) spread over as many blocks as they have chunks, and a block keeps its chunk in registers.
+constexpr int kPer = 4;
+constexpr long long kChunk = kPer * kThreads;
+constexpr int kDotRows = 4;  // blocks that share a chunk's dot products, each with every kDotRows-th vector
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -40,24 +43,61 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;  // valid in thread 0
 }
 
+// partial[i * nch + c] = V_i . w over the block's chunk c for i = i0, i0 + step, ... < nv, w given by its values in
+// registers: eight vectors at a time, one reduction across the block for the eight.
+__device__ __forceinline__ void chunk_dots(const double* __restrict__ V, long long ldv, int i0, int step, int nv,
+                                           const SegChunk& q, const double (&we)[kPer], int nch, int c,
+                                           double* __restrict__ partial) {
+  constexpr int B = 8, W = kThreads / 32;
+  __shared__ double red[B][W];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int ib = i0; ib < nv; ib += B * step) {
+    double acc[B];
+#pragma unroll
+    for (int h = 0; h < B; ++h) {
+      acc[h] = 0.0;
+      const int i = ib + h * step;
+      if (i < nv) {
+        const double* v = V + ldv * i;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+          const long long e = q.b + threadIdx.x + (long long)k * kThreads;
+          if (e < q.e) acc[h] = fma(v[e], we[k], acc[h]);
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < B; ++h) {
+      for (int o = 16; o > 0; o >>= 1) acc[h] += __shfl_xor_sync(0xffffffffu, acc[h], o);
+      if (lane == 0) red[h][warp] = acc[h];
+    }
+    __syncthreads();
+    const int i = ib + (int)threadIdx.x * step;
+    if (threadIdx.x < B && i < nv) {
+      double s = 0.0;
+      for (int w = 0; w < W; ++w) s += red[threadIdx.x][w];
+      partial[(long long)i * nch + c] = s;
+    }
+    __syncthreads();
+  }
+}
+
 // partial[i * nch + c] = V_i . w over chunk c, for i < nv; nv = ctrl[0] + nv_add, or nv_fixed when
 // ctrl is null.
 __global__ void __launch_bounds__(kThreads) k_seg_dot(const double* __restrict__ V, long long ldv,
                                                       const int* __restrict__ ctrl, int nv_add, int nv_fixed,
                                                       const double* __restrict__ w, const SegChunk* __restrict__ ch,
                                                       int nch, double* __restrict__ partial) {
-  __shared__ double red[kThreads / 32];
-  const int i = blockIdx.y;
   const int nv = ctrl ? ctrl[0] + nv_add : nv_fixed;
-  if (i >= nv) return;
-  const double* v = V + ldv * i;
-  for (int c = blockIdx.x; c < nch; c += gridDim.x) {
-    const SegChunk q = ch[c];
-    double acc = 0.0;
-    for (long long e = q.b + threadIdx.x; e < q.e; e += kThreads) acc = fma(v[e], w[e], acc);
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) partial[(long long)i * nch + c] = acc;
+  if ((int)blockIdx.y >= nv) return;
+  const SegChunk q = ch[blockIdx.x];
+  double we[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const long long e = q.b + threadIdx.x + (long long)k * kThreads;
+    we[k] = e < q.e ? w[e] : 0.0;
   }
+  chunk_dots(V, ldv, blockIdx.y, gridDim.y, nv, q, we, nch, blockIdx.x, partial);
 }
 
 // Sums the chunk partials of segment s = blockIdx.x for vector i = blockIdx.y.  Gram-Schmidt mode
@@ -87,50 +127,69 @@ __global__ void __launch_bounds__(kThreads) k_seg_reduce(const double* __restric
 }
 
 // w = alpha w + sign * sum_{i < nv} coef[i * S + seg] V_i on every chunk; nv = ctrl[0] + nv_add, or
-// nv_fixed when ctrl is null.
-__global__ void __launch_bounds__(kThreads) k_seg_combine(double* __restrict__ w, double alpha,
+// nv_fixed when ctrl is null.  With partial, the block then forms the dot products of its new chunk:
+// partial[i * nch + c] = V_i . w for i < nv when dots is 1, and w . w at i = 0 when dots is 2.
+__global__ void __launch_bounds__(kThreads) k_seg_combine(double* w, double alpha,
                                                           const double* __restrict__ V, long long ldv,
                                                           const int* __restrict__ ctrl, int nv_add, int nv_fixed,
                                                           const double* __restrict__ coef, int S, double sign,
-                                                          const SegChunk* __restrict__ ch, int nch) {
+                                                          const SegChunk* __restrict__ ch, int nch, int dots,
+                                                          double* __restrict__ partial) {
   extern __shared__ double sc[];
   const int nv = ctrl ? ctrl[0] + nv_add : nv_fixed;
-  for (int c = blockIdx.x; c < nch; c += gridDim.x) {
-    const SegChunk q = ch[c];
-    for (int i = threadIdx.x; i < nv; i += kThreads) sc[i] = sign * coef[(long long)i * S + q.seg];
-    __syncthreads();
-    for (long long e = q.b + threadIdx.x; e < q.e; e += kThreads) {
-      double acc = (alpha == 0.0) ? 0.0 : alpha * w[e];
-      for (int i = 0; i < nv; ++i) acc = fma(sc[i], V[ldv * i + e], acc);
-      w[e] = acc;
+  const SegChunk q = ch[blockIdx.x];
+  for (int i = threadIdx.x; i < nv; i += kThreads) sc[i] = sign * coef[(long long)i * S + q.seg];
+  __syncthreads();
+  double we[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const long long e = q.b + threadIdx.x + (long long)k * kThreads;
+    we[k] = (alpha != 0.0 && e < q.e) ? alpha * w[e] : 0.0;
+  }
+  // (elements beyond the chunk's end stay zero)
+#pragma unroll 4
+  for (int i = 0; i < nv; ++i) {
+    const double* v = V + ldv * i;
+    const double f = sc[i];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const long long e = q.b + threadIdx.x + (long long)k * kThreads;
+      if (e < q.e) we[k] = fma(f, v[e], we[k]);
     }
-    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const long long e = q.b + threadIdx.x + (long long)k * kThreads;
+    if (e < q.e) w[e] = we[k];
+  }
+  if (dots == 1) chunk_dots(V, ldv, 0, 1, nv, q, we, nch, blockIdx.x, partial);
+  if (dots == 2) {
+    __shared__ double red[kThreads / 32];
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) acc = fma(we[k], we[k], acc);
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = acc;
   }
 }
 
-// out = V + ldv * (ctrl ? ctrl[0] + 1 : 0):  out = w / den[seg] on the chunks of active segments with
-// den > 0, and 0 elsewhere.
+// out = V + ldv * (ctrl ? ctrl[0] : 0):  out = w / den[seg] on the chunks of active segments with den > 0,
+// and 0 elsewhere; the same to vin.
 __global__ void __launch_bounds__(kThreads) k_seg_scale(double* __restrict__ V, long long ldv,
                                                         const int* __restrict__ ctrl, const double* __restrict__ w,
                                                         const double* __restrict__ den,
                                                         const int* __restrict__ active,
-                                                        const SegChunk* __restrict__ ch, int nch) {
-  double* out = V + ldv * (ctrl ? ctrl[0] + 1 : 0);
-  for (int c = blockIdx.x; c < nch; c += gridDim.x) {
-    const SegChunk q = ch[c];
-    const double d = den[q.seg];
-    const bool on = active[q.seg] && d > 0.0;
-    const double f = on ? 1.0 / d : 0.0;
-    for (long long e = q.b + threadIdx.x; e < q.e; e += kThreads) out[e] = on ? w[e] * f : 0.0;
+                                                        const SegChunk* __restrict__ ch, double* __restrict__ vin) {
+  double* out = V + ldv * (ctrl ? ctrl[0] : 0);
+  const SegChunk q = ch[blockIdx.x];
+  const double d = den[q.seg];
+  const bool on = active[q.seg] && d > 0.0;
+  const double f = on ? 1.0 / d : 0.0;
+  for (long long e = q.b + threadIdx.x; e < q.e; e += kThreads) {
+    const double v = on ? w[e] * f : 0.0;
+    out[e] = v;
+    vin[e] = v;
   }
-}
-
-// vin = V_k, k = ctrl[0].
-__global__ void k_seg_gather(double* __restrict__ vin, const double* __restrict__ V, long long ldv,
-                             const int* __restrict__ ctrl, long long n) {
-  const double* v = V + ldv * ctrl[0];
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-    vin[e] = v[e];
 }
 
 // Start of a restart cycle from beta2[s] = ||r_s||^2: the least-squares right-hand side g_s =
@@ -183,12 +242,15 @@ __global__ void k_seg_cycle_init(int S, const double* __restrict__ beta2, const 
 // leading dimension ld, hs entries per segment).  On entry wn2[s] = ||w_s||^2 after the
 // orthogonalisation; hn[s] receives the new basis norm.  A segment stops when its residual estimate
 // |g_s(k + 1)| is within tol[s] (converged) or is not a number, or when it has used ctrl[3]
-// iterations.  ctrl[1] = the number of segments still active; ctrl[2] counts NaN estimates.
+// iterations.  ctrl[1] = the number of segments still active; ctrl[2] counts NaN estimates.  Ends the step's
+// bookkeeping: ctrl[0] = k + 1, and with a graph condition the loop body is re-entered while a segment is active
+// and the basis has room (k + 1 < m).
 __global__ void k_seg_givens(int S, double* __restrict__ H, int ld, long long hs, double* __restrict__ cs,
                              double* __restrict__ sn, double* __restrict__ g, int gs, const double* __restrict__ wn2,
                              double* __restrict__ hn, const double* __restrict__ tol, double* __restrict__ res,
                              int* __restrict__ active, int* __restrict__ conv, int* __restrict__ kdone,
-                             int* __restrict__ iters, int* __restrict__ ctrl) {
+                             int* __restrict__ iters, int* __restrict__ ctrl, int m,
+                             cudaGraphConditionalHandle handle, int use_handle) {
   __shared__ int cnt[kThreads / 32], bad[kThreads / 32];
   const int k = ctrl[0];
   const int max_iters = ctrl[3];
@@ -247,18 +309,11 @@ __global__ void k_seg_givens(int S, double* __restrict__ H, int ld, long long hs
       a_ += cnt[q];
       b_ += bad[q];
     }
+    ctrl[0] = k + 1;
     ctrl[1] = a_;
     ctrl[2] += b_;
+    if (use_handle) cudaGraphSetConditional(handle, (a_ > 0 && k + 1 < m) ? 1u : 0u);
   }
-}
-
-// End of an Arnoldi step: k += 1; with a graph condition, re-enter the loop body while a segment is
-// active and the basis has room.
-__global__ void k_seg_step_end(int* __restrict__ ctrl, int m, cudaGraphConditionalHandle handle, int use_handle) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int k = ctrl[0] + 1;
-  ctrl[0] = k;
-  if (use_handle) cudaGraphSetConditional(handle, (ctrl[1] > 0 && k < m) ? 1u : 0u);
 }
 
 // y_s = R_s^{-1} g_s for the kdone[s] x kdone[s] triangle of each segment, stored as y[i * S + s]
@@ -382,15 +437,20 @@ static Status ensure_work(Context& c, const SegSet& sg, long long n, int m) {
   return Status::Ok();
 }
 
+// The chunk partials of one vector summed per segment into out (S doubles).
+static void seg_reduce(Context& c, const SegSet& sg, double* out) {
+  k_seg_reduce<<<dim3(sg.S, 1), kThreads, 0, c.stream>>>(c.gw.partial.ptr, sg.nch, sg.d_c0.ptr, sg.S, nullptr, 0, 1,
+                                                         nullptr, nullptr, nullptr, 0, 0, out);
+}
+
 // Per-segment squared norms (or dot products) of vectors of sg.n elements into the device array out
 // (S doubles).
 Status seg_dot(Context& c, const SegSet& sg, const double* a, const double* b, double* out) {
   GmresWork& g = c.gw;
-  dim3 gd(std::min(std::max(1, sg.nch), kDotBlocksX), 1);
   c.stats.launches += 2;
-  k_seg_dot<<<gd, kThreads, 0, c.stream>>>(a, 0, nullptr, 0, 1, b, sg.d_chunks.ptr, sg.nch, g.partial.ptr);
-  k_seg_reduce<<<dim3(sg.S, 1), kThreads, 0, c.stream>>>(g.partial.ptr, sg.nch, sg.d_c0.ptr, sg.S, nullptr, 0, 1,
-                                                         nullptr, nullptr, nullptr, 0, 0, out);
+  k_seg_dot<<<std::max(1, sg.nch), kThreads, 0, c.stream>>>(a, 0, nullptr, 0, 1, b, sg.d_chunks.ptr, sg.nch,
+                                                            g.partial.ptr);
+  seg_reduce(c, sg, out);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
@@ -422,29 +482,27 @@ static Status arnoldi_step(Context& c, const LinOp& op, const SegSet& sg, int m,
   double* res = tol + S;
   double* hn = res + S;
   double* wn2 = hn + S;
-  const int nb = grid_for(c, n);
-  c.stats.launches += 1;
-  k_seg_gather<<<nb, 256, 0, c.stream>>>(g.vin.ptr, g.V.ptr, n, ctrl, n);
+  // vin holds basis vector k (k_seg_scale of the previous step or of the cycle's start)
   RBS_TRY(op.apply_AP(g.vin.ptr, g.w.ptr, g.z.ptr));
-  const dim3 gdot(std::min(std::max(1, sg.nch), kDotBlocksX), m + 1);
+  const int nch = std::max(1, sg.nch);
   const dim3 gred(S, m + 1);
-  const int gcomb = std::min(std::max(1, sg.nch), 8 * std::max(1, c.sm_count));
+  // first Gram-Schmidt pass: coefficients, then w less its projections together with the second pass's dot
+  // products; second pass together with w's norm
+  c.stats.launches += 7;
+  k_seg_dot<<<dim3(nch, kDotRows), kThreads, 0, c.stream>>>(g.V.ptr, n, ctrl, 1, 0, g.w.ptr, sg.d_chunks.ptr, sg.nch,
+                                                            g.partial.ptr);
   for (int pass = 0; pass < 2; ++pass) {
-    c.stats.launches += 3;
-    k_seg_dot<<<gdot, kThreads, 0, c.stream>>>(g.V.ptr, n, ctrl, 1, 0, g.w.ptr, sg.d_chunks.ptr, sg.nch,
-                                                g.partial.ptr);
     k_seg_reduce<<<gred, kThreads, 0, c.stream>>>(g.partial.ptr, sg.nch, sg.d_c0.ptr, S, ctrl, 1, 0, active,
                                                    g.coef.ptr, g.H.ptr, ld, hs, nullptr);
-    k_seg_combine<<<gcomb, kThreads, sizeof(double) * (m + 1), c.stream>>>(g.w.ptr, 1.0, g.V.ptr, n, ctrl, 1, 0,
-                                                                           g.coef.ptr, S, -1.0, sg.d_chunks.ptr,
-                                                                           sg.nch);
+    k_seg_combine<<<nch, kThreads, sizeof(double) * (m + 1), c.stream>>>(
+        g.w.ptr, 1.0, g.V.ptr, n, ctrl, 1, 0, g.coef.ptr, S, -1.0, sg.d_chunks.ptr, sg.nch, pass == 0 ? 1 : 2,
+        g.partial.ptr);
   }
-  RBS_TRY(seg_dot(c, sg, g.w.ptr, g.w.ptr, wn2));
-  c.stats.launches += 3;
+  seg_reduce(c, sg, wn2);
   k_seg_givens<<<1, kThreads, 0, c.stream>>>(S, g.H.ptr, ld, hs, g.cs.ptr, g.sn.ptr, g.g.ptr, gs, wn2, hn, tol, res,
-                                             active, conv, kdone, iters, ctrl);
-  k_seg_scale<<<gcomb, kThreads, 0, c.stream>>>(g.V.ptr, n, ctrl, g.w.ptr, hn, active, sg.d_chunks.ptr, sg.nch);
-  k_seg_step_end<<<1, 32, 0, c.stream>>>(ctrl, m, handle, use_handle ? 1 : 0);
+                                             active, conv, kdone, iters, ctrl, m, handle, use_handle ? 1 : 0);
+  c.stats.launches += 1;
+  k_seg_scale<<<nch, kThreads, 0, c.stream>>>(g.V.ptr, n, ctrl, g.w.ptr, hn, active, sg.d_chunks.ptr, g.vin.ptr);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
@@ -529,7 +587,7 @@ Status gmres_seg(Context& c, const LinOp& op, const SegSet& sg, const double* b,
   double* res = tol + S;
   double* beta2 = res + 3 * S;
   const int nb = grid_for(c, n);
-  const int gcomb = std::min(std::max(1, sg.nch), 8 * std::max(1, c.sm_count));
+  const int nch = std::max(1, sg.nch);
   double* r = g.r.ptr;
 
   // tolerances in, iteration counts zeroed
@@ -576,7 +634,7 @@ Status gmres_seg(Context& c, const LinOp& op, const SegSet& sg, const double* b,
     ++cycles;
     RBS_CUDA_TRY(cudaMemsetAsync(g.H.ptr, 0, sizeof(double) * (size_t)S * hs, c.stream));
     c.stats.launches++;
-    k_seg_scale<<<gcomb, kThreads, 0, c.stream>>>(g.V.ptr, n, nullptr, r, res, active, sg.d_chunks.ptr, sg.nch);
+    k_seg_scale<<<nch, kThreads, 0, c.stream>>>(g.V.ptr, n, nullptr, r, res, active, sg.d_chunks.ptr, g.vin.ptr);
     int k_host = 0;
     bool cont = true;
     if (slot && !slot->exec) {
@@ -614,17 +672,17 @@ Status gmres_seg(Context& c, const LinOp& op, const SegSet& sg, const double* b,
     k_seg_trisolve<<<cdiv(S, 128), 128, 0, c.stream>>>(S, g.H.ptr, ld, hs, g.g.ptr, gs, kdone, m, g.y.ptr);
     if (op.apply_P) {
       c.stats.launches++;
-      k_seg_combine<<<gcomb, kThreads, sizeof(double) * (m + 1), c.stream>>>(g.w.ptr, 0.0, g.V.ptr, n, nullptr, 0,
-                                                                             k_host, g.y.ptr, S, 1.0,
-                                                                             sg.d_chunks.ptr, sg.nch);
+      k_seg_combine<<<nch, kThreads, sizeof(double) * (m + 1), c.stream>>>(g.w.ptr, 0.0, g.V.ptr, n, nullptr, 0, k_host,
+                                                                           g.y.ptr, S, 1.0, sg.d_chunks.ptr, sg.nch, 0,
+                                                                           nullptr);
       RBS_TRY(op.apply_P(g.w.ptr, g.z.ptr, r));
       c.stats.launches++;
       k_axpby_g<<<nb, 256, 0, c.stream>>>(x, 1.0, g.z.ptr, 1.0, n);
     } else {
       c.stats.launches++;
-      k_seg_combine<<<gcomb, kThreads, sizeof(double) * (m + 1), c.stream>>>(x, 1.0, g.V.ptr, n, nullptr, 0, k_host,
-                                                                             g.y.ptr, S, 1.0, sg.d_chunks.ptr,
-                                                                             sg.nch);
+      k_seg_combine<<<nch, kThreads, sizeof(double) * (m + 1), c.stream>>>(x, 1.0, g.V.ptr, n, nullptr, 0, k_host,
+                                                                           g.y.ptr, S, 1.0, sg.d_chunks.ptr, sg.nch, 0,
+                                                                           nullptr);
     }
     RBS_CUDA_TRY(cudaGetLastError());
     // every segment within its tolerance (by the estimate) or out of iterations: done

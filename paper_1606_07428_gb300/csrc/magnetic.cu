@@ -7,7 +7,7 @@
 // the smooth rule over distinct particles, upsampled sources for near pairs, and the rotated-pole
 // singular rule on each particle's own surface (scalar blocks, invariant under the particle's rotation,
 // stored per shape with every row).  The smooth pair sums run in double-float arithmetic (about 1e-12),
-// the near corrections and blocks in float64; the solve is float64 GMRES, right-preconditioned by the
+// and so do the near corrections, the blocks in float64; the solve is float64 GMRES, right-preconditioned by the
 // inverse of each particle's own 1/2 I + eta K^L block.
 //
 // On the fluid side of each surface the field is H = -grad_s phi + H_n n, the tangential gradient by
@@ -19,6 +19,8 @@
 
 #include "common.cuh"
 #include "dfloat.cuh"
+#include "near.cuh"
+#include "pairsdf.cuh"
 #include "surface.cuh"
 
 namespace rbs {
@@ -145,101 +147,101 @@ __global__ void k_weight_df1(long long N, const double4* __restrict__ x, const d
   wq[t] = make_float2(a.h, a.l);
 }
 
-// The smooth scalar pair sums in double-float arithmetic (about 1e-12 relative, like float64 here, on
-// the float32 pipes): positions staged from exact three-float splits relative to the item's first
-// target, the weighted density as double-float pairs, tiles accumulated in double-float.
+// The smooth scalar pair sums in double-float arithmetic on the float32 pipes: two sources per packed
+// instruction, tiles and work units as the mobility operators' (pairsdf.cuh).  One pair takes 97 float32
+// operations (K^L) or 71 (S^L), 9 fewer where the tile is on a grid.
+template <int KIND, int MODE>
+__device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const int* spid, int l0, int l1,
+                                               const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2& acc) {
+#pragma unroll 1
+  for (int l = l0; l < l1; l += 2) {
+    df2 d[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2 yh = *reinterpret_cast<const float2*>(&sa[2 * c][l]), yl = *reinterpret_cast<const float2*>(&sa[2 * c + 1][l]);
+      d[c] = df_separation<MODE>(xt[c], df2{yh, yl});
+    }
+    const df2 q = {*reinterpret_cast<const float2*>(&sa[6][l]), *reinterpret_cast<const float2*>(&sa[7][l])};
+    int2 pp = make_int2(0, 0);
+    if (MODE == kDfMask) pp = *reinterpret_cast<const int2*>(&spid[l]);
+    float2 R;
+    const inv_powers p = df_inv_powers<MODE>(d, pp, pt, R);
+    if (KIND == 0) {
+      const float2 r = __fmul2_rn(R, p.y0);
+      const df2 rn = bdot2(d[0], nt[0], d[1], nt[1], d[2], nt[2], __fmul2_rn(r, dup2(kBiasFactor)));
+      df2 a = mul2(rn, p.y3());
+      a.l = __ffma2_rn(p.w3(), a.h, a.l);
+      acc2_add(acc, mul2(a, q));
+    } else {
+      acc2_add(acc, mul2(p.inv(), q));
+    }
+  }
+}
+
 template <int KIND>
-__global__ void __launch_bounds__(128, 8) k_lap_df(int nitems, const longlong4* __restrict__ work,
+__global__ void __launch_bounds__(128, 5) k_lap_df(int nunits, int* __restrict__ counter,
+                                                   const longlong4* __restrict__ work,
                                                    const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                                    const float4* __restrict__ x3l, const float4* __restrict__ nh,
                                                    const float4* __restrict__ nl, const float2* __restrict__ wq,
                                                    double scale, double* __restrict__ y) {
-  constexpr int TS = 128;
-  __shared__ float4 sph[TS], spl[TS];
-  __shared__ float2 sq[TS];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const longlong4 w = work[it];
-    const float4 oh = x3h[w.x], om = x3m[w.x], ol = x3l[w.x];
-    const long long t = w.x + threadIdx.x;
-    const bool valid = t < w.y;
-    float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
-    int pt = -1;
-    if (valid) {
-      ah = x3h[t];
-      am = x3m[t];
-      al = x3l[t];
-      bh = nh[t];
-      bl = nl[t];
-      pt = __float_as_int(ah.w);
-    }
-    const dflt xt[3] = {df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x), df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y),
+  __shared__ __align__(16) float tiles[4][9][kTileDf];
+  float(*sa)[kTileDf] = tiles[threadIdx.x >> 5];
+  int* const spid = reinterpret_cast<int*>(&sa[8][0]);
+  const int lane = threadIdx.x & 31;
+  while (true) {
+    int unit = 0;
+    if (lane == 0) unit = atomicAdd(counter, 1);
+    unit = __shfl_sync(0xffffffffu, unit, 0);
+    if (unit >= nunits) return;
+    const longlong4 w = work[unit >> 2];
+    const int t0 = (int)w.x + 32 * (unit & 3), t1 = (int)w.y;
+    if (t0 >= t1) continue;
+    const bool split = t1 - t0 <= 16;  // the half-warps take alternate halves of the sources
+    const int half = split ? lane >> 4 : 0;
+    const int t = t0 + (split ? lane & 15 : lane);
+    const bool valid = t < t1;
+    const float4 oh = x3h[t0], om = x3m[t0], ol = x3l[t0], zero = make_float4(0, 0, 0, 0);
+    const float4 ah = valid ? x3h[t] : oh, am = valid ? x3m[t] : om, al = valid ? x3l[t] : ol;
+    const float4 bh = valid ? nh[t] : zero, bl = valid ? nl[t] : zero;
+    const int pt = valid ? __float_as_int(ah.w) : -1;
+    const dflt x0[3] = {df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x), df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y),
                         df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z)};
-    const dflt nt[3] = {{bh.x, bl.x}, {bh.y, bl.y}, {bh.z, bl.z}};
+    const df2 nt[3] = {{dup2(bh.x), dup2(bl.x)}, {dup2(bh.y), dup2(bl.y)}, {dup2(bh.z), dup2(bl.z)}};
+    const float xm = warp_max_abs(fmaxf(fabsf(x0[0].h), fmaxf(fabsf(x0[1].h), fabsf(x0[2].h))));
+    const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(x3h[min(t0 + 32, t1) - 1].w);
     dflt a = {0.0f, 0.0f};
-    for (long long s0 = w.z; s0 < w.w; s0 += TS) {
-      const int cnt = (int)min((long long)TS, w.w - s0);
-      __syncthreads();
-      if ((int)threadIdx.x < cnt) {
-        const long long s = s0 + threadIdx.x;
-        const float4 ph = x3h[s], pm = x3m[s], pl = x3l[s];
-        const dflt px = df_diff3(ph.x, pm.x, pl.x, oh.x, om.x, ol.x);
-        const dflt py = df_diff3(ph.y, pm.y, pl.y, oh.y, om.y, ol.y);
-        const dflt pz = df_diff3(ph.z, pm.z, pl.z, oh.z, om.z, ol.z);
-        sph[threadIdx.x] = make_float4(px.h, py.h, pz.h, ph.w);
-        spl[threadIdx.x] = make_float4(px.l, py.l, pz.l, 0.0f);
-        sq[threadIdx.x] = wq[s];
-      }
-      __syncthreads();
-      dflt acc = {0.0f, 0.0f};
-      for (int l = 0; l < cnt; ++l) {
-        const float4 yh = sph[l], yl = spl[l];
-        const float2 qq = sq[l];
-        dflt d[3];
-        d[0] = df_two_sum(xt[0].h, -yh.x);
-        d[0].l += xt[0].l - yl.x;
-        d[1] = df_two_sum(xt[1].h, -yh.y);
-        d[1].l += xt[1].l - yl.y;
-        d[2] = df_two_sum(xt[2].h, -yh.z);
-        d[2].l += xt[2].l - yl.z;
-        float p[3], e[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          p[c] = d[c].h * d[c].h;
-          e[c] = fmaf(d[c].h, d[c].h, -p[c]);
-          e[c] = fmaf(d[c].h + d[c].h, d[c].l, e[c]);
-        }
-        const dflt s1 = df_two_sum(p[0], p[1]);
-        const dflt s2 = df_two_sum(s1.h, p[2]);
-        const float r2l = s1.l + s2.l + e[0] + e[1] + e[2];
-        const float r2h = s2.h;
-        const float y0 = rsqrt_hw(r2h);
-        const float q0 = y0 * y0;
-        const float qe = fmaf(y0, y0, -q0);
-        float tt = fmaf(r2h, q0, -1.0f);
-        tt = fmaf(r2h, qe, tt);
-        tt = fmaf(r2l, q0, tt);
-        dflt inv = {y0, -0.5f * tt * y0};
-        if (__float_as_int(yh.w) == pt) inv = {0.0f, 0.0f};
-        const dflt wqv = {qq.x, qq.y};
-        if (KIND == 0) {
-          const dflt rn = df_dot3(d[0], nt[0], d[1], nt[1], d[2], nt[2]);
-          const dflt inv3 = df_mul(df_mul(inv, inv), inv);
-          df_acc(acc, df_mul(df_mul(rn, inv3), wqv));
-        } else {
-          df_acc(acc, df_mul(inv, wqv));
-        }
-      }
-      a = df_add_accurate(a, acc);
+    for (int s0 = (int)w.z; s0 < (int)w.w; s0 += kTileDf) {
+      const int cnt = min(kTileDf, (int)w.w - s0), cnt4 = (cnt + 3) & ~3;
+      const int sidx[2] = {s0 + lane, s0 + lane + 32};
+      const int tlo = __float_as_int(x3h[s0].w), thi = __float_as_int(x3h[s0 + cnt - 1].w);
+      const bool masked = !(thi < pid_lo || tlo > pid_hi);
+      df2 xt[3];
+      const bool grid = df_stage(sa, spid, sidx, cnt, masked, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
+        const float2 q = s >= 0 ? wq[s] : make_float2(0.0f, 0.0f);
+        sa[6][l] = q.x;
+        sa[7][l] = q.y;
+      });
+      df2 acc = {dup2(0.0f), dup2(0.0f)};
+      const int m = split ? cnt4 / 2 : cnt4, l0 = half * m;
+      if (masked)
+        lap_tile_pairs<KIND, kDfMask>(sa, spid, l0, l0 + m, xt, nt, pt, acc);
+      else if (grid)
+        lap_tile_pairs<KIND, kDfGrid>(sa, spid, l0, l0 + m, xt, nt, pt, acc);
+      else
+        lap_tile_pairs<KIND, kDfPlain>(sa, spid, l0, l0 + m, xt, nt, pt, acc);
+      a = df_add_accurate(a, fold2(acc));
     }
     if (valid) atomicAdd(y + t, (KIND == 0 ? -scale : scale) * kInv4Pi * ((double)a.h + (double)a.l));
   }
 }
 
-// Upsampled scalar densities of the near-source particles: q_up = U q_j (U stored N_p x N_up).
+// Upsampled weighted scalar densities of the near-source particles, w U q_j in float64 (U stored N_p x N_up)
+// rounded to float32 pairs.
 __global__ void k_lap_upsample(int n_up, const int* __restrict__ up_particle, const long long* __restrict__ up_off,
                                const long long* __restrict__ offset, const int* __restrict__ nodes,
                                const double* const* __restrict__ Umats, const double* __restrict__ q,
-                               double* __restrict__ qup) {
+                               const double4* __restrict__ up_x, float2* __restrict__ qup) {
   for (int u = blockIdx.y; u < n_up; u += gridDim.y) {
     const int j = up_particle[u];
     const int np = nodes[j];
@@ -248,45 +250,71 @@ __global__ void k_lap_upsample(int n_up, const int* __restrict__ up_particle, co
     const double* Ut = Umats[u];
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nup; r += gridDim.x * blockDim.x) {
       double a = 0.0;
-      for (int s = 0; s < np; ++s) a = fma(Ut[(long long)s * nup + r], q[o + s], a);
-      qup[base + r] = a;
+#pragma unroll 8
+      for (int s = 0; s < np; ++s) a = fma(__ldg(Ut + (long long)s * nup + r), __ldg(q + o + s), a);
+      const dflt v = df_split(up_x[base + r].w * a);
+      qup[base + r] = make_float2(v.h, v.l);
     }
   }
 }
 
-// Near correction for one ordered near pair (i, j) per block: for targets of i, add the upsampled
-// contribution of j and remove the smooth-rule one.
+// Near correction by the units of near.cuh: for targets of i, the upsampled contribution of j is added and the
+// smooth-rule one removed, both in the double-float arithmetic of the smooth sum, so that what is removed
+// is what was added (float64 here took 1.7 ms a launch on 454 pairs of 144-node particles, bound by the
+// float64 pipe, and left the smooth sum's rounding uncancelled).
 template <int KIND>
-__global__ void __launch_bounds__(128) k_lap_near(const int2* __restrict__ near, const long long* __restrict__ offset,
-                                                  const int* __restrict__ nodes, const int* __restrict__ up_index,
-                                                  const long long* __restrict__ up_off, const double4* __restrict__ x,
-                                                  const double4* __restrict__ nrm, const double* __restrict__ q,
-                                                  const double4* __restrict__ up_x, const double* __restrict__ qup,
-                                                  double scale, double* __restrict__ y) {
-  const int2 pr = near[blockIdx.x];
-  const long long oi = offset[pr.x], oj = offset[pr.y];
-  const int ni = nodes[pr.x], nj = nodes[pr.y];
-  const int u = up_index[pr.y];
-  const long long ou = up_off[u];
-  const int nu = (int)(up_off[u + 1] - ou);
-  for (int tt = threadIdx.x; tt < ni; tt += blockDim.x) {
-    const double4 xt = x[oi + tt], nt = nrm[oi + tt];
-    double acc = 0.0;
-    for (int a = 0; a < nu; ++a) {
-      const double4 ps = up_x[ou + a];
-      const double dx = xt.x - ps.x, dy = xt.y - ps.y, dz = xt.z - ps.z;
-      const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
-      const double kv = KIND == 0 ? -(dx * nt.x + dy * nt.y + dz * nt.z) * inv * inv * inv : inv;
-      acc = fma(kv, ps.w * qup[ou + a], acc);
+__global__ void __launch_bounds__(128, 5) k_lap_near(NearArgs A, const float4* __restrict__ x3h,
+                                                     const float4* __restrict__ x3m, const float4* __restrict__ x3l,
+                                                     const float4* __restrict__ nh, const float4* __restrict__ nl,
+                                                     const float2* __restrict__ wq, const float4* __restrict__ up3h,
+                                                     const float4* __restrict__ up3m, const float4* __restrict__ up3l,
+                                                     const float2* __restrict__ upq, double scale,
+                                                     double* __restrict__ y) {
+  __shared__ __align__(16) float tiles[4][9][kTileDf];
+  float(*sa)[kTileDf] = tiles[threadIdx.x >> 5];
+  int* const spid = reinterpret_cast<int*>(&sa[8][0]);
+  const int lane = threadIdx.x & 31;
+  NearUnit n;
+  while (next_near_unit(A, n)) {
+    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    const bool split = n.t1 - n.t0 <= 16;
+    const int half = split ? lane >> 4 : 0;
+    const int t = n.t0 + (split ? lane & 15 : lane);
+    const bool valid = t < n.t1;
+    const float4 oh = x3h[n.t0], om = x3m[n.t0], ol = x3l[n.t0], zero = make_float4(0, 0, 0, 0);
+    const float4 ah = valid ? x3h[t] : oh, am = valid ? x3m[t] : om, al = valid ? x3l[t] : ol;
+    const float4 bh = valid ? nh[t] : zero, bl = valid ? nl[t] : zero;
+    const dflt x0[3] = {df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x), df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y),
+                        df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z)};
+    const df2 nt[3] = {{dup2(bh.x), dup2(bl.x)}, {dup2(bh.y), dup2(bl.y)}, {dup2(bh.z), dup2(bl.z)}};
+    const float xm = warp_max_abs(fmaxf(fabsf(x0[0].h), fmaxf(fabsf(x0[1].h), fabsf(x0[2].h))));
+    dflt a = {0.0f, 0.0f};
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {  // upsampled nodes, then base nodes with the opposite sign
+      const int b = pass == 0 ? n.s0 : max(n.s0, n.nup), e = pass == 0 ? min(n.s1, n.nup) : n.s1;
+      const long long g0 = pass == 0 ? n.ub : n.oj - n.nup;
+      const float2* qs = pass == 0 ? upq : wq;
+      const float sign = pass == 0 ? 1.0f : -1.0f;
+      for (int sb = b; sb < e; sb += kTileDf) {
+        const int cnt = min(kTileDf, e - sb), cnt4 = (cnt + 3) & ~3;
+        const int sidx[2] = {(int)(g0 + sb) + lane, (int)(g0 + sb) + lane + 32};
+        df2 xt[3];
+        const bool grid = df_stage(sa, spid, sidx, cnt, false, pass == 0 ? up3h : x3h, pass == 0 ? up3m : x3m,
+                                   pass == 0 ? up3l : x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
+                                     const float2 q = s >= 0 ? qs[s] : make_float2(0.0f, 0.0f);
+                                     sa[6][l] = sign * q.x;
+                                     sa[7][l] = sign * q.y;
+                                   });
+        df2 acc = {dup2(0.0f), dup2(0.0f)};
+        const int m = split ? cnt4 / 2 : cnt4, l0 = half * m;
+        if (grid)
+          lap_tile_pairs<KIND, kDfGrid>(sa, spid, l0, l0 + m, xt, nt, -1, acc);
+        else
+          lap_tile_pairs<KIND, kDfPlain>(sa, spid, l0, l0 + m, xt, nt, -1, acc);
+        a = df_add_accurate(a, fold2(acc));
+      }
     }
-    for (int s = 0; s < nj; ++s) {
-      const double4 ps = x[oj + s];
-      const double dx = xt.x - ps.x, dy = xt.y - ps.y, dz = xt.z - ps.z;
-      const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
-      const double kv = KIND == 0 ? -(dx * nt.x + dy * nt.y + dz * nt.z) * inv * inv * inv : inv;
-      acc = fma(-kv, ps.w * q[oj + s], acc);
-    }
-    atomicAdd(y + oi + tt, scale * kInv4Pi * acc);
+    if (valid) atomicAdd(y + t, (KIND == 0 ? -scale : scale) * kInv4Pi * ((double)a.h + (double)a.l));
   }
 }
 
@@ -563,11 +591,13 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
   k_lap_blocks<<<c.n, 256, 0, s>>>(c.d_offset.ptr, c.d_nodes.ptr, c.d_shape.ptr, M.d_block_off.ptr, B, x, scale, half, y);
   const int nw = (int)c.work.size();
   if (nw > 0) {
-    RBS_TRY(M.d_wq.alloc(c.N));
+    if (M.d_wq.n != (size_t)c.N) RBS_TRY(M.d_wq.alloc(c.N));
     c.stats.launches += 2;
     k_weight_df1<<<cdiv(c.N, 256), 256, 0, s>>>(c.N, c.d_x.ptr, x, M.d_wq.ptr);
-    const int grid = std::min(nw, 8 * std::max(1, c.sm_count));
-#define RBS_LAP_ARGS nw, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
+    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), s));
+    const int grid = std::min(nw, 5 * std::max(1, c.sm_count));
+#define RBS_LAP_ARGS \
+  4 * nw, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
     if (kind == 0)
       k_lap_df<0><<<grid, 128, 0, s>>>(RBS_LAP_ARGS);
     else
@@ -576,20 +606,26 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
   }
   const int nn = (int)c.near_pairs.size();
   if (nn > 0) {
-    RBS_TRY(M.d_qup.alloc(std::max<long long>(1, c.n_up_nodes)));
+    if (M.d_qup.n != (size_t)c.n_up_nodes) RBS_TRY(M.d_qup.alloc(std::max<long long>(1, c.n_up_nodes)));
     int maxup = 0;
     for (Grid* g : c.grids) maxup = std::max(maxup, g->nup);
     const int nup_p = (int)c.up_particle.size();
     dim3 gu(cdiv(maxup, 128), (unsigned)std::min(nup_p, 65535));
     c.stats.launches += 2;
     k_lap_upsample<<<gu, 128, 0, s>>>(nup_p, c.d_up_particle.ptr, c.d_up_off.ptr, c.d_offset.ptr, c.d_nodes.ptr,
-                                     M.d_upU.ptr, x, M.d_qup.ptr);
+                                     M.d_upU.ptr, x, c.d_up_x.ptr, M.d_qup.ptr);
+    NearArgs A;
+    int blocks = 0;
+    RBS_TRY(near_args(c, A, blocks));
+    blocks = std::min(blocks, 5 * std::max(1, c.sm_count));
+#define RBS_LAP_NEAR                                                                                              \
+  A, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, c.d_up3h.ptr, c.d_up3m.ptr, \
+      c.d_up3l.ptr, M.d_qup.ptr, scale, y
     if (kind == 0)
-      k_lap_near<0><<<nn, 128, 0, s>>>(c.d_near.ptr, c.d_offset.ptr, c.d_nodes.ptr, c.d_up_index.ptr, c.d_up_off.ptr,
-                                       c.d_x.ptr, c.d_nrm.ptr, x, c.d_up_x.ptr, M.d_qup.ptr, scale, y);
+      k_lap_near<0><<<blocks, 128, 0, s>>>(RBS_LAP_NEAR);
     else
-      k_lap_near<1><<<nn, 128, 0, s>>>(c.d_near.ptr, c.d_offset.ptr, c.d_nodes.ptr, c.d_up_index.ptr, c.d_up_off.ptr,
-                                       c.d_x.ptr, c.d_nrm.ptr, x, c.d_up_x.ptr, M.d_qup.ptr, scale, y);
+      k_lap_near<1><<<blocks, 128, 0, s>>>(RBS_LAP_NEAR);
+#undef RBS_LAP_NEAR
   }
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();

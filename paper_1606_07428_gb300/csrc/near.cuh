@@ -1,0 +1,80 @@
+// Work units of the near corrections (mobility and magnetostatic operators).
+#pragma once
+
+#include <climits>
+
+#include "common.cuh"
+
+namespace rbs {
+
+// Near correction.  For a near pair (target particle i, source particle j) the contribution of j's
+// upsampled nodes is added and that of its base nodes (already in the smooth sum) removed.  A unit is
+// (pair, 32 targets of i, one of `parts` equal runs of the N_up + N_j sources), taken by warps from a
+// counter; parts grows until small near lists fill the GPU.  A pair of 144-node particles is 688 sources
+// against five units of targets, so one block per pair left most of the SMs idle on lists of a few hundred
+// pairs and most of its threads idle where orders mix.
+struct NearArgs {
+  int nunits, chunks, parts;
+  int* counter;
+  const int2* near;
+  const long long* offset;
+  const int* nodes;
+  const int* up_index;
+  const long long* up_off;
+};
+struct NearUnit {
+  int t0, t1;           // targets [t0, t1) of particle i that the unit holds, 32 at most (t0 >= t1: none)
+  long long ub, oj;     // first upsampled node and first base node of j
+  int s0, s1, nup;      // sources [s0, s1): below nup upsampled nodes, then base nodes
+};
+__device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
+  int unit = 0;
+  if ((threadIdx.x & 31) == 0) unit = atomicAdd(A.counter, 1);
+  unit = __shfl_sync(0xffffffffu, unit, 0);
+  if (unit >= A.nunits) return false;
+  const int part = unit % A.parts, q = unit / A.parts;
+  const int chunk = q % A.chunks;
+  const int2 pr = A.near[q / A.chunks];
+  const long long oi = A.offset[pr.x];
+  n.t0 = (int)oi + 32 * chunk;
+  n.t1 = min(n.t0 + 32, (int)oi + A.nodes[pr.x]);
+  const int u = A.up_index[pr.y];
+  n.ub = A.up_off[u];
+  n.nup = (int)(A.up_off[u + 1] - n.ub);
+  n.oj = A.offset[pr.y];
+  const int total = n.nup + A.nodes[pr.y];
+  const int step = ((total + A.parts - 1) / A.parts + 3) & ~3;
+  n.s0 = min(total, part * step);
+  n.s1 = min(total, n.s0 + step);
+  return true;
+}
+
+
+// The units of the context's near list, with the counter zeroed on its stream; blocks: as many 128-thread
+// blocks as have a unit per warp.
+inline Status near_args(Context& c, NearArgs& A, int& blocks) {
+  const long long nn = (long long)c.near_pairs.size();
+  A.chunks = (c.max_np + 31) / 32;
+  // source runs: about 16 units per SM, of at least 128 sources and at most about 512 (a unit of one p = 16
+  // source particle, 2,656 sources, would outlast a list of mixed orders)
+  int most = 1;
+  for (Grid* g : c.grids) most = std::max(most, g->nup + g->np);
+  const long long units1 = std::max(1LL, nn * A.chunks);
+  A.parts = (int)std::max((most + 511LL) / 512, std::min<long long>((16LL * c.sm_count + units1 - 1) / units1, most / 128));
+  // a float64 context's targets with one near source each keep one addition, the same bits on every run
+  if (!prec_f32(c.opt.precision) && !c.near_multi) A.parts = 1;
+  const long long units = units1 * A.parts;
+  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "near correction: more than 2^31 work units");
+  A.nunits = (int)units;
+  A.counter = c.d_unit.ptr;
+  A.near = c.d_near.ptr;
+  A.offset = c.d_offset.ptr;
+  A.nodes = c.d_nodes.ptr;
+  A.up_index = c.d_up_index.ptr;
+  A.up_off = c.d_up_off.ptr;
+  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
+  blocks = (int)((units + 3) / 4);
+  return Status::Ok();
+}
+
+}  // namespace rbs

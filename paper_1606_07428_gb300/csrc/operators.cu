@@ -15,6 +15,7 @@
 
 #include "common.cuh"
 #include "dfloat.cuh"
+#include "near.cuh"
 #include "pairs32.cuh"
 #include "pairsdf.cuh"
 
@@ -227,7 +228,9 @@ __device__ __forceinline__ void cp_async_wait() {
 // reflected inputs z_g, g = 4h .. 4h + 3, keeping twelve partial sums; at the end of r a reduce-scatter
 // over the sixteen column groups leaves reflection g's three sums in lanes 4g .. 4g + 3.  In float32
 // arithmetic the row sums go to shared memory and every node is finished by the whole CTA at the end;
-// in float64 lane 4g finishes node g(r) at once.
+// in float64 lane 4g finishes node g(r) at once.  gridDim.y CTAs share a particle, each taking every
+// gridDim.y-th run of kSymWarps representatives: a float64 particle of 144 nodes is 65 us of one SM's float64
+// pipe, so a list of few particles, or of few large ones, would leave the other SMs idle.
 template <typename TS, typename TB>
 __global__ void __launch_bounds__(kSymWarps * 32, sizeof(TB) == 4 ? 3 : 2)
     k_blocks_sym(int mode, const int* __restrict__ sym_list, const long long* __restrict__ offset,
@@ -260,6 +263,8 @@ __global__ void __launch_bounds__(kSymWarps * 32, sizeof(TB) == 4 ? 3 : 2)
   const int i = sym_list[blockIdx.x];
   const int p = pvec[i], nphi = nphivec[i], np = (p + 1) * nphi, dim = 3 * np;
   const int nk = nphi / 4 + 1, nrep = (p / 2 + 1) * nk;
+  const int part = blockIdx.y, nparts = gridDim.y;
+  if (kSymWarps * part >= nrep) return;  // (no block, mode L: one part)
   const int zs = sym_zstride(dim, sizeof(TB));
   TB* zg = reinterpret_cast<TB*>(zraw + kRingBytes);  // 8 rows of stride zs
   TB* ynode = zg + 8 * zs;                            // float32: 3 N_p row sums
@@ -279,10 +284,11 @@ __global__ void __launch_bounds__(kSymWarps * 32, sizeof(TB) == 4 ? 3 : 2)
   const int nst = (dim + SC - 1) / SC;
   const bool al16 = ((reinterpret_cast<uintptr_t>(A) & 15u) == 0) && (dim % E == 0);
   const uint32_t ring_l = static_cast<uint32_t>(__cvta_generic_to_shared(zraw)) + warp * (S * 3 * 512) + lane * 16;
-  int iss_left = (has_block && warp < nrep) ? ((nrep - 1 - warp) / kSymWarps + 1) * nst : 0;
+  const int rep0 = warp + kSymWarps * part, rep_step = kSymWarps * nparts;
+  int iss_left = (has_block && rep0 < nrep) ? ((nrep - 1 - rep0) / rep_step + 1) * nst : 0;
   int iss_it = 0, iss_slot = 0;
-  const TS* iss_src = A + (long long)(3 * warp) * dim + E * lane;
-  const long long rep_jump = (long long)3 * kSymWarps * dim - (long long)SC * nst;
+  const TS* iss_src = A + (long long)(3 * rep0) * dim + E * lane;
+  const long long rep_jump = (long long)3 * rep_step * dim - (long long)SC * nst;
   auto issue = [&]() {
     if (iss_left > 0) {
       // entries past the row end are zero-filled (nothing is read there)
@@ -409,7 +415,7 @@ __global__ void __launch_bounds__(kSymWarps * 32, sizeof(TB) == 4 ? 3 : 2)
   const TS* ring_k = reinterpret_cast<const TS*>(zraw) + warp * (S * 3 * SC) + 4 * kc;
   const TB* zl = zg + (4 * hg) * zs + 4 * kc;
   int slot = 0;
-  for (int r = warp; r < nrep; r += kSymWarps) {
+  for (int r = rep0; r < nrep; r += rep_step) {
     float2 y2[4][3];
     TB yd[4][3];
 #pragma unroll
@@ -502,7 +508,14 @@ __global__ void __launch_bounds__(kSymWarps * 32, sizeof(TB) == 4 ? 3 : 2)
   cp_async_wait<0>();
   if constexpr (kF32) {
     __syncthreads();
-    for (int t = threadIdx.x; t < np; t += blockDim.x) finish(t, ynode[3 * t], ynode[3 * t + 1], ynode[3 * t + 2]);
+    for (int t = threadIdx.x; t < np; t += blockDim.x) {
+      if (nparts > 1) {  // the nodes of this part's representatives
+        const int j = t / nphi, k = t - j * nphi;
+        const int kh = min(k, nphi - k), kr = min(kh, nphi / 2 - kh);
+        if ((min(j, p - j) * nk + kr) / kSymWarps % nparts != part) continue;
+      }
+      finish(t, ynode[3 * t], ynode[3 * t + 1], ynode[3 * t + 2]);
+    }
   }
 }
 
@@ -577,116 +590,6 @@ __global__ void __launch_bounds__(128) k_pairs64(int nitems, const longlong4* __
 }
 
 // ------------------------------------------------------------------------------------------
-// Smooth pair sums in float32.  Coordinates are taken relative to the first target of the block in
-// float64 before rounding, so a float32 difference keeps the relative accuracy of the separation
-// rather than of the absolute position.  Each 256-source tile is summed in float32 and added into
-// a compensated (two-sum) float32 accumulator.  Tiles whose particles cannot meet the block's
-// targets skip the same-particle test.
-
-template <int KIND, bool MASK, int NT>
-__device__ __forceinline__ void pair_tile32(const float4* __restrict__ sp, const float4* __restrict__ sd, int cnt,
-                                            const float (&xt)[NT][3], const float (&nt)[NT][3], const int (&pt)[NT],
-                                            float (&acc)[NT][3]) {
-#pragma unroll 4
-  for (int l = 0; l < cnt; ++l) {
-    const float4 ps = sp[l];
-    const float4 ds = sd[l];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) {
-      const float dx = xt[u][0] - ps.x, dy = xt[u][1] - ps.y, dz = xt[u][2] - ps.z;
-      const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-      float inv = rsqrt_hw(r2);
-      if (MASK && __float_as_int(ps.w) == pt[u]) inv = 0.0f;
-      const float rr = fmaf(dx, ds.x, fmaf(dy, ds.y, dz * ds.z));
-      if (KIND == 0) {
-        const float inv2 = inv * inv;
-        const float rn = fmaf(dx, nt[u][0], fmaf(dy, nt[u][1], dz * nt[u][2]));
-        const float c = (rn * rr) * (inv2 * inv2 * inv);
-        acc[u][0] = fmaf(c, dx, acc[u][0]);
-        acc[u][1] = fmaf(c, dy, acc[u][1]);
-        acc[u][2] = fmaf(c, dz, acc[u][2]);
-      } else {
-        const float c = rr * (inv * inv * inv);
-        acc[u][0] = fmaf(c, dx, fmaf(ds.x, inv, acc[u][0]));
-        acc[u][1] = fmaf(c, dy, fmaf(ds.y, inv, acc[u][1]));
-        acc[u][2] = fmaf(c, dz, fmaf(ds.z, inv, acc[u][2]));
-      }
-    }
-  }
-}
-
-// NT targets per thread (block = 128 / NT threads over a 128-target work item): each staged source
-// feeds NT independent pair evaluations.
-template <int KIND, int NT>
-__global__ void __launch_bounds__(128 / NT, NT == 1 ? 1 : (NT == 2 ? 16 : 12)) k_pairs32(int nitems, const longlong4* __restrict__ work, const double4* __restrict__ x,
-                                                      const double4* __restrict__ nrm, const int* __restrict__ pid,
-                                                      const double* __restrict__ dens, double* __restrict__ y) {
-  constexpr int TS = 256, NTH = 128 / NT;
-  __shared__ float4 sp[TS];
-  __shared__ float4 sd[TS];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-  const longlong4 w = work[it];
-  const double4 org = x[w.x];
-  float xt[NT][3], nt[NT][3];
-  int pt[NT];
-  bool valid[NT];
-#pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    const long long t = w.x + threadIdx.x + NTH * u;
-    valid[u] = t < w.y;
-    xt[u][0] = xt[u][1] = xt[u][2] = nt[u][0] = nt[u][1] = nt[u][2] = 0.0f;
-    pt[u] = -1;
-    if (valid[u]) {
-      const double4 a = x[t], nn = nrm[t];
-      xt[u][0] = (float)(a.x - org.x);
-      xt[u][1] = (float)(a.y - org.y);
-      xt[u][2] = (float)(a.z - org.z);
-      nt[u][0] = (float)nn.x;
-      nt[u][1] = (float)nn.y;
-      nt[u][2] = (float)nn.z;
-      pt[u] = pid[t];
-    }
-  }
-  const int pid_lo = pid[w.x], pid_hi = pid[w.y - 1];
-  float sa[NT][3], ea[NT][3];
-#pragma unroll
-  for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
-  for (long long s0 = w.z; s0 < w.w; s0 += TS) {
-    const int cnt = (int)min((long long)TS, w.w - s0);
-    __syncthreads();
-    for (int l = threadIdx.x; l < cnt; l += NTH) {
-      const long long s = s0 + l;
-      const double4 ps = x[s];
-      const double* d = dens + 3 * s;
-      sp[l] = make_float4((float)(ps.x - org.x), (float)(ps.y - org.y), (float)(ps.z - org.z), __int_as_float(pid[s]));
-      sd[l] = make_float4((float)(ps.w * d[0]), (float)(ps.w * d[1]), (float)(ps.w * d[2]), 0.0f);
-    }
-    __syncthreads();
-    const int tlo = pid[s0], thi = pid[s0 + cnt - 1];
-    float p[NT][3];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) p[u][0] = p[u][1] = p[u][2] = 0.0f;
-    if (thi < pid_lo || tlo > pid_hi)
-      pair_tile32<KIND, false, NT>(sp, sd, cnt, xt, nt, pt, p);
-    else
-      pair_tile32<KIND, true, NT>(sp, sd, cnt, xt, nt, pt, p);
-#pragma unroll
-    for (int u = 0; u < NT; ++u)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c]);
-  }
-  const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
-#pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    if (!valid[u]) continue;
-    const long long t = w.x + threadIdx.x + NTH * u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
-  }
-  }
-}
-
-// ------------------------------------------------------------------------------------------
 // Weighted density in float32 for the packed kernels: wmu[t] = (w_t mu_t, 0).
 __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
                              float4* __restrict__ wmu) {
@@ -696,92 +599,121 @@ __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const d
   wmu[t] = make_float4((float)(w * dens[3 * t]), (float)(w * dens[3 * t + 1]), (float)(w * dens[3 * t + 2]), 0.0f);
 }
 
-// Sources and targets are read as float32 hi + lo position pairs and float32 weighted densities, so
-// the kernel runs no float64 arithmetic but its final accumulation: a coordinate relative to the work
-// item's origin o is (y_hi - o_hi) + (y_lo - o_lo), within one rounding of the exact difference.
+// Direct float32 pair sums.  Sources and targets are read as float32 hi + lo position pairs and float32
+// weighted densities, so the kernel runs no float64 arithmetic but its final accumulation: a coordinate
+// relative to the unit's origin o (its first target) is (y_hi - o_hi) + (y_lo - o_lo), within one rounding
+// of the exact difference.  A unit is 32 NT targets of a work item against its sources; warps take units
+// from a counter and stage their own tiles of 128 sources, summed in float32 and added into a compensated
+// accumulator.  Tiles whose particles cannot meet the unit's targets skip the same-particle test.
+// Bound by the float32 pipe (20 operations a traction pair, 18 a Stokeslet pair).
 template <int KIND, int NT>
-__global__ void __launch_bounds__(128 / NT, NT == 4 ? 12 : (NT == 2 ? 10 : 8)) k_pairs32x2(int nitems, const longlong4* __restrict__ work, const float4* __restrict__ xhi,
-                                                       const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
-                                                       const float4* __restrict__ wmu, double* __restrict__ y) {
-  constexpr int TS = 512, NTH = 128 / NT;  // 512 sources per tile: the staging latency is amortised over more pairs
-  __shared__ __align__(16) float ssx[TS], ssy[TS], ssz[TS], srx[TS], sry[TS], srz[TS];
-  __shared__ __align__(16) int spid[TS];
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-  const longlong4 w = work[it];
-  const float4 oh = xhi[w.x], ol = xlo[w.x];
-  float2 xt[NT][3], nt[NT][3];
-  int pt[NT];
-  bool valid[NT];
+__global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
+    k_pairs32x2(int nunits, int* __restrict__ counter, const longlong4* __restrict__ work,
+                const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
+                const float4* __restrict__ wmu, double* __restrict__ y) {
+  constexpr int TW = 128, kPerItem = 4 / NT;
+  __shared__ __align__(16) float tiles[4][7 * TW];
+  const int lane = threadIdx.x & 31;
+  float* const ssx = tiles[threadIdx.x >> 5];
+  int* const spid = reinterpret_cast<int*>(ssx + 6 * TW);
+  while (true) {
+    int unit = 0;
+    if (lane == 0) unit = atomicAdd(counter, 1);
+    unit = __shfl_sync(0xffffffffu, unit, 0);
+    if (unit >= nunits) return;
+    const longlong4 w = work[unit / kPerItem];
+    const int t0 = (int)w.x + 32 * NT * (unit % kPerItem), t1 = (int)w.y;
+    if (t0 >= t1) continue;
+    const bool split = t1 - t0 <= 16;  // the two half-warps take alternate halves of the sources
+    const int half = split ? lane >> 4 : 0;
+    const int nu = min(NT, (t1 - t0 + 31) / 32);
+    const float4 oh = xhi[t0], ol = xlo[t0];
+    float2 xt[NT][3], nt[NT][3];
+    int pt[NT];
+    bool valid[NT];
 #pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    const long long t = w.x + threadIdx.x + NTH * u;
-    valid[u] = t < w.y;
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, n0 = 0.0f, n1 = 0.0f, n2 = 0.0f;
-    pt[u] = -1;
-    if (valid[u]) {
-      const float4 ah = xhi[t], al = xlo[t], nn = nrm32[t];
-      a0 = (ah.x - oh.x) + (al.x - ol.x);
-      a1 = (ah.y - oh.y) + (al.y - ol.y);
-      a2 = (ah.z - oh.z) + (al.z - ol.z);
-      n0 = nn.x;
-      n1 = nn.y;
-      n2 = nn.z;
-      pt[u] = __float_as_int(ah.w);
-    }
-    xt[u][0] = f2(a0, a0);
-    xt[u][1] = f2(a1, a1);
-    xt[u][2] = f2(a2, a2);
-    nt[u][0] = f2(n0, n0);
-    nt[u][1] = f2(n1, n1);
-    nt[u][2] = f2(n2, n2);
-  }
-  const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(xhi[w.y - 1].w);
-  float sa[NT][3], ea[NT][3];
-#pragma unroll
-  for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
-  for (long long s0 = w.z; s0 < w.w; s0 += TS) {
-    const int cnt = (int)min((long long)TS, w.w - s0);
-    const int cnt4 = (cnt + 3) & ~3;
-    __syncthreads();
-    for (int l = threadIdx.x; l < cnt4; l += NTH) {
-      if (l < cnt) {
-        const long long s = s0 + l;
-        const float4 ph = xhi[s], pl = xlo[s], q = wmu[s];
-        ssx[l] = (oh.x - ph.x) + (ol.x - pl.x);
-        ssy[l] = (oh.y - ph.y) + (ol.y - pl.y);
-        ssz[l] = (oh.z - ph.z) + (ol.z - pl.z);
-        srx[l] = q.x;
-        sry[l] = q.y;
-        srz[l] = q.z;
-        spid[l] = __float_as_int(ph.w);
-      } else {
-        ssx[l] = ssy[l] = ssz[l] = 1.0e4f;
-        srx[l] = sry[l] = srz[l] = 0.0f;
-        spid[l] = -2;
+    for (int u = 0; u < NT; ++u) {
+      const int t = t0 + 32 * u + (split ? lane & 15 : lane);
+      valid[u] = t < t1;
+      float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, n0 = 0.0f, n1 = 0.0f, n2 = 0.0f;
+      pt[u] = -1;
+      if (valid[u]) {
+        const float4 ah = xhi[t], al = xlo[t], nn = nrm32[t];
+        a0 = (ah.x - oh.x) + (al.x - ol.x);
+        a1 = (ah.y - oh.y) + (al.y - ol.y);
+        a2 = (ah.z - oh.z) + (al.z - ol.z);
+        n0 = nn.x;
+        n1 = nn.y;
+        n2 = nn.z;
+        pt[u] = __float_as_int(ah.w);
       }
+      xt[u][0] = f2(a0, a0);
+      xt[u][1] = f2(a1, a1);
+      xt[u][2] = f2(a2, a2);
+      nt[u][0] = f2(n0, n0);
+      nt[u][1] = f2(n1, n1);
+      nt[u][2] = f2(n2, n2);
     }
-    __syncthreads();
-    const int tlo = spid[0], thi = spid[cnt - 1];
-    float2 p[NT][3];
+    const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(xhi[min(t0 + 32 * NT, t1) - 1].w);
+    float sa[NT][3], ea[NT][3];
 #pragma unroll
-    for (int u = 0; u < NT; ++u) p[u][0] = p[u][1] = p[u][2] = f2(0.0f, 0.0f);
-    if (thi < pid_lo || tlo > pid_hi)
-      pair_tile32x2<KIND, false, NT>(ssx, ssy, ssz, srx, sry, srz, spid, cnt4, xt, nt, pt, p);
-    else
-      pair_tile32x2<KIND, true, NT>(ssx, ssy, ssz, srx, sry, srz, spid, cnt4, xt, nt, pt, p);
+    for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
+    for (int s0 = (int)w.z; s0 < (int)w.w; s0 += TW) {
+      const int cnt = min(TW, (int)w.w - s0), cnt8 = (cnt + 7) & ~7;
+      __syncwarp();  // the warp's reads of the previous tile are done
 #pragma unroll
-    for (int u = 0; u < NT; ++u)
+      for (int l = lane; l < TW; l += 32) {
+        if (l < cnt) {
+          const int s = s0 + l;
+          const float4 ph = xhi[s], pl = xlo[s], q = wmu[s];
+          ssx[l] = (oh.x - ph.x) + (ol.x - pl.x);
+          ssx[TW + l] = (oh.y - ph.y) + (ol.y - pl.y);
+          ssx[2 * TW + l] = (oh.z - ph.z) + (ol.z - pl.z);
+          ssx[3 * TW + l] = q.x;
+          ssx[4 * TW + l] = q.y;
+          ssx[5 * TW + l] = q.z;
+          spid[l] = __float_as_int(ph.w);
+        } else if (l < cnt8) {
+          ssx[l] = ssx[TW + l] = ssx[2 * TW + l] = 1.0e4f;
+          ssx[3 * TW + l] = ssx[4 * TW + l] = ssx[5 * TW + l] = 0.0f;
+          spid[l] = -2;
+        }
+      }
+      __syncwarp();
+      const int tlo = spid[0], thi = spid[cnt - 1];
+      float2 p[NT][3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c].x + p[u][c].y);
-  }
-  const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
+      for (int u = 0; u < NT; ++u) p[u][0] = p[u][1] = p[u][2] = f2(0.0f, 0.0f);
+      const int m = split ? cnt8 / 2 : cnt8, l0 = half * m;
+      const float* b = ssx + l0;
+#define RBS_TILE(NUV)                                                                                               \
+  do {                                                                                                              \
+    if (thi < pid_lo || tlo > pid_hi)                                                                               \
+      pair_tile32x2<KIND, false, NT, NUV>(b, b + TW, b + 2 * TW, b + 3 * TW, b + 4 * TW, b + 5 * TW, spid + l0, m, \
+                                          xt, nt, pt, p);                                                          \
+    else                                                                                                            \
+      pair_tile32x2<KIND, true, NT, NUV>(b, b + TW, b + 2 * TW, b + 3 * TW, b + 4 * TW, b + 5 * TW, spid + l0, m,  \
+                                         xt, nt, pt, p);                                                           \
+  } while (0)
+      if (nu == NT) {
+        RBS_TILE(NT);
+      } else if constexpr (NT > 1) {
+        RBS_TILE(1);
+      }
+#undef RBS_TILE
 #pragma unroll
-  for (int u = 0; u < NT; ++u) {
-    if (!valid[u]) continue;
-    const long long t = w.x + threadIdx.x + NTH * u;
+      for (int u = 0; u < NT; ++u)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
-  }
+        for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c].x + p[u][c].y);
+    }
+    const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+      if (!valid[u]) continue;
+      const long long t = t0 + 32 * u + (split ? lane & 15 : lane);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
+    }
   }
 }
 
@@ -869,93 +801,82 @@ __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restric
 }
 
 // ------------------------------------------------------------------------------------------
-// Upsampled densities of the near-source particles: mu_up = U mu_j with U stored transposed
-// (N_p x N_up), one thread per upsampled node reading U coalesced and mu_j from shared memory; the
-// arithmetic is that of U's storage type (float32 for the inner solve, float64 otherwise).  The near
-// sums take them weighted: FORM 0 w mu as float64 (qd), 1 as float32 (qh), 2 as float32 pairs (qh, ql).
+// Upsampled densities of the near-source particles: mu_up = U mu_j with U stored transposed (N_p x N_up),
+// in the arithmetic of U's storage type (float32 for the inner solve, float64 otherwise).  One block takes
+// 64 upsampled nodes of up to four particles of one grid: its threads read U coalesced, each entry once for
+// the four, in four groups that share the sum over the grid's nodes (kUpTile of them staged at a time), so that
+// a few particles still fill a block and many read U from L2 a quarter as often.  The near sums take the
+// results weighted: FORM 0 w mu as float64 (qd), 1 as float32 (qh), 2 as float32 pairs (qh, ql).
+constexpr int kUpRows = 64, kUpTile = 64;
+
 template <typename TU, int FORM>
-__global__ void __launch_bounds__(128) k_upsample(int n_up, const int* __restrict__ up_particle,
+__global__ void __launch_bounds__(256) k_upsample(const int4* __restrict__ groups, const int* __restrict__ up_particle,
                                                   const long long* __restrict__ up_off,
                                                   const long long* __restrict__ offset, const int* __restrict__ nodes,
                                                   const TU* const* __restrict__ Umats, const double* __restrict__ dens,
                                                   const double4* __restrict__ upx, double4* __restrict__ qd,
                                                   float4* __restrict__ qh, float4* __restrict__ ql) {
-  extern __shared__ double mus_raw[];  // 3 N_p values of type TU
-  TU* mus = reinterpret_cast<TU*>(mus_raw);
-  for (int u = blockIdx.y; u < n_up; u += gridDim.y) {
-    const int j = up_particle[u];
-    const int np = nodes[j];
-    const long long o = offset[j];
-    const long long base = up_off[u];
-    const int nup = (int)(up_off[u + 1] - base);
-    if ((int)(blockIdx.x * blockDim.x) >= nup) continue;
+  __shared__ __align__(16) TU mus[kUpTile][12];
+  __shared__ TU part[3][12][kUpRows];
+  const int4 gr = groups[blockIdx.y];
+  const int us[4] = {gr.x, gr.y, gr.z, gr.w};
+  const int np = nodes[up_particle[gr.x]];
+  const int nup = (int)(up_off[gr.x + 1] - up_off[gr.x]);
+  const int r0 = blockIdx.x * kUpRows;
+  if (r0 >= nup) return;
+  const int row = threadIdx.x % kUpRows, sg = threadIdx.x / kUpRows;
+  const int r = min(r0 + row, nup - 1);
+  const TU* Ut = Umats[gr.x] + r;
+  TU acc[12];
+#pragma unroll
+  for (int q = 0; q < 12; ++q) acc[q] = 0;
+  for (int s0 = 0; s0 < np; s0 += kUpTile) {
+    const int cnt = min(kUpTile, np - s0);
     __syncthreads();
-    for (int l = threadIdx.x; l < 3 * np; l += blockDim.x) mus[l] = (TU)dens[3 * o + l];
-    __syncthreads();
-    const TU* Ut = Umats[u];
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nup; r += gridDim.x * blockDim.x) {
-      TU a0 = 0, a1 = 0, a2 = 0;
-#pragma unroll 8
-      for (int s = 0; s < np; ++s) {
-        const TU uv = __ldg(Ut + (long long)s * nup + r);
-        a0 = fma_t(uv, mus[3 * s], a0);
-        a1 = fma_t(uv, mus[3 * s + 1], a1);
-        a2 = fma_t(uv, mus[3 * s + 2], a2);
-      }
-      const double w = upx[base + r].w;
-      const double q0 = w * (double)a0, q1 = w * (double)a1, q2 = w * (double)a2;
-      if (FORM == 0) qd[base + r] = make_double4(q0, q1, q2, 0.0);
-      if (FORM == 1) qh[base + r] = make_float4((float)q0, (float)q1, (float)q2, 0.0f);
-      if (FORM == 2) {
-        const dflt d0 = df_split(q0), d1 = df_split(q1), d2 = df_split(q2);
-        qh[base + r] = make_float4(d0.h, d1.h, d2.h, 0.0f);
-        ql[base + r] = make_float4(d0.l, d1.l, d2.l, 0.0f);
-      }
+    for (int e = threadIdx.x; e < 12 * kUpTile; e += 256) {
+      const int s = (e / 3) % kUpTile, p = e / (3 * kUpTile), k = e % 3;
+      TU v = 0;
+      if (us[p] >= 0 && s < cnt) v = (TU)dens[3 * (offset[up_particle[us[p]]] + s0 + s) + k];
+      mus[s][3 * p + k] = v;
     }
+    __syncthreads();
+    // the tile's rows of this group: sg, sg + 4, ... (zero densities beyond cnt; U stays in bounds)
+#pragma unroll 8
+    for (int s = sg; s < kUpTile; s += 4) {
+      const TU u = __ldg(Ut + (long long)min(s0 + s, np - 1) * nup);
+#pragma unroll
+      for (int q = 0; q < 12; ++q) acc[q] = fma_t(u, mus[s][q], acc[q]);
+    }
+  }
+  __syncthreads();
+  if (sg > 0)
+#pragma unroll
+    for (int q = 0; q < 12; ++q) part[sg - 1][q][row] = acc[q];
+  __syncthreads();
+  // group sg finishes particle sg
+  if (sg == 0)
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {
+      const TU v = acc[q] + part[0][q][row] + part[1][q][row] + part[2][q][row];
+      part[0][q][row] = v;
+    }
+  __syncthreads();
+  const int u = us[sg];
+  if (u < 0 || r0 + row >= nup) return;
+  const long long o = up_off[u] + r0 + row;
+  const double w = upx[o].w;
+  const double q0 = w * (double)part[0][3 * sg][row], q1 = w * (double)part[0][3 * sg + 1][row],
+               q2 = w * (double)part[0][3 * sg + 2][row];
+  if (FORM == 0) qd[o] = make_double4(q0, q1, q2, 0.0);
+  if (FORM == 1) qh[o] = make_float4((float)q0, (float)q1, (float)q2, 0.0f);
+  if (FORM == 2) {
+    const dflt d0 = df_split(q0), d1 = df_split(q1), d2 = df_split(q2);
+    qh[o] = make_float4(d0.h, d1.h, d2.h, 0.0f);
+    ql[o] = make_float4(d0.l, d1.l, d2.l, 0.0f);
   }
 }
 
-// Near correction.  For a near pair (target particle i, source particle j) the contribution of j's
-// upsampled nodes is added and that of its base nodes (already in the smooth sum) removed.  A unit is
-// (pair, 32 targets of i, one of `parts` equal runs of the N_up + N_j sources), taken by warps from a
-// counter; parts grows until small near lists fill the GPU.  A pair of 144-node particles is 688 sources
-// against five units of targets, so one block per pair left most of the SMs idle on lists of a few hundred
-// pairs and most of its threads idle where orders mix.
-struct NearArgs {
-  int nunits, chunks, parts;
-  int* counter;
-  const int2* near;
-  const long long* offset;
-  const int* nodes;
-  const int* up_index;
-  const long long* up_off;
-};
-struct NearUnit {
-  int t0, t1;           // targets [t0, t1) of particle i that the unit holds, 32 at most (t0 >= t1: none)
-  long long ub, oj;     // first upsampled node and first base node of j
-  int s0, s1, nup;      // sources [s0, s1): below nup upsampled nodes, then base nodes
-};
-__device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
-  int unit = 0;
-  if ((threadIdx.x & 31) == 0) unit = atomicAdd(A.counter, 1);
-  unit = __shfl_sync(0xffffffffu, unit, 0);
-  if (unit >= A.nunits) return false;
-  const int part = unit % A.parts, q = unit / A.parts;
-  const int chunk = q % A.chunks;
-  const int2 pr = A.near[q / A.chunks];
-  const long long oi = A.offset[pr.x];
-  n.t0 = (int)oi + 32 * chunk;
-  n.t1 = min(n.t0 + 32, (int)oi + A.nodes[pr.x]);
-  const int u = A.up_index[pr.y];
-  n.ub = A.up_off[u];
-  n.nup = (int)(A.up_off[u + 1] - n.ub);
-  n.oj = A.offset[pr.y];
-  const int total = n.nup + A.nodes[pr.y];
-  const int step = ((total + A.parts - 1) / A.parts + 3) & ~3;
-  n.s0 = min(total, part * step);
-  n.s1 = min(total, n.s0 + step);
-  return true;
-}
+// Near correction by the units of near.cuh.
 
 // Float32: the packed tile loop of the smooth sum over per-warp tiles of 128 sources.
 template <int KIND>
@@ -1189,90 +1110,58 @@ static int resident_grid(Context& c, const void* kernel, int threads, int items)
   return std::max(1, std::min(items, per_sm * std::max(1, c.sm_count)));
 }
 
-// Launch of the smooth pair sum over the first `items` work items with NT targets per thread.
-// KIND 2 (traction into y and Stokeslet into y2 in one pass) exists in double-float only.
-template <int KIND>
-static void launch_pairs_kind(Context& c, int prec, int nt, int items, const double* x, double* y, double* y2) {
-#define RBS_PAIR_ARGS items, c.d_work.ptr, c.d_x.ptr, c.d_nrm.ptr, c.d_pid.ptr, x, y
-  if (prec == RBS_PREC_DF) {
-    cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream);
-    const int units = 4 * items;
-    k_pairs_df2<KIND><<<resident_grid(c, (const void*)k_pairs_df2<KIND>, 128, items), 128, 0, c.stream>>>(
-        units, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
-        c.d_wmuh.ptr, c.d_wmul.ptr, y, y2);
-  } else if constexpr (KIND == 2) {
-    return;
-  } else if (prec == RBS_PREC_FP64) {
-    k_pairs64<KIND><<<resident_grid(c, (const void*)k_pairs64<KIND>, 128, items), 128, 0, c.stream>>>(RBS_PAIR_ARGS);
-  } else {
-    if (nt == 1)
-      k_pairs32<KIND, 1><<<resident_grid(c, (const void*)k_pairs32<KIND, 1>, 128, items), 128, 0, c.stream>>>(RBS_PAIR_ARGS);
-    else if (nt == 2)
-      k_pairs32<KIND, 2><<<resident_grid(c, (const void*)k_pairs32<KIND, 2>, 64, items), 64, 0, c.stream>>>(RBS_PAIR_ARGS);
-    else if (nt == 4)
-      k_pairs32<KIND, 4><<<resident_grid(c, (const void*)k_pairs32<KIND, 4>, 32, items), 32, 0, c.stream>>>(RBS_PAIR_ARGS);
-    else {
-#define RBS_PACKED_ARGS items, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y
-      if (nt == kPacked + 1)
-        k_pairs32x2<KIND, 1><<<resident_grid(c, (const void*)k_pairs32x2<KIND, 1>, 128, items), 128, 0, c.stream>>>(RBS_PACKED_ARGS);
-      else if (nt == kPacked + 2)
-        k_pairs32x2<KIND, 2><<<resident_grid(c, (const void*)k_pairs32x2<KIND, 2>, 64, items), 64, 0, c.stream>>>(RBS_PACKED_ARGS);
-      else
-        k_pairs32x2<KIND, 4><<<resident_grid(c, (const void*)k_pairs32x2<KIND, 4>, 32, items), 32, 0, c.stream>>>(RBS_PACKED_ARGS);
-#undef RBS_PACKED_ARGS
-    }
-  }
-#undef RBS_PAIR_ARGS
+// Targets per lane of the direct float32 sums: two, which share each source's loads, once that still makes
+// 64 units per SM (three rounds of its warps); one below, and where rbs_options.pair_variant asks for it.
+static int pairs32_targets(const Context& c) {
+  const int v = c.opt.pair_variant;
+  if (v > 0) return v == 1 || v == kPacked + 1 ? 1 : 2;
+  return 2 * (long long)c.work.size() >= 64LL * c.sm_count ? 2 : 1;
 }
 
-static Status launch_pairs(Context& c, int kind, int prec, int nt, int items, const double* x, double* y,
-                           double* y2 = nullptr) {
-  if (kind == 0)
-    launch_pairs_kind<0>(c, prec, nt, items, x, y, y2);
-  else if (kind == 1)
-    launch_pairs_kind<1>(c, prec, nt, items, x, y, y2);
-  else
-    launch_pairs_kind<2>(c, prec, nt, items, x, y, y2);
+int direct_variant(const Context& c) { return kPacked + pairs32_targets(c); }
+
+template <int KIND, int NT>
+static void launch_pairs32(Context& c, double* y) {
+  const int items = (int)c.work.size();
+  const auto kernel = k_pairs32x2<KIND, NT>;
+  kernel<<<resident_grid(c, (const void*)kernel, 128, items), 128, 0, c.stream>>>(
+      4 / NT * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y);
+}
+
+template <int KIND>
+static void launch_pairs_df(Context& c, double* y, double* y2) {
+  const int items = (int)c.work.size();
+  k_pairs_df2<KIND><<<resident_grid(c, (const void*)k_pairs_df2<KIND>, 128, items), 128, 0, c.stream>>>(
+      4 * items, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
+      c.d_wmuh.ptr, c.d_wmul.ptr, y, y2);
+}
+
+// Launch of the direct smooth pair sum; kind 2 (traction into y and Stokeslet into y2 in one pass) exists in
+// double-float only.  The float32 and double-float sums read the weighted densities of this x.
+static Status launch_pairs(Context& c, int kind, int prec, const double* x, double* y, double* y2 = nullptr) {
+  const int items = (int)c.work.size();
+  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
+  if (prec == RBS_PREC_DF) {
+    if (kind == 0)
+      launch_pairs_df<0>(c, y, y2);
+    else if (kind == 1)
+      launch_pairs_df<1>(c, y, y2);
+    else
+      launch_pairs_df<2>(c, y, y2);
+  } else if (prec == RBS_PREC_FP64) {
+#define RBS_PAIR_ARGS items, c.d_work.ptr, c.d_x.ptr, c.d_nrm.ptr, c.d_pid.ptr, x, y
+    if (kind == 0)
+      k_pairs64<0><<<resident_grid(c, (const void*)k_pairs64<0>, 128, items), 128, 0, c.stream>>>(RBS_PAIR_ARGS);
+    else
+      k_pairs64<1><<<resident_grid(c, (const void*)k_pairs64<1>, 128, items), 128, 0, c.stream>>>(RBS_PAIR_ARGS);
+#undef RBS_PAIR_ARGS
+  } else if (pairs32_targets(c) == 1) {
+    kind == 0 ? launch_pairs32<0, 1>(c, y) : launch_pairs32<1, 1>(c, y);
+  } else {
+    kind == 0 ? launch_pairs32<0, 2>(c, y) : launch_pairs32<1, 2>(c, y);
+  }
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
-}
-
-// Pair-kernel variant: targets per thread (1, 2 or 4), plus kPacked for the float32 kernels that take
-// two sources per packed instruction.  rbs_options.pair_variant when set (its targets per thread for
-// the double-float kernels), otherwise the fastest candidate timed once per (kernel, arithmetic) on a
-// prefix of the work list (the same items for every variant, into a scratch output).
-static int pair_variant(Context& c, int kind, int prec, const double* x) {
-  if (prec == RBS_PREC_DF) return kPacked + 1;
-  if (c.opt.pair_variant > 0) return c.opt.pair_variant;
-  const int key = kind;
-  if (c.tuned[key]) return c.tuned[key];
-  int best = 2;
-  const int items = std::min<int>((int)c.work.size(), 2 * 32 * std::max(1, c.sm_count));
-  double* scratch = nullptr;
-  cudaEvent_t a = nullptr, b = nullptr;
-  if (cudaMalloc(&scratch, sizeof(double) * 6 * c.N) == cudaSuccess && cudaEventCreate(&a) == cudaSuccess &&
-      cudaEventCreate(&b) == cudaSuccess) {
-    float best_ms = 1e30f;
-    for (int nt : {1, 2, 4, kPacked + 1, kPacked + 2, kPacked + 4}) {
-      launch_pairs(c, kind, prec, nt, items, x, scratch, scratch + 3 * c.N);  // warm (first launch of this variant)
-      cudaEventRecord(a, c.stream);
-      launch_pairs(c, kind, prec, nt, items, x, scratch, scratch + 3 * c.N);
-      cudaEventRecord(b, c.stream);
-      float ms = 0.0f;
-      if (cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&ms, a, b) == cudaSuccess && ms < best_ms) {
-        best_ms = ms;
-        best = nt;
-      }
-      c.stats.launches += 2;
-    }
-    c.tune_ms[key] = best_ms;
-  }
-  if (a) cudaEventDestroy(a);
-  if (b) cudaEventDestroy(b);
-  if (scratch) cudaFree(scratch);
-  cudaGetLastError();
-  c.tuned[key] = best;
-  return best;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1300,6 +1189,11 @@ Status apply_blocks(Context& c, int mode, int prec, const double* x, double* y, 
   if (gemm) RBS_TRY(apply_self_gemm(c, mode, x, y, aux, scale));
   if (nsym > 0) {
     const size_t zs = (size_t)sym_smem_bytes(c.max_np_sym, use16 ? 2 : use32 ? 4 : 8, use32 ? 4 : 8);
+    // parts of a particle: about six CTAs per SM, and no more than its runs of kSymWarps representatives
+    int runs = 1;
+    for (Grid* g : c.grids) runs = std::max(runs, (g->nrep + kSymWarps - 1) / kSymWarps);
+    const int parts = mode == kModeL ? 1 : std::max(1, std::min(runs, (6 * c.sm_count + nsym - 1) / nsym));
+    const dim3 grid(nsym, parts);
 #define RBS_SYM_ARGS                                                                                              \
   mode, sym_ids, c.d_offset.ptr, c.d_p.ptr, c.d_nphi.ptr, c.d_rot.ptr, c.d_centre.ptr, c.d_shape.ptr, \
       c.d_block_off.ptr, B, c.d_x.ptr, x, y, aux, scale
@@ -1310,26 +1204,26 @@ Status apply_blocks(Context& c, int mode, int prec, const double* x, double* y, 
         if (zs > 48 * 1024)
           RBS_CUDA_TRY(cudaFuncSetAttribute(k_blocks_sym<F16Bits, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)zs));
-        k_blocks_sym<F16Bits, float><<<nsym, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
+        k_blocks_sym<F16Bits, float><<<grid, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
       } else {
         const BF16Bits* B = reinterpret_cast<const BF16Bits*>(B16);
         if (zs > 48 * 1024)
           RBS_CUDA_TRY(cudaFuncSetAttribute(k_blocks_sym<BF16Bits, float>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zs));
-        k_blocks_sym<BF16Bits, float><<<nsym, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
+        k_blocks_sym<BF16Bits, float><<<grid, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
       }
     } else if (use32) {
       const float* B = (mode == kModePrecond) ? c.d_precond32.ptr : c.d_blockK32.ptr;
       if (zs > 48 * 1024)
         RBS_CUDA_TRY(cudaFuncSetAttribute(k_blocks_sym<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)zs));
-      k_blocks_sym<float, float><<<nsym, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
+      k_blocks_sym<float, float><<<grid, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
     } else {
       const double* B = (mode == kModePrecond) ? c.d_precond.ptr : (mode == kModeSelfS ? c.d_blockS.ptr : c.d_blockK.ptr);
       if (zs > 48 * 1024)
         RBS_CUDA_TRY(cudaFuncSetAttribute(k_blocks_sym<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)zs));
-      k_blocks_sym<double, double><<<nsym, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
+      k_blocks_sym<double, double><<<grid, kSymWarps * 32, zs, c.stream>>>(RBS_SYM_ARGS);
     }
 #undef RBS_SYM_ARGS
     RBS_CUDA_TRY(cudaGetLastError());
@@ -1362,26 +1256,22 @@ Status apply_blocks(Context& c, int mode, int prec, const double* x, double* y, 
 // Near correction, step 1: upsampled weighted densities of the near-source particles (float32
 // interpolation for the inner solve, float64 otherwise), in the form the sums of arithmetic prec read.
 static Status near_upsample(Context& c, int prec, const double* x) {
-  const bool f32 = prec_f32(prec);
-  const size_t smem = (f32 ? sizeof(float) : sizeof(double)) * 3 * (size_t)c.max_np;
   int maxup = 0;
   for (Grid* g : c.grids) maxup = std::max(maxup, g->nup);
-  const int nup_p = (int)c.up_particle.size();
-  dim3 gu(cdiv(maxup, 128), (unsigned)std::min(nup_p, 65535));
-#define RBS_UPSAMPLE(TU, FORM, U)                                                                                       \
-  do {                                                                                                                  \
-    if (smem > 48 * 1024)                                                                                               \
-      RBS_CUDA_TRY(cudaFuncSetAttribute(k_upsample<TU, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-    k_upsample<TU, FORM><<<gu, 128, smem, c.stream>>>(nup_p, c.d_up_particle.ptr, c.d_up_off.ptr, c.d_offset.ptr,       \
-                                                      c.d_nodes.ptr, U, x, c.d_up_x.ptr, c.d_up_q.ptr, c.d_up_qh.ptr,   \
-                                                      c.d_up_ql.ptr);                                                   \
-  } while (0)
-  if (f32)
-    RBS_UPSAMPLE(float, 1, c.d_upU32.ptr);
-  else if (prec == RBS_PREC_DF)
-    RBS_UPSAMPLE(double, 2, c.d_upU.ptr);
-  else
-    RBS_UPSAMPLE(double, 0, c.d_upU.ptr);
+  const int ng = (int)c.up_groups.size();
+#define RBS_UPSAMPLE(TU, FORM, U)                                                                                     \
+  k_upsample<TU, FORM><<<dim3(cdiv(maxup, kUpRows), cnt), 256, 0, c.stream>>>(                                        \
+      c.d_up_groups.ptr + g0, c.d_up_particle.ptr, c.d_up_off.ptr, c.d_offset.ptr, c.d_nodes.ptr, U, x, c.d_up_x.ptr, \
+      c.d_up_q.ptr, c.d_up_qh.ptr, c.d_up_ql.ptr)
+  for (int g0 = 0; g0 < ng; g0 += 65535) {
+    const int cnt = std::min(65535, ng - g0);
+    if (prec_f32(prec))
+      RBS_UPSAMPLE(float, 1, c.d_upU32.ptr);
+    else if (prec == RBS_PREC_DF)
+      RBS_UPSAMPLE(double, 2, c.d_upU.ptr);
+    else
+      RBS_UPSAMPLE(double, 0, c.d_upU.ptr);
+  }
 #undef RBS_UPSAMPLE
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
@@ -1390,25 +1280,9 @@ static Status near_upsample(Context& c, int prec, const double* x) {
 // Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one; kind 0
 // traction into y, 1 Stokeslet into y, 2 (double-float only) traction into y and Stokeslet into y2.
 static Status near_sums(Context& c, int kind, int prec, const double* x, double* y, double* y2) {
-  const long long nn = (long long)c.near_pairs.size();
   NearArgs A;
-  A.chunks = (c.max_np + 31) / 32;
-  // source runs: about 16 units per SM, of at least 128 sources
-  int most = 1;
-  for (Grid* g : c.grids) most = std::max(most, g->nup + g->np);
-  const long long units1 = nn * A.chunks;
-  A.parts = (int)std::max(1LL, std::min<long long>((16LL * c.sm_count + units1 - 1) / units1, most / 128));
-  const long long units = units1 * A.parts;
-  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "near correction: more than 2^31 work units");
-  A.nunits = (int)units;
-  A.counter = c.d_unit.ptr;
-  A.near = c.d_near.ptr;
-  A.offset = c.d_offset.ptr;
-  A.nodes = c.d_nodes.ptr;
-  A.up_index = c.d_up_index.ptr;
-  A.up_off = c.d_up_off.ptr;
-  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
-  const int blocks = (int)std::min<long long>((units + 3) / 4, INT_MAX);
+  int blocks = 0;
+  RBS_TRY(near_args(c, A, blocks));
 #define RBS_NEAR_LAUNCH(KERNEL, ...) \
   KERNEL<<<resident_grid(c, (const void*)KERNEL, 128, blocks), 128, 0, c.stream>>>(A, __VA_ARGS__)
   if (prec == RBS_PREC_DF) {
@@ -1453,16 +1327,14 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     RBS_TRY(weight_df(c, x));
   }
   if (f32 && c.tree.active) {
-    RBS_TRY(apply_tree(c, kind, x, y));  // treecode in place of the direct float32 sum
+    RBS_TRY(apply_tree(c, kind, y));  // treecode in place of the direct float32 sum
   } else if (prec == RBS_PREC_DF && c.tree_df.active) {
     RBS_TRY(apply_tree_df(c, kind, x, y, nullptr));  // and of the direct double-float sum
   } else if (nw > 0) {
     int cls = f32 ? (kind == 0 ? RBS_KC_PAIR_K32 : RBS_KC_PAIR_S32) : (kind == 0 ? RBS_KC_PAIR_K64 : RBS_KC_PAIR_S64);
     if (prec == RBS_PREC_DF) cls = kind == 0 ? RBS_KC_PAIR_KDF : RBS_KC_PAIR_SDF;
-    const int nt = (prec == RBS_PREC_FP64) ? 1 : pair_variant(c, kind, prec, x);
     KernelTimer timer(c, cls);
-    RBS_TRY(launch_pairs(c, kind, prec, nt, nw, x, y));
-    RBS_CUDA_TRY(cudaGetLastError());
+    RBS_TRY(launch_pairs(c, kind, prec, x, y));
     timer.done((double)c.stats.far_pairs);
   }
   if (!c.near_pairs.empty()) {
@@ -1488,18 +1360,17 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
     RBS_TRY(apply_tree_df(c, 2, x, yK, yS));
   } else if (nw > 0) {
     if (prec == RBS_PREC_DF) {
-      const int nt = pair_variant(c, 2, prec, x);
       KernelTimer timer(c, RBS_KC_PAIR_KSDF);
-      RBS_TRY(launch_pairs(c, 2, prec, nt, nw, x, yK, yS));
+      RBS_TRY(launch_pairs(c, 2, prec, x, yK, yS));
       timer.done((double)c.stats.far_pairs);
     } else {
       {
         KernelTimer timer(c, RBS_KC_PAIR_K64);
-        RBS_TRY(launch_pairs(c, 0, prec, 1, nw, x, yK));
+        RBS_TRY(launch_pairs(c, 0, prec, x, yK));
         timer.done((double)c.stats.far_pairs);
       }
       KernelTimer timer(c, RBS_KC_PAIR_S64);
-      RBS_TRY(launch_pairs(c, 1, prec, 1, nw, x, yS));
+      RBS_TRY(launch_pairs(c, 1, prec, x, yS));
       timer.done((double)c.stats.far_pairs);
     }
   }

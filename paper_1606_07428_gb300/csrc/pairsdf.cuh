@@ -88,25 +88,22 @@ struct inv_powers {
 // or on a common grid (df_tile).
 enum DfMode { kDfPlain = 0, kDfMask = 1, kDfGrid = 2 };
 
-// One target against two sources, KIND 0 traction into acc, 1 Stokeslet into acc, 2 traction into acc and
-// Stokeslet into acc2; fb = kBiasFactor |density| of the sources.  With two-sums 221 float32 operations
-// for both kernels, 154 for the traction alone and 139 for the Stokeslet alone; 9 fewer on the grid.
-template <int KIND, int MODE>
-__device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], float2 fb, int2 spid,
-                                         const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
-  df2 d[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    if (MODE == kDfGrid) {
-      d[c] = norm2(__fadd2_rn(xt[c].h, y[c].h), __fadd2_rn(xt[c].l, y[c].l));
-    } else {
-      d[c] = two_sum2(xt[c].h, y[c].h);
-      d[c].l = __fadd2_rn(d[c].l, __fadd2_rn(xt[c].l, y[c].l));
-    }
-  }
+// One component of the separation from the target's coordinate and the source's negated one.
+template <int MODE>
+__device__ __forceinline__ df2 df_separation(df2 x, df2 y) {
+  if (MODE == kDfGrid) return norm2(__fadd2_rn(x.h, y.h), __fadd2_rn(x.l, y.l));
+  df2 d = two_sum2(x.h, y.h);
+  d.l = __fadd2_rn(d.l, __fadd2_rn(x.l, y.l));
+  return d;
+}
+
+// Powers of 1 / r for the separation d, and R = r^2 in float32; MODE kDfMask zeroes them for sources of the
+// target's own particle.
+template <int MODE>
+__device__ __forceinline__ inv_powers df_inv_powers(const df2 (&d)[3], int2 spid, int pt, float2& R) {
   // r^2 by biased accumulation over 5/4 of its own float32 value R (over R itself the sum can round to
   // just above 2 R, where the difference from R is inexact)
-  const float2 R = __ffma2_rn(d[2].h, d[2].h, __ffma2_rn(d[1].h, d[1].h, __fmul2_rn(d[0].h, d[0].h)));
+  R = __ffma2_rn(d[2].h, d[2].h, __ffma2_rn(d[1].h, d[1].h, __fmul2_rn(d[0].h, d[0].h)));
   float2 y0 = make_float2(rsqrt_hw(R.x), rsqrt_hw(R.y));
   if (MODE == kDfMask) {  // the target's own particle: every power of 1 / r becomes zero
     if (spid.x == pt) y0.x = 0.0f;
@@ -120,7 +117,21 @@ __device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3],
   e0 = __ffma2_rn(__ffma2_rn(dup2(2.0f), d[0].h, d[0].l), d[0].l, e0);
   e1 = __ffma2_rn(__ffma2_rn(dup2(2.0f), d[1].h, d[1].l), d[1].l, e1);
   e2 = __ffma2_rn(__ffma2_rn(dup2(2.0f), d[2].h, d[2].l), d[2].l, e2);
-  const inv_powers p(__fadd2_rn(s2, ng2(Rb)), __fadd2_rn(__fadd2_rn(e0, e1), e2), y0);
+  return inv_powers(__fadd2_rn(s2, ng2(Rb)), __fadd2_rn(__fadd2_rn(e0, e1), e2), y0);
+}
+
+// One target against two sources, KIND 0 traction into acc, 1 Stokeslet into acc, 2 traction into acc and
+// Stokeslet into acc2; fb = kBiasFactor |density| of the sources.  With two-sums 221 float32 operations
+// for both kernels, 154 for the traction alone and 139 for the Stokeslet alone; 9 fewer on the grid.
+template <int KIND, int MODE>
+__device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], float2 fb, int2 spid,
+                                         const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
+  df2 d[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) d[c] = df_separation<MODE>(xt[c], y[c]);
+  float2 R;
+  const inv_powers p = df_inv_powers<MODE>(d, spid, pt, R);
+  const float2 y0 = p.y0;
   const float2 r = __fmul2_rn(R, y0);
   const df2 rr = bdot2(d[0], den[0], d[1], den[1], d[2], den[2], __fmul2_rn(r, fb));
   const df2 a = mul2(rr, p.y3());  // r . q / r^3 but for the series
@@ -191,23 +202,25 @@ __device__ __forceinline__ void df_tile_pairs(const float (*sa)[kTileDf], const 
   }
 }
 
-template <int KIND>
-__device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int filled, bool masked, bool split, int half,
-                                        const float4* __restrict__ x3h, const float4* __restrict__ x3m,
-                                        const float4* __restrict__ x3l, const float4* __restrict__ qh_,
-                                        const float4* __restrict__ ql_, const float4& oh, const float4& om,
-                                        const float4& ol, const dflt (&x0)[3], const dflt (&n0)[3], float xm, int pt,
-                                        dflt (&tot)[3], dflt (&tot2)[3], float sign = 1.0f) {
+// Stages the coordinates of a tile and the target's in the tile's form (xt); stage_q(l, s) stores what else
+// slot l needs of source s (s < 0: a padding slot, to be given zero density).  Returns whether the tile is
+// on a grid.
+template <typename StageQ>
+__device__ __forceinline__ bool df_stage(float (*sa)[kTileDf], int* spid, const int (&sidx)[2], int filled, bool masked,
+                                         const float4* __restrict__ x3h, const float4* __restrict__ x3m,
+                                         const float4* __restrict__ x3l, const float4& oh, const float4& om,
+                                         const float4& ol, const dflt (&x0)[3], float xm, df2 (&xt)[3], StageQ stage_q) {
   const int lane = threadIdx.x & 31;
-  float(*sa)[kTileDf] = reinterpret_cast<float(*)[kTileDf]>(wsm);
-  int* const spid = reinterpret_cast<int*>(&sa[13][0]);
   dflt p[2][3];
+  int pid[2];
   float m = 0.0f, mn = 3.0e38f;
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     p[k][0] = p[k][1] = p[k][2] = dflt{0.0f, 0.0f};
+    pid[k] = -2;
     if (lane + 32 * k < filled) {
       const float4 ph = x3h[sidx[k]], pm = x3m[sidx[k]], pl = x3l[sidx[k]];
+      pid[k] = __float_as_int(ph.w);
       p[k][0] = df_diff3(oh.x, om.x, ol.x, ph.x, pm.x, pl.x);
       p[k][1] = df_diff3(oh.y, om.y, ol.y, ph.y, pm.y, pl.y);
       p[k][2] = df_diff3(oh.z, om.z, ol.z, ph.z, pm.z, pl.z);
@@ -233,36 +246,57 @@ __device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int fi
   for (int k = 0; k < 2; ++k) {
     const int l = lane + 32 * k;
     if (l < filled) {
-      const float4 qh = qh_[sidx[k]], ql = ql_[sidx[k]];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const dflt v = on_grid(p[k][c]);
         sa[2 * c][l] = v.h;
         sa[2 * c + 1][l] = v.l;
       }
-      sa[6][l] = sign * qh.x;
-      sa[7][l] = sign * ql.x;
-      sa[8][l] = sign * qh.y;
-      sa[9][l] = sign * ql.y;
-      sa[10][l] = sign * qh.z;
-      sa[11][l] = sign * ql.z;
-      sa[12][l] = kBiasFactor * sqrtf(fmaf(qh.x, qh.x, fmaf(qh.y, qh.y, qh.z * qh.z)));
-      spid[l] = __float_as_int(x3h[sidx[k]].w);
+      stage_q(l, sidx[k]);
+      spid[l] = pid[k];
     } else if (l < cnt4) {  // zero-density sources away from every target: they add exactly zero
       sa[0][l] = sa[2][l] = sa[4][l] = 8.0f * m;
       sa[1][l] = sa[3][l] = sa[5][l] = 0.0f;
-      for (int q = 6; q < 13; ++q) sa[q][l] = 0.0f;
+      stage_q(l, -1);
       spid[l] = -2;
     }
   }
-  df2 xt[3], nt[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const dflt v = on_grid(x0[c]);
     xt[c] = {dup2(v.h), dup2(v.l)};
-    nt[c] = {dup2(n0[c].h), dup2(n0[c].l)};
   }
   __syncwarp();
+  return grid;
+}
+
+template <int KIND>
+__device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int filled, bool masked, bool split, int half,
+                                        const float4* __restrict__ x3h, const float4* __restrict__ x3m,
+                                        const float4* __restrict__ x3l, const float4* __restrict__ qh_,
+                                        const float4* __restrict__ ql_, const float4& oh, const float4& om,
+                                        const float4& ol, const dflt (&x0)[3], const dflt (&n0)[3], float xm, int pt,
+                                        dflt (&tot)[3], dflt (&tot2)[3], float sign = 1.0f) {
+  float(*sa)[kTileDf] = reinterpret_cast<float(*)[kTileDf]>(wsm);
+  int* const spid = reinterpret_cast<int*>(&sa[13][0]);
+  df2 xt[3], nt[3];
+  const bool grid = df_stage(sa, spid, sidx, filled, masked, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
+    float4 qh = make_float4(0, 0, 0, 0), ql = qh;
+    if (s >= 0) {
+      qh = qh_[s];
+      ql = ql_[s];
+    }
+    sa[6][l] = sign * qh.x;
+    sa[7][l] = sign * ql.x;
+    sa[8][l] = sign * qh.y;
+    sa[9][l] = sign * ql.y;
+    sa[10][l] = sign * qh.z;
+    sa[11][l] = sign * ql.z;
+    sa[12][l] = kBiasFactor * sqrtf(fmaf(qh.x, qh.x, fmaf(qh.y, qh.y, qh.z * qh.z)));
+  });
+#pragma unroll
+  for (int c = 0; c < 3; ++c) nt[c] = {dup2(n0[c].h), dup2(n0[c].l)};
+  const int cnt4 = (filled + 3) & ~3;
   df2 acc[3], acc2[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) acc[c] = acc2[c] = df2{dup2(0.0f), dup2(0.0f)};

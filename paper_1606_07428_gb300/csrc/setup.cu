@@ -918,6 +918,16 @@ Status build_near(Context& c) {
     RBS_TRY(upload(c.d_upU, U, s));
     RBS_TRY(upload(c.d_upU32, U32, s));
   }
+  c.up_groups.clear();
+  for (size_t gi = 0; gi < c.grids.size(); ++gi) {
+    std::vector<int> ids;
+    for (size_t u = 0; u < c.up_particle.size(); ++u)
+      if (c.grid_of[c.up_particle[u]] == (int)gi) ids.push_back((int)u);
+    for (size_t k = 0; k < ids.size(); k += 4)
+      c.up_groups.push_back(make_int4(ids[k], k + 1 < ids.size() ? ids[k + 1] : -1, k + 2 < ids.size() ? ids[k + 2] : -1,
+                                      k + 3 < ids.size() ? ids[k + 3] : -1));
+  }
+  RBS_TRY(upload(c.d_up_groups, c.up_groups, s));
   RBS_TRY(upload(c.d_up_particle, c.up_particle, s));
   RBS_TRY(upload(c.d_up_off, c.up_offset, s));
   RBS_TRY(upload(c.d_up_index, c.up_index, s));
@@ -935,6 +945,9 @@ Status build_near(Context& c) {
     RBS_CUDA_TRY(cudaGetLastError());
   }
 
+  c.near_multi = false;
+  for (size_t k = 1; k < c.near_pairs.size(); ++k)  // (the list is ordered by target)
+    if (c.near_pairs[k].x == c.near_pairs[k - 1].x) c.near_multi = true;
   c.near_pair_nodes = 0;
   for (const int2& pr : c.near_pairs)
     c.near_pair_nodes += (double)(c.offset[pr.x + 1] - c.offset[pr.x]) *
@@ -1247,8 +1260,12 @@ Status build_geometry(Context& c) {
     int splits = (int)std::max(1LL, (want + tiles - 1) / std::max(1LL, tiles));
     for (auto& sp : susp) {
       long long ns = sp.second - sp.first;
-      // small systems: as many chunks as give every SM eight items, of 128 sources at least
-      const long long few = std::min((8LL * c.sm_count + tiles - 1) / tiles, ns / 128);
+      // small systems: as many chunks as give every SM 32 items (128 warps' units, some seven rounds of the
+      // double-float sums' 16 warps), of 128 sources at least
+      // (a float64 context's suspension below two chunks of 2,048 stays one chunk: its sums, one addition per
+      // target, are the same bits on every run)
+      const bool one = !prec_f32(c.opt.precision) && ns < 4096;
+      const long long few = one ? 1 : std::min((32LL * c.sm_count + tiles - 1) / tiles, ns / 128);
       int sc = (int)std::max(few, std::min<long long>(splits, std::max(1LL, ns / 2048)));
       long long chunk = (ns + sc - 1) / sc;
       for (long long tb = sp.first; tb < sp.second; tb += TT)

@@ -33,13 +33,10 @@ namespace rbs {
 
 namespace {
 
-constexpr int kTreeMaxQ = 11;        // degree <= 10
 constexpr int kTreeMaxTargets = 512; // targets per work item at most
 constexpr int kTreeTile32 = 128;     // sources per warp tile of the float32 treecode sum
 constexpr int kTreeMaxQ64 = 13;      // degree <= 12 (double-float passes)
 
-__device__ __forceinline__ float fma_any(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_any(double a, double b, double c) { return fma(a, b, c); }
 
 // Bounding box of each particle's nodes: lo (3) then hi (3) per particle.
 __global__ void __launch_bounds__(128) k_particle_boxes(int n, const long long* __restrict__ offset,
@@ -101,75 +98,175 @@ __device__ __forceinline__ void lagrange_row(T u, const T* s, const T* bw, int n
     if (k < nq) L[k] = hit >= 0 ? (k == hit ? (T)1 : (T)0) : t[k] / sum;
 }
 
-// Cluster charges, one block per (cluster, run of its particles); T = float or double.  Nodes are staged
-// kChargeTile at a time with their Lagrange rows in x and y and the products L_c(z) q_k (k = 0, 1, 2); a
-// thread owns NB values of b for one a of the proxy grid and every c, so a node costs it NB products
-// L_a L_b and 3 multiply-adds per proxy.  The threads form groups of one (a, b) plane each that take the
-// staged nodes in turn; in float32 the groups add up in shared memory first, then one group's worth of
-// partial charges is added atomically to the cluster's (zeroed before).  Charges are stored by rows of the
-// grid's last axis, the layout that the pair kernels read: q[(((cluster nq + a) nbp + b) 3 + k) ncp + c],
-// rows padded to ncp and planes to nbp rows with zeros.
+// Cluster charges, one block per (cluster, run of its particles), from the nodes' weighted densities.
+// They are stored by rows of the proxy grid's last axis, the layout that the pair kernels read:
+// q[(((cluster nq + a) nbp + b) 3 + k) ncp + c], rows padded to ncp and planes to nbp rows with zeros (all
+// zeroed before; blocks add theirs atomically).  A node costs one product L_a L_b per row and 3
+// multiply-adds per proxy on the products L_c(z) q_k.
 constexpr int kChargeThreads = 256;
-constexpr int kChargeTile = 64;
 
-template <typename T, int MAXQ, int NB>
-__global__ void __launch_bounds__(kChargeThreads) k_tree_charges(const int4* __restrict__ items,
-                                                                 const int* __restrict__ order,
-                                                                 const long long* __restrict__ offset,
-                                                                 const double4* __restrict__ x,
-                                                                 const double* __restrict__ dens,
-                                                                 const double* __restrict__ box,
-                                                                 const T* __restrict__ cheb, int nq, int nbp, int ncp,
-                                                                 T* __restrict__ qproxy) {
-  constexpr int TS = kChargeTile;
-  constexpr int MC = (MAXQ + 3) & ~3, MB = (MAXQ + NB - 1) / NB * NB;
-  constexpr bool kReduce = sizeof(T) == 4;
-  __shared__ T sLx[TS][MAXQ];
-  __shared__ __align__(16) T sLy[TS][MB];
-  __shared__ __align__(16) T sq[TS][3][MC];
-  __shared__ T s_sum[kReduce ? 3 * MAXQ * MAXQ * MAXQ : 1];
-  __shared__ T s_pts[MAXQ], s_bw[MAXQ];
+// Float32.  Warps take batches of 32 nodes of the run on their own: each lane forms the three Lagrange rows
+// of one node, then owns two (a, b) rows of the proxy grid and every c over the batch's nodes (12 packed
+// multiply-adds a node and row, loads shared by the two rows).  Grids of more than 64 rows take several passes.
+constexpr int kChargeThreads32 = 128;
+
+template <int MAXQ>
+__global__ void __launch_bounds__(kChargeThreads32) k_tree_charges32(const int4* __restrict__ items,
+                                                                   const int* __restrict__ order,
+                                                                   const long long* __restrict__ offset,
+                                                                   const double4* __restrict__ x,
+                                                                   const float4* __restrict__ wmu,
+                                                                   const double* __restrict__ box,
+                                                                   const float* __restrict__ cheb, int nq, int nbp,
+                                                                   int ncp, float* __restrict__ qproxy) {
+  constexpr int W = kChargeThreads32 / 32, MQ = 3 * MAXQ + 4;  // row pitch of 4 mod 32 words: no bank conflicts
+  __shared__ float sL[W][32][2 * MAXQ + 1];
+  __shared__ __align__(16) float sq[W][32][MQ];
+  __shared__ float s_pts[MAXQ], s_bw[MAXQ];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if ((int)threadIdx.x < nq) {
     s_pts[threadIdx.x] = cheb[threadIdx.x];
     s_bw[threadIdx.x] = cheb[nq + threadIdx.x];
   }
-  if (kReduce)
-    for (int k = threadIdx.x; k < 3 * nq * nq * nq; k += kChargeThreads) s_sum[k] = 0;
+  __syncthreads();
   const int4 it = items[blockIdx.x];
   const int u = it.x;
-  const int nbt = (nq + NB - 1) / NB, plane = nq * nbt;
+  const double* bx = box + 6 * (size_t)u;
+  const double m0 = bx[0], m1 = bx[1], m2 = bx[2], h0 = bx[3], h1 = bx[4], h2 = bx[5];
+  for (int pass = 0; pass < nq * nq; pass += 64) {
+    int ra[2], rb[2];
+    bool own[2];
+    float2 acc[2][3][MAXQ / 2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int ab = pass + lane + 32 * h;
+      own[h] = ab < nq * nq;
+      ra[h] = own[h] ? ab / nq : 0;
+      rb[h] = own[h] ? ab - ra[h] * nq : 0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < MAXQ / 2; ++c) acc[h][k][c] = make_float2(0.0f, 0.0f);
+    }
+    int batch = 0;
+    bool any = false;
+    for (int pi = it.y; pi < it.z; ++pi) {
+      const int j = order[pi];
+      const long long e = offset[j + 1];
+      for (long long s0 = offset[j]; s0 < e; s0 += 32, ++batch) {
+        if (batch % W != warp) continue;
+        any = true;
+        const int cnt = (int)min(32LL, e - s0);
+        __syncwarp();  // the previous batch is read
+        if (lane < cnt) {
+          const double4 p = x[s0 + lane];
+          const float4 q = wmu[s0 + lane];
+          float L[MAXQ];
+          lagrange_row<float, MAXQ>((float)((p.x - m0) * h0), s_pts, s_bw, nq, L);
+#pragma unroll
+          for (int k = 0; k < MAXQ; ++k)
+            if (k < nq) sL[warp][lane][k] = L[k];
+          lagrange_row<float, MAXQ>((float)((p.y - m1) * h1), s_pts, s_bw, nq, L);
+#pragma unroll
+          for (int k = 0; k < MAXQ; ++k)
+            if (k < nq) sL[warp][lane][MAXQ + k] = L[k];
+          lagrange_row<float, MAXQ>((float)((p.z - m2) * h2), s_pts, s_bw, nq, L);
+#pragma unroll
+          for (int k = 0; k < MAXQ; ++k) {
+            const float l = k < nq ? L[k] : 0.0f;
+            sq[warp][lane][k] = l * q.x;
+            sq[warp][lane][MAXQ + k] = l * q.y;
+            sq[warp][lane][2 * MAXQ + k] = l * q.z;
+          }
+        }
+        __syncwarp();
+#pragma unroll 2
+        for (int l = 0; l < cnt; ++l) {
+          float2 w[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float v = sL[warp][l][ra[h]] * sL[warp][l][MAXQ + rb[h]];
+            w[h] = make_float2(v, v);
+          }
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int c = 0; c < MAXQ / 4; ++c) {
+              const float4 q = *reinterpret_cast<const float4*>(&sq[warp][l][k * MAXQ + 4 * c]);
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                acc[h][k][2 * c] = __ffma2_rn(w[h], make_float2(q.x, q.y), acc[h][k][2 * c]);
+                acc[h][k][2 * c + 1] = __ffma2_rn(w[h], make_float2(q.z, q.w), acc[h][k][2 * c + 1]);
+              }
+            }
+        }
+      }
+    }
+    if (!any) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!own[h]) continue;
+      float* dst = qproxy + ((size_t)(u * nq + ra[h]) * nbp + rb[h]) * 3 * ncp;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < MAXQ / 4; ++c)
+          if (4 * c < ncp)
+            atomicAdd(reinterpret_cast<float4*>(dst + k * ncp + 4 * c),
+                      make_float4(acc[h][k][2 * c].x, acc[h][k][2 * c].y, acc[h][k][2 * c + 1].x, acc[h][k][2 * c + 1].y));
+    }
+  }
+}
+
+// Float64: nodes are staged kChargeTile at a time by the block, one thread per (node, axis); a thread owns
+// one (a, b) row, and threads beyond the first plane take the staged nodes in turn.  Bound by the float64 pipe.
+constexpr int kChargeTile = 64;
+
+__global__ void __launch_bounds__(kChargeThreads) k_tree_charges64(const int4* __restrict__ items,
+                                                                   const int* __restrict__ order,
+                                                                   const long long* __restrict__ offset,
+                                                                   const double4* __restrict__ x,
+                                                                   const double* __restrict__ dens,
+                                                                   const double* __restrict__ box,
+                                                                   const double* __restrict__ cheb, int nq, int nbp,
+                                                                   int ncp, double* __restrict__ qproxy) {
+  constexpr int TS = kChargeTile, MAXQ = kTreeMaxQ64;
+  __shared__ double sL[TS][2][MAXQ];
+  __shared__ __align__(16) double sq[TS][3][MAXQ + 1];
+  __shared__ double s_pts[MAXQ], s_bw[MAXQ];
+  if ((int)threadIdx.x < nq) {
+    s_pts[threadIdx.x] = cheb[threadIdx.x];
+    s_bw[threadIdx.x] = cheb[nq + threadIdx.x];
+  }
+  const int4 it = items[blockIdx.x];
+  const int u = it.x;
+  const int plane = nq * nq;
   const int groups = kChargeThreads / plane;  // at least one: plane <= 169
   const int g = threadIdx.x / plane;
-  const int ab = threadIdx.x - g * plane, a = ab / nbt, b = NB * (ab - a * nbt);
-  T acc[NB][3][MAXQ];
+  const int ab = threadIdx.x - g * plane, a = ab / nq, b = ab - a * nq;
+  double acc[3][MAXQ];
 #pragma unroll
-  for (int h = 0; h < NB; ++h)
-#pragma unroll
-    for (int c = 0; c < MAXQ; ++c) acc[h][0][c] = acc[h][1][c] = acc[h][2][c] = 0;
+  for (int c = 0; c < MAXQ; ++c) acc[0][c] = acc[1][c] = acc[2][c] = 0;
   for (int pi = it.y; pi < it.z; ++pi) {
     const int j = order[pi];
     const long long o = offset[j], e = offset[j + 1];
     for (long long s0 = o; s0 < e; s0 += TS) {
       const int cnt = (int)min((long long)TS, e - s0);
       __syncthreads();
-      // one thread per (node, axis)
       const int ax = threadIdx.x / TS, l = threadIdx.x - TS * ax;
       if (ax < 3 && l < cnt) {
         const double4 p = x[s0 + l];
         const double v = ax == 0 ? p.x : (ax == 1 ? p.y : p.z);
         const double m = box[6 * (size_t)u + ax], h = box[6 * (size_t)u + 3 + ax];
-        T L[MAXQ];
-        lagrange_row<T, MAXQ>((T)((v - m) * h), s_pts, s_bw, nq, L);
-        if (ax == 0) {
+        double L[MAXQ];
+        lagrange_row<double, MAXQ>((v - m) * h, s_pts, s_bw, nq, L);
+        if (ax < 2) {
 #pragma unroll
           for (int k = 0; k < MAXQ; ++k)
-            if (k < nq) sLx[l][k] = L[k];
-        } else if (ax == 1) {
-#pragma unroll
-          for (int k = 0; k < MB; ++k) sLy[l][k] = k < nq && k < MAXQ ? L[k < MAXQ ? k : 0] : (T)0;
+            if (k < nq) sL[l][ax][k] = L[k];
         } else {
           const double* d = dens + 3 * (s0 + l);
-          const T q0 = (T)(p.w * d[0]), q1 = (T)(p.w * d[1]), q2 = (T)(p.w * d[2]);
+          const double q0 = p.w * d[0], q1 = p.w * d[1], q2 = p.w * d[2];
 #pragma unroll
           for (int k = 0; k < MAXQ; ++k)
             if (k < nq) {
@@ -182,48 +279,24 @@ __global__ void __launch_bounds__(kChargeThreads) k_tree_charges(const int4* __r
       __syncthreads();
       if (g < groups) {
         for (int l2 = g; l2 < cnt; l2 += groups) {
-          T w[NB];
+          const double w = sL[l2][0][a] * sL[l2][1][b];
 #pragma unroll
-          for (int h = 0; h < NB; ++h) w[h] = sLx[l2][a] * sLy[l2][b + h];
-#pragma unroll
-          for (int k = 0; k < 3; ++k)
-#pragma unroll
-            for (int c = 0; c < MAXQ; ++c)
-              if (c < nq) {
-                const T v = sq[l2][k][c];
-#pragma unroll
-                for (int h = 0; h < NB; ++h) acc[h][k][c] = fma_any(w[h], v, acc[h][k][c]);
-              }
+          for (int c = 0; c < MAXQ; ++c)
+            if (c < nq) {
+              acc[0][c] = fma(w, sq[l2][0][c], acc[0][c]);
+              acc[1][c] = fma(w, sq[l2][1][c], acc[1][c]);
+              acc[2][c] = fma(w, sq[l2][2][c], acc[2][c]);
+            }
         }
       }
     }
   }
-  // the groups add their sums in turn
-  for (int gg = 0; gg < (kReduce ? groups : 1); ++gg) {
-    if (kReduce) __syncthreads();
-    if (kReduce ? g == gg : g < groups) {
+  if (g < groups) {
+    double* dst = qproxy + ((size_t)(u * nq + a) * nbp + b) * 3 * ncp;
 #pragma unroll
-      for (int h = 0; h < NB; ++h) {
-        if (b + h >= nq) continue;
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-          for (int c = 0; c < MAXQ; ++c)
-            if (c < nq) {
-              if (kReduce)
-                s_sum[((a * nq + b + h) * 3 + k) * nq + c] += acc[h][k][c];
-              else
-                atomicAdd(qproxy + (((size_t)(u * nq + a) * nbp + b + h) * 3 + k) * ncp + c, acc[h][k][c]);
-            }
-      }
-    }
-  }
-  if (kReduce) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < 3 * nq * nq * nq; e += kChargeThreads) {
-      const int row = e / nq, c = e - row * nq, r3 = row / 3, k = row - 3 * r3, aa = r3 / nq, bb = r3 - aa * nq;
-      atomicAdd(qproxy + (((size_t)(u * nq + aa) * nbp + bb) * 3 + k) * ncp + c, s_sum[e]);
-    }
+    for (int c = 0; c < MAXQ; ++c)
+      if (c < nq)
+        for (int k = 0; k < 3; ++k) atomicAdd(dst + k * ncp + c, acc[k][c]);
   }
 }
 
@@ -1213,7 +1286,7 @@ int tree_variant(const Context& c) {
   return c.tree.degree > 7 || c.opt.pair_variant == 1 || c.opt.pair_variant == kPacked + 1 ? 1 : 2;
 }
 
-Status apply_tree(Context& c, int kind, const double* x, double* y) {
+Status apply_tree(Context& c, int kind, double* y) {
   TreeState& T = c.tree;
   {
     KernelTimer timer(c, RBS_KC_TREE);
@@ -1221,14 +1294,14 @@ Status apply_tree(Context& c, int kind, const double* x, double* y) {
     if (T.n_cells > 0) {
       RBS_CUDA_TRY(cudaMemsetAsync(T.d_pq.ptr, 0, sizeof(float) * T.d_pq.n, c.stream));
       const int nq = T.degree + 1;
+#define RBS_CHARGE_ARGS                                                                                            \
+  T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, c.d_wmu32.ptr, T.d_box.ptr, T.d_cheb.ptr, nq, T.nbp, \
+      T.ncp, T.d_pq.ptr
       if (nq <= 8)
-        k_tree_charges<float, 8, 2><<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
-            T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb.ptr, nq, T.nbp,
-            T.ncp, T.d_pq.ptr);
+        k_tree_charges32<8><<<(unsigned)T.charge_items.size(), kChargeThreads32, 0, c.stream>>>(RBS_CHARGE_ARGS);
       else
-        k_tree_charges<float, kTreeMaxQ, 2><<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
-            T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb.ptr, nq, T.nbp,
-            T.ncp, T.d_pq.ptr);
+        k_tree_charges32<12><<<(unsigned)T.charge_items.size(), kChargeThreads32, 0, c.stream>>>(RBS_CHARGE_ARGS);
+#undef RBS_CHARGE_ARGS
       launches = 1;
     }
     RBS_CUDA_TRY(cudaGetLastError());
@@ -1269,7 +1342,7 @@ Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y
       const int nq = T.degree + 1;
       const long long rows = (long long)T.n_cells * nq * T.nbp;
       RBS_CUDA_TRY(cudaMemsetAsync(T.d_q64.ptr, 0, sizeof(double) * T.d_q64.n, c.stream));
-      k_tree_charges<double, kTreeMaxQ64, 1><<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
+      k_tree_charges64<<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
           T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb64.ptr, nq, T.nbp,
           T.ncp, T.d_q64.ptr);
       k_tree_q64_split<<<cdiv(rows * T.ncp, 256), 256, 0, c.stream>>>(rows, T.ncp, T.d_q64.ptr, T.d_pq.ptr);
