@@ -89,7 +89,13 @@ struct Grid {
   std::vector<double> t, lam;         // Gauss-Legendre nodes (ascending) and weights, p + 1
   std::vector<double> t_up, lam_up;   // the same for the upsampled grid
   DevBuf<double> d_t, d_lam, d_t_up, d_lam_up;
-  DevBuf<double> d_interp;  // (p + 1) x nrot x np: singular-rule interpolation, target (j, 0)
+  // singular-rule interpolation for target (j, 0) in two factors: harmonics of all orders (nfull = (p + 1)^2) at
+  // the rule's points in their own frame, as products of d_rule_trig (nb / 2 + 1 rows of cos and sin (m phi'),
+  // nf = 2 p + 1 columns) and d_rule_leg ((ps + 1) x nfull), times d_rule ((p + 1) x nfull x np): the rotation
+  // to the target's frame and the analysis of the grid values
+  int nfull = 0, nf = 0;
+  DevBuf<double> d_rule, d_rule_trig, d_rule_leg;
+  DevBuf<int> d_rule_col;   // per harmonic: its trig column
   DevBuf<double> d_rotpts;  // (p + 1) x nrot x 4: rotated-rule points (x, y, z, weight)
   DevBuf<double> d_up;      // nup x np: interpolation to the upsampled grid
   DevBuf<double> d_an;      // nbasis x np: analysis (grid values -> coefficients)
@@ -495,6 +501,11 @@ void gauss_legendre_newton(int n, std::vector<double>& t, std::vector<double>& w
 Status build_self_gemm(Context& c);
 Status apply_self_gemm(Context& c, int mode, const double* x, double* y, double* aux, double scale);
 Status check_self_gemm(Context& c);
+
+// Rule sums of `rows` rows of kernel values (nrot each; per shape stride strideC) against the rule's harmonics:
+// out (rows x nfull per shape, stride strideOut).
+Status rule_transform(Context& c, const Grid& g, int rows, int shapes, const double* C, long long strideC, double* out,
+                      long long strideOut);
 
 // ---- dense kernels (linalg.cu)
 Status dgemm_batched(cudaStream_t s, int M, int N, int K, const double* A, long long lda, long long strideA,

@@ -484,13 +484,14 @@ static Status build_laplace(Context& c) {
       }
     if (ids.empty()) continue;
     const long long rowsC = 2LL * g.nphi;
-    const size_t perC = (size_t)rowsC * g.nrot, perG = (size_t)rowsC * g.np;
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(ids.size(), ((size_t)1 << 27) / (perC + perG)));
-    DevBuf<double> C, G;
+    const size_t perC = (size_t)rowsC * g.nrot, perG = (size_t)rowsC * g.np, perH = (size_t)rowsC * g.nfull;
+    const int chunk = (int)std::max<size_t>(1, std::min<size_t>(ids.size(), ((size_t)1 << 27) / (perC + perG + perH)));
+    DevBuf<double> C, G, H;
     DevBuf<int> d_ids;
     DevBuf<long long> d_off;
     RBS_TRY(C.alloc(perC * chunk));
     RBS_TRY(G.alloc(perG * chunk));
+    RBS_TRY(H.alloc(perH * chunk));
     RBS_TRY(d_ids.alloc(ids.size()));
     RBS_TRY(d_off.alloc(goff.size()));
     RBS_CUDA_TRY(cudaMemcpyAsync(d_ids.ptr, ids.data(), sizeof(int) * ids.size(), cudaMemcpyHostToDevice, s));
@@ -502,8 +503,9 @@ static Status build_laplace(Context& c) {
         k_lap_kernel_values<<<grd, 128, 0, s>>>(g.nphi, g.nrot, g.t[j], d_ids.ptr + st, RBS_SHAPE_PASS,
                                                 (const double4*)g.d_rotpts.ptr + (size_t)j * g.nrot, C.ptr, perC);
         RBS_CUDA_TRY(cudaGetLastError());
-        RBS_TRY(dgemm_batched(s, (int)rowsC, g.np, g.nrot, C.ptr, g.nrot, (long long)perC,
-                              g.d_interp.ptr + (size_t)j * g.nrot * g.np, g.np, 0, G.ptr, g.np, (long long)perG, cnt));
+        RBS_TRY(rule_transform(c, g, (int)rowsC, cnt, C.ptr, (long long)perC, H.ptr, (long long)perH));
+        RBS_TRY(dgemm_batched(s, (int)rowsC, g.np, g.nfull, H.ptr, g.nfull, (long long)perH,
+                              g.d_rule.ptr + (size_t)j * g.nfull * g.np, g.np, 0, G.ptr, g.np, (long long)perG, cnt));
         dim3 grs(cdiv(2LL * g.nphi * g.np, 256), cnt);
         k_lap_scatter<<<grs, 256, 0, s>>>(g.nphi, g.np, j, G.ptr, perG, d_off.ptr + st, M.d_blockK.ptr,
                                           M.d_blockS.ptr);

@@ -134,6 +134,60 @@ __global__ void k_analysis(int np, int nbasis, const double* Yg, const double4* 
 
 
 
+// Points R_y(theta_j) s of every polar node j: out[j * npts + i].
+__global__ void k_rotate_points(int npts, int nj, const double* t, const double4* pts, double4* out) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= (long long)npts * nj) return;
+  const int j = (int)(e / npts);
+  const double4 s = pts[e - (long long)j * npts];
+  const double ct = t[j], st = sqrt(fmax(0.0, 1.0 - ct * ct));
+  out[e] = make_double4(ct * s.x + st * s.z, s.y, -st * s.x + ct * s.z, s.w);
+}
+
+// Sums of kernel-value rows over the singular rule against every harmonic of degree <= p at the rule's points
+// in their own frame, where the harmonics are products: out[row][b] = sum over theta' of leg[theta'][b] sum
+// over phi' of trig[phi'][col(b)] C[row][theta'][phi'].  One block per (row, shape); the phi' sums run over the
+// half circle, on the sums (cosines) and differences (sines) of opposite points.  About 20,000
+// multiply-adds a row at p = 12 where the rule's nrot x N_p interpolation matrix takes 390,000.
+__global__ void __launch_bounds__(256) k_rule_transform(int na, int slab, int nb, int nf, int nfull, const double* trig,
+                                                        const double* leg, const int* col, const double* C,
+                                                        long long strideC, double* out, long long strideOut) {
+  extern __shared__ double rule_smem[];
+  const int nh = nb / 2 + 1;
+  double* H = rule_smem;                // na x nf
+  double* sum = H + na * nf;            // slab x nh: `slab` values of theta' at a time
+  double* dif = sum + slab * nh;        // slab x nh
+  const double* row = C + strideC * blockIdx.y + (long long)blockIdx.x * na * nb;
+  for (int a0 = 0; a0 < na; a0 += slab) {
+    const int ns = min(slab, na - a0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < ns * nh; e += blockDim.x) {
+      const int a = e / nh, b = e - a * nh;
+      const double* r = row + (a0 + a) * nb;
+      const bool paired = b > 0 && 2 * b != nb;
+      const double u = r[b], v = paired ? r[nb - b] : 0.0;
+      sum[e] = u + v;
+      dif[e] = paired ? u - v : 0.0;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < ns * nf; e += blockDim.x) {
+      const int a = e / nf, f = e - a * nf;
+      const double* src = ((f & 1) || f == 0 ? sum : dif) + a * nh;  // columns: 1, cos, sin, cos 2, sin 2, ...
+      double acc = 0.0;
+      for (int b = 0; b < nh; ++b) acc = fma(src[b], __ldg(trig + b * nf + f), acc);
+      H[(a0 + a) * nf + f] = acc;
+    }
+  }
+  __syncthreads();
+  double* dst = out + strideOut * blockIdx.y + (long long)blockIdx.x * nfull;
+  for (int k = threadIdx.x; k < nfull; k += blockDim.x) {
+    const int f = col[k];
+    double acc = 0.0;
+    for (int a = 0; a < na; ++a) acc = fma(H[a * nf + f], __ldg(leg + (long long)a * nfull + k), acc);
+    dst[k] = acc;
+  }
+}
+
 // Surface nodes of all particles (lab frame): x = c + R x_b(s), n = R n_b(s) and weight
 // (2 pi / nphi) lambda_j J(s) (Eq. 35 with W / sin(theta) = J), s the grid point of Eq. 33.
 __global__ void k_nodes(int n, const long long* offset, const int* pvec, const int* nphivec, const int* shape_of,
@@ -724,14 +778,74 @@ static Status build_grid(Context& c, Grid& g) {
   k_analysis<<<cdiv((long long)g.np * g.nbasis, 256), 256, 0, s>>>(g.np, g.nbasis, Yg.ptr, gp.ptr, An.ptr);
   RBS_CUDA_TRY(cudaGetLastError());
 
-  // singular-rule interpolation: Interp_j = Y(rotated points of j) x An
-  DevBuf<double> Yr;
-  long long nrp = (long long)(g.p + 1) * g.nrot;
-  RBS_TRY(Yr.alloc((size_t)nrp * g.nbasis));
-  k_sh_at_points<<<cdiv(nrp, 128), 128, 0, s>>>(g.p, g.mmax, g.nbasis, (const double4*)g.d_rotpts.ptr, (int)nrp,
-                                                Yr.ptr);
-  RBS_TRY(g.d_interp.alloc((size_t)nrp * g.np));
-  RBS_TRY(dgemm_batched(s, (int)nrp, g.np, g.nbasis, Yr.ptr, g.nbasis, 0, An.ptr, g.np, 0, g.d_interp.ptr, g.np, 0, 1));
+  // singular-rule interpolation: Y(rotated points of j) An = Y'(rule's points) D_j An, D_j the rotation of the
+  // harmonics of degree <= p by R_y(theta_j), D_j[b', b] = integral of Y_b'(s) Y_b(R_j s), exact on a grid of p + 1
+  // Gauss-Legendre by 2 p + 2 uniform points
+  {
+    const int na = g.ps + 1, nphi_q = 2 * g.p + 2, nq = (g.p + 1) * nphi_q, nj = g.p + 1;
+    g.nfull = (g.p + 1) * (g.p + 1);
+    g.nf = 2 * g.p + 1;
+    std::vector<double> trig((size_t)(nb / 2 + 1) * g.nf), leg((size_t)na * g.nfull);
+    std::vector<int> col(g.nfull), deg(g.nfull), ord(g.nfull);
+    int k = 0;
+    for (int m = 0; m <= g.p; ++m)
+      for (int n = m; n <= g.p; ++n)
+        for (int v = 0; v < (m == 0 ? 1 : 2); ++v, ++k) {
+          col[k] = m == 0 ? 0 : 2 * m - 1 + v;
+          deg[k] = n;
+          ord[k] = m;
+        }
+    for (int b = 0; b <= nb / 2; ++b)
+      for (int f = 0; f < g.nf; ++f) {
+        const int m = (f + 1) / 2;
+        const double ph = 2.0 * kPi * ((long long)m * b % nb) / nb;
+        trig[(size_t)b * g.nf + f] = (f == 0 || (f & 1)) ? std::cos(ph) : std::sin(ph);
+      }
+    std::vector<double> P((size_t)(g.p + 1) * (g.p + 1));  // normalised associated Legendre values at one angle
+    for (int a = 0; a < na; ++a) {
+      const double th = 0.5 * kPi * (u[a] + 1.0), ct = std::cos(th), st = std::sin(th);
+      double pmm = std::sqrt(1.0 / (4.0 * kPi));
+      for (int m = 0; m <= g.p; ++m) {
+        if (m > 0) pmm *= std::sqrt((2.0 * m + 1.0) / (2.0 * m)) * st;
+        double p2 = 0.0, p1 = pmm;
+        for (int n = m; n <= g.p; ++n) {
+          double pn = p1;
+          if (n > m) {
+            const double x = std::sqrt((4.0 * n * n - 1.0) / ((double)n * n - (double)m * m));
+            const double y = n > m + 1 ? std::sqrt(((n - 1.0) * (n - 1.0) - (double)m * m) / (4.0 * (n - 1.0) * (n - 1.0) - 1.0)) : 0.0;
+            pn = x * (ct * p1 - y * p2);
+            p2 = p1;
+            p1 = pn;
+          }
+          P[(size_t)n * (g.p + 1) + m] = m == 0 ? pn : std::sqrt(2.0) * pn;
+        }
+      }
+      for (int q = 0; q < g.nfull; ++q) leg[(size_t)a * g.nfull + q] = P[(size_t)deg[q] * (g.p + 1) + ord[q]];
+    }
+    RBS_TRY(upload(g.d_rule_trig, trig, s));
+    RBS_TRY(upload(g.d_rule_leg, leg, s));
+    RBS_TRY(upload(g.d_rule_col, col, s));
+    DevBuf<double4> qp, qr;
+    DevBuf<double> Yq, Aq, Yr, D;
+    RBS_TRY(qp.alloc(nq));
+    RBS_TRY(qr.alloc((size_t)nj * nq));
+    RBS_TRY(Yq.alloc((size_t)nq * g.nfull));
+    RBS_TRY(Aq.alloc((size_t)nq * g.nfull));
+    RBS_TRY(Yr.alloc((size_t)nj * nq * g.nbasis));
+    RBS_TRY(D.alloc((size_t)nj * g.nfull * g.nbasis));
+    RBS_TRY(g.d_rule.alloc((size_t)nj * g.nfull * g.np));
+    k_grid_points<<<cdiv(nq, 128), 128, 0, s>>>(g.p, nphi_q, g.d_t.ptr, g.d_lam.ptr, qp.ptr);
+    k_rotate_points<<<cdiv((long long)nj * nq, 128), 128, 0, s>>>(nq, nj, g.d_t.ptr, qp.ptr, qr.ptr);
+    k_sh_at_points<<<cdiv(nq, 128), 128, 0, s>>>(g.p, g.p, g.nfull, qp.ptr, nq, Yq.ptr);
+    k_analysis<<<cdiv((long long)nq * g.nfull, 256), 256, 0, s>>>(nq, g.nfull, Yq.ptr, qp.ptr, Aq.ptr);
+    k_sh_at_points<<<cdiv((long long)nj * nq, 128), 128, 0, s>>>(g.p, g.mmax, g.nbasis, qr.ptr, nj * nq, Yr.ptr);
+    RBS_CUDA_TRY(cudaGetLastError());
+    RBS_TRY(dgemm_batched(s, g.nfull, g.nbasis, nq, Aq.ptr, nq, 0, Yr.ptr, g.nbasis, (long long)nq * g.nbasis, D.ptr,
+                          g.nbasis, (long long)g.nfull * g.nbasis, nj));
+    RBS_TRY(dgemm_batched(s, g.nfull, g.np, g.nbasis, D.ptr, g.nbasis, (long long)g.nfull * g.nbasis, An.ptr, g.np, 0,
+                          g.d_rule.ptr, g.np, (long long)g.nfull * g.np, nj));
+    RBS_CUDA_TRY(cudaStreamSynchronize(s));  // temporaries and host tables are released here
+  }
 
   // upsampling interpolation U = Y(upsampled grid) x An
   DevBuf<double4> gup;
@@ -758,9 +872,24 @@ static Status build_grid(Context& c, Grid& g) {
   return Status::Ok();
 }
 
+Status rule_transform(Context& c, const Grid& g, int rows, int shapes, const double* C, long long strideC, double* out,
+                      long long strideOut) {
+  const int na = g.ps + 1, nb = 2 * g.ps + 2;
+  const int nh = nb / 2 + 1;
+  const int slab = std::min(na, std::max(1, 4096 / (2 * nh)));  // 32 KB of folded values
+  const size_t smem = sizeof(double) * ((size_t)na * g.nf + 2 * (size_t)slab * nh);
+  if (smem > 48 * 1024)
+    RBS_CUDA_TRY(cudaFuncSetAttribute(k_rule_transform, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_rule_transform<<<dim3(rows, shapes), 256, smem, c.stream>>>(na, slab, nb, g.nf, g.nfull, g.d_rule_trig.ptr,
+                                                               g.d_rule_leg.ptr, g.d_rule_col.ptr, C, strideC, out,
+                                                               strideOut);
+  RBS_CUDA_TRY(cudaGetLastError());
+  return Status::Ok();
+}
+
 // Self blocks of every shape of one grid, in chunks of shapes.  For each chunk and polar index j:
-// kernel values C (18 nkc x nrot per shape), one batched GEMM G = C x Interp_j, and the scatter
-// into the body-frame blocks with the azimuthal shift.  Shapes stored by representative rows (sym)
+// kernel values C (18 nkc x nrot per shape), their sums against the rule's harmonics (rule_transform), one
+// batched GEMM with the rotation and analysis G = C' x Rule_j, and the scatter into the body-frame blocks with the azimuthal shift.  Shapes stored by representative rows (sym)
 // need the targets j <= p / 2, k <= nphi / 4 only.
 static Status build_self_blocks(Context& c, int gi, const std::vector<int>& shape_ids, bool sym) {
   cudaStream_t s = c.stream;
@@ -768,14 +897,15 @@ static Status build_self_blocks(Context& c, int gi, const std::vector<int>& shap
   const int nkc = sym ? g.nk : g.nphi;
   const int jmax = sym ? g.nj - 1 : g.p;
   long long rowsC = 18LL * nkc;
-  size_t perC = (size_t)rowsC * g.nrot, perG = (size_t)rowsC * g.np;
+  size_t perC = (size_t)rowsC * g.nrot, perG = (size_t)rowsC * g.np, perH = (size_t)rowsC * g.nfull;
   size_t budget = (size_t)1 << 27;  // doubles, 1 GB
-  int per_chunk = (int)std::max<size_t>(1, budget / (perC + perG));
+  int per_chunk = (int)std::max<size_t>(1, budget / (perC + perG + perH));
   int nsh = (int)shape_ids.size();
   int chunk = std::min(std::min(per_chunk, nsh), 65535);
-  DevBuf<double> C, G;
+  DevBuf<double> C, G, H;
   RBS_TRY(C.alloc(perC * chunk));
   RBS_TRY(G.alloc(perG * chunk));
+  RBS_TRY(H.alloc(perH * chunk));
   std::vector<long long> off(nsh);
   for (int k = 0; k < nsh; ++k) off[k] = (long long)c.shapes[shape_ids[k]].block_off;
   DevBuf<int> d_ids;
@@ -789,8 +919,9 @@ static Status build_self_blocks(Context& c, int gi, const std::vector<int>& shap
       k_self_kernel_values<<<grd, 128, 0, s>>>(g.nphi, nkc, g.nrot, g.t[j], d_ids.ptr + start, RBS_SHAPE_PASS,
                                                (const double4*)g.d_rotpts.ptr + (size_t)j * g.nrot, C.ptr, perC);
       RBS_CUDA_TRY(cudaGetLastError());
-      RBS_TRY(dgemm_batched(s, (int)rowsC, g.np, g.nrot, C.ptr, g.nrot, (long long)perC,
-                            g.d_interp.ptr + (size_t)j * g.nrot * g.np, g.np, 0, G.ptr, g.np, (long long)perG, cnt));
+      RBS_TRY(rule_transform(c, g, (int)rowsC, cnt, C.ptr, (long long)perC, H.ptr, (long long)perH));
+      RBS_TRY(dgemm_batched(s, (int)rowsC, g.np, g.nfull, H.ptr, g.nfull, (long long)perH,
+                            g.d_rule.ptr + (size_t)j * g.nfull * g.np, g.np, 0, G.ptr, g.np, (long long)perG, cnt));
       long long tot = 2LL * nkc * 9 * g.np;
       dim3 grs(cdiv(tot, 256), cnt);
       k_self_scatter<<<grs, 256, 0, s>>>(g.nphi, nkc, g.np, j, G.ptr, perG, d_off.ptr + start, c.d_blockK.ptr,
