@@ -480,6 +480,9 @@ Status apply_tree(Context& c, int kind, double* y);
 int tree_variant(const Context& c);  // its targets per lane
 // The same for the double-float passes (d_wmuh, d_wmul): y += kind 0 or 1 sum; kind 2: y += traction, y2 += Stokeslet.
 Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y2);
+// y += traction and y2 += Stokeslet sum over the double-float passes' lists in float32 arithmetic (d_wmu32; the
+// charges formed in float64).
+Status apply_tree_df_f32(Context& c, const double* x, double* y, double* y2);
 // Relative error assumed for a float32 operator application: rounding plus, with the treecode,
 // its approximation model C(theta) rho^-n.
 double f32_operator_error(const Context& c);
@@ -533,6 +536,9 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y); 
 // yK += off-diagonal K x and yS += off-diagonal S x in one pass over the pairs (double-float)
 Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, double* yS);
 Status apply_operator(Context& c, int op, int prec, const double* x, double* y);
+// w = A d and v = S d for a correction d: float64 blocks and the near correction in double-float, only the smooth
+// sums in float32, over the same lists as the double-float passes.
+Status apply_correction(Context& c, const double* d, double* w, double* v);
 
 // ---- solver (solver.cu)
 Status mobility_solve(Context& c, const double* F, const double* T, double tol, double* v, double* om,

@@ -29,8 +29,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double rsq(double v) { return rsqrt(v); }
-
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
 
@@ -606,11 +604,13 @@ __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const d
 // from a counter and stage their own tiles of 128 sources, summed in float32 and added into a compensated
 // accumulator.  Tiles whose particles cannot meet the unit's targets skip the same-particle test.
 // Bound by the float32 pipe (20 operations a traction pair, 18 a Stokeslet pair).
+// KIND 2 (one target per lane): traction into y and Stokeslet into y2 in one pass, 26 operations.
 template <int KIND, int NT>
-__global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
+__global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
     k_pairs32x2(int nunits, int* __restrict__ counter, const longlong4* __restrict__ work,
                 const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
-                const float4* __restrict__ wmu, double* __restrict__ y) {
+                const float4* __restrict__ wmu, double* __restrict__ y, double* __restrict__ y2) {
+  static_assert(KIND != 2 || NT == 1, "both sums: one target per lane");
   constexpr int TW = 128, kPerItem = 4 / NT;
   __shared__ __align__(16) float tiles[4][7 * TW];
   const int lane = threadIdx.x & 31;
@@ -656,6 +656,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
     }
     const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(xhi[min(t0 + 32 * NT, t1) - 1].w);
     float sa[NT][3], ea[NT][3];
+    float sb[3] = {0.0f, 0.0f, 0.0f}, eb[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
     for (int s0 = (int)w.z; s0 < (int)w.w; s0 += TW) {
@@ -695,7 +696,15 @@ __global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
       pair_tile32x2<KIND, true, NT, NUV>(b, b + TW, b + 2 * TW, b + 3 * TW, b + 4 * TW, b + 5 * TW, spid + l0, m,  \
                                          xt, nt, pt, p);                                                           \
   } while (0)
-      if (nu == NT) {
+      if constexpr (KIND == 2) {
+        float2 p2[3] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
+        if (thi < pid_lo || tlo > pid_hi)
+          pair_tile32_both<false, TW>(ssx, spid, l0, m, xt[0], nt[0], pt[0], p[0], p2);
+        else
+          pair_tile32_both<true, TW>(ssx, spid, l0, m, xt[0], nt[0], pt[0], p[0], p2);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) two_sum_acc(sb[c], eb[c], p2[c].x + p2[c].y);
+      } else if (nu == NT) {
         RBS_TILE(NT);
       } else if constexpr (NT > 1) {
         RBS_TILE(1);
@@ -706,13 +715,16 @@ __global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
 #pragma unroll
         for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c].x + p[u][c].y);
     }
-    const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
+    const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
       if (!valid[u]) continue;
       const long long t = t0 + 32 * u + (split ? lane & 15 : lane);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
+      for (int c = 0; c < 3; ++c) {
+        atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
+        if (KIND == 2) atomicAdd(y2 + 3 * t + c, kStokesletScale * ((double)sb[c] + (double)eb[c]));
+      }
     }
   }
 }
@@ -1054,7 +1066,7 @@ __global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __res
       for (int l = 0; l < cnt; ++l) {
         const double4 ps = sp[warp][l], q = sq[warp][l];
         const double dx = xt.x - ps.x, dy = xt.y - ps.y, dz = xt.z - ps.z;
-        const double inv = rsq(dx * dx + dy * dy + dz * dz);
+        const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
         const double rr = dx * q.x + dy * q.y + dz * q.z;
         if (KIND == 0) {
           const double inv2 = inv * inv;
@@ -1121,11 +1133,11 @@ static int pairs32_targets(const Context& c) {
 int direct_variant(const Context& c) { return kPacked + pairs32_targets(c); }
 
 template <int KIND, int NT>
-static void launch_pairs32(Context& c, double* y) {
+static void launch_pairs32(Context& c, double* y, double* y2 = nullptr) {
   const int items = (int)c.work.size();
   const auto kernel = k_pairs32x2<KIND, NT>;
   kernel<<<resident_grid(c, (const void*)kernel, 128, items), 128, 0, c.stream>>>(
-      4 / NT * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y);
+      4 / NT * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y, y2);
 }
 
 template <int KIND>
@@ -1385,6 +1397,30 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
       RBS_TRY(near_sums(c, 1, prec, x, yS, nullptr));
       timer.done(2.0 * c.near_pair_nodes, 3);
     }
+  }
+  return Status::Ok();
+}
+
+Status apply_correction(Context& c, const double* d, double* w, double* v) {
+  RBS_TRY(apply_blocks(c, kModeSelfK, RBS_PREC_DF, d, w, nullptr, 1.0));
+  RBS_TRY(apply_blocks(c, kModeSelfS, RBS_PREC_DF, d, v, nullptr, 1.0));
+  c.stats.launches += 2;
+  RBS_TRY(weight_f32(c, d));
+  RBS_TRY(weight_df(c, d));
+  if (c.tree_df.active) {
+    RBS_TRY(apply_tree_df_f32(c, d, w, v));
+  } else if (!c.work.empty()) {
+    KernelTimer timer(c, RBS_KC_PAIR_K32);
+    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
+    launch_pairs32<2, 1>(c, w, v);
+    RBS_CUDA_TRY(cudaGetLastError());
+    timer.done(2.0 * (double)c.stats.far_pairs);
+  }
+  if (!c.near_pairs.empty()) {
+    KernelTimer timer(c, RBS_KC_NEAR);
+    RBS_TRY(near_upsample(c, RBS_PREC_DF, d));
+    RBS_TRY(near_sums(c, 2, RBS_PREC_DF, d, w, v));
+    timer.done(2.0 * c.near_pair_nodes, 2);
   }
   return Status::Ok();
 }

@@ -1398,7 +1398,8 @@ Status build_geometry(Context& c) {
       const bool one = !prec_f32(c.opt.precision) && ns < 4096;
       const long long few = one ? 1 : std::min((32LL * c.sm_count + tiles - 1) / tiles, ns / 128);
       int sc = (int)std::max(few, std::min<long long>(splits, std::max(1LL, ns / 2048)));
-      long long chunk = (ns + sc - 1) / sc;
+      // whole tiles of 128 sources (a chunk of 129 would stage a tile for its last source)
+      long long chunk = sc > 1 ? ((ns + sc - 1) / sc + 127) / 128 * 128 : ns;
       for (long long tb = sp.first; tb < sp.second; tb += TT)
         for (long long sb = sp.first; sb < sp.second; sb += chunk) {
           longlong4 w;

@@ -168,6 +168,9 @@ __global__ void k_unpack_vo(int n, const double* vo, double* v, double* om) {
 // L2 error of a few 1e-7 on the 1,000-ellipsoid p = 12 suspension, plus the treecode's model when it
 // is on) decides when a refinement residual may be updated in float32.
 
+// Relative error assumed for apply_correction.
+constexpr double kCorrectionError = 5e-7;
+
 // Float64-class residual and surface velocity of one iterate x, sharing one pass over the pairs:
 // with sigma = rho + x,  r = b - A x = -(1/2 I + K) sigma - L x = L rho - A sigma  (Eq. 25, A the
 // operator 1/2 I + K + L) and  u = S sigma  (the velocity of Section 2.3).
@@ -267,11 +270,12 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
   } else {
     // Iterative refinement around float32 inner solves.  A float64-class pass gives the true
     // residual r = b - A x and, from the same pair sums, u = S[rho + x].  After a pass, a small
-    // correction d may instead update r -= A d and u += S d in float32: the float32 operator's error
-    // on d is f32_operator_error ||A d||, and these updates are taken only while that error, summed
-    // since the last pass, stays below a tenth of the tolerance in every suspension the correction
-    // touched.  Suspensions within tolerance after a float64-class pass take no further inner
-    // iterations.
+    // correction d may instead update r -= A d and u += S d by a cheaper operator of relative error e: these
+    // updates are taken only while e ||A d||, summed since the last pass, stays below a tenth of the
+    // tolerance in every suspension the correction touched.  The cheapest that allows it is chosen:
+    //   the inner solve's float32 operator (f32_operator_error: 1e-5, plus the treecode's model), or
+    //   apply_correction, whose smooth sums alone are float32 (kCorrectionError; a tenth of a pass's time).
+    // Suspensions within tolerance after a float64-class pass take no further inner iterations.
     double* lrho = c.d_vec[8].ptr;  // L rho (Eq. 26), float64
     RBS_TRY(apply_blocks(c, kModeL, RBS_PREC_FP64, rho, lrho, nullptr, 1.0));
     std::vector<double> rn = bn;
@@ -288,7 +292,8 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
       RBS_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(double) * n3, c.stream));
       RBS_CUDA_TRY(cudaMemcpyAsync(r, b, sizeof(double) * n3, cudaMemcpyDeviceToDevice, c.stream));
     }
-    // sigma accumulates the corrections applied in float32 since the last float64-class pass
+    // sigma accumulates the corrections applied by the float32 operator since the last float64-class pass
+    bool sigma_used = false;
     std::vector<double> pending(S, 0.0);
     std::vector<int> used(S, 0);
     const double ferr = f32_operator_error(c);
@@ -320,20 +325,33 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
       ++refinements;
       c.stats.launches++;
       k_axpby<<<nbk, 256, 0, c.stream>>>(x, 1.0, d, 1.0, n3);
-      bool f32_ok = u_done;
-      for (int s = 0; s < S && f32_ok; ++s)
-        if (R.iters[s] > 0 && ferr * (pending[s] + rn[s]) > 0.1 * tol * bn[s]) f32_ok = false;
-      if (f32_ok) {
+      // pending[s]: the error of the updates since the last pass
+      auto allowed = [&](double err) {
+        for (int s = 0; s < S; ++s)
+          if (R.iters[s] > 0 && pending[s] + err * rn[s] > 0.1 * tol * bn[s]) return false;
+        return u_done;
+      };
+      if (allowed(ferr)) {
         RBS_TRY(apply_operator(c, RBS_OP_A, RBS_PREC_MIXED, d, w));
         c.stats.launches += 2;
         k_axpby<<<nbk, 256, 0, c.stream>>>(r, -1.0, w, 1.0, n3);
         k_axpby<<<nbk, 256, 0, c.stream>>>(sigma, 1.0, d, 1.0, n3);
+        sigma_used = true;
         for (int s = 0; s < S; ++s)
-          if (R.iters[s] > 0) pending[s] += rn[s];
+          if (R.iters[s] > 0) pending[s] += ferr * rn[s];
+      } else if (hi == RBS_PREC_DF && allowed(kCorrectionError)) {
+        double* v = c.d_vec[6].ptr;
+        RBS_TRY(apply_correction(c, d, w, v));
+        c.stats.launches += 2;
+        k_axpby<<<nbk, 256, 0, c.stream>>>(r, -1.0, w, 1.0, n3);
+        k_axpby<<<nbk, 256, 0, c.stream>>>(u, 1.0, v, 1.0, n3);
+        for (int s = 0; s < S; ++s)
+          if (R.iters[s] > 0) pending[s] += kCorrectionError * rn[s];
       } else {
         RBS_TRY(residual_and_velocity(c, hi, rho, lrho, x, sigma, r, u));
         u_done = true;
         RBS_CUDA_TRY(cudaMemsetAsync(sigma, 0, sizeof(double) * n3, c.stream));
+        sigma_used = false;
         std::fill(pending.begin(), pending.end(), 0.0);
       }
       RBS_TRY(seg_norms_host(c, c.seg3, r, rn));
@@ -343,9 +361,7 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
       if (moved == 0) break;  // the inner solves could not move
     }
     for (int s = 0; s < S; ++s) rel[s] = bn[s] > 0.0 ? rn[s] / bn[s] : 0.0;
-    bool any_pending = false;
-    for (double p : pending) any_pending = any_pending || p > 0.0;
-    if (u_done && any_pending) {
+    if (u_done && sigma_used) {
       RBS_TRY(apply_operator(c, RBS_OP_S, RBS_PREC_MIXED, sigma, w));
       c.stats.launches++;
       k_axpby<<<nbk, 256, 0, c.stream>>>(u, 1.0, w, 1.0, n3);

@@ -350,16 +350,18 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 // NQ2 = ceil((n + 1) / 2).  Charges come in slabs (one a) through a per-warp ring of asynchronous
 // copies.
 //
-// A unit with at most 16 targets gives its two half-warps alternate halves of the sources.
+// A unit with at most 16 targets gives its two half-warps alternate halves of the sources.  KIND 0 traction,
+// 1 Stokeslet into y; 2 traction into y and Stokeslet into y2 (26 and 17 operations a pair, one target per lane).
 constexpr int kRing32 = 4;
 
 template <int KIND, int NT, int NQ2>
-__global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
+__global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 : 5)) : 4)
     k_tree32x2(int nunits, int per_item, int* __restrict__ counter, const TreeItem* __restrict__ items,
                const int2* __restrict__ segs, long long N, int npx, int nq, int nbp, int ncp,
                const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
                const float4* __restrict__ sq, const float4* __restrict__ axis, const float* __restrict__ pq,
-               int warp_floats, double* __restrict__ y) {
+               int warp_floats, double* __restrict__ y, double* __restrict__ y2) {
+  static_assert(KIND != 2 || NT == 1, "both sums: one target per lane");
   constexpr int TW = kTreeTile32, SL = TW / 32;
   const int lane = threadIdx.x & 31;
   extern __shared__ __align__(16) float tree_smem32[];
@@ -411,6 +413,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
       nt[u][2] = f2(n2, n2);
     }
     float sa[NT][3], ea[NT][3];
+    float sb[3] = {0.0f, 0.0f, 0.0f}, eb[3] = {0.0f, 0.0f, 0.0f};  // KIND 2: the Stokeslet sums
 #pragma unroll
     for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
     int seg = w.s0, off = 0, done = 0;
@@ -473,7 +476,15 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
       pair_tile32x2<KIND, false, NT, NUV>(ssx + l0, ssy + l0, ssz + l0, srx + l0, sry + l0, srz + l0, spid + l0, \
                                           cnt, xt, nt, pt, p);                                               \
   } while (0)
-      if (nu == NT) {
+      if constexpr (KIND == 2) {
+        float2 p2[3] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
+        if (done < w.nmask)
+          pair_tile32_both<true, TW>(ssx, spid, l0, cnt, xt[0], nt[0], pt[0], p[0], p2);
+        else
+          pair_tile32_both<false, TW>(ssx, spid, l0, cnt, xt[0], nt[0], pt[0], p[0], p2);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) two_sum_acc(sb[c], eb[c], p2[c].x + p2[c].y);
+      } else if (nu == NT) {
         RBS_TILE(NT);
       } else if constexpr (NT > 1) {
         RBS_TILE(1);
@@ -531,6 +542,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
           __syncwarp();
           const float* row = ring + slot * slab + half * 3 * ncp;
           float2 dx[NT], dx2[NT], rnx[NT], p[NT][3], s0x[NT], s0y[NT];
+          float2 p2[3] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f), f2(0.0f, 0.0f)}, t0x = p2[0], t0y = p2[0];  // KIND 2
           const float sxa = sax[a];
 #pragma unroll
           for (int u = 0; u < NT; ++u) {
@@ -552,7 +564,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
               const float2 dy = __fadd2_rn(xt[u][1], f2(syb, syb));
               const float2 sab = __ffma2_rn(dy, dy, dx2[u]);
               const float2 rnab = __ffma2_rn(dy, nt[u][1], rnx[u]);
-              float2 s0 = f2(0.0f, 0.0f);
+              float2 s0 = f2(0.0f, 0.0f), t0 = s0;
 #pragma unroll
               for (int i = 0; i < NQ2; ++i) {
                 const float2 qx = (i & 1) ? f2(q[0][i / 2].z, q[0][i / 2].w) : f2(q[0][i / 2].x, q[0][i / 2].y);
@@ -568,6 +580,13 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
                 if (KIND == 0) {
                   const float2 rn = __ffma2_rn(d, nt[u][2], rnab);
                   c = __fmul2_rn(__fmul2_rn(__fmul2_rn(rn, rr), inv2), inv3);
+                } else if (KIND == 2) {
+                  const float2 cs = __fmul2_rn(rr, inv3);
+                  c = __fmul2_rn(__fmul2_rn(__ffma2_rn(d, nt[u][2], rnab), inv2), cs);
+                  p2[0] = __ffma2_rn(qx, inv, p2[0]);
+                  p2[1] = __ffma2_rn(qy, inv, p2[1]);
+                  p2[2] = __ffma2_rn(cs, d, __ffma2_rn(qz, inv, p2[2]));
+                  t0 = __fadd2_rn(t0, cs);
                 } else {
                   c = __fmul2_rn(rr, inv3);
                   p[u][0] = __ffma2_rn(qx, inv, p[u][0]);
@@ -579,6 +598,10 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
               }
               s0x[u] = __fadd2_rn(s0x[u], s0);
               s0y[u] = __ffma2_rn(dy, s0, s0y[u]);
+              if (KIND == 2) {
+                t0x = __fadd2_rn(t0x, t0);
+                t0y = __ffma2_rn(dy, t0, t0y);
+              }
             }
           }
 #pragma unroll
@@ -588,19 +611,28 @@ __global__ void __launch_bounds__(128, NT == 1 ? (NQ2 <= 4 ? 6 : 5) : 4)
 #pragma unroll
             for (int c = 0; c < 3; ++c) two_sum_acc(sa[u][c], ea[u][c], p[u][c].x + p[u][c].y);
           }
+          if (KIND == 2) {
+            p2[0] = __ffma2_rn(dx[0], t0x, p2[0]);
+            p2[1] = __fadd2_rn(p2[1], t0y);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) two_sum_acc(sb[c], eb[c], p2[c].x + p2[c].y);
+          }
           __syncwarp();  // every lane has read the slab before its slot is refilled
           slot = slot + 1 == kRing32 ? 0 : slot + 1;
         }
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
+    const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
       if (!valid[u]) continue;
       const long long t = tb + 32 * u + (split ? lane & 15 : lane);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
+      for (int c = 0; c < 3; ++c) {
+        atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
+        if (KIND == 2) atomicAdd(y2 + 3 * t + c, kStokesletScale * ((double)sb[c] + (double)eb[c]));
+      }
     }
   }
 }
@@ -1244,8 +1276,7 @@ static int tree_grid(Context& c, const void* kernel, size_t smem, long long unit
 }
 
 template <int KIND, int NT, int NQ2>
-static Status launch_tree(Context& c, double* y) {
-  TreeState& T = c.tree;
+static Status launch_tree(Context& c, const TreeState& T, double* y, double* y2 = nullptr) {
   const int nq = T.degree + 1;
   const int slab = 3 * T.nbp * T.ncp;
   const int warp_floats = std::max(7 * kTreeTile32, (kRing32 * slab + 3 * nq + 3) & ~3);
@@ -1257,24 +1288,25 @@ static Status launch_tree(Context& c, double* y) {
   const auto kernel = k_tree32x2<KIND, NT, NQ2>;
   kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
       (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_xhi.ptr,
-      c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, T.d_axis.ptr, T.d_pq.ptr, warp_floats, y);
+      c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, T.d_axis.ptr, T.d_pq.ptr, warp_floats, y, y2);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
 
 template <int KIND>
 static Status launch_tree(Context& c, double* y) {
-  const int nq2 = (c.tree.degree + 2) / 2;  // pairs of the last proxy axis; degree 2 to 10
+  const TreeState& T = c.tree;
+  const int nq2 = (T.degree + 2) / 2;  // pairs of the last proxy axis; degree 2 to 10
   if (tree_variant(c) == 2) {
-    if (nq2 == 2) return launch_tree<KIND, 2, 2>(c, y);
-    return nq2 == 3 ? launch_tree<KIND, 2, 3>(c, y) : launch_tree<KIND, 2, 4>(c, y);
+    if (nq2 == 2) return launch_tree<KIND, 2, 2>(c, T, y);
+    return nq2 == 3 ? launch_tree<KIND, 2, 3>(c, T, y) : launch_tree<KIND, 2, 4>(c, T, y);
   }
   switch (nq2) {
-    case 2: return launch_tree<KIND, 1, 2>(c, y);
-    case 3: return launch_tree<KIND, 1, 3>(c, y);
-    case 4: return launch_tree<KIND, 1, 4>(c, y);
-    case 5: return launch_tree<KIND, 1, 5>(c, y);
-    default: return launch_tree<KIND, 1, 6>(c, y);
+    case 2: return launch_tree<KIND, 1, 2>(c, T, y);
+    case 3: return launch_tree<KIND, 1, 3>(c, T, y);
+    case 4: return launch_tree<KIND, 1, 4>(c, T, y);
+    case 5: return launch_tree<KIND, 1, 5>(c, T, y);
+    default: return launch_tree<KIND, 1, 6>(c, T, y);
   }
 }
 
@@ -1314,6 +1346,46 @@ Status apply_tree(Context& c, int kind, double* y) {
   return Status::Ok();
 }
 
+// Float64 cluster charges of the double-float lists, as the float32 kernel reads them.
+__global__ void k_tree_q64_round(long long count, const double* __restrict__ q64, float* __restrict__ q) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (k < count) q[k] = (float)q64[k];
+}
+
+static Status charges_df(Context& c, const double* x) {
+  TreeState& T = c.tree_df;
+  RBS_CUDA_TRY(cudaMemsetAsync(T.d_q64.ptr, 0, sizeof(double) * T.d_q64.n, c.stream));
+  k_tree_charges64<<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
+      T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb64.ptr, T.degree + 1,
+      T.nbp, T.ncp, T.d_q64.ptr);
+  RBS_CUDA_TRY(cudaGetLastError());
+  return Status::Ok();
+}
+
+Status apply_tree_df_f32(Context& c, const double* x, double* y, double* y2) {
+  TreeState& T = c.tree_df;
+  if (T.n_cells > 0) {
+    KernelTimer timer(c, RBS_KC_TREE);
+    RBS_TRY(charges_df(c, x));
+    const long long count = (long long)T.n_cells * (T.degree + 1) * T.nbp * 3 * T.ncp;
+    k_tree_q64_round<<<cdiv(count, 256), 256, 0, c.stream>>>(count, T.d_q64.ptr, T.d_pq.ptr);
+    RBS_CUDA_TRY(cudaGetLastError());
+    timer.done((double)T.charge_work, 2);
+  }
+  if (T.items.empty()) return Status::Ok();
+  KernelTimer timer(c, RBS_KC_PAIR_K32);
+  switch ((T.degree + 2) / 2) {  // degree 2 to 12
+    case 2: RBS_TRY((launch_tree<2, 1, 2>(c, T, y, y2))); break;
+    case 3: RBS_TRY((launch_tree<2, 1, 3>(c, T, y, y2))); break;
+    case 4: RBS_TRY((launch_tree<2, 1, 4>(c, T, y, y2))); break;
+    case 5: RBS_TRY((launch_tree<2, 1, 5>(c, T, y, y2))); break;
+    case 6: RBS_TRY((launch_tree<2, 1, 6>(c, T, y, y2))); break;
+    default: RBS_TRY((launch_tree<2, 1, 7>(c, T, y, y2)));
+  }
+  timer.done(2.0 * (double)(T.direct_pairs + T.proxy_pairs));
+  return Status::Ok();
+}
+
 template <int KIND>
 static Status launch_tree_df(Context& c, double* y, double* y2) {
   TreeState& T = c.tree_df;
@@ -1341,10 +1413,7 @@ Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y
     if (T.n_cells > 0) {
       const int nq = T.degree + 1;
       const long long rows = (long long)T.n_cells * nq * T.nbp;
-      RBS_CUDA_TRY(cudaMemsetAsync(T.d_q64.ptr, 0, sizeof(double) * T.d_q64.n, c.stream));
-      k_tree_charges64<<<(unsigned)T.charge_items.size(), kChargeThreads, 0, c.stream>>>(
-          T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, x, T.d_box.ptr, T.d_cheb64.ptr, nq, T.nbp,
-          T.ncp, T.d_q64.ptr);
+      RBS_TRY(charges_df(c, x));
       k_tree_q64_split<<<cdiv(rows * T.ncp, 256), 256, 0, c.stream>>>(rows, T.ncp, T.d_q64.ptr, T.d_pq.ptr);
       launches = 2;
     }
