@@ -66,7 +66,20 @@ Status Context::harvest() {
   return Status::Ok();
 }
 
+Status Context::side_stream() {
+  if (!side) RBS_CUDA_TRY(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+  if (!fork_ev) RBS_CUDA_TRY(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
+  if (!join_ev) RBS_CUDA_TRY(cudaEventCreateWithFlags(&join_ev, cudaEventDisableTiming));
+  return Status::Ok();
+}
+
 Context::~Context() {
+  if (side) {  // (an error between fork and join may have left work on it)
+    cudaStreamSynchronize(side);
+    cudaStreamDestroy(side);
+  }
+  if (fork_ev) cudaEventDestroy(fork_ev);
+  if (join_ev) cudaEventDestroy(join_ev);
   warm_release(*this);
   for (const Timed& t : pending) {
     free_events.push_back(t.a);

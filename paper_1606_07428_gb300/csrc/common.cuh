@@ -268,9 +268,16 @@ struct GemmGroup {
   double flops = 0.0;  // tensor-core flops issued since creation
 };
 
+// Largest system whose float32 near correction runs beside the smooth sum.
+constexpr long long kBesideNodes = 131072;
+
 struct Context {
   rbs_options opt{};
   cudaStream_t stream = nullptr;
+  // a second stream for work beside it, with the events of the fork and the join (side_stream, created by the
+  // set-up of a system that uses it); the join is always waited for on `stream`
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   std::string err;
   int device = 0;
   int sm_count = 0;
@@ -352,7 +359,6 @@ struct Context {
   DevBuf<int> d_gemm_err;
   int max_np_sym = 0;
   int max_np = 0;
-  int max_np_shape = 0;
   // per upsampled-source particle: interpolation matrix of its grid (float64 and float32)
   DevBuf<const double*> d_upU;
   DevBuf<const float*> d_upU32;
@@ -364,7 +370,7 @@ struct Context {
   // smooth pair-sum work list: (target begin, target end, source begin, source end)
   std::vector<longlong4> work;
   DevBuf<longlong4> d_work;
-  DevBuf<int> d_unit;  // the next work unit of the running pair sum (zeroed before each launch)
+  DevBuf<int> d_unit;  // next work unit of the running smooth sum and near correction (zeroed before each launch)
 
   // scratch vectors (3N doubles each) and GMRES workspace
   DevBuf<double> d_vec[10];
@@ -412,6 +418,7 @@ struct Context {
   Status time_begin(int cls, Timed* t);
   Status time_end(Timed* t, double units);
   Status harvest();
+  Status side_stream();
 
   Context() = default;
   ~Context();

@@ -153,7 +153,7 @@ __global__ void k_weight_df1(long long N, const double4* __restrict__ x, const d
 template <int KIND, int MODE>
 __device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const int* spid, int l0, int l1,
                                                const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2& acc) {
-#pragma unroll 1
+#pragma unroll 2
   for (int l = l0; l < l1; l += 2) {
     df2 d[3];
 #pragma unroll
@@ -179,7 +179,7 @@ __device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(128, 5) k_lap_df(int nunits, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 4) k_lap_df(int nunits, int* __restrict__ counter,
                                                    const longlong4* __restrict__ work,
                                                    const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                                    const float4* __restrict__ x3l, const float4* __restrict__ nh,
@@ -596,8 +596,8 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
     if (M.d_wq.n != (size_t)c.N) RBS_TRY(M.d_wq.alloc(c.N));
     c.stats.launches += 2;
     k_weight_df1<<<cdiv(c.N, 256), 256, 0, s>>>(c.N, c.d_x.ptr, x, M.d_wq.ptr);
-    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), s));
-    const int grid = std::min(nw, 5 * std::max(1, c.sm_count));
+    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, 2 * sizeof(int), s));
+    const int grid = std::min(nw, 4 * std::max(1, c.sm_count));
 #define RBS_LAP_ARGS \
   4 * nw, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
     if (kind == 0)

@@ -50,8 +50,8 @@ __device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
 }
 
 
-// The units of the context's near list, with the counter zeroed on its stream; blocks: as many 128-thread
-// blocks as have a unit per warp.
+// The units of the context's near list (its counter, d_unit[1], is zeroed by the caller or the weight kernels);
+// blocks: as many 128-thread blocks as have a unit per warp.
 inline Status near_args(Context& c, NearArgs& A, int& blocks) {
   const long long nn = (long long)c.near_pairs.size();
   A.chunks = (c.max_np + 31) / 32;
@@ -66,13 +66,12 @@ inline Status near_args(Context& c, NearArgs& A, int& blocks) {
   const long long units = units1 * A.parts;
   if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "near correction: more than 2^31 work units");
   A.nunits = (int)units;
-  A.counter = c.d_unit.ptr;
+  A.counter = c.d_unit.ptr + 1;
   A.near = c.d_near.ptr;
   A.offset = c.d_offset.ptr;
   A.nodes = c.d_nodes.ptr;
   A.up_index = c.d_up_index.ptr;
   A.up_off = c.d_up_off.ptr;
-  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
   blocks = (int)((units + 3) / 4);
   return Status::Ok();
 }

@@ -590,8 +590,9 @@ __global__ void __launch_bounds__(128) k_pairs64(int nitems, const longlong4* __
 // ------------------------------------------------------------------------------------------
 // Weighted density in float32 for the packed kernels: wmu[t] = (w_t mu_t, 0).
 __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
-                             float4* __restrict__ wmu) {
+                             float4* __restrict__ wmu, int* __restrict__ units) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t < 2) units[t] = 0;  // the unit counters of the smooth sum and the near correction that follow
   if (t >= N) return;
   const double w = x[t].w;
   wmu[t] = make_float4((float)(w * dens[3 * t]), (float)(w * dens[3 * t + 1]), (float)(w * dens[3 * t + 2]), 0.0f);
@@ -733,8 +734,9 @@ __global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
 // Weighted density as double-float pairs for the double-float kernels: (w mu) rounded to float32 and
 // the rounded remainder.
 __global__ void k_weight_df(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
-                            float4* __restrict__ wh, float4* __restrict__ wl) {
+                            float4* __restrict__ wh, float4* __restrict__ wl, int* __restrict__ units) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t < 2) units[t] = 0;
   if (t >= N) return;
   const double w = x[t].w;
   const dflt a = df_split(w * dens[3 * t]), b = df_split(w * dens[3 * t + 1]), c = df_split(w * dens[3 * t + 2]);
@@ -1042,7 +1044,9 @@ __global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __res
   NearUnit n;
   while (next_near_unit(A, n)) {
     if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
-    const int t = n.t0 + lane;
+    const bool split = n.t1 - n.t0 <= 16;  // the half-warps take alternate halves of the sources
+    const int half = split ? lane >> 4 : 0;
+    const int t = n.t0 + (split ? lane & 15 : lane);
     const bool valid = t < n.t1;
     const double4 xt = x[valid ? t : n.t0], nt = nrm[valid ? t : n.t0];
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
@@ -1063,7 +1067,7 @@ __global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __res
       }
       __syncwarp();
 #pragma unroll 4
-      for (int l = 0; l < cnt; ++l) {
+      for (int l = half; l < cnt; l += split ? 2 : 1) {
         const double4 ps = sp[warp][l], q = sq[warp][l];
         const double dx = xt.x - ps.x, dy = xt.y - ps.y, dz = xt.z - ps.z;
         const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
@@ -1083,7 +1087,12 @@ __global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __res
         }
       }
     }
-    if (valid) {
+    if (split) {  // one addition per target
+      a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
+      a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
+    }
+    if (valid && half == 0) {
       const double sc = KIND == 0 ? kTractionScale : kStokesletScale;
       atomicAdd(y + 3 * (long long)t + 0, sc * a0);
       atomicAdd(y + 3 * (long long)t + 1, sc * a1);
@@ -1094,14 +1103,16 @@ __global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __res
 
 }  // namespace
 
-// Weighted densities of the float32 and double-float pair sums.
+// Weighted densities of the float32 and double-float pair sums; they also zero the unit counters (d_unit: smooth
+// sum, near correction), so each is followed by at most one of either sum.
 static Status weight_f32(Context& c, const double* x) {
-  k_weight_f32<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmu32.ptr);
+  k_weight_f32<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmu32.ptr, c.d_unit.ptr);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
 static Status weight_df(Context& c, const double* x) {
-  k_weight_df<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmuh.ptr, c.d_wmul.ptr);
+  k_weight_df<<<cdiv(c.N, 256), 256, 0, c.stream>>>(c.N, c.d_x.ptr, x, c.d_wmuh.ptr, c.d_wmul.ptr,
+                                                           c.d_unit.ptr);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
 }
@@ -1152,7 +1163,6 @@ static void launch_pairs_df(Context& c, double* y, double* y2) {
 // double-float only.  The float32 and double-float sums read the weighted densities of this x.
 static Status launch_pairs(Context& c, int kind, int prec, const double* x, double* y, double* y2 = nullptr) {
   const int items = (int)c.work.size();
-  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
   if (prec == RBS_PREC_DF) {
     if (kind == 0)
       launch_pairs_df<0>(c, y, y2);
@@ -1295,6 +1305,7 @@ static Status near_sums(Context& c, int kind, int prec, const double* x, double*
   NearArgs A;
   int blocks = 0;
   RBS_TRY(near_args(c, A, blocks));
+  if (prec == RBS_PREC_FP64) RBS_CUDA_TRY(cudaMemsetAsync(A.counter, 0, sizeof(int), c.stream));
 #define RBS_NEAR_LAUNCH(KERNEL, ...) \
   KERNEL<<<resident_grid(c, (const void*)KERNEL, 128, blocks), 128, 0, c.stream>>>(A, __VA_ARGS__)
   if (prec == RBS_PREC_DF) {
@@ -1338,18 +1349,42 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     c.stats.launches++;
     RBS_TRY(weight_df(c, x));
   }
+  // The float32 near correction of a small system runs beside the smooth sum (both add into y atomically): each
+  // alone leaves SMs idle at its end, and below about 10^5 nodes that is a tenth of an apply.  Not while kernel
+  // classes are timed.
+  const bool beside = f32 && c.side && !c.near_pairs.empty() && c.N <= kBesideNodes && c.opt.timing == 0;
+  if (beside) {
+    RBS_CUDA_TRY(cudaEventRecord(c.fork_ev, c.stream));
+    RBS_CUDA_TRY(cudaStreamWaitEvent(c.side, c.fork_ev, 0));
+    const cudaStream_t main = c.stream;
+    c.stream = c.side;
+    Status st = near_upsample(c, prec, x);
+    if (st.ok()) st = near_sums(c, kind, prec, x, y, nullptr);
+    c.stream = main;
+    c.stats.launches += 2;
+    c.stats.kernel_count[RBS_KC_NEAR] += 2;
+    c.stats.kernel_units[RBS_KC_NEAR] += (double)c.near_pair_nodes;
+    RBS_CUDA_TRY(cudaEventRecord(c.join_ev, c.side));
+    if (!st.ok()) {
+      cudaStreamWaitEvent(c.stream, c.join_ev, 0);
+      return st;
+    }
+  }
+  Status st;
   if (f32 && c.tree.active) {
-    RBS_TRY(apply_tree(c, kind, y));  // treecode in place of the direct float32 sum
+    st = apply_tree(c, kind, y);  // treecode in place of the direct float32 sum
   } else if (prec == RBS_PREC_DF && c.tree_df.active) {
-    RBS_TRY(apply_tree_df(c, kind, x, y, nullptr));  // and of the direct double-float sum
+    st = apply_tree_df(c, kind, x, y, nullptr);  // and of the direct double-float sum
   } else if (nw > 0) {
     int cls = f32 ? (kind == 0 ? RBS_KC_PAIR_K32 : RBS_KC_PAIR_S32) : (kind == 0 ? RBS_KC_PAIR_K64 : RBS_KC_PAIR_S64);
     if (prec == RBS_PREC_DF) cls = kind == 0 ? RBS_KC_PAIR_KDF : RBS_KC_PAIR_SDF;
     KernelTimer timer(c, cls);
-    RBS_TRY(launch_pairs(c, kind, prec, x, y));
+    st = launch_pairs(c, kind, prec, x, y);
     timer.done((double)c.stats.far_pairs);
   }
-  if (!c.near_pairs.empty()) {
+  if (beside) RBS_CUDA_TRY(cudaStreamWaitEvent(c.stream, c.join_ev, 0));  // (also when the smooth sum failed)
+  RBS_TRY(st);
+  if (!beside && !c.near_pairs.empty()) {
     KernelTimer timer(c, RBS_KC_NEAR);
     RBS_TRY(near_upsample(c, prec, x));
     RBS_TRY(near_sums(c, kind, prec, x, y, nullptr));
@@ -1411,7 +1446,6 @@ Status apply_correction(Context& c, const double* d, double* w, double* v) {
     RBS_TRY(apply_tree_df_f32(c, d, w, v));
   } else if (!c.work.empty()) {
     KernelTimer timer(c, RBS_KC_PAIR_K32);
-    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
     launch_pairs32<2, 1>(c, w, v);
     RBS_CUDA_TRY(cudaGetLastError());
     timer.done(2.0 * (double)c.stats.far_pairs);

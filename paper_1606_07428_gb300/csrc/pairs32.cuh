@@ -27,7 +27,8 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& e, float v) {
 // pipe rather than by instruction issue.  Sources are staged structure-of-arrays in shared memory,
 // four per 128-bit load, coordinates negated (x_t + (-y_s) is the separation) and relative to the
 // work item's first target; the tile is padded to a multiple of four with zero-density sources far
-// away (they add exactly zero).  The reciprocal square root stays one hardware instruction per pair.
+// away (they add exactly zero).  The reciprocal square root stays one hardware instruction per pair: a second
+// one for 1 / r^2 in place of a product would make the transcendental pipe (16 lanes a clock) the bound.
 // Each target thread keeps float2 partial sums over the two source streams and adds their total into
 // a compensated (two-sum) accumulator once per tile.
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
@@ -52,7 +53,8 @@ __device__ __forceinline__ void pair2_f32(float2 sx, float2 sy, float2 sz, float
     acc[1] = __ffma2_rn(c, dy, acc[1]);
     acc[2] = __ffma2_rn(c, dz, acc[2]);
   } else {
-    const float2 inv3 = __fmul2_rn(__fmul2_rn(inv, inv), inv);
+    const float2 inv2 = __fmul2_rn(inv, inv);
+    const float2 inv3 = __fmul2_rn(inv2, inv);
     const float2 c = __fmul2_rn(rr, inv3);
     acc[0] = __ffma2_rn(c, dx, __ffma2_rn(rx, inv, acc[0]));
     acc[1] = __ffma2_rn(c, dy, __ffma2_rn(ry, inv, acc[1]));

@@ -306,12 +306,13 @@ __global__ void k_shape_extent(const ShapeGrid* sg, RBS_SHAPE_ARGS, double* shif
   }
 }
 
-// Body-frame nodes (x_b, weight) of one shape on its own grid.
-__global__ void k_body_nodes(int np, int nphi, const double* t, const double* lam, int shape, RBS_SHAPE_ARGS,
+// Body-frame nodes (x_b, weight) of the listed shapes of one grid, np per shape (blockIdx.y).
+__global__ void k_body_nodes(int np, int nphi, const double* t, const double* lam, const int* shapes, RBS_SHAPE_ARGS,
                              double4* out) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= np) return;
-  const ShapeRef S = RBS_SHAPE_REF(shape);
+  out += (long long)blockIdx.y * np;
+  const ShapeRef S = RBS_SHAPE_REF(shapes[blockIdx.y]);
   const int j = l / nphi, k = l % nphi;
   const double ct = t[j], st = sqrt(fmax(0.0, 1.0 - ct * ct));
   double sp, cp;
@@ -452,11 +453,16 @@ __global__ void k_self_scatter(int nphi, int nkc, int np, int j, const double* G
 
 // Preconditioner matrix before inversion: M = 1/2 I + K0 + L0 in the body frame, with
 // L0_ts = w_s (I - [r_t]x [r_s]x) (Eq. 26 written as a block; r the body-frame node).
-// Stored row 3 r + al belongs to node (r / nk) nphi + r % nk (the node r itself when nk = nphi).
-__global__ void k_precond_matrix(int np, int nphi, int nk, int rows, const double4* body, const double* BK, double* M) {
+// Stored row 3 r + al belongs to node (r / nk) nphi + r % nk (the node r itself when nk = nphi).  One shape per
+// blockIdx.y, its block at block_off.
+__global__ void k_precond_matrix(int np, int nphi, int nk, int rows, const double4* body, const long long* block_off,
+                                 const double* BK, double* M) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   long long dim = 3LL * np;
   if (i >= (long long)rows * dim) return;
+  body += (long long)blockIdx.y * np;
+  BK += block_off[blockIdx.y];
+  M += block_off[blockIdx.y];
   int row = (int)(i / dim), col = (int)(i % dim);
   int r = row / 3, al = row % 3, sn = col / 3, be = col % 3;
   int tn = (r / nk) * nphi + r % nk;
@@ -1106,10 +1112,8 @@ static Status build_shape_tables(Context& c, const std::vector<long long>& grid_
   std::vector<double> axes(3 * (size_t)ns, 0.0), shift(3 * (size_t)ns, 0.0);
   std::vector<long long> coef_off(ns, -1);
   std::vector<ShapeGrid> sg;
-  c.max_np_shape = 0;
   for (int k = 0; k < ns; ++k) {
     const Shape& sh = c.shapes[k];
-    c.max_np_shape = std::max(c.max_np_shape, sh.np);
     kind[k] = sh.kind;
     axes[3 * k] = sh.a;
     axes[3 * k + 1] = sh.b;
@@ -1288,18 +1292,37 @@ Status build_geometry(Context& c) {
   // block-diagonal preconditioner P0 = (1/2 I + K0 + L0)^{-1} per shape (Section 3.2)
   if (c.opt.preconditioner) {
     RBS_TRY(c.d_precond.alloc(c.block_elems));
-    DevBuf<double4> body;
-    RBS_TRY(body.alloc(c.max_np_shape));
-    for (size_t k = 0; k < c.shapes.size(); ++k) {
-      const Shape& sh = c.shapes[k];
-      Grid& g = *c.grids[sh.grid];
-      long long elems = (long long)sh.rows * 3 * sh.np;
-      k_body_nodes<<<cdiv(sh.np, 128), 128, 0, s>>>(sh.np, g.nphi, g.d_t.ptr, g.d_lam.ptr, (int)k, RBS_SHAPE_PASS,
-                                                    body.ptr);
-      k_precond_matrix<<<cdiv(elems, 256), 256, 0, s>>>(sh.np, g.nphi, sh.sym ? g.nk : g.nphi, sh.rows, body.ptr,
-                                                        c.d_blockK.ptr + sh.block_off, c.d_precond.ptr + sh.block_off);
+    {
+      std::vector<std::vector<int>> by_grid(2 * c.grids.size());
+      for (size_t k = 0; k < c.shapes.size(); ++k)
+        by_grid[2 * c.shapes[k].grid + (c.shapes[k].sym ? 1 : 0)].push_back((int)k);
+      for (size_t q = 0; q < by_grid.size(); ++q) {
+        const std::vector<int>& ids = by_grid[q];
+        if (ids.empty()) continue;
+        const Shape& sh = c.shapes[ids[0]];
+        const Grid& g = *c.grids[sh.grid];
+        const long long elems = (long long)sh.rows * 3 * sh.np;
+        const int most = std::min<int>((int)ids.size(), 16384);
+        DevBuf<int> d_ids;
+        DevBuf<long long> d_off;
+        DevBuf<double4> body;
+        std::vector<long long> off;
+        for (int k : ids) off.push_back((long long)c.shapes[k].block_off);
+        RBS_TRY(upload(d_ids, ids, s));
+        RBS_TRY(upload(d_off, off, s));
+        RBS_TRY(body.alloc((size_t)most * sh.np));
+        for (int b0 = 0; b0 < (int)ids.size(); b0 += most) {
+          const int cnt = std::min(most, (int)ids.size() - b0);
+          k_body_nodes<<<dim3(cdiv(sh.np, 128), cnt), 128, 0, s>>>(sh.np, g.nphi, g.d_t.ptr, g.d_lam.ptr, d_ids.ptr + b0,
+                                                                   RBS_SHAPE_PASS, body.ptr);
+          k_precond_matrix<<<dim3(cdiv(elems, 256), cnt), 256, 0, s>>>(sh.np, g.nphi, sh.sym ? g.nk : g.nphi, sh.rows,
+                                                                       body.ptr, d_off.ptr + b0, c.d_blockK.ptr,
+                                                                       c.d_precond.ptr);
+        }
+        RBS_CUDA_TRY(cudaGetLastError());
+        RBS_CUDA_TRY(cudaStreamSynchronize(s));  // the lists go out of scope
+      }
     }
-    RBS_CUDA_TRY(cudaGetLastError());
     // shapes storing every row: invert runs of consecutive (hence contiguous) shapes of one size
     size_t k = 0;
     while (k < c.shapes.size()) {
@@ -1399,7 +1422,7 @@ Status build_geometry(Context& c) {
       const long long few = one ? 1 : std::min((32LL * c.sm_count + tiles - 1) / tiles, ns / 128);
       int sc = (int)std::max(few, std::min<long long>(splits, std::max(1LL, ns / 2048)));
       // whole tiles of 128 sources (a chunk of 129 would stage a tile for its last source)
-      long long chunk = sc > 1 ? ((ns + sc - 1) / sc + 127) / 128 * 128 : ns;
+      long long chunk = sc > 1 ? std::max(128LL, (ns + sc - 1) / sc / 128 * 128) : ns;
       for (long long tb = sp.first; tb < sp.second; tb += TT)
         for (long long sb = sp.first; sb < sp.second; sb += chunk) {
           longlong4 w;
@@ -1412,7 +1435,8 @@ Status build_geometry(Context& c) {
     }
   }
   RBS_TRY(upload(c.d_work, c.work, s));
-  RBS_TRY(c.d_unit.alloc(1));
+  RBS_TRY(c.d_unit.alloc(2));
+  if (!c.near_pairs.empty() && c.N <= kBesideNodes) RBS_TRY(c.side_stream());
 
   // particle-block work list
   c.bwork.clear();

@@ -1284,7 +1284,6 @@ static Status launch_tree(Context& c, const TreeState& T, double* y, double* y2 
   const int per_item = (T.tmax + 32 * NT - 1) / (32 * NT);
   const long long units = (long long)T.items.size() * per_item;
   if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "treecode: more than 2^31 work units");
-  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
   const auto kernel = k_tree32x2<KIND, NT, NQ2>;
   kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
       (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_xhi.ptr,
@@ -1395,7 +1394,6 @@ static Status launch_tree_df(Context& c, double* y, double* y2) {
   const int per_item = (T.tmax + 31) / 32;
   const long long units = (long long)T.items.size() * per_item;
   if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "treecode: more than 2^31 work units");
-  RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, sizeof(int), c.stream));
   const auto kernel = k_tree_df2<KIND>;
   kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
       (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_x3h.ptr,
