@@ -56,11 +56,16 @@ FP64_OPS_PER_PAIR = {"traction": 27.0, "stokeslet": 25.0}
 # once (sources are re-read from L2), so traffic grows with N, not with the N^2 pairs
 NCU_TRAFFIC = {"pair_traction_df": (6.404864e6, 57600), "pair_traction_f32": (4.872192e6, 57600),
                "pair_both_df": (8.511744e6, 57600)}
-# float32-pipe operations per pair the double-float kernels issue, counted from the source of
-# pair2_df (separation 24, r^2 28, reciprocal square root 8, r . density 28, powers 8, then the
-# traction tail 76, the Stokeslet tail 76, or both tails sharing 1/r^5 and r . n: 152): the issue
-# efficiency of a double-float kernel is measured against this count, its roofline against the flops
+# float32-pipe operations of a double-float pair with every sum and product error-free on its own (separation
+# 24, r^2 28, reciprocal square root 8, r . density 28, powers 8, then the traction tail 76, the Stokeslet
+# tail 76, or both tails sharing 1/r^5 and r . n: 152)
 DF_INSTR_PER_PAIR = {"traction": 172.0, "stokeslet": 172.0, "both": 248.0}
+# the same as the kernels issue them, counted from their source: per node pair (pair2_df with two-sum
+# separations; 9 fewer where a tile's coordinates are on a grid), and per (node, proxy point) pair of the
+# double-float treecode, whose proxies share a row's separations.  A double-float kernel's issue efficiency
+# is measured against these, its roofline against the flops
+DF_INSTR_NODE = {"traction": 154.0, "stokeslet": 139.0, "both": 221.0}
+DF_INSTR_PROXY = {"traction": 82.0, "stokeslet": 105.0, "both": 144.0}
 # DRAM bytes per launch of the fused double-float treecode kernel from an ncu capture on the
 # 2,000-ellipsoid profiling case (288,000 nodes; 83.27 MB read + 6.95 MB written, theta 0.45, degree 11,
 # one target per thread), scaled by node count like the direct kernels' figures
@@ -88,7 +93,7 @@ def parse_args():
     ap.add_argument("--cpu-seconds", type=float, default=15.0, help="budget of the oracle CPU sample")
     ap.add_argument("--cpu-procs", type=int, default=0, help="oracle sample processes (0: every host core)")
     ap.add_argument("--pair-variant", type=int, default=0,
-                    help="pair-kernel variant (rbs_options.pair_variant); 0 lets the library's autotuner choose")
+                    help="pair-kernel variant (rbs_options.pair_variant); 0 lets the library choose by size")
     ap.add_argument("--far-field", default="tree-df", choices=["direct", "tree", "tree-df"],
                     help="direct sums over all node pairs; tree: the treecode for the float32 inner applies "
                          "(double-float passes stay direct); tree-df: treecodes for both "
@@ -291,10 +296,16 @@ def pair_kind(name: str) -> str:
     return "traction" if "traction" in name else ("both" if "both" in name else "stokeslet")
 
 
-def kernel_rooflines(kernels, f_mhz, hbm_gbs):
+def df_instr(kind: str, proxy_share: float) -> float:
+    """Float32 operations a double-float pair issues on average, proxy_share of the pairs being proxy pairs."""
+    return (1.0 - proxy_share) * DF_INSTR_NODE[kind] + proxy_share * DF_INSTR_PROXY[kind]
+
+
+def kernel_rooflines(kernels, f_mhz, hbm_gbs, proxy_share=None):
     """Achieved rate of every timed kernel class against the roofline that bounds it: the float32 FMA
     peak (algorithmic flops per pair) for float32 and double-float pair sums, with the issue efficiency
-    of the double-float kernels beside it; the float64 FMA rate for float64 pair sums; HBM bandwidth
+    of the double-float kernels beside it (against the operations they issue where proxy_share, the share of
+    proxy pairs, is given; else against DF_INSTR_PER_PAIR); the float64 FMA rate for float64 pair sums; HBM bandwidth
     for the particle-block kernel (bytes of block entries)."""
     f = f_mhz * 1e6
     fp32 = SMS * FP32_LANES_PER_SM * 2 * f
@@ -312,7 +323,8 @@ def kernel_rooflines(kernels, f_mhz, hbm_gbs):
                 row.update({"achieved_tflops": tf / 1e12, "peak_tflops": fp32 / 1e12, "frac": tf / fp32,
                             "bound": "alu"})
                 if name.endswith("_df"):
-                    row["issue_efficiency"] = rate * DF_INSTR_PER_PAIR[kind] / (SMS * FP32_LANES_PER_SM * f)
+                    ops = DF_INSTR_PER_PAIR[kind] if proxy_share is None else df_instr(kind, proxy_share)
+                    row["issue_efficiency"] = rate * ops / (SMS * FP32_LANES_PER_SM * f)
             else:
                 peak = SMS * FP64_DFMA_PER_CLK_SM * f / FP64_OPS_PER_PAIR[kind]
                 row.update({"peak_gpair_s": peak / 1e9, "frac": rate / peak, "bound": "alu"})
@@ -587,6 +599,7 @@ def run_ours(args):
     if plain and "traction_f64_gpair_s" in plain:
         gpairs["traction_f64_plain"] = plain["traction_f64_gpair_s"]
         gpairs["stokeslet_f64_plain"] = plain["stokeslet_f64_gpair_s"]
+    proxy_share = stats["tree_df_proxy_pairs"] / stats["tree_df_pairs"] if stats.get("tree_df_pairs") else 0.0
     timed = {k: v for k, v in kernels.items() if k != "gmres_graph"}
     dom = max(timed.items(), key=lambda kv: kv[1]["ms"])
     name, e = dom
@@ -604,8 +617,9 @@ def run_ours(args):
                                   f"x {units_per_launch:.4g} pairs per launch / CUDA-event time per launch",
                 "gpair_s": pairs_s / 1e9}
         if name.endswith("_df"):
-            roof["issue_efficiency"] = pairs_s * DF_INSTR_PER_PAIR[kind] / (SMS * FP32_LANES_PER_SM * f_mhz * 1e6)
-            roof["issue_basis"] = (f"{DF_INSTR_PER_PAIR[kind]:.0f} float32 operations the double-float kernel issues "
+            ops = df_instr(kind, proxy_share)
+            roof["issue_efficiency"] = pairs_s * ops / (SMS * FP32_LANES_PER_SM * f_mhz * 1e6)
+            roof["issue_basis"] = (f"{ops:.0f} float32 operations the double-float kernel issues "
                                    f"per pair against {SMS} SMs x 128 lanes x {f_mhz:.0f} MHz")
     elif name.startswith("pair_"):
         kind = pair_kind(name)
@@ -630,7 +644,7 @@ def run_ours(args):
         hbm_peak = 6800.0
     # the block kernel with float32 entries (HBM-bound) and with float64 entries (float64-pipe-bound)
     rooflines = kernel_rooflines({**op_kernels, **{k: v for k, v in kernels.items() if k != "particle_blocks"}},
-                                 f_mhz, hbm_peak)
+                                 f_mhz, hbm_peak, proxy_share)
     if "particle_blocks_f64" in kernels and kernels["particle_blocks_f64"]["ms"] > 0:
         rooflines["particle_blocks_f64"] = block_f64_roofline(kernels["particle_blocks_f64"], f_mhz)
     # the captured counters belong to the direct kernels (and the double-float treecode kernel, captured

@@ -92,11 +92,10 @@ typedef struct {
                           (default 0); results in rbs_stats.kernel_ms */
   int refine_precision; /* RBS_PREC_MIXED: arithmetic of the right-hand side, refinement residuals
                           and velocity evaluation, RBS_PREC_DF (default) or RBS_PREC_FP64 */
-  int pair_variant;    /* pair-kernel variant: targets per thread 1, 2 or 4, or for the float32
-                          kernels 9, 10 or 12 = 8 + targets per thread of the packed kernels that
-                          evaluate two sources per instruction (the double-float kernels then use
-                          the targets per thread alone); 0 (default) times the candidates once per
-                          context and kernel and keeps the fastest */
+  int pair_variant;    /* targets per lane of the float32 pair kernels, which evaluate two sources per
+                          instruction: 1 or 9 for one, 2, 4, 10 or 12 for two (one where the kernel has
+                          no other form); 0 (default) chooses by the size of the system.  The
+                          double-float and float64 kernels have one form and ignore it */
   int warm_start;      /* initial GMRES guess: RBS_WARM_ZERO (default), RBS_WARM_PREVIOUS (the last
                           solved density of this context), RBS_WARM_LEARNED (the trained network's
                           density for the current configuration) or RBS_WARM_LEARNED_DELTA (the last
@@ -190,11 +189,9 @@ typedef struct {
   double kernel_units[RBS_KC_COUNT];     /* work per class: node pairs (pair sums, near), bytes of
                                             block entries read (particle blocks) */
   int n_contacts;        /* contacts found by the last mobility solve (rbs_options.contact_gap > 0) */
-  int pair_variant[5];   /* variant in use (as rbs_options.pair_variant): float32 traction, float32
-                            Stokeslet (the treecode kernel's with RBS_FAR_TREECODE), double-float
-                            traction, double-float Stokeslet, fused double-float traction and
-                            Stokeslet (the double-float treecode kernel's targets per thread with
-                            RBS_FAR_TREECODE_DF; 0 = not yet chosen) */
+  int pair_variant[5];   /* variant in use, 8 + targets per lane: float32 traction, float32 Stokeslet (the
+                            treecode kernel's with RBS_FAR_TREECODE), double-float traction, double-float
+                            Stokeslet, fused double-float traction and Stokeslet (9 for these three) */
   long long tree_pairs;  /* RBS_FAR_TREECODE: (target node, source) pairs one treecode apply evaluates,
                             direct node pairs (the target's own particle included, masked) plus
                             proxy pairs; 0 without a treecode */

@@ -44,14 +44,6 @@ __device__ __forceinline__ dflt df_add(dflt a, dflt b) {
   const float h = s.h + s.l;
   return {h, s.l - (h - s.h)};
 }
-// a0 b0 + a1 b1 + a2 b2: products exact to the low part, the three high parts added with two-sums
-// and every low part folded into one float32 sum (unnormalised result)
-__device__ __forceinline__ dflt df_dot3(dflt a0, dflt b0, dflt a1, dflt b1, dflt a2, dflt b2) {
-  const dflt p0 = df_mul(a0, b0), p1 = df_mul(a1, b1), p2 = df_mul(a2, b2);
-  const dflt s1 = df_two_sum(p0.h, p1.h);
-  const dflt s2 = df_two_sum(s1.h, p2.h);
-  return {s2.h, ((s1.l + s2.l) + (p0.l + p1.l)) + p2.l};
-}
 // acc += v with the low parts carried unnormalised (renormalised when the tile is flushed)
 __device__ __forceinline__ void df_acc(dflt& acc, dflt v) {
   const dflt s = df_two_sum(acc.h, v.h);

@@ -14,8 +14,8 @@
 // the steps of a restart cycle run as one CUDA graph: a conditional WHILE node whose body is the
 // captured step, re-entered by the device as long as some segment is active, so a cycle costs one
 // graph launch and no host round trip per iteration.  The first step on a configuration runs eagerly
-// (it also lets the autotuners pick their variants before capture); contexts that cannot build the
-// graph run the same kernels eagerly with one host read per step.
+// (kernels load and occupancies are looked up before capture); contexts that cannot build the graph run
+// the same kernels eagerly with one host read per step.
 #include <algorithm>
 #include <cmath>
 
@@ -638,7 +638,7 @@ Status gmres_seg(Context& c, const LinOp& op, const SegSet& sg, const double* b,
     int k_host = 0;
     bool cont = true;
     if (slot && !slot->exec) {
-      // the first step on this configuration runs eagerly (autotuners settle), then the graph is captured
+      // the first step on this configuration runs eagerly, then the graph is captured
       RBS_TRY(arnoldi_step(c, op, sg, m, cudaGraphConditionalHandle{}, false));
       RBS_CUDA_TRY(cudaMemcpyAsync(g.hctrl, ctrl, sizeof(int) * 3, cudaMemcpyDeviceToHost, c.stream));
       RBS_CUDA_TRY(cudaStreamSynchronize(c.stream));

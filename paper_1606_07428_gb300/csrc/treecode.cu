@@ -352,6 +352,9 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 //
 // A unit with at most 16 targets gives its two half-warps alternate halves of the sources.  KIND 0 traction,
 // 1 Stokeslet into y; 2 traction into y and Stokeslet into y2 (26 and 17 operations a pair, one target per lane).
+//
+// Bound by the float32 pipe, 76% busy.  With every source in one tile loop and blocks of whole particles, and
+// now: 1,150 to 1,770 Gpair/s on 1,500 particles of 144 nodes, 1,350 to 1,820 on 700 of 312.
 constexpr int kRing32 = 4;
 
 template <int KIND, int NT, int NQ2>
@@ -646,6 +649,9 @@ __global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 
 // memory for the whole cluster, the row sums d_x^2 + d_y^2 and d_x n_x + d_y n_y in registers, so a proxy
 // pair takes 144 float32 operations (traction and Stokeslet) where the node pair takes pairsdf.cuh's.
 // Charge rows are read through L1: a warp spends thousands of cycles on each 128-byte line.
+//
+// Bound by the float32 pipe, 83% busy.  Both sums with 248 operations for every pair, and now: 113 to 171 Gpair/s
+// on 1,500 particles of 144 nodes, 128 to 154 on 700 of 312 (fewer of whose pairs are with proxies).
 template <int KIND>
 __global__ void __launch_bounds__(128, 4)
     k_tree_df2(int nunits, int per_item, int* __restrict__ counter, const TreeItem* __restrict__ items,
