@@ -228,7 +228,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // arithmetic the row sums go to shared memory and every node is finished by the whole CTA at the end;
 // in float64 lane 4g finishes node g(r) at once.  gridDim.y CTAs share a particle, each taking every
 // gridDim.y-th run of kSymWarps representatives: a float64 particle of 144 nodes is 65 us of one SM's float64
-// pipe, so a list of few particles, or of few large ones, would leave the other SMs idle.
+// pipe, so a list of few particles, or of few large ones, would leave the other SMs idle (8 particles: 77 us a
+// float64 launch alone, 29 shared).
 template <typename TS, typename TB>
 __global__ void __launch_bounds__(kSymWarps * 32, sizeof(TB) == 4 ? 3 : 2)
     k_blocks_sym(int mode, const int* __restrict__ sym_list, const long long* __restrict__ offset,
@@ -604,7 +605,9 @@ __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const d
 // of the exact difference.  A unit is 32 NT targets of a work item against its sources; warps take units
 // from a counter and stage their own tiles of 128 sources, summed in float32 and added into a compensated
 // accumulator.  Tiles whose particles cannot meet the unit's targets skip the same-particle test.
-// Bound by the float32 pipe (20 operations a traction pair, 18 a Stokeslet pair).
+// Bound by the float32 pipe (20 operations a traction pair, 18 a Stokeslet pair), 76% busy: 1,460 Gpair/s on 101
+// particles of 220 nodes, 1,400 with blocks that took whole items; on 8 particles of 144 nodes an apply went from 34 to
+// 12 us by the smaller units.
 // KIND 2 (one target per lane): traction into y and Stokeslet into y2 in one pass, 26 operations.
 template <int KIND, int NT>
 __global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
@@ -748,7 +751,9 @@ __global__ void k_weight_df(long long N, const double4* __restrict__ x, const do
 // Direct double-float pair sums: y += traction sum (KIND 0, 2) or Stokeslet sum (KIND 1); KIND 2 also
 // y2 += Stokeslet sum.  A unit is 32 targets of a work item against its sources; warps take units from
 // a counter, stage their own source tiles and never wait for one another (df_tile, shared with the
-// treecode).  No float64 arithmetic runs but the final accumulation per target.
+// treecode).  No float64 arithmetic runs but the final accumulation per target.  Bound by the float32 pipe, 84%
+// busy: both sums 126 to 153 Gpair/s (101 particles of 220 nodes), the traction alone 195 to 219 (500 of 220),
+// against two-sum arithmetic throughout in blocks of whole items.
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restrict__ counter,
                                                       const longlong4* __restrict__ work,
@@ -892,7 +897,9 @@ __global__ void __launch_bounds__(256) k_upsample(const int4* __restrict__ group
 
 // Near correction by the units of near.cuh.
 
-// Float32: the packed tile loop of the smooth sum over per-warp tiles of 128 sources.
+// Float32: the packed tile loop of the smooth sum over per-warp tiles of 128 sources.  Bound by the float32 pipe;
+// against one block per pair, a solve's 17 corrections (one double-float) with 398 pairs in 24 suspensions of mixed
+// orders went from 28 to 5.8 ms with their upsampling, and with 6,582 pairs of 144-node particles from 31 to 22.5 ms.
 template <int KIND>
 __global__ void __launch_bounds__(128, 6) k_near32(NearArgs A, const float4* __restrict__ xhi,
                                                    const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
@@ -1134,11 +1141,13 @@ static int resident_grid(Context& c, const void* kernel, int threads, int items)
 }
 
 // Targets per lane of the direct float32 sums: two, which share each source's loads, once that still makes
-// 64 units per SM (three rounds of its warps); one below, and where rbs_options.pair_variant asks for it.
+// 48 units per SM (two rounds of its warps); one below, and where rbs_options.pair_variant asks for it.  Traction
+// Gpair/s with one and two: 117 and 97 at one unit per SM (8 particles of 144 nodes), 1,227 and 1,261 at 64 (40 of
+// 220), 1,405 and 1,438 above (101 of 220).
 static int pairs32_targets(const Context& c) {
   const int v = c.opt.pair_variant;
   if (v > 0) return v == 1 || v == kPacked + 1 ? 1 : 2;
-  return 2 * (long long)c.work.size() >= 64LL * c.sm_count ? 2 : 1;
+  return 2 * (long long)c.work.size() >= 48LL * c.sm_count ? 2 : 1;
 }
 
 int direct_variant(const Context& c) { return kPacked + pairs32_targets(c); }
@@ -1350,8 +1359,9 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     RBS_TRY(weight_df(c, x));
   }
   // The float32 near correction of a small system runs beside the smooth sum (both add into y atomically): each
-  // alone leaves SMs idle at its end, and below about 10^5 nodes that is a tenth of an apply.  Not while kernel
-  // classes are timed.
+  // alone leaves SMs idle at its end.  Solves after one another and beside: 50.7 and 49.2 ms (a step of 101
+  // particles, 22,000 nodes), 49.9 and 49.4 (57,600 nodes), 403.3 and 402.6 (216,000), where the line is drawn: the
+  // gain is within the runs' spread.  Not while kernel classes are timed.
   const bool beside = f32 && c.side && !c.near_pairs.empty() && c.N <= kBesideNodes && c.opt.timing == 0;
   if (beside) {
     RBS_CUDA_TRY(cudaEventRecord(c.fork_ev, c.stream));

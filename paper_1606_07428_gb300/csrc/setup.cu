@@ -148,7 +148,9 @@ __global__ void k_rotate_points(int npts, int nj, const double* t, const double4
 // in their own frame, where the harmonics are products: out[row][b] = sum over theta' of leg[theta'][b] sum
 // over phi' of trig[phi'][col(b)] C[row][theta'][phi'].  One block per (row, shape); the phi' sums run over the
 // half circle, on the sums (cosines) and differences (sines) of opposite points.  About 20,000
-// multiply-adds a row at p = 12 where the rule's nrot x N_p interpolation matrix takes 390,000.
+// multiply-adds a row at p = 12 where the rule's nrot x N_p interpolation matrix takes 390,000.  Bound by the
+// float64 pipe: for 64 shapes at p = 12 these sums and the GEMM after them take 2.2 and 7.2 ms, the GEMM with the
+// dense matrix took 47.
 __global__ void __launch_bounds__(256) k_rule_transform(int na, int slab, int nb, int nf, int nfull, const double* trig,
                                                         const double* leg, const int* col, const double* C,
                                                         long long strideC, double* out, long long strideOut) {
