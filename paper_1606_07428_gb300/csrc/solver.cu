@@ -168,7 +168,9 @@ __global__ void k_unpack_vo(int n, const double* vo, double* v, double* om) {
 // L2 error of a few 1e-7 on the 1,000-ellipsoid p = 12 suspension, plus the treecode's model when it
 // is on) decides when a refinement residual may be updated in float32.
 
-// Relative error assumed for apply_correction.
+// Relative error assumed for apply_correction.  Measured for float32 smooth and near sums together against
+// double-float, 8 to 700 ellipsoids of orders 6 to 12, random and smooth densities: at most 1.3e-8 of |A d| in K and
+// 3.0e-7 of |S_off d| in S.
 constexpr double kCorrectionError = 5e-7;
 
 // Float64-class residual and surface velocity of one iterate x, sharing one pass over the pairs:
