@@ -161,7 +161,8 @@ struct TreeItem {  // one work item of the treecode pair sum
   int t0, t1;      // target nodes [t0, t1), all on one particle
   int s0, s1;      // source segments [s0, s1) of that particle's list
   int nmask;       // leading sources of the item that may lie on the target's own particle
-  int pad0, pad1, pad2;
+  int nskip;       // leading segments of the item that are the target's own particle or its near ones
+  int pad0, pad1;
 };
 struct TreeState {
   bool active = false;
@@ -190,6 +191,8 @@ struct TreeState {
   DevBuf<float> d_pq;
   DevBuf<double> d_q64;
   long long direct_pairs = 0, proxy_pairs = 0, charge_work = 0;
+  // node pairs of the leading segments (the own particle and its near ones), and how many near pairs these hold
+  long long lead_pairs = 0, near_listed = 0;
   void release();
 };
 
@@ -293,6 +296,7 @@ struct Context {
   size_t block_elems = 0;  // sum over shapes of (3 np)^2
   double particle_block_entries = 0;  // sum over particles of (3 np)^2 (entries read per block apply)
   double near_pair_nodes = 0;         // sum over near pairs of np_i (nup_j + np_j)
+  double near_base_nodes = 0;         // sum over near pairs of np_i np_j
   bool have_geometry = false;
 
   // per-particle device data
@@ -335,6 +339,7 @@ struct Context {
   std::vector<int2> near_pairs;   // (target particle, source particle)
   bool near_multi = false;        // some target particle has several near sources
   DevBuf<int2> d_near;
+  DevBuf<int> d_near_first;       // n + 1: first near pair of each target particle
   std::vector<int> up_index;      // per particle: index into upsampled-source list or -1
   std::vector<long long> up_offset;  // per upsampled source particle: first upsampled node
   std::vector<int> up_particle;
@@ -476,6 +481,7 @@ struct TreePlan {
   std::vector<double> box, proxy;
   int n_cells = 0, tmax = 0;
   long long n_src = 0, direct_pairs = 0, proxy_pairs = 0, charge_work = 0;
+  long long lead_pairs = 0, near_listed = 0;  // as in TreeState
 };
 // Host only: no device work (also usable without a GPU).
 Status plan_treecode(const PlanInput& in, double theta, int degree, TreePlan& plan);
@@ -488,11 +494,8 @@ int tree_variant(const Context& c);  // its targets per lane
 // The same for the double-float passes (d_wmuh, d_wmul): y += kind 0 or 1 sum; kind 2: y += traction, y2 += Stokeslet.
 Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y2);
 // y += traction and y2 += Stokeslet sum over the double-float passes' lists in float32 arithmetic (d_wmu32; the
-// charges formed in float64).
+// charges formed in float64), without the sources on particles near the target's.
 Status apply_tree_df_f32(Context& c, const double* x, double* y, double* y2);
-// Relative error assumed for a float32 operator application: rounding plus, with the treecode,
-// its approximation model C(theta) rho^-n.
-double f32_operator_error(const Context& c);
 
 // ---- setup (setup.cu)
 Status build_geometry(Context& c);
@@ -501,6 +504,8 @@ Status build_near(Context& c);
 // Host only: the reflection-symmetry tables of a (p, n_phi) grid (see rbs_grid_symmetry).
 Status grid_symmetry_host(int p, int nphi, std::vector<int>& rep_of, std::vector<int>& g_of, int irrep_dim[8],
                           int* nrep);
+// Host only: whether particles i and j of one suspension are near.
+bool near_particles(const double* centres, const double* R, int i, int j, double delta);
 // Host only: the near pairs of centres with bounding radii R and inscribed radii rmin (see build_near).
 Status plan_near(int n, const double* centres, const double* R, const double* rmin, const int* sid, double delta,
                  std::vector<int2>& out);
@@ -543,8 +548,8 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y); 
 // yK += off-diagonal K x and yS += off-diagonal S x in one pass over the pairs (double-float)
 Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, double* yS);
 Status apply_operator(Context& c, int op, int prec, const double* x, double* y);
-// w = A d and v = S d for a correction d: float64 blocks and the near correction in double-float, only the smooth
-// sums in float32, over the same lists as the double-float passes.
+// w = A d and v = S d for a correction d: float64 blocks, the near pairs' upsampled sums in double-float, and the
+// smooth sums between particles that are not near in float32, over the same lists as the double-float passes.
 Status apply_correction(Context& c, const double* d, double* w, double* v);
 
 // ---- solver (solver.cu)

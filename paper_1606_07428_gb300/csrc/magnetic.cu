@@ -619,7 +619,7 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
                                      M.d_upU.ptr, x, c.d_up_x.ptr, M.d_qup.ptr);
     NearArgs A;
     int blocks = 0;
-    RBS_TRY(near_args(c, A, blocks));
+    RBS_TRY(near_args(c, true, A, blocks));
     blocks = std::min(blocks, 5 * std::max(1, c.sm_count));
 #define RBS_LAP_NEAR                                                                                              \
   A, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, c.d_up3h.ptr, c.d_up3m.ptr, \

@@ -13,8 +13,10 @@ namespace rbs {
 // counter; parts grows until small near lists fill the GPU.  A pair of 144-node particles is 688 sources
 // against five units of targets, so one block per pair left most of the SMs idle on lists of a few hundred
 // pairs and most of its threads idle where orders mix.
+// base: with the base nodes; else the upsampled nodes alone (for sums that leave near sources out).
 struct NearArgs {
   int nunits, chunks, parts;
+  bool base;
   int* counter;
   const int2* near;
   const long long* offset;
@@ -42,7 +44,7 @@ __device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
   n.ub = A.up_off[u];
   n.nup = (int)(A.up_off[u + 1] - n.ub);
   n.oj = A.offset[pr.y];
-  const int total = n.nup + A.nodes[pr.y];
+  const int total = n.nup + (A.base ? A.nodes[pr.y] : 0);
   const int step = ((total + A.parts - 1) / A.parts + 3) & ~3;
   n.s0 = min(total, part * step);
   n.s1 = min(total, n.s0 + step);
@@ -52,7 +54,8 @@ __device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
 
 // The units of the context's near list (its counter, d_unit[1], is zeroed by the caller or the weight kernels);
 // blocks: as many 128-thread blocks as have a unit per warp.
-inline Status near_args(Context& c, NearArgs& A, int& blocks) {
+inline Status near_args(Context& c, bool base, NearArgs& A, int& blocks) {
+  A.base = base;
   const long long nn = (long long)c.near_pairs.size();
   A.chunks = (c.max_np + 31) / 32;
   // source runs: about 16 units per SM, of at least 128 sources and at most about 512 (a unit of one p = 16

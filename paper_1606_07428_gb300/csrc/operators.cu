@@ -608,13 +608,11 @@ __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const d
 // Bound by the float32 pipe (20 operations a traction pair, 18 a Stokeslet pair), 76% busy: 1,460 Gpair/s on 101
 // particles of 220 nodes, 1,400 with blocks that took whole items; on 8 particles of 144 nodes an apply went from 34 to
 // 12 us by the smaller units.
-// KIND 2 (one target per lane): traction into y and Stokeslet into y2 in one pass, 26 operations.
 template <int KIND, int NT>
-__global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
+__global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
     k_pairs32x2(int nunits, int* __restrict__ counter, const longlong4* __restrict__ work,
                 const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
-                const float4* __restrict__ wmu, double* __restrict__ y, double* __restrict__ y2) {
-  static_assert(KIND != 2 || NT == 1, "both sums: one target per lane");
+                const float4* __restrict__ wmu, double* __restrict__ y) {
   constexpr int TW = 128, kPerItem = 4 / NT;
   __shared__ __align__(16) float tiles[4][7 * TW];
   const int lane = threadIdx.x & 31;
@@ -660,7 +658,6 @@ __global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
     }
     const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(xhi[min(t0 + 32 * NT, t1) - 1].w);
     float sa[NT][3], ea[NT][3];
-    float sb[3] = {0.0f, 0.0f, 0.0f}, eb[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
     for (int s0 = (int)w.z; s0 < (int)w.w; s0 += TW) {
@@ -700,15 +697,7 @@ __global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
       pair_tile32x2<KIND, true, NT, NUV>(b, b + TW, b + 2 * TW, b + 3 * TW, b + 4 * TW, b + 5 * TW, spid + l0, m,  \
                                          xt, nt, pt, p);                                                           \
   } while (0)
-      if constexpr (KIND == 2) {
-        float2 p2[3] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
-        if (thi < pid_lo || tlo > pid_hi)
-          pair_tile32_both<false, TW>(ssx, spid, l0, m, xt[0], nt[0], pt[0], p[0], p2);
-        else
-          pair_tile32_both<true, TW>(ssx, spid, l0, m, xt[0], nt[0], pt[0], p[0], p2);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) two_sum_acc(sb[c], eb[c], p2[c].x + p2[c].y);
-      } else if (nu == NT) {
+      if (nu == NT) {
         RBS_TILE(NT);
       } else if constexpr (NT > 1) {
         RBS_TILE(1);
@@ -725,10 +714,113 @@ __global__ void __launch_bounds__(128, KIND == 2 ? 5 : (NT == 1 ? 7 : 5))
       if (!valid[u]) continue;
       const long long t = t0 + 32 * u + (split ? lane & 15 : lane);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
-        if (KIND == 2) atomicAdd(y2 + 3 * t + c, kStokesletScale * ((double)sb[c] + (double)eb[c]));
+      for (int c = 0; c < 3; ++c) atomicAdd(y + 3 * t + c, sc * ((double)sa[u][c] + (double)ea[u][c]));
+    }
+  }
+}
+
+// Direct float32 sums of a refinement correction: traction into y and Stokeslet into y2 in one pass (26 operations a
+// pair), over the sources that lie neither on the target's own particle nor on one near it.  Near terms grow as the
+// inverse square of a gap and their float32 rounding as its inverse cube, so a sum that adds them for the near correction to
+// remove keeps an error without bound (with one pair of spheres 0.01 apart, a solve to 1e-10 ended at 2e-9); without
+// them every separation is at least near_delta.  A unit is 32 targets of a work item, taken one target particle at a
+// time: sources are relative to the run's first target, a particle's diameter away at most.  Excluded sources become
+// zero-density ones far away.  The near pairs of a particle are ordered by source, so a pointer walks them beside
+// the tiles.
+__global__ void __launch_bounds__(128, 5)
+    k_far32_both(int nunits, int* __restrict__ counter, const longlong4* __restrict__ work,
+                 const long long* __restrict__ offset, const int* __restrict__ near_first, const int2* __restrict__ near,
+                 const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
+                 const float4* __restrict__ wmu, double* __restrict__ y, double* __restrict__ y2) {
+  constexpr int TW = 128, SL = TW / 32;
+  __shared__ __align__(16) float tiles[4][6 * TW];
+  const int lane = threadIdx.x & 31;
+  float* const ssx = tiles[threadIdx.x >> 5];
+  while (true) {
+    int unit = 0;
+    if (lane == 0) unit = atomicAdd(counter, 1);
+    unit = __shfl_sync(0xffffffffu, unit, 0);
+    if (unit >= nunits) return;
+    const longlong4 w = work[unit >> 2];
+    const int ub = (int)w.x + 32 * (unit & 3), ue = min(ub + 32, (int)w.y);
+    for (int t0 = ub; t0 < ue;) {
+      const float4 oh = xhi[t0], ol = xlo[t0];
+      const int i = __float_as_int(oh.w);
+      const int t1 = (int)min((long long)ue, offset[i + 1]);
+      const bool split = t1 - t0 <= 16;  // the two half-warps take alternate halves of the sources
+      const int half = split ? lane >> 4 : 0;
+      const int t = t0 + (split ? lane & 15 : lane);
+      const bool valid = t < t1;
+      float2 xt[3], nt[3];
+      {
+        const float4 ah = valid ? xhi[t] : oh, al = valid ? xlo[t] : ol;
+        const float4 nn = valid ? nrm32[t] : make_float4(0, 0, 0, 0);
+        const float a0 = (ah.x - oh.x) + (al.x - ol.x), a1 = (ah.y - oh.y) + (al.y - ol.y),
+                    a2 = (ah.z - oh.z) + (al.z - ol.z);
+        xt[0] = f2(a0, a0);
+        xt[1] = f2(a1, a1);
+        xt[2] = f2(a2, a2);
+        nt[0] = f2(nn.x, nn.x);
+        nt[1] = f2(nn.y, nn.y);
+        nt[2] = f2(nn.z, nn.z);
       }
+      float sa[3] = {0, 0, 0}, ea[3] = {0, 0, 0}, sb[3] = {0, 0, 0}, eb[3] = {0, 0, 0};
+      int k = near_first[i];
+      const int ke = near_first[i + 1];
+      for (int s0 = (int)w.z; s0 < (int)w.w; s0 += TW) {
+        const int cnt = min(TW, (int)w.w - s0), cnt8 = (cnt + 7) & ~7;
+        float4 ph[SL];
+        bool out[SL];
+#pragma unroll
+        for (int q = 0; q < SL; ++q) {
+          const int l = lane + 32 * q;
+          out[q] = l >= cnt;
+          ph[q] = l < cnt ? xhi[s0 + l] : make_float4(0, 0, 0, 0);
+          if (__float_as_int(ph[q].w) == i) out[q] = true;
+        }
+        const int tlo = __float_as_int(xhi[s0].w), thi = __float_as_int(xhi[s0 + cnt - 1].w);
+        while (k < ke && near[k].y < tlo) ++k;
+        for (int e = k; e < ke && near[e].y <= thi; ++e) {
+          const int j = near[e].y;
+#pragma unroll
+          for (int q = 0; q < SL; ++q)
+            if (__float_as_int(ph[q].w) == j) out[q] = true;
+        }
+        __syncwarp();  // the warp's reads of the previous tile are done
+#pragma unroll
+        for (int q = 0; q < SL; ++q) {
+          const int l = lane + 32 * q;
+          if (!out[q]) {
+            const float4 pl = xlo[s0 + l], d = wmu[s0 + l];
+            ssx[l] = (oh.x - ph[q].x) + (ol.x - pl.x);
+            ssx[TW + l] = (oh.y - ph[q].y) + (ol.y - pl.y);
+            ssx[2 * TW + l] = (oh.z - ph[q].z) + (ol.z - pl.z);
+            ssx[3 * TW + l] = d.x;
+            ssx[4 * TW + l] = d.y;
+            ssx[5 * TW + l] = d.z;
+          } else {
+            ssx[l] = ssx[TW + l] = ssx[2 * TW + l] = 1.0e4f;
+            ssx[3 * TW + l] = ssx[4 * TW + l] = ssx[5 * TW + l] = 0.0f;
+          }
+        }
+        __syncwarp();
+        const int m = split ? cnt8 / 2 : cnt8;
+        float2 p[3] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f), f2(0.0f, 0.0f)}, p2[3] = {p[0], p[0], p[0]};
+        pair_tile32_both<TW>(ssx, half * m, m, xt, nt, p, p2);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          two_sum_acc(sa[c], ea[c], p[c].x + p[c].y);
+          two_sum_acc(sb[c], eb[c], p2[c].x + p2[c].y);
+        }
+      }
+      if (valid) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          atomicAdd(y + 3 * (long long)t + c, kTractionScale * ((double)sa[c] + (double)ea[c]));
+          atomicAdd(y2 + 3 * (long long)t + c, kStokesletScale * ((double)sb[c] + (double)eb[c]));
+        }
+      }
+      t0 = t1;
     }
   }
 }
@@ -980,7 +1072,7 @@ __global__ void __launch_bounds__(128, 6) k_near32(NearArgs A, const float4* __r
   }
 }
 
-// Double-float: the arithmetic of the smooth sums (df_tile), so that what is removed is what they added;
+// Double-float: the arithmetic of the smooth sums (df_tile), whose base terms it removes to about 1e-13 of each;
 // KIND 2 both kernels in one pass.
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_near_df(NearArgs A, const float4* __restrict__ x3h,
@@ -1153,11 +1245,11 @@ static int pairs32_targets(const Context& c) {
 int direct_variant(const Context& c) { return kPacked + pairs32_targets(c); }
 
 template <int KIND, int NT>
-static void launch_pairs32(Context& c, double* y, double* y2 = nullptr) {
+static void launch_pairs32(Context& c, double* y) {
   const int items = (int)c.work.size();
   const auto kernel = k_pairs32x2<KIND, NT>;
   kernel<<<resident_grid(c, (const void*)kernel, 128, items), 128, 0, c.stream>>>(
-      4 / NT * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y, y2);
+      4 / NT * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y);
 }
 
 template <int KIND>
@@ -1308,12 +1400,13 @@ static Status near_upsample(Context& c, int prec, const double* x) {
   return Status::Ok();
 }
 
-// Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one; kind 0
-// traction into y, 1 Stokeslet into y, 2 (double-float only) traction into y and Stokeslet into y2.
-static Status near_sums(Context& c, int kind, int prec, const double* x, double* y, double* y2) {
+// Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one (base false: the
+// upsampled one is added); kind 0 traction into y, 1 Stokeslet into y, 2 (double-float only) traction into y and
+// Stokeslet into y2.
+static Status near_sums(Context& c, int kind, int prec, const double* x, double* y, double* y2, bool base = true) {
   NearArgs A;
   int blocks = 0;
-  RBS_TRY(near_args(c, A, blocks));
+  RBS_TRY(near_args(c, base, A, blocks));
   if (prec == RBS_PREC_FP64) RBS_CUDA_TRY(cudaMemsetAsync(A.counter, 0, sizeof(int), c.stream));
 #define RBS_NEAR_LAUNCH(KERNEL, ...) \
   KERNEL<<<resident_grid(c, (const void*)KERNEL, 128, blocks), 128, 0, c.stream>>>(A, __VA_ARGS__)
@@ -1456,15 +1549,18 @@ Status apply_correction(Context& c, const double* d, double* w, double* v) {
     RBS_TRY(apply_tree_df_f32(c, d, w, v));
   } else if (!c.work.empty()) {
     KernelTimer timer(c, RBS_KC_PAIR_K32);
-    launch_pairs32<2, 1>(c, w, v);
+    const int items = (int)c.work.size();
+    k_far32_both<<<resident_grid(c, (const void*)k_far32_both, 128, items), 128, 0, c.stream>>>(
+        4 * items, c.d_unit.ptr, c.d_work.ptr, c.d_offset.ptr, c.d_near_first.ptr, c.d_near.ptr, c.d_xhi.ptr, c.d_xlo.ptr,
+        c.d_nrm32.ptr, c.d_wmu32.ptr, w, v);
     RBS_CUDA_TRY(cudaGetLastError());
-    timer.done(2.0 * (double)c.stats.far_pairs);
+    timer.done(2.0 * ((double)c.stats.far_pairs - c.near_base_nodes));
   }
   if (!c.near_pairs.empty()) {
     KernelTimer timer(c, RBS_KC_NEAR);
     RBS_TRY(near_upsample(c, RBS_PREC_DF, d));
-    RBS_TRY(near_sums(c, 2, RBS_PREC_DF, d, w, v));
-    timer.done(2.0 * c.near_pair_nodes, 2);
+    RBS_TRY(near_sums(c, 2, RBS_PREC_DF, d, w, v, false));
+    timer.done(2.0 * (c.near_pair_nodes - c.near_base_nodes), 2);
   }
   return Status::Ok();
 }

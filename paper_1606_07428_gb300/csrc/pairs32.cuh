@@ -88,18 +88,13 @@ __device__ __forceinline__ void pair_tile32x2(const float* __restrict__ ssx, con
 }
 
 // Both sums of one density for one target: traction into acc, Stokeslet into acc2 (26 operations a pair, where
-// the two separately take 38).
-template <bool MASK>
-__device__ __forceinline__ void pair2_both_f32(float2 sx, float2 sy, float2 sz, float2 rx, float2 ry, float2 rz, int2 spid,
-                                               const float2 (&xt)[3], const float2 (&nt)[3], int pt, float2 (&acc)[3],
+// the two separately take 38).  No source is on the target's own particle.
+__device__ __forceinline__ void pair2_both_f32(float2 sx, float2 sy, float2 sz, float2 rx, float2 ry, float2 rz,
+                                               const float2 (&xt)[3], const float2 (&nt)[3], float2 (&acc)[3],
                                                float2 (&acc2)[3]) {
   const float2 dx = __fadd2_rn(xt[0], sx), dy = __fadd2_rn(xt[1], sy), dz = __fadd2_rn(xt[2], sz);
   const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-  float2 inv = f2(rsqrt_hw(r2.x), rsqrt_hw(r2.y));
-  if (MASK) {
-    if (spid.x == pt) inv.x = 0.0f;
-    if (spid.y == pt) inv.y = 0.0f;
-  }
+  const float2 inv = f2(rsqrt_hw(r2.x), rsqrt_hw(r2.y));
   const float2 rr = __ffma2_rn(dz, rz, __ffma2_rn(dy, ry, __fmul2_rn(dx, rx)));
   const float2 rn = __ffma2_rn(dz, nt[2], __ffma2_rn(dy, nt[1], __fmul2_rn(dx, nt[0])));
   const float2 inv2 = __fmul2_rn(inv, inv);
@@ -113,23 +108,20 @@ __device__ __forceinline__ void pair2_both_f32(float2 sx, float2 sy, float2 sz, 
   acc2[2] = __ffma2_rn(cs, dz, __ffma2_rn(rz, inv, acc2[2]));
 }
 
-// One target per lane against a warp's tile (rows of TW floats: x, y, z, density x, y, z, then particle ids),
-// sources [l0, l0 + cnt), cnt a multiple of four.
-template <bool MASK, int TW>
-__device__ __forceinline__ void pair_tile32_both(const float* __restrict__ t, const int* __restrict__ spid, int l0, int cnt,
-                                                 const float2 (&xt)[3], const float2 (&nt)[3], int pt, float2 (&acc)[3],
-                                                 float2 (&acc2)[3]) {
+// One target per lane against a warp's tile (rows of TW floats: x, y, z, density x, y, z), sources
+// [l0, l0 + cnt), cnt a multiple of four.
+template <int TW>
+__device__ __forceinline__ void pair_tile32_both(const float* __restrict__ t, int l0, int cnt, const float2 (&xt)[3],
+                                                 const float2 (&nt)[3], float2 (&acc)[3], float2 (&acc2)[3]) {
 #pragma unroll 2
   for (int l = l0; l < l0 + cnt; l += 4) {
     const float4 ax = *reinterpret_cast<const float4*>(t + l), ay = *reinterpret_cast<const float4*>(t + TW + l);
     const float4 az = *reinterpret_cast<const float4*>(t + 2 * TW + l), bx = *reinterpret_cast<const float4*>(t + 3 * TW + l);
     const float4 by = *reinterpret_cast<const float4*>(t + 4 * TW + l), bz = *reinterpret_cast<const float4*>(t + 5 * TW + l);
-    int4 pp = make_int4(-1, -1, -1, -1);
-    if (MASK) pp = *reinterpret_cast<const int4*>(spid + l);
-    pair2_both_f32<MASK>(f2(ax.x, ax.y), f2(ay.x, ay.y), f2(az.x, az.y), f2(bx.x, bx.y), f2(by.x, by.y), f2(bz.x, bz.y),
-                         make_int2(pp.x, pp.y), xt, nt, pt, acc, acc2);
-    pair2_both_f32<MASK>(f2(ax.z, ax.w), f2(ay.z, ay.w), f2(az.z, az.w), f2(bx.z, bx.w), f2(by.z, by.w), f2(bz.z, bz.w),
-                         make_int2(pp.z, pp.w), xt, nt, pt, acc, acc2);
+    pair2_both_f32(f2(ax.x, ax.y), f2(ay.x, ay.y), f2(az.x, az.y), f2(bx.x, bx.y), f2(by.x, by.y), f2(bz.x, bz.y), xt,
+                   nt, acc, acc2);
+    pair2_both_f32(f2(ax.z, ax.w), f2(ay.z, ay.w), f2(az.z, az.w), f2(bx.z, bx.w), f2(by.z, by.w), f2(bz.z, bz.w), xt,
+                   nt, acc, acc2);
   }
 }
 

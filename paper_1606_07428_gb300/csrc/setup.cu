@@ -974,6 +974,12 @@ Status place_particles(Context& c) {
   return Status::Ok();
 }
 
+bool near_particles(const double* centres, const double* R, int i, int j, double delta) {
+  const double dx = centres[3 * i] - centres[3 * j], dy = centres[3 * i + 1] - centres[3 * j + 1],
+               dz = centres[3 * i + 2] - centres[3 * j + 2];
+  return std::sqrt(dx * dx + dy * dy + dz * dz) < R[i] + R[j] + delta;
+}
+
 // Near pairs (Section 3, upsampling for close particles): ordered pairs (i, j), i != j of one
 // suspension with |c_i - c_j| < R_i + R_j + delta, found with a cell list; RBS_EOVERLAP when two
 // inscribed spheres (radius rmin) intersect.  Host only.
@@ -1012,7 +1018,7 @@ Status plan_near(int n, const double* centres, const double* R, const double* rm
       if (d < rmin[i] + rmin[j])
         return Status::Err(RBS_EOVERLAP, "particles " + std::to_string(i) + " and " + std::to_string(j) +
                                              " overlap (inscribed spheres intersect)");
-      if (d < R[i] + R[j] + delta) out.push_back(make_int2(i, j));
+      if (near_particles(centres, R, i, j, delta)) out.push_back(make_int2(i, j));
     }
   }
   return Status::Ok();
@@ -1032,6 +1038,10 @@ Status build_near(Context& c) {
     RBS_TRY(plan_near(n, c.centres.data(), R.data(), rmin.data(), c.sid.data(), c.opt.near_delta, c.near_pairs));
   }
   RBS_TRY(upload(c.d_near, c.near_pairs, s));
+  std::vector<int> first(n + 1, 0);  // (the list is ordered by target)
+  for (const int2& pr : c.near_pairs) ++first[pr.x + 1];
+  for (int i = 0; i < n; ++i) first[i + 1] += first[i];
+  RBS_TRY(upload(c.d_near_first, first, s));
   // upsampled sources
   c.up_index.assign(n, -1);
   c.up_particle.clear();
@@ -1085,12 +1095,14 @@ Status build_near(Context& c) {
   }
 
   c.near_multi = false;
-  for (size_t k = 1; k < c.near_pairs.size(); ++k)  // (the list is ordered by target)
-    if (c.near_pairs[k].x == c.near_pairs[k - 1].x) c.near_multi = true;
-  c.near_pair_nodes = 0;
-  for (const int2& pr : c.near_pairs)
-    c.near_pair_nodes += (double)(c.offset[pr.x + 1] - c.offset[pr.x]) *
-                         (c.grids[c.grid_of[pr.y]]->nup + (c.offset[pr.y + 1] - c.offset[pr.y]));
+  for (int i = 0; i < n; ++i)
+    if (first[i + 1] - first[i] > 1) c.near_multi = true;
+  c.near_pair_nodes = c.near_base_nodes = 0;
+  for (const int2& pr : c.near_pairs) {
+    const double base = (double)(c.offset[pr.x + 1] - c.offset[pr.x]) * (c.offset[pr.y + 1] - c.offset[pr.y]);
+    c.near_base_nodes += base;
+    c.near_pair_nodes += base + (double)(c.offset[pr.x + 1] - c.offset[pr.x]) * c.grids[c.grid_of[pr.y]]->nup;
+  }
   c.stats.near_pairs = (long long)c.near_pairs.size();
   return build_far_field(c);
 }

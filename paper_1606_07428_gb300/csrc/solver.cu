@@ -163,15 +163,23 @@ __global__ void k_unpack_vo(int n, const double* vo, double* v, double* om) {
   }
 }
 
-// The relative error of a float32 operator application (f32_operator_error: 1e-5 for float32 pair
-// sums with per-tile compensation, float32 blocks and interpolation, a bound on the measured relative
-// L2 error of a few 1e-7 on the 1,000-ellipsoid p = 12 suspension, plus the treecode's model when it
-// is on) decides when a refinement residual may be updated in float32.
-
-// Relative error assumed for apply_correction.  Measured for float32 smooth and near sums together against
-// double-float, 8 to 700 ellipsoids of orders 6 to 12, random and smooth densities: at most 1.3e-8 of |A d| in K and
-// 3.0e-7 of |S_off d| in S.
+// Relative error assumed for apply_correction, infinite where it is not to be used.  Its float32 sums hold no near pair,
+// so their separations are at least near_delta and the error does not grow as gaps close.  Measured against
+// double-float applies for random, smooth and solution densities, orders 2 to 24, 2 to 1,000 particles, direct and with
+// proxies: at most 9e-8 of |A d| at gaps 0.2 to 0.003 with near_delta the particles' radius, 1.0e-7, 4.5e-7, 5.9e-7 and
+// 1.7e-6 with radii of 2, 4, 8 and 16 near_delta (coordinates are rounded at a particle's size, terms are as steep as
+// near_delta); of |S d| at most 2e-7 in all of these.
 constexpr double kCorrectionError = 5e-7;
+
+static double correction_error(const Context& c) {
+  double rmax = 0.0;
+  for (const Shape& sh : c.shapes) rmax = std::max(rmax, sh.radius);
+  if (!(c.opt.near_delta > 0.0)) return INFINITY;
+  // every near pair has to be among the directly evaluated ones of the tree (a cluster is accepted only beyond
+  // near_delta, but for rounding)
+  if (c.tree_df.active && c.tree_df.near_listed != (long long)c.near_pairs.size()) return INFINITY;
+  return kCorrectionError * std::max(1.0, rmax / (2.0 * c.opt.near_delta));
+}
 
 // Float64-class residual and surface velocity of one iterate x, sharing one pass over the pairs:
 // with sigma = rho + x,  r = b - A x = -(1/2 I + K) sigma - L x = L rho - A sigma  (Eq. 25, A the
@@ -272,12 +280,11 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
   } else {
     // Iterative refinement around float32 inner solves.  A float64-class pass gives the true
     // residual r = b - A x and, from the same pair sums, u = S[rho + x].  After a pass, a small
-    // correction d may instead update r -= A d and u += S d by a cheaper operator of relative error e: these
-    // updates are taken only while e ||A d||, summed since the last pass, stays below a tenth of the
-    // tolerance in every suspension the correction touched.  The cheapest that allows it is chosen:
-    //   the inner solve's float32 operator (f32_operator_error: 1e-5, plus the treecode's model), or
-    //   apply_correction, whose smooth sums alone are float32 (kCorrectionError; a tenth of a pass's time).
-    // Suspensions within tolerance after a float64-class pass take no further inner iterations.
+    // correction d may instead update r -= A d and u += S d by apply_correction, of relative error e (a
+    // tenth of a pass's time): these updates are taken only while e ||A d||, summed since the last pass, stays
+    // below a tenth of the tolerance in every suspension the correction touched.  (The inner solve's float32
+    // operator is no substitute at any size of d: it adds near pairs' base terms and removes them again, and
+    // with one pair 0.02 apart its updates left 9e-9 of a solve to 1e-10.)  Suspensions within tolerance after a float64-class pass take no further inner iterations.
     double* lrho = c.d_vec[8].ptr;  // L rho (Eq. 26), float64
     RBS_TRY(apply_blocks(c, kModeL, RBS_PREC_FP64, rho, lrho, nullptr, 1.0));
     std::vector<double> rn = bn;
@@ -294,11 +301,10 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
       RBS_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(double) * n3, c.stream));
       RBS_CUDA_TRY(cudaMemcpyAsync(r, b, sizeof(double) * n3, cudaMemcpyDeviceToDevice, c.stream));
     }
-    // sigma accumulates the corrections applied by the float32 operator since the last float64-class pass
-    bool sigma_used = false;
-    std::vector<double> pending(S, 0.0);
+    std::vector<double> pending(S, 0.0);  // the error of the updates since the last pass
     std::vector<int> used(S, 0);
-    const double ferr = f32_operator_error(c);
+    // (passes asked for in float64 are replaced only by updates that change nothing in their last digits)
+    const double err = hi == RBS_PREC_DF ? correction_error(c) : std::max(1e-5, correction_error(c));
     converged = false;
     int used_max = 0;
     while (!converged && refinements < c.opt.max_refinements && used_max < c.opt.max_iters) {
@@ -327,33 +333,20 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
       ++refinements;
       c.stats.launches++;
       k_axpby<<<nbk, 256, 0, c.stream>>>(x, 1.0, d, 1.0, n3);
-      // pending[s]: the error of the updates since the last pass
-      auto allowed = [&](double err) {
-        for (int s = 0; s < S; ++s)
-          if (R.iters[s] > 0 && pending[s] + err * rn[s] > 0.1 * tol * bn[s]) return false;
-        return u_done;
-      };
-      if (allowed(ferr)) {
-        RBS_TRY(apply_operator(c, RBS_OP_A, RBS_PREC_MIXED, d, w));
-        c.stats.launches += 2;
-        k_axpby<<<nbk, 256, 0, c.stream>>>(r, -1.0, w, 1.0, n3);
-        k_axpby<<<nbk, 256, 0, c.stream>>>(sigma, 1.0, d, 1.0, n3);
-        sigma_used = true;
-        for (int s = 0; s < S; ++s)
-          if (R.iters[s] > 0) pending[s] += ferr * rn[s];
-      } else if (hi == RBS_PREC_DF && allowed(kCorrectionError)) {
+      bool update = u_done;
+      for (int s = 0; s < S; ++s)
+        if (R.iters[s] > 0 && !(pending[s] + err * rn[s] <= 0.1 * tol * bn[s])) update = false;
+      if (update) {
         double* v = c.d_vec[6].ptr;
         RBS_TRY(apply_correction(c, d, w, v));
         c.stats.launches += 2;
         k_axpby<<<nbk, 256, 0, c.stream>>>(r, -1.0, w, 1.0, n3);
         k_axpby<<<nbk, 256, 0, c.stream>>>(u, 1.0, v, 1.0, n3);
         for (int s = 0; s < S; ++s)
-          if (R.iters[s] > 0) pending[s] += kCorrectionError * rn[s];
+          if (R.iters[s] > 0) pending[s] += err * rn[s];
       } else {
         RBS_TRY(residual_and_velocity(c, hi, rho, lrho, x, sigma, r, u));
         u_done = true;
-        RBS_CUDA_TRY(cudaMemsetAsync(sigma, 0, sizeof(double) * n3, c.stream));
-        sigma_used = false;
         std::fill(pending.begin(), pending.end(), 0.0);
       }
       RBS_TRY(seg_norms_host(c, c.seg3, r, rn));
@@ -363,11 +356,6 @@ static Status solve_core(Context& c, double tol, bool warm, std::vector<int>& it
       if (moved == 0) break;  // the inner solves could not move
     }
     for (int s = 0; s < S; ++s) rel[s] = bn[s] > 0.0 ? rn[s] / bn[s] : 0.0;
-    if (u_done && sigma_used) {
-      RBS_TRY(apply_operator(c, RBS_OP_S, RBS_PREC_MIXED, sigma, w));
-      c.stats.launches++;
-      k_axpby<<<nbk, 256, 0, c.stream>>>(u, 1.0, w, 1.0, n3);
-    }
   }
   // 3. u = S[rho + mu] (already formed by the mixed path's float64-class passes) and the rigid velocities
   if (!u_done) {

@@ -16,8 +16,8 @@
 // Layout: one source array holds the N nodes followed by the proxy points of every accepted cell
 // (float32: hi + lo positions and weighted density; double-float: three-float positions and float32
 // pairs of weighted density, with float64 cluster charges); each target particle has a list of
-// (first, count) segments into it: its own particle first (masked by particle id), then the directly
-// evaluated particles, then its accepted cells.  Work items pair the targets of one particle (or a
+// (first, count) segments into it: its own particle first (masked by particle id), then the particles near
+// it, then the other directly evaluated ones, then its accepted cells.  Work items pair the targets of one particle (or a
 // near-equal part of it, at most 512) with a run of those segments.  The host plan (plan_treecode)
 // does no device work, so it also serves the host-only entry point rbs_treecode_plan.
 #include <algorithm>
@@ -351,7 +351,8 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 // copies.
 //
 // A unit with at most 16 targets gives its two half-warps alternate halves of the sources.  KIND 0 traction,
-// 1 Stokeslet into y; 2 traction into y and Stokeslet into y2 (26 and 17 operations a pair, one target per lane).
+// 1 Stokeslet into y; 2 traction into y and Stokeslet into y2 (26 and 17 operations a pair, one target per lane),
+// without the leading nskip segments (the own particle and its near ones).
 //
 // Bound by the float32 pipe, 76% busy.  With every source in one tile loop and blocks of whole particles, and
 // now: 1,150 to 1,770 Gpair/s on 1,500 particles of 144 nodes, 1,350 to 1,820 on 700 of 312.
@@ -419,8 +420,8 @@ __global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 
     float sb[3] = {0.0f, 0.0f, 0.0f}, eb[3] = {0.0f, 0.0f, 0.0f};  // KIND 2: the Stokeslet sums
 #pragma unroll
     for (int u = 0; u < NT; ++u) sa[u][0] = sa[u][1] = sa[u][2] = ea[u][0] = ea[u][1] = ea[u][2] = 0.0f;
-    int seg = w.s0, off = 0, done = 0;
-    int2 sg = segs[seg];
+    int seg = w.s0 + (KIND == 2 ? w.nskip : 0), off = 0, done = 0;
+    int2 sg = seg < w.s1 ? segs[seg] : make_int2(0, 0);
     // nodes
     while (seg < w.s1 && sg.x < N) {
       // the source of each of this lane's slots (lane + 32 k) from a walk over consecutive segments
@@ -481,10 +482,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 
   } while (0)
       if constexpr (KIND == 2) {
         float2 p2[3] = {f2(0.0f, 0.0f), f2(0.0f, 0.0f), f2(0.0f, 0.0f)};
-        if (done < w.nmask)
-          pair_tile32_both<true, TW>(ssx, spid, l0, cnt, xt[0], nt[0], pt[0], p[0], p2);
-        else
-          pair_tile32_both<false, TW>(ssx, spid, l0, cnt, xt[0], nt[0], pt[0], p[0], p2);
+        pair_tile32_both<TW>(ssx, l0, cnt, xt[0], nt[0], p[0], p2);
 #pragma unroll
         for (int c = 0; c < 3; ++c) two_sum_acc(sb[c], eb[c], p2[c].x + p2[c].y);
       } else if (nu == NT) {
@@ -961,17 +959,7 @@ void TreeState::release() {
   d_cheb64.release();
   d_q64.release();
   df = false;
-  direct_pairs = proxy_pairs = charge_work = 0;
-}
-
-double f32_operator_error(const Context& c) {
-  constexpr double kF32OperatorError = 1e-5;  // float32 rounding of one apply (measured: a few 1e-7)
-  if (!c.tree.active) return kF32OperatorError;
-  // empirical model of the treecode's relative error: C(theta) rho^-n with rho the Bernstein ellipse
-  // parameter 1/theta + sqrt(1/theta^2 - 1) and C = 0.25 max(1, (theta / 0.5)^2)
-  const double th = c.tree.theta, a = 1.0 / th;
-  const double C = 0.25 * std::max(1.0, (th / 0.5) * (th / 0.5));
-  return kF32OperatorError + C * std::pow(a + std::sqrt(a * a - 1.0), -c.tree.degree);
+  direct_pairs = proxy_pairs = charge_work = lead_pairs = near_listed = 0;
 }
 
 Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) {
@@ -997,6 +985,8 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
   const long long N = c.offset[n];
   std::vector<std::vector<int2>> seg_of(n);
   std::vector<long long> proxy_src(n, 0);
+  std::vector<int> lead(n, 1);  // leading segments: the own particle and its near ones
+  T.near_listed = T.lead_pairs = 0;
   int n_used = 0;
   std::vector<int> used_cells;
   std::vector<int> stack;
@@ -1005,7 +995,7 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
     std::vector<int2>& L = seg_of[i];
     const int np_i = (int)(c.offset[i + 1] - c.offset[i]);
     L.push_back(make_int2((int)c.offset[i], np_i));
-    std::vector<int> approx;
+    std::vector<int> approx, direct;
     stack.clear();
     stack.push_back(root_of[i]);
     while (!stack.empty()) {
@@ -1020,12 +1010,17 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
       } else if (C.nkid > 0) {
         for (int k = C.nkid - 1; k >= 0; --k) stack.push_back(C.kid[k]);
       } else {
-        for (int q = C.pb; q < C.pe; ++q) {
-          const int j = order[q];
-          if (j != i) L.push_back(make_int2((int)c.offset[j], (int)(c.offset[j + 1] - c.offset[j])));
-        }
+        for (int q = C.pb; q < C.pe; ++q)
+          if (order[q] != i) direct.push_back(order[q]);
       }
     }
+    const auto far = std::stable_partition(direct.begin(), direct.end(), [&](int j) {
+      return near_particles(c.centres, c.radius, i, j, c.near_delta);
+    });
+    lead[i] += (int)(far - direct.begin());
+    T.near_listed += far - direct.begin();
+    for (int j : direct) L.push_back(make_int2((int)c.offset[j], (int)(c.offset[j + 1] - c.offset[j])));
+    for (int k = 0; k < lead[i]; ++k) T.lead_pairs += (long long)np_i * L[k].y;
     for (int id : approx) {
       if (cells[id].used < 0) {
         cells[id].used = n_used++;
@@ -1111,6 +1106,7 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
         it.s0 = base + cut[r];
         it.s1 = base + cut[r + 1];
         it.nmask = r == 0 ? np_i : 0;
+        it.nskip = std::max(0, std::min(cut[r + 1], lead[i]) - cut[r]);
         T.items.push_back(it);
       }
     }
@@ -1187,6 +1183,8 @@ static Status build_lists(Context& c, TreeState& T, const std::vector<double>& p
   T.direct_pairs = P.direct_pairs;
   T.proxy_pairs = P.proxy_pairs;
   T.charge_work = P.charge_work;
+  T.lead_pairs = P.lead_pairs;
+  T.near_listed = P.near_listed;
   T.items.swap(P.items);
   T.segs.swap(P.segs);
   T.charge_items.swap(P.charge_items);
@@ -1387,7 +1385,7 @@ Status apply_tree_df_f32(Context& c, const double* x, double* y, double* y2) {
     case 6: RBS_TRY((launch_tree<2, 1, 6>(c, T, y, y2))); break;
     default: RBS_TRY((launch_tree<2, 1, 7>(c, T, y, y2)));
   }
-  timer.done(2.0 * (double)(T.direct_pairs + T.proxy_pairs));
+  timer.done(2.0 * (double)(T.direct_pairs - T.lead_pairs + T.proxy_pairs));
   return Status::Ok();
 }
 
