@@ -191,8 +191,7 @@ struct TreeState {
   DevBuf<float> d_pq;
   DevBuf<double> d_q64;
   long long direct_pairs = 0, proxy_pairs = 0, charge_work = 0;
-  // node pairs of the leading segments (the own particle and its near ones), and how many near pairs these hold
-  long long lead_pairs = 0, near_listed = 0;
+  long long lead_pairs = 0;  // node pairs of the leading segments (the own particle and its near ones)
   void release();
 };
 
@@ -481,7 +480,7 @@ struct TreePlan {
   std::vector<double> box, proxy;
   int n_cells = 0, tmax = 0;
   long long n_src = 0, direct_pairs = 0, proxy_pairs = 0, charge_work = 0;
-  long long lead_pairs = 0, near_listed = 0;  // as in TreeState
+  long long lead_pairs = 0;  // as in TreeState
 };
 // Host only: no device work (also usable without a GPU).
 Status plan_treecode(const PlanInput& in, double theta, int degree, TreePlan& plan);

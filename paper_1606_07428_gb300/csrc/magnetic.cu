@@ -152,8 +152,8 @@ __global__ void k_weight_df1(long long N, const double4* __restrict__ x, const d
 // operations (K^L) or 71 (S^L), 9 fewer where the tile is on a grid.  Bound by the float32 pipe: the forces on 216
 // particles of 144 nodes went from 49.4 to 27.4 ms with these sums and the near corrections below.
 template <int KIND, int MODE>
-__device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const int* spid, int l0, int l1,
-                                               const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2& acc) {
+__device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const int* smask, int l0, int l1,
+                                               const df2 (&xt)[3], const df2 (&nt)[3], int bit, df2& acc) {
 #pragma unroll 2
   for (int l = l0; l < l1; l += 2) {
     df2 d[3];
@@ -164,9 +164,9 @@ __device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const
     }
     const df2 q = {*reinterpret_cast<const float2*>(&sa[6][l]), *reinterpret_cast<const float2*>(&sa[7][l])};
     int2 pp = make_int2(0, 0);
-    if (MODE == kDfMask) pp = *reinterpret_cast<const int2*>(&spid[l]);
+    if (MODE == kDfMask) pp = *reinterpret_cast<const int2*>(&smask[l]);
     float2 R;
-    const inv_powers p = df_inv_powers<MODE>(d, pp, pt, R);
+    const inv_powers p = df_inv_powers<MODE>(d, pp, bit, R);
     if (KIND == 0) {
       const float2 r = __fmul2_rn(R, p.y0);
       const df2 rn = bdot2(d[0], nt[0], d[1], nt[1], d[2], nt[2], __fmul2_rn(r, dup2(kBiasFactor)));
@@ -181,14 +181,16 @@ __device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const
 
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_lap_df(int nunits, int* __restrict__ counter,
-                                                   const longlong4* __restrict__ work,
+                                                   const longlong4* __restrict__ work, DfSkip skip,
                                                    const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                                    const float4* __restrict__ x3l, const float4* __restrict__ nh,
                                                    const float4* __restrict__ nl, const float2* __restrict__ wq,
                                                    double scale, double* __restrict__ y) {
   __shared__ __align__(16) float tiles[4][9][kTileDf];
+  __shared__ int skips[4][kDfSkipInts];
+  int* const sk = skips[threadIdx.x >> 5];
   float(*sa)[kTileDf] = tiles[threadIdx.x >> 5];
-  int* const spid = reinterpret_cast<int*>(&sa[8][0]);
+  int* const smask = reinterpret_cast<int*>(&sa[8][0]);
   const int lane = threadIdx.x & 31;
   while (true) {
     int unit = 0;
@@ -205,32 +207,32 @@ __global__ void __launch_bounds__(128, 4) k_lap_df(int nunits, int* __restrict__
     const float4 oh = x3h[t0], om = x3m[t0], ol = x3l[t0], zero = make_float4(0, 0, 0, 0);
     const float4 ah = valid ? x3h[t] : oh, am = valid ? x3m[t] : om, al = valid ? x3l[t] : ol;
     const float4 bh = valid ? nh[t] : zero, bl = valid ? nl[t] : zero;
-    const int pt = valid ? __float_as_int(ah.w) : -1;
+    df_skip_targets(skip, __float_as_int(oh.w), __float_as_int(x3h[min(t0 + 32, t1) - 1].w), sk);
+    const int bit = valid ? 1 << (__float_as_int(ah.w) - __float_as_int(oh.w)) : 0;
     const dflt x0[3] = {df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x), df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y),
                         df_diff3(ah.z, am.z, al.z, oh.z, om.z, ol.z)};
     const df2 nt[3] = {{dup2(bh.x), dup2(bl.x)}, {dup2(bh.y), dup2(bl.y)}, {dup2(bh.z), dup2(bl.z)}};
     const float xm = warp_max_abs(fmaxf(fabsf(x0[0].h), fmaxf(fabsf(x0[1].h), fabsf(x0[2].h))));
-    const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(x3h[min(t0 + 32, t1) - 1].w);
     dflt a = {0.0f, 0.0f};
     for (int s0 = (int)w.z; s0 < (int)w.w; s0 += kTileDf) {
       const int cnt = min(kTileDf, (int)w.w - s0), cnt4 = (cnt + 3) & ~3;
       const int sidx[2] = {s0 + lane, s0 + lane + 32};
       const int tlo = __float_as_int(x3h[s0].w), thi = __float_as_int(x3h[s0 + cnt - 1].w);
-      const bool masked = !(thi < pid_lo || tlo > pid_hi);
-      df2 xt[3];
-      const bool grid = df_stage(sa, spid, sidx, cnt, masked, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
+      const int m = split ? cnt4 / 2 : cnt4, l0 = half * m;
+      auto stage_q = [&](int l, int s) {
         const float2 q = s >= 0 ? wq[s] : make_float2(0.0f, 0.0f);
         sa[6][l] = q.x;
         sa[7][l] = q.y;
-      });
-      df2 acc = {dup2(0.0f), dup2(0.0f)};
-      const int m = split ? cnt4 / 2 : cnt4, l0 = half * m;
-      if (masked)
-        lap_tile_pairs<KIND, kDfMask>(sa, spid, l0, l0 + m, xt, nt, pt, acc);
-      else if (grid)
-        lap_tile_pairs<KIND, kDfGrid>(sa, spid, l0, l0 + m, xt, nt, pt, acc);
-      else
-        lap_tile_pairs<KIND, kDfPlain>(sa, spid, l0, l0 + m, xt, nt, pt, acc);
+      };
+      df2 xt[3], acc = {dup2(0.0f), dup2(0.0f)};
+      if (df_skip_any(sk, tlo, thi)) {
+        if (df_stage<true>(sa, smask, sidx, cnt, skip, sk, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, stage_q) == kDfNone) continue;
+        lap_tile_pairs<KIND, kDfMask>(sa, smask, l0, l0 + m, xt, nt, bit, acc);
+      } else if (df_stage<false>(sa, smask, sidx, cnt, skip, sk, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, stage_q) == kDfGrid) {
+        lap_tile_pairs<KIND, kDfGrid>(sa, smask, l0, l0 + m, xt, nt, bit, acc);
+      } else {
+        lap_tile_pairs<KIND, kDfPlain>(sa, smask, l0, l0 + m, xt, nt, bit, acc);
+      }
       a = df_add_accurate(a, fold2(acc));
     }
     if (valid) atomicAdd(y + t, (KIND == 0 ? -scale : scale) * kInv4Pi * ((double)a.h + (double)a.l));
@@ -259,21 +261,20 @@ __global__ void k_lap_upsample(int n_up, const int* __restrict__ up_particle, co
   }
 }
 
-// Near correction by the units of near.cuh: for targets of i, the upsampled contribution of j is added and the
-// smooth-rule one removed, both in the double-float arithmetic of the smooth sum, so that what is removed
-// is what was added (float64 here took 1.7 ms a launch on 454 pairs of 144-node particles, bound by the
-// float64 pipe, and left the smooth sum's rounding uncancelled).
+// Near correction by the units of near.cuh: for targets of i, the upsampled contribution of j (the smooth sum
+// leaves near sources out) in the double-float arithmetic of the smooth sum (float64 here took 1.7 ms a launch
+// on 454 pairs of 144-node particles with the base nodes, bound by the float64 pipe).
 template <int KIND>
 __global__ void __launch_bounds__(128, 5) k_lap_near(NearArgs A, const float4* __restrict__ x3h,
                                                      const float4* __restrict__ x3m, const float4* __restrict__ x3l,
                                                      const float4* __restrict__ nh, const float4* __restrict__ nl,
-                                                     const float2* __restrict__ wq, const float4* __restrict__ up3h,
+                                                     const float4* __restrict__ up3h,
                                                      const float4* __restrict__ up3m, const float4* __restrict__ up3l,
                                                      const float2* __restrict__ upq, double scale,
                                                      double* __restrict__ y) {
   __shared__ __align__(16) float tiles[4][9][kTileDf];
   float(*sa)[kTileDf] = tiles[threadIdx.x >> 5];
-  int* const spid = reinterpret_cast<int*>(&sa[8][0]);
+  int* const smask = reinterpret_cast<int*>(&sa[8][0]);
   const int lane = threadIdx.x & 31;
   NearUnit n;
   while (next_near_unit(A, n)) {
@@ -290,30 +291,22 @@ __global__ void __launch_bounds__(128, 5) k_lap_near(NearArgs A, const float4* _
     const df2 nt[3] = {{dup2(bh.x), dup2(bl.x)}, {dup2(bh.y), dup2(bl.y)}, {dup2(bh.z), dup2(bl.z)}};
     const float xm = warp_max_abs(fmaxf(fabsf(x0[0].h), fmaxf(fabsf(x0[1].h), fabsf(x0[2].h))));
     dflt a = {0.0f, 0.0f};
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {  // upsampled nodes, then base nodes with the opposite sign
-      const int b = pass == 0 ? n.s0 : max(n.s0, n.nup), e = pass == 0 ? min(n.s1, n.nup) : n.s1;
-      const long long g0 = pass == 0 ? n.ub : n.oj - n.nup;
-      const float2* qs = pass == 0 ? upq : wq;
-      const float sign = pass == 0 ? 1.0f : -1.0f;
-      for (int sb = b; sb < e; sb += kTileDf) {
-        const int cnt = min(kTileDf, e - sb), cnt4 = (cnt + 3) & ~3;
-        const int sidx[2] = {(int)(g0 + sb) + lane, (int)(g0 + sb) + lane + 32};
-        df2 xt[3];
-        const bool grid = df_stage(sa, spid, sidx, cnt, false, pass == 0 ? up3h : x3h, pass == 0 ? up3m : x3m,
-                                   pass == 0 ? up3l : x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
-                                     const float2 q = s >= 0 ? qs[s] : make_float2(0.0f, 0.0f);
-                                     sa[6][l] = sign * q.x;
-                                     sa[7][l] = sign * q.y;
-                                   });
-        df2 acc = {dup2(0.0f), dup2(0.0f)};
-        const int m = split ? cnt4 / 2 : cnt4, l0 = half * m;
-        if (grid)
-          lap_tile_pairs<KIND, kDfGrid>(sa, spid, l0, l0 + m, xt, nt, -1, acc);
-        else
-          lap_tile_pairs<KIND, kDfPlain>(sa, spid, l0, l0 + m, xt, nt, -1, acc);
-        a = df_add_accurate(a, fold2(acc));
-      }
+    for (int sb = n.s0; sb < n.s1; sb += kTileDf) {
+      const int cnt = min(kTileDf, n.s1 - sb), cnt4 = (cnt + 3) & ~3;
+      const int sidx[2] = {(int)(n.ub + sb) + lane, (int)(n.ub + sb) + lane + 32};
+      df2 xt[3];
+      const DfMode mode = df_stage<false>(sa, smask, sidx, cnt, DfSkip{}, nullptr, up3h, up3m, up3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
+        const float2 q = s >= 0 ? upq[s] : make_float2(0.0f, 0.0f);
+        sa[6][l] = q.x;
+        sa[7][l] = q.y;
+      });
+      df2 acc = {dup2(0.0f), dup2(0.0f)};
+      const int m = split ? cnt4 / 2 : cnt4, l0 = half * m;
+      if (mode == kDfGrid)
+        lap_tile_pairs<KIND, kDfGrid>(sa, smask, l0, l0 + m, xt, nt, 0, acc);
+      else
+        lap_tile_pairs<KIND, kDfPlain>(sa, smask, l0, l0 + m, xt, nt, 0, acc);
+      a = df_add_accurate(a, fold2(acc));
     }
     if (valid) atomicAdd(y + t, (KIND == 0 ? -scale : scale) * kInv4Pi * ((double)a.h + (double)a.l));
   }
@@ -600,7 +593,7 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
     RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, 2 * sizeof(int), s));
     const int grid = std::min(nw, 4 * std::max(1, c.sm_count));
 #define RBS_LAP_ARGS \
-  4 * nw, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
+  4 * nw, c.d_unit.ptr, c.d_work.ptr, DfSkip{c.d_near_first.ptr, c.d_near.ptr}, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
     if (kind == 0)
       k_lap_df<0><<<grid, 128, 0, s>>>(RBS_LAP_ARGS);
     else
@@ -619,11 +612,11 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
                                      M.d_upU.ptr, x, c.d_up_x.ptr, M.d_qup.ptr);
     NearArgs A;
     int blocks = 0;
-    RBS_TRY(near_args(c, true, A, blocks));
+    RBS_TRY(near_args(c, false, A, blocks));
     blocks = std::min(blocks, 5 * std::max(1, c.sm_count));
 #define RBS_LAP_NEAR                                                                                              \
-  A, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, c.d_up3h.ptr, c.d_up3m.ptr, \
-      c.d_up3l.ptr, M.d_qup.ptr, scale, y
+  A, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, c.d_up3h.ptr, c.d_up3m.ptr, c.d_up3l.ptr, \
+      M.d_qup.ptr, scale, y
     if (kind == 0)
       k_lap_near<0><<<blocks, 128, 0, s>>>(RBS_LAP_NEAR);
     else

@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(128, 5)
                  const long long* __restrict__ offset, const int* __restrict__ near_first, const int2* __restrict__ near,
                  const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
                  const float4* __restrict__ wmu, double* __restrict__ y, double* __restrict__ y2) {
-  constexpr int TW = 128, SL = TW / 32;
+  constexpr int TW = 128, SL = 4;
   __shared__ __align__(16) float tiles[4][6 * TW];
   const int lane = threadIdx.x & 31;
   float* const ssx = tiles[threadIdx.x >> 5];
@@ -786,6 +786,7 @@ __global__ void __launch_bounds__(128, 5)
           for (int q = 0; q < SL; ++q)
             if (__float_as_int(ph[q].w) == j) out[q] = true;
         }
+        if (__all_sync(0xffffffffu, out[0] && out[1] && out[2] && out[3])) continue;
         __syncwarp();  // the warp's reads of the previous tile are done
 #pragma unroll
         for (int q = 0; q < SL; ++q) {
@@ -848,13 +849,15 @@ __global__ void k_weight_df(long long N, const double4* __restrict__ x, const do
 // against two-sum arithmetic throughout in blocks of whole items.
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restrict__ counter,
-                                                      const longlong4* __restrict__ work,
+                                                      const longlong4* __restrict__ work, DfSkip skip,
                                                       const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                                       const float4* __restrict__ x3l, const float4* __restrict__ nh,
                                                       const float4* __restrict__ nl, const float4* __restrict__ wh,
                                                       const float4* __restrict__ wl, double* __restrict__ y,
                                                       double* __restrict__ y2) {
   __shared__ __align__(16) float tiles[4 * kTileDfFloats];
+  __shared__ int skips[4][kDfSkipInts];
+  int* const sk = skips[threadIdx.x >> 5];
   float* const wsm = tiles + (threadIdx.x >> 5) * kTileDfFloats;
   const int lane = threadIdx.x & 31;
   while (true) {
@@ -871,7 +874,9 @@ __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restric
     const bool valid = t < t1;
     const float4 oh = x3h[t0], om = x3m[t0], ol = x3l[t0];
     dflt xt[3], nt[3], a[3], a2[3];
-    int pt = -1;
+    const int pid0 = __float_as_int(oh.w);
+    int bit = 0;
+    df_skip_targets(skip, pid0, __float_as_int(x3h[min(t0 + 32, t1) - 1].w), sk);
     {
       float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
       if (valid) {
@@ -880,7 +885,7 @@ __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restric
         al = x3l[t];
         bh = nh[t];
         bl = nl[t];
-        pt = __float_as_int(ah.w);
+        bit = 1 << (__float_as_int(ah.w) - pid0);
       }
       xt[0] = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x);
       xt[1] = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y);
@@ -892,13 +897,16 @@ __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restric
     const float xm = warp_max_abs(fmaxf(fabsf(xt[0].h), fmaxf(fabsf(xt[1].h), fabsf(xt[2].h))));
 #pragma unroll
     for (int c = 0; c < 3; ++c) a[c] = a2[c] = dflt{0.0f, 0.0f};
-    const int pid_lo = __float_as_int(oh.w), pid_hi = __float_as_int(x3h[min(t0 + 32, t1) - 1].w);
     for (int s0 = (int)w.z; s0 < (int)w.w; s0 += kTileDf) {
       const int cnt = min(kTileDf, (int)w.w - s0);
       const int sidx[2] = {s0 + lane, s0 + lane + 32};
       const int tlo = __float_as_int(x3h[s0].w), thi = __float_as_int(x3h[s0 + cnt - 1].w);
-      df_tile<KIND>(wsm, sidx, cnt, !(thi < pid_lo || tlo > pid_hi), split, half, x3h, x3m, x3l, wh, wl, oh, om, ol, xt,
-                    nt, xm, pt, a, a2);
+      if (df_skip_any(sk, tlo, thi))
+        df_tile<KIND, true>(wsm, sidx, cnt, skip, sk, split, half, x3h, x3m, x3l, wh, wl, oh, om, ol, xt, nt, xm, bit, a,
+                            a2);
+      else
+        df_tile<KIND, false>(wsm, sidx, cnt, skip, sk, split, half, x3h, x3m, x3l, wh, wl, oh, om, ol, xt, nt, xm, bit, a,
+                             a2);
     }
     const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
     if (valid) {
@@ -1072,13 +1080,12 @@ __global__ void __launch_bounds__(128, 6) k_near32(NearArgs A, const float4* __r
   }
 }
 
-// Double-float: the arithmetic of the smooth sums (df_tile), whose base terms it removes to about 1e-13 of each;
-// KIND 2 both kernels in one pass.
+// Double-float, upsampled nodes alone (df_tile: the smooth sums leave near sources out); KIND 2 both kernels in one
+// pass.
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_near_df(NearArgs A, const float4* __restrict__ x3h,
                                                     const float4* __restrict__ x3m, const float4* __restrict__ x3l,
                                                     const float4* __restrict__ nh, const float4* __restrict__ nl,
-                                                    const float4* __restrict__ wh, const float4* __restrict__ wl,
                                                     const float4* __restrict__ up3h, const float4* __restrict__ up3m,
                                                     const float4* __restrict__ up3l, const float4* __restrict__ upqh,
                                                     const float4* __restrict__ upql, double* __restrict__ y,
@@ -1109,16 +1116,10 @@ __global__ void __launch_bounds__(128, 4) k_near_df(NearArgs A, const float4* __
     const float xm = warp_max_abs(fmaxf(fabsf(xt[0].h), fmaxf(fabsf(xt[1].h), fabsf(xt[2].h))));
 #pragma unroll
     for (int c = 0; c < 3; ++c) a[c] = a2[c] = dflt{0.0f, 0.0f};
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {  // upsampled nodes, then base nodes with the opposite sign
-      const int b = pass == 0 ? n.s0 : max(n.s0, n.nup), e = pass == 0 ? min(n.s1, n.nup) : n.s1;
-      const long long g0 = pass == 0 ? n.ub : n.oj - n.nup;
-      for (int sb = b; sb < e; sb += kTileDf) {
-        const int sidx[2] = {(int)(g0 + sb) + lane, (int)(g0 + sb) + lane + 32};
-        df_tile<KIND>(wsm, sidx, min(kTileDf, e - sb), false, split, half, pass == 0 ? up3h : x3h,
-                      pass == 0 ? up3m : x3m, pass == 0 ? up3l : x3l, pass == 0 ? upqh : wh, pass == 0 ? upql : wl, oh,
-                      om, ol, xt, nt, xm, -1, a, a2, pass == 0 ? 1.0f : -1.0f);
-      }
+    for (int sb = n.s0; sb < n.s1; sb += kTileDf) {
+      const int sidx[2] = {(int)(n.ub + sb) + lane, (int)(n.ub + sb) + lane + 32};
+      df_tile<KIND, false>(wsm, sidx, min(kTileDf, n.s1 - sb), DfSkip{}, nullptr, split, half, up3h, up3m, up3l, upqh, upql, oh, om, ol, xt, nt,
+                    xm, 0, a, a2);
     }
     if (valid) {
       const double sc = KIND == 1 ? kStokesletScale : kTractionScale;
@@ -1256,7 +1257,7 @@ template <int KIND>
 static void launch_pairs_df(Context& c, double* y, double* y2) {
   const int items = (int)c.work.size();
   k_pairs_df2<KIND><<<resident_grid(c, (const void*)k_pairs_df2<KIND>, 128, items), 128, 0, c.stream>>>(
-      4 * items, c.d_unit.ptr, c.d_work.ptr, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
+      4 * items, c.d_unit.ptr, c.d_work.ptr, DfSkip{c.d_near_first.ptr, c.d_near.ptr}, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
       c.d_wmuh.ptr, c.d_wmul.ptr, y, y2);
 }
 
@@ -1400,18 +1401,23 @@ static Status near_upsample(Context& c, int prec, const double* x) {
   return Status::Ok();
 }
 
-// Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one (base false: the
+// Node pairs of one near correction.
+static double near_units(const Context& c, int prec) {
+  return prec == RBS_PREC_DF ? c.near_pair_nodes - c.near_base_nodes : c.near_pair_nodes;
+}
+
+// Near correction, step 2: for every near pair, the base-grid term is replaced by the upsampled one (double-float: the
 // upsampled one is added); kind 0 traction into y, 1 Stokeslet into y, 2 (double-float only) traction into y and
 // Stokeslet into y2.
-static Status near_sums(Context& c, int kind, int prec, const double* x, double* y, double* y2, bool base = true) {
+static Status near_sums(Context& c, int kind, int prec, const double* x, double* y, double* y2) {
   NearArgs A;
   int blocks = 0;
-  RBS_TRY(near_args(c, base, A, blocks));
+  RBS_TRY(near_args(c, prec != RBS_PREC_DF, A, blocks));
   if (prec == RBS_PREC_FP64) RBS_CUDA_TRY(cudaMemsetAsync(A.counter, 0, sizeof(int), c.stream));
 #define RBS_NEAR_LAUNCH(KERNEL, ...) \
   KERNEL<<<resident_grid(c, (const void*)KERNEL, 128, blocks), 128, 0, c.stream>>>(A, __VA_ARGS__)
   if (prec == RBS_PREC_DF) {
-#define RBS_NEAR_DF c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, c.d_wmuh.ptr, c.d_wmul.ptr, \
+#define RBS_NEAR_DF c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, \
                     c.d_up3h.ptr, c.d_up3m.ptr, c.d_up3l.ptr, c.d_up_qh.ptr, c.d_up_ql.ptr, y, y2
     if (kind == 0)
       RBS_NEAR_LAUNCH(k_near_df<0>, RBS_NEAR_DF);
@@ -1466,7 +1472,7 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     c.stream = main;
     c.stats.launches += 2;
     c.stats.kernel_count[RBS_KC_NEAR] += 2;
-    c.stats.kernel_units[RBS_KC_NEAR] += (double)c.near_pair_nodes;
+    c.stats.kernel_units[RBS_KC_NEAR] += near_units(c, prec);
     RBS_CUDA_TRY(cudaEventRecord(c.join_ev, c.side));
     if (!st.ok()) {
       cudaStreamWaitEvent(c.stream, c.join_ev, 0);
@@ -1483,7 +1489,7 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     if (prec == RBS_PREC_DF) cls = kind == 0 ? RBS_KC_PAIR_KDF : RBS_KC_PAIR_SDF;
     KernelTimer timer(c, cls);
     st = launch_pairs(c, kind, prec, x, y);
-    timer.done((double)c.stats.far_pairs);
+    timer.done((double)c.stats.far_pairs - (prec == RBS_PREC_DF ? c.near_base_nodes : 0.0));
   }
   if (beside) RBS_CUDA_TRY(cudaStreamWaitEvent(c.stream, c.join_ev, 0));  // (also when the smooth sum failed)
   RBS_TRY(st);
@@ -1491,7 +1497,7 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     KernelTimer timer(c, RBS_KC_NEAR);
     RBS_TRY(near_upsample(c, prec, x));
     RBS_TRY(near_sums(c, kind, prec, x, y, nullptr));
-    timer.done((double)c.near_pair_nodes, 2);
+    timer.done(near_units(c, prec), 2);
   }
   return Status::Ok();
 }
@@ -1512,7 +1518,7 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
     if (prec == RBS_PREC_DF) {
       KernelTimer timer(c, RBS_KC_PAIR_KSDF);
       RBS_TRY(launch_pairs(c, 2, prec, x, yK, yS));
-      timer.done((double)c.stats.far_pairs);
+      timer.done((double)c.stats.far_pairs - c.near_base_nodes);
     } else {
       {
         KernelTimer timer(c, RBS_KC_PAIR_K64);
@@ -1529,11 +1535,11 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
     RBS_TRY(near_upsample(c, prec, x));
     if (prec == RBS_PREC_DF) {
       RBS_TRY(near_sums(c, 2, prec, x, yK, yS));
-      timer.done(2.0 * c.near_pair_nodes, 2);
+      timer.done(2.0 * near_units(c, prec), 2);
     } else {
       RBS_TRY(near_sums(c, 0, prec, x, yK, nullptr));
       RBS_TRY(near_sums(c, 1, prec, x, yS, nullptr));
-      timer.done(2.0 * c.near_pair_nodes, 3);
+      timer.done(2.0 * near_units(c, prec), 3);
     }
   }
   return Status::Ok();
@@ -1559,8 +1565,8 @@ Status apply_correction(Context& c, const double* d, double* w, double* v) {
   if (!c.near_pairs.empty()) {
     KernelTimer timer(c, RBS_KC_NEAR);
     RBS_TRY(near_upsample(c, RBS_PREC_DF, d));
-    RBS_TRY(near_sums(c, 2, RBS_PREC_DF, d, w, v, false));
-    timer.done(2.0 * (c.near_pair_nodes - c.near_base_nodes), 2);
+    RBS_TRY(near_sums(c, 2, RBS_PREC_DF, d, w, v));
+    timer.done(2.0 * near_units(c, RBS_PREC_DF), 2);
   }
   return Status::Ok();
 }

@@ -2,6 +2,8 @@
 // (treecode.cu).
 #pragma once
 
+#include <climits>
+
 #include "common.cuh"
 #include "dfloat.cuh"
 
@@ -84,9 +86,9 @@ struct inv_powers {
   __device__ __forceinline__ df2 inv() const { return {y0, __fmul2_rn(y0, series(-0.5f, 0.375f))}; }
 };
 
-// How a tile forms separations: by two-sums, the same with the target's own particle masked by its id,
-// or on a common grid (df_tile).
-enum DfMode { kDfPlain = 0, kDfMask = 1, kDfGrid = 2 };
+// How a tile forms separations: by two-sums, the same with sources masked per target particle (DfSkip), or on a
+// common grid (df_tile); kDfNone: every source of the tile is left out for every target.
+enum DfMode { kDfPlain = 0, kDfMask = 1, kDfGrid = 2, kDfNone = 3 };
 
 // One component of the separation from the target's coordinate and the source's negated one.
 template <int MODE>
@@ -97,17 +99,17 @@ __device__ __forceinline__ df2 df_separation(df2 x, df2 y) {
   return d;
 }
 
-// Powers of 1 / r for the separation d, and R = r^2 in float32; MODE kDfMask zeroes them for sources of the
-// target's own particle.
+// Powers of 1 / r for the separation d, and R = r^2 in float32; MODE kDfMask zeroes them for the sources whose
+// mask holds the target's bit.
 template <int MODE>
-__device__ __forceinline__ inv_powers df_inv_powers(const df2 (&d)[3], int2 spid, int pt, float2& R) {
+__device__ __forceinline__ inv_powers df_inv_powers(const df2 (&d)[3], int2 mask, int bit, float2& R) {
   // r^2 by biased accumulation over 5/4 of its own float32 value R (over R itself the sum can round to
   // just above 2 R, where the difference from R is inexact)
   R = __ffma2_rn(d[2].h, d[2].h, __ffma2_rn(d[1].h, d[1].h, __fmul2_rn(d[0].h, d[0].h)));
   float2 y0 = make_float2(rsqrt_hw(R.x), rsqrt_hw(R.y));
-  if (MODE == kDfMask) {  // the target's own particle: every power of 1 / r becomes zero
-    if (spid.x == pt) y0.x = 0.0f;
-    if (spid.y == pt) y0.y = 0.0f;
+  if (MODE == kDfMask) {  // every power of 1 / r becomes zero
+    if (mask.x & bit) y0.x = 0.0f;
+    if (mask.y & bit) y0.y = 0.0f;
   }
   const float2 Rb = __fmul2_rn(dup2(1.25f), R);
   const float2 s0 = __ffma2_rn(d[0].h, d[0].h, Rb), s1 = __ffma2_rn(d[1].h, d[1].h, s0), s2 = __ffma2_rn(d[2].h, d[2].h, s1);
@@ -124,13 +126,13 @@ __device__ __forceinline__ inv_powers df_inv_powers(const df2 (&d)[3], int2 spid
 // Stokeslet into acc2; fb = kBiasFactor |density| of the sources.  With two-sums 221 float32 operations
 // for both kernels, 154 for the traction alone and 139 for the Stokeslet alone; 9 fewer on the grid.
 template <int KIND, int MODE>
-__device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], float2 fb, int2 spid,
-                                         const df2 (&xt)[3], const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
+__device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], float2 fb, int2 mask,
+                                         const df2 (&xt)[3], const df2 (&nt)[3], int bit, df2 (&acc)[3], df2 (&acc2)[3]) {
   df2 d[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) d[c] = df_separation<MODE>(xt[c], y[c]);
   float2 R;
-  const inv_powers p = df_inv_powers<MODE>(d, spid, pt, R);
+  const inv_powers p = df_inv_powers<MODE>(d, mask, bit, R);
   const float2 y0 = p.y0;
   const float2 r = __fmul2_rn(R, y0);
   const df2 rr = bdot2(d[0], den[0], d[1], den[1], d[2], den[2], __fmul2_rn(r, fb));
@@ -173,8 +175,38 @@ constexpr int kTileDfFloats = 14 * kTileDf;
 // two above the largest separation: differences of hi parts are exact without a two-sum, and the lo parts
 // (at most g / 2) keep the separation within a few times 2^-50 of itself.  Closer tiles take two-sums.
 // split: each half-warp holds the same 16 targets and takes its half of the tile.  xm = the
-// warp's largest target coordinate; sign (1 or -1) multiplies the densities; totals go to tot (and tot2
-// for KIND 2).
+// warp's largest target coordinate; totals go to tot (and tot2 for KIND 2).
+//
+// Sources on a target's own particle, and on the particles near it, are left out (the near corrections add the
+// latter's upsampled contribution).  Near terms grow as the inverse square of a gap, and what a sum adds
+// another one removes only to its own rounding of their separations: with a pair of spheres 0.003 apart a pass that
+// did so was 1.5e-9 of the right-hand side away from its residual.
+struct DfSkip {
+  const int* first;   // per particle, its first near pair
+  const int2* near;   // near pairs (target, source), by target
+};
+// The part of it that belongs to a warp's targets, in shared memory (the pair loops have no register to spare): one of
+// the first 32 near sources of particles lo and lo + 1 per lane (-1: none), lo and hi, and whether there are others.
+constexpr int kDfSkipInts = 68;
+__device__ __forceinline__ void df_skip_targets(const DfSkip& skip, int lo, int hi, int* sk) {
+  const int lane = threadIdx.x & 31;
+  const int e0 = skip.first[lo], n0 = skip.first[lo + 1], n1 = hi > lo ? skip.first[lo + 2] : n0;
+  __syncwarp();  // the previous unit's reads are done
+  sk[lane] = e0 + lane < n0 ? skip.near[e0 + lane].y : -1;
+  sk[32 + lane] = n0 + lane < n1 ? skip.near[n0 + lane].y : -1;
+  if (lane == 0) {
+    sk[64] = lo;
+    sk[65] = hi;  // a particle has 12 nodes at least: at most lo + 3
+    sk[66] = n0 - e0 > 32 || n1 - n0 > 32 || hi > lo + 1;
+  }
+  __syncwarp();
+}
+// Whether a tile of nodes of particles tlo to thi may hold a source to leave out.
+__device__ __forceinline__ bool df_skip_any(const int* sk, int tlo, int thi) {
+  const int a = sk[threadIdx.x & 31], b = sk[32 + (threadIdx.x & 31)];
+  return __any_sync(0xffffffffu, (a >= tlo && a <= thi) || (b >= tlo && b <= thi)) || (thi >= sk[64] && tlo <= sk[65]) ||
+         sk[66];
+}
 
 __device__ __forceinline__ float warp_max_abs(float v) {  // of non-negative values
   return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
@@ -185,8 +217,8 @@ __device__ __forceinline__ float warp_min_abs(float v) {
 }
 
 template <int KIND, int MODE>
-__device__ __forceinline__ void df_tile_pairs(const float (*sa)[kTileDf], const int* spid, int l0, int l1, const df2 (&xt)[3],
-                                              const df2 (&nt)[3], int pt, df2 (&acc)[3], df2 (&acc2)[3]) {
+__device__ __forceinline__ void df_tile_pairs(const float (*sa)[kTileDf], const int* smask, int l0, int l1, const df2 (&xt)[3],
+                                              const df2 (&nt)[3], int bit, df2 (&acc)[3], df2 (&acc2)[3]) {
 #pragma unroll 1
   for (int l = l0; l < l1; l += 2) {
     df2 ys[3], den[3];
@@ -197,17 +229,19 @@ __device__ __forceinline__ void df_tile_pairs(const float (*sa)[kTileDf], const 
     }
     const float2 fb = *reinterpret_cast<const float2*>(&sa[12][l]);
     int2 pp = make_int2(0, 0);
-    if (MODE == kDfMask) pp = *reinterpret_cast<const int2*>(&spid[l]);
-    pair2_df<KIND, MODE>(ys, den, fb, pp, xt, nt, pt, acc, acc2);
+    if (MODE == kDfMask) pp = *reinterpret_cast<const int2*>(&smask[l]);
+    pair2_df<KIND, MODE>(ys, den, fb, pp, xt, nt, bit, acc, acc2);
   }
 }
 
 // Stages the coordinates of a tile and the target's in the tile's form (xt); stage_q(l, s) stores what else
-// slot l needs of source s (s < 0: a padding slot, to be given zero density).  Returns whether the tile is
-// on a grid.
-template <typename StageQ>
-__device__ __forceinline__ bool df_stage(float (*sa)[kTileDf], int* spid, const int (&sidx)[2], int filled, bool masked,
-                                         const float4* __restrict__ x3h, const float4* __restrict__ x3m,
+// slot l needs of source s (s < 0: a padding slot, to be given zero density).  With SKIP, where df_skip_any says so
+// (sk: df_skip_targets' part), bit i - lo of a slot's mask in smask leaves it out for targets of particle i, and the mode
+// is kDfMask or kDfNone (grid and plain tiles, nearly all of them, carry none of this);
+// else kDfGrid or kDfPlain.
+template <bool SKIP, typename StageQ>
+__device__ __forceinline__ DfMode df_stage(float (*sa)[kTileDf], int* smask, const int (&sidx)[2], int filled, const DfSkip& skip,
+                                         const int* sk, const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                          const float4* __restrict__ x3l, const float4& oh, const float4& om,
                                          const float4& ol, const dflt (&x0)[3], float xm, df2 (&xt)[3], StageQ stage_q) {
   const int lane = threadIdx.x & 31;
@@ -229,9 +263,35 @@ __device__ __forceinline__ bool df_stage(float (*sa)[kTileDf], int* spid, const 
       mn = fminf(mn, far);
     }
   }
+  int mask[2] = {0, 0};
+  if constexpr (SKIP) {
+    const int lo = sk[64], hi = sk[65];
+    const int tlo = __reduce_min_sync(0xffffffffu, pid[0] < 0 ? INT_MAX : pid[0]);
+    const int thi = __reduce_max_sync(0xffffffffu, max(pid[0], pid[1]));
+    auto near_bit = [&](int j, int bit) {  // j: a near source per lane
+      for (unsigned hits = __ballot_sync(0xffffffffu, j >= tlo && j <= thi); hits; hits &= hits - 1) {
+        const int jj = __shfl_sync(0xffffffffu, j, __ffs(hits) - 1);
+        if (pid[0] == jj) mask[0] |= bit;
+        if (pid[1] == jj) mask[1] |= bit;
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (pid[k] >= lo && pid[k] <= hi) mask[k] = 1 << (pid[k] - lo);
+    near_bit(sk[lane], 1);
+    near_bit(sk[32 + lane], 2);
+    if (sk[66])
+      for (int i = lo; i <= hi; ++i) {
+        const int end = skip.first[i + 1];
+        for (int e = skip.first[i] + (i < lo + 2 ? 32 : 0); e < end; e += 32)
+          near_bit(e + lane < end ? skip.near[e + lane].y : -1, 1 << (i - lo));
+      }
+    const int all = (2 << (hi - lo)) - 1;
+    if (__all_sync(0xffffffffu, (pid[0] < 0 || mask[0] == all) && (pid[1] < 0 || mask[1] == all))) return kDfNone;
+  }
   m = warp_max_abs(m) + xm;
   // in the largest coordinate alone a source is at least mn - xm away
-  const bool grid = !masked && warp_min_abs(mn) - xm >= 0.25f * m;
+  const bool grid = !SKIP && warp_min_abs(mn) - xm >= 0.25f * m;
   // g = 2^(e - 24), 2^e > m; its exponent field is that of m less 23
   const int ge = max(1, (int)(__float_as_uint(m) >> 23) - 23);
   const float g = __uint_as_float((unsigned)ge << 23), ginv = __uint_as_float((unsigned)(254 - ge) << 23);
@@ -253,12 +313,12 @@ __device__ __forceinline__ bool df_stage(float (*sa)[kTileDf], int* spid, const 
         sa[2 * c + 1][l] = v.l;
       }
       stage_q(l, sidx[k]);
-      spid[l] = pid[k];
+      if (SKIP) smask[l] = mask[k];
     } else if (l < cnt4) {  // zero-density sources away from every target: they add exactly zero
       sa[0][l] = sa[2][l] = sa[4][l] = 8.0f * m;
       sa[1][l] = sa[3][l] = sa[5][l] = 0.0f;
       stage_q(l, -1);
-      spid[l] = -2;
+      if (SKIP) smask[l] = 0;
     }
   }
 #pragma unroll
@@ -267,46 +327,47 @@ __device__ __forceinline__ bool df_stage(float (*sa)[kTileDf], int* spid, const 
     xt[c] = {dup2(v.h), dup2(v.l)};
   }
   __syncwarp();
-  return grid;
+  return SKIP ? kDfMask : (grid ? kDfGrid : kDfPlain);
 }
 
-template <int KIND>
-__device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int filled, bool masked, bool split, int half,
-                                        const float4* __restrict__ x3h, const float4* __restrict__ x3m,
+template <int KIND, bool SKIP>
+__device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int filled, const DfSkip& skip, const int* sk, bool split,
+                                        int half, const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                         const float4* __restrict__ x3l, const float4* __restrict__ qh_,
                                         const float4* __restrict__ ql_, const float4& oh, const float4& om,
-                                        const float4& ol, const dflt (&x0)[3], const dflt (&n0)[3], float xm, int pt,
-                                        dflt (&tot)[3], dflt (&tot2)[3], float sign = 1.0f) {
+                                        const float4& ol, const dflt (&x0)[3], const dflt (&n0)[3], float xm, int bit,
+                                        dflt (&tot)[3], dflt (&tot2)[3]) {
   float(*sa)[kTileDf] = reinterpret_cast<float(*)[kTileDf]>(wsm);
-  int* const spid = reinterpret_cast<int*>(&sa[13][0]);
+  int* const smask = reinterpret_cast<int*>(&sa[13][0]);
   df2 xt[3], nt[3];
-  const bool grid = df_stage(sa, spid, sidx, filled, masked, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
+  const DfMode mode = df_stage<SKIP>(sa, smask, sidx, filled, skip, sk, x3h, x3m, x3l, oh, om, ol, x0, xm, xt, [&](int l, int s) {
     float4 qh = make_float4(0, 0, 0, 0), ql = qh;
     if (s >= 0) {
       qh = qh_[s];
       ql = ql_[s];
     }
-    sa[6][l] = sign * qh.x;
-    sa[7][l] = sign * ql.x;
-    sa[8][l] = sign * qh.y;
-    sa[9][l] = sign * ql.y;
-    sa[10][l] = sign * qh.z;
-    sa[11][l] = sign * ql.z;
+    sa[6][l] = qh.x;
+    sa[7][l] = ql.x;
+    sa[8][l] = qh.y;
+    sa[9][l] = ql.y;
+    sa[10][l] = qh.z;
+    sa[11][l] = ql.z;
     sa[12][l] = kBiasFactor * sqrtf(fmaf(qh.x, qh.x, fmaf(qh.y, qh.y, qh.z * qh.z)));
   });
 #pragma unroll
   for (int c = 0; c < 3; ++c) nt[c] = {dup2(n0[c].h), dup2(n0[c].l)};
+  if (mode == kDfNone) return;
   const int cnt4 = (filled + 3) & ~3;
   df2 acc[3], acc2[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) acc[c] = acc2[c] = df2{dup2(0.0f), dup2(0.0f)};
   const int cnt = split ? cnt4 / 2 : cnt4, l0 = half * cnt;
-  if (masked)
-    df_tile_pairs<KIND, kDfMask>(sa, spid, l0, l0 + cnt, xt, nt, pt, acc, acc2);
-  else if (grid)
-    df_tile_pairs<KIND, kDfGrid>(sa, spid, l0, l0 + cnt, xt, nt, pt, acc, acc2);
+  if constexpr (SKIP)
+    df_tile_pairs<KIND, kDfMask>(sa, smask, l0, l0 + cnt, xt, nt, bit, acc, acc2);
+  else if (mode == kDfGrid)
+    df_tile_pairs<KIND, kDfGrid>(sa, smask, l0, l0 + cnt, xt, nt, bit, acc, acc2);
   else
-    df_tile_pairs<KIND, kDfPlain>(sa, spid, l0, l0 + cnt, xt, nt, pt, acc, acc2);
+    df_tile_pairs<KIND, kDfPlain>(sa, smask, l0, l0 + cnt, xt, nt, bit, acc, acc2);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     tot[c] = df_add_accurate(tot[c], fold2(acc[c]));

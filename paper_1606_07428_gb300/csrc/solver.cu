@@ -175,9 +175,6 @@ static double correction_error(const Context& c) {
   double rmax = 0.0;
   for (const Shape& sh : c.shapes) rmax = std::max(rmax, sh.radius);
   if (!(c.opt.near_delta > 0.0)) return INFINITY;
-  // every near pair has to be among the directly evaluated ones of the tree (a cluster is accepted only beyond
-  // near_delta, but for rounding)
-  if (c.tree_df.active && c.tree_df.near_listed != (long long)c.near_pairs.size()) return INFINITY;
   return kCorrectionError * std::max(1.0, rmax / (2.0 * c.opt.near_delta));
 }
 

@@ -677,7 +677,6 @@ __global__ void __launch_bounds__(128, 4)
     const float4 oh = x3h[w.t0], om = x3m[w.t0], ol = x3l[w.t0];
     const bool valid = t < w.t1;
     dflt xt[3], nt[3], a[3], a2[3];
-    int pt = -1;
     {
       float4 ah = oh, am = om, al = ol, bh = make_float4(0, 0, 0, 0), bl = make_float4(0, 0, 0, 0);
       if (valid) {
@@ -686,7 +685,6 @@ __global__ void __launch_bounds__(128, 4)
         al = x3l[t];
         bh = nh[t];
         bl = nl[t];
-        pt = __float_as_int(ah.w);
       }
       xt[0] = df_diff3(ah.x, am.x, al.x, oh.x, om.x, ol.x);
       xt[1] = df_diff3(ah.y, am.y, al.y, oh.y, om.y, ol.y);
@@ -698,9 +696,9 @@ __global__ void __launch_bounds__(128, 4)
     const float xm = warp_max_abs(fmaxf(fabsf(xt[0].h), fmaxf(fabsf(xt[1].h), fabsf(xt[2].h))));
 #pragma unroll
     for (int c = 0; c < 3; ++c) a[c] = a2[c] = dflt{0.0f, 0.0f};
-    int seg = w.s0, off = 0, done = 0;
-    int2 sg = segs[seg];
-    // nodes
+    int seg = w.s0 + w.nskip, off = 0;
+    int2 sg = seg < w.s1 ? segs[seg] : make_int2(0, 0);
+    // nodes (the leading segments are the own particle and its near ones)
     while (seg < w.s1 && sg.x < N) {
       int sidx[2] = {0, 0};
       int filled = 0;
@@ -719,9 +717,7 @@ __global__ void __launch_bounds__(128, 4)
           if (seg < w.s1) sg = segs[seg];
         }
       }
-      df_tile<KIND>(wsm, sidx, filled, done < w.nmask, split, half, x3h, x3m, x3l, sqh, sql, oh, om, ol, xt, nt, xm,
-                    pt, a, a2);
-      done += filled;
+      df_tile<KIND, false>(wsm, sidx, filled, DfSkip{}, nullptr, split, half, x3h, x3m, x3l, sqh, sql, oh, om, ol, xt, nt, xm, 0, a, a2);
     }
     // clusters
     for (; seg < w.s1; ++seg) {
@@ -959,7 +955,7 @@ void TreeState::release() {
   d_cheb64.release();
   d_q64.release();
   df = false;
-  direct_pairs = proxy_pairs = charge_work = lead_pairs = near_listed = 0;
+  direct_pairs = proxy_pairs = charge_work = lead_pairs = 0;
 }
 
 Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) {
@@ -986,7 +982,9 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
   std::vector<std::vector<int2>> seg_of(n);
   std::vector<long long> proxy_src(n, 0);
   std::vector<int> lead(n, 1);  // leading segments: the own particle and its near ones
-  T.near_listed = T.lead_pairs = 0;
+  T.lead_pairs = 0;
+  double reach = 0.0;  // of the coordinates, whose rounding d has
+  for (size_t k = 0; k < 3 * (size_t)n; ++k) reach = std::max(reach, std::fabs(c.centres[k]));
   int n_used = 0;
   std::vector<int> used_cells;
   std::vector<int> stack;
@@ -1005,7 +1003,12 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
       const double dx = B.cen[0] - C.cen[0], dy = B.cen[1] - C.cen[1], dz = B.cen[2] - C.cen[2];
       const double d = std::sqrt(dx * dx + dy * dy + dz * dz);
       const double rr = B.r + C.r;
-      if (rr < theta * d && d >= rr + c.near_delta && (long long)npx < C.nodes) {
+      bool accept = rr < theta * d && d >= rr + c.near_delta && (long long)npx < C.nodes;
+      // (near particles stay out of clusters whatever the rounding of d)
+      if (accept && d - (rr + c.near_delta) <= 1e-9 * (d + reach))
+        for (int q = C.pb; q < C.pe && accept; ++q)
+          accept = !near_particles(c.centres, c.radius, i, order[q], c.near_delta);
+      if (accept) {
         approx.push_back(id);
       } else if (C.nkid > 0) {
         for (int k = C.nkid - 1; k >= 0; --k) stack.push_back(C.kid[k]);
@@ -1018,7 +1021,6 @@ Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) 
       return near_particles(c.centres, c.radius, i, j, c.near_delta);
     });
     lead[i] += (int)(far - direct.begin());
-    T.near_listed += far - direct.begin();
     for (int j : direct) L.push_back(make_int2((int)c.offset[j], (int)(c.offset[j + 1] - c.offset[j])));
     for (int k = 0; k < lead[i]; ++k) T.lead_pairs += (long long)np_i * L[k].y;
     for (int id : approx) {
@@ -1184,7 +1186,6 @@ static Status build_lists(Context& c, TreeState& T, const std::vector<double>& p
   T.proxy_pairs = P.proxy_pairs;
   T.charge_work = P.charge_work;
   T.lead_pairs = P.lead_pairs;
-  T.near_listed = P.near_listed;
   T.items.swap(P.items);
   T.segs.swap(P.segs);
   T.charge_items.swap(P.charge_items);
@@ -1425,7 +1426,7 @@ Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y
   if (T.items.empty()) return Status::Ok();
   KernelTimer timer(c, kind == 0 ? RBS_KC_PAIR_KDF : (kind == 1 ? RBS_KC_PAIR_SDF : RBS_KC_PAIR_KSDF));
   RBS_TRY(kind == 0 ? launch_tree_df<0>(c, y, y2) : (kind == 1 ? launch_tree_df<1>(c, y, y2) : launch_tree_df<2>(c, y, y2)));
-  timer.done((double)(T.direct_pairs + T.proxy_pairs));
+  timer.done((double)(T.direct_pairs - T.lead_pairs + T.proxy_pairs));
   return Status::Ok();
 }
 
