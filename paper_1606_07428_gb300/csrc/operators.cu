@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(128, 5)
 
 // ------------------------------------------------------------------------------------------
 // Weighted density as double-float pairs for the double-float kernels: (w mu) rounded to float32 and
-// the rounded remainder.
+// the rounded remainder, with the bound of their biased sums.
 __global__ void k_weight_df(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
                             float4* __restrict__ wh, float4* __restrict__ wl, int* __restrict__ units) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -836,7 +836,7 @@ __global__ void k_weight_df(long long N, const double4* __restrict__ x, const do
   if (t >= N) return;
   const double w = x[t].w;
   const dflt a = df_split(w * dens[3 * t]), b = df_split(w * dens[3 * t + 1]), c = df_split(w * dens[3 * t + 2]);
-  wh[t] = make_float4(a.h, b.h, c.h, 0.0f);
+  wh[t] = make_float4(a.h, b.h, c.h, bias_bound(a.h, b.h, c.h));
   wl[t] = make_float4(a.l, b.l, c.l, 0.0f);
 }
 
@@ -990,7 +990,7 @@ __global__ void __launch_bounds__(256) k_upsample(const int4* __restrict__ group
   if (FORM == 1) qh[o] = make_float4((float)q0, (float)q1, (float)q2, 0.0f);
   if (FORM == 2) {
     const dflt d0 = df_split(q0), d1 = df_split(q1), d2 = df_split(q2);
-    qh[o] = make_float4(d0.h, d1.h, d2.h, 0.0f);
+    qh[o] = make_float4(d0.h, d1.h, d2.h, bias_bound(d0.h, d1.h, d2.h));
     ql[o] = make_float4(d0.l, d1.l, d2.l, 0.0f);
   }
 }

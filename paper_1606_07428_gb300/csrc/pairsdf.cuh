@@ -48,6 +48,11 @@ __device__ __forceinline__ dflt fold2(const df2& a) {
 // kBiasFactor is 2 with a margin for the rounded norms.
 constexpr float kBiasFactor = 2.002f;
 
+// kBiasFactor |q|, without overflow or underflow of the squares: a plain root of their sum is infinite from 2e19 up (the
+// bias less a partial sum then is not a number) and loses its digits from 1e-19 down (the bias no longer bounds the
+// partial sums, whose rounding falls to float32's).  The double-float weighted densities carry it in hi's fourth component.
+__device__ __forceinline__ float bias_bound(float x, float y, float z) { return kBiasFactor * norm3df(x, y, z); }
+
 __device__ __forceinline__ df2 norm2(float2 h, float2 l) {  // h + l, renormalised
   const float2 s = __fadd2_rn(h, l);
   return {s, __fadd2_rn(l, ng2(__fadd2_rn(s, ng2(h))))};
@@ -123,7 +128,7 @@ __device__ __forceinline__ inv_powers df_inv_powers(const df2 (&d)[3], int2 mask
 }
 
 // One target against two sources, KIND 0 traction into acc, 1 Stokeslet into acc, 2 traction into acc and
-// Stokeslet into acc2; fb = kBiasFactor |density| of the sources.  With two-sums 221 float32 operations
+// Stokeslet into acc2; fb = bias_bound of the sources.  With two-sums 221 float32 operations
 // for both kernels, 154 for the traction alone and 139 for the Stokeslet alone; 9 fewer on the grid.
 template <int KIND, int MODE>
 __device__ __forceinline__ void pair2_df(const df2 (&y)[3], const df2 (&den)[3], float2 fb, int2 mask,
@@ -352,7 +357,7 @@ __device__ __forceinline__ void df_tile(float* wsm, const int (&sidx)[2], int fi
     sa[9][l] = ql.y;
     sa[10][l] = qh.z;
     sa[11][l] = ql.z;
-    sa[12][l] = kBiasFactor * sqrtf(fmaf(qh.x, qh.x, fmaf(qh.y, qh.y, qh.z * qh.z)));
+    sa[12][l] = qh.w;
   });
 #pragma unroll
   for (int c = 0; c < 3; ++c) nt[c] = {dup2(n0[c].h), dup2(n0[c].l)};

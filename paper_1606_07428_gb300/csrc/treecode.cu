@@ -301,22 +301,22 @@ __global__ void __launch_bounds__(kChargeThreads) k_tree_charges64(const int4* _
 }
 
 // Float64 cluster charges to the rows the double-float kernel reads, per row of the last proxy axis:
-// (x, y, z hi, x, y, z lo, bound) x ncp, bound = 2 |q| rounded up (the bias of the biased sums).
+// (x, y, z hi, x, y, z lo, bound) x ncp, the bound of their biased sums.
 __global__ void k_tree_q64_split(long long rows, int ncp, const double* __restrict__ q64, float* __restrict__ q) {
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (k >= rows * ncp) return;
   const long long r = k / ncp;
   const int c = (int)(k - r * ncp);
   float* dst = q + r * 7 * ncp + c;
-  float s = 0.0f;
+  float h[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const dflt v = df_split(q64[(r * 3 + d) * ncp + c]);
     dst[d * ncp] = v.h;
     dst[(3 + d) * ncp] = v.l;
-    s = fmaf(v.h, v.h, s);
+    h[d] = v.h;
   }
-  dst[6 * ncp] = kBiasFactor * sqrtf(s);
+  dst[6 * ncp] = bias_bound(h[0], h[1], h[2]);
 }
 
 // Next unit of a warp: units are (work item, run of 32 NT of its targets) in item order, taken from a
