@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/rbs.h"
+#include "units.cuh"
 
 namespace rbs {
 
@@ -374,7 +375,7 @@ struct Context {
   // smooth pair-sum work list: (target begin, target end, source begin, source end)
   std::vector<longlong4> work;
   DevBuf<longlong4> d_work;
-  DevBuf<int> d_unit;  // next work unit of the running smooth sum and near correction (zeroed before each launch)
+  DevBuf<unit_t> d_unit;  // next work unit of the running smooth sum and near correction (zeroed before each launch)
 
   // scratch vectors (3N doubles each) and GMRES workspace
   DevBuf<double> d_vec[10];

@@ -180,7 +180,7 @@ __device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(128, 4) k_lap_df(int nunits, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 4) k_lap_df(unit_t nunits, unit_t* __restrict__ counter,
                                                    const longlong4* __restrict__ work, DfSkip skip,
                                                    const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                                    const float4* __restrict__ x3l, const float4* __restrict__ nh,
@@ -193,12 +193,11 @@ __global__ void __launch_bounds__(128, 4) k_lap_df(int nunits, int* __restrict__
   int* const smask = reinterpret_cast<int*>(&sa[8][0]);
   const int lane = threadIdx.x & 31;
   while (true) {
-    int unit = 0;
-    if (lane == 0) unit = atomicAdd(counter, 1);
-    unit = __shfl_sync(0xffffffffu, unit, 0);
+    const unit_t unit = take_unit(counter);
     if (unit >= nunits) return;
-    const longlong4 w = work[unit >> 2];
-    const int t0 = (int)w.x + 32 * (unit & 3), t1 = (int)w.y;
+    const UnitPart u = unit_part(unit, 4);
+    const longlong4 w = work[u.item];
+    const int t0 = (int)w.x + 32 * u.part, t1 = (int)w.y;
     if (t0 >= t1) continue;
     const bool split = t1 - t0 <= 16;  // the half-warps take alternate halves of the sources
     const int half = split ? lane >> 4 : 0;
@@ -590,10 +589,11 @@ static Status apply_laplace(Context& c, int kind, double half, double scale, con
     if (M.d_wq.n != (size_t)c.N) RBS_TRY(M.d_wq.alloc(c.N));
     c.stats.launches += 2;
     k_weight_df1<<<cdiv(c.N, 256), 256, 0, s>>>(c.N, c.d_x.ptr, x, M.d_wq.ptr);
-    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, 2 * sizeof(int), s));
+    RBS_CUDA_TRY(cudaMemsetAsync(c.d_unit.ptr, 0, 2 * sizeof(unit_t), s));
     const int grid = std::min(nw, 4 * std::max(1, c.sm_count));
-#define RBS_LAP_ARGS \
-  4 * nw, c.d_unit.ptr, c.d_work.ptr, DfSkip{c.d_near_first.ptr, c.d_near.ptr}, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
+#define RBS_LAP_ARGS                                                                                                  \
+  (unit_t)4 * nw, c.d_unit.ptr, c.d_work.ptr, DfSkip{c.d_near_first.ptr, c.d_near.ptr}, c.d_x3h.ptr, c.d_x3m.ptr, \
+      c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, M.d_wq.ptr, scale, y
     if (kind == 0)
       k_lap_df<0><<<grid, 128, 0, s>>>(RBS_LAP_ARGS);
     else

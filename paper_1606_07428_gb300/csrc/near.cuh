@@ -15,9 +15,10 @@ namespace rbs {
 // pairs and most of its threads idle where orders mix.
 // base: with the base nodes; else the upsampled nodes alone (for sums that leave near sources out).
 struct NearArgs {
-  int nunits, chunks, parts;
+  unit_t nunits;
+  int chunks, parts;
   bool base;
-  int* counter;
+  unit_t* counter;
   const int2* near;
   const long long* offset;
   const int* nodes;
@@ -30,13 +31,11 @@ struct NearUnit {
   int s0, s1, nup;      // sources [s0, s1): below nup upsampled nodes, then base nodes
 };
 __device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
-  int unit = 0;
-  if ((threadIdx.x & 31) == 0) unit = atomicAdd(A.counter, 1);
-  unit = __shfl_sync(0xffffffffu, unit, 0);
+  const unit_t unit = take_unit(A.counter);
   if (unit >= A.nunits) return false;
-  const int part = unit % A.parts, q = unit / A.parts;
-  const int chunk = q % A.chunks;
-  const int2 pr = A.near[q / A.chunks];
+  const UnitPart u1 = unit_part(unit, A.parts), u2 = unit_part(u1.item, A.chunks);
+  const int part = u1.part, chunk = u2.part;
+  const int2 pr = A.near[u2.item];
   const long long oi = A.offset[pr.x];
   n.t0 = (int)oi + 32 * chunk;
   n.t1 = min(n.t0 + 32, (int)oi + A.nodes[pr.x]);
@@ -67,15 +66,15 @@ inline Status near_args(Context& c, bool base, NearArgs& A, int& blocks) {
   // a float64 context's targets with one near source each keep one addition, the same bits on every run
   if (!prec_f32(c.opt.precision) && !c.near_multi) A.parts = 1;
   const long long units = units1 * A.parts;
-  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "near correction: more than 2^31 work units");
-  A.nunits = (int)units;
+  if (!units_fit(units)) return Status::Err(RBS_ENOMEM, "near correction: more than 2^32 work units");
+  A.nunits = (unit_t)units;
   A.counter = c.d_unit.ptr + 1;
   A.near = c.d_near.ptr;
   A.offset = c.d_offset.ptr;
   A.nodes = c.d_nodes.ptr;
   A.up_index = c.d_up_index.ptr;
   A.up_off = c.d_up_off.ptr;
-  blocks = (int)((units + 3) / 4);
+  blocks = (int)std::min<long long>((units + 3) / 4, INT_MAX);
   return Status::Ok();
 }
 

@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(128) k_pairs64(int nitems, const longlong4* __
 // ------------------------------------------------------------------------------------------
 // Weighted density in float32 for the packed kernels: wmu[t] = (w_t mu_t, 0).
 __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
-                             float4* __restrict__ wmu, int* __restrict__ units) {
+                             float4* __restrict__ wmu, unit_t* __restrict__ units) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t < 2) units[t] = 0;  // the unit counters of the smooth sum and the near correction that follow
   if (t >= N) return;
@@ -610,7 +610,7 @@ __global__ void k_weight_f32(long long N, const double4* __restrict__ x, const d
 // 12 us by the smaller units.
 template <int KIND, int NT>
 __global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
-    k_pairs32x2(int nunits, int* __restrict__ counter, const longlong4* __restrict__ work,
+    k_pairs32x2(unit_t nunits, unit_t* __restrict__ counter, const longlong4* __restrict__ work,
                 const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
                 const float4* __restrict__ wmu, double* __restrict__ y) {
   constexpr int TW = 128, kPerItem = 4 / NT;
@@ -619,12 +619,11 @@ __global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
   float* const ssx = tiles[threadIdx.x >> 5];
   int* const spid = reinterpret_cast<int*>(ssx + 6 * TW);
   while (true) {
-    int unit = 0;
-    if (lane == 0) unit = atomicAdd(counter, 1);
-    unit = __shfl_sync(0xffffffffu, unit, 0);
+    const unit_t unit = take_unit(counter);
     if (unit >= nunits) return;
-    const longlong4 w = work[unit / kPerItem];
-    const int t0 = (int)w.x + 32 * NT * (unit % kPerItem), t1 = (int)w.y;
+    const UnitPart u = unit_part(unit, kPerItem);
+    const longlong4 w = work[u.item];
+    const int t0 = (int)w.x + 32 * NT * u.part, t1 = (int)w.y;
     if (t0 >= t1) continue;
     const bool split = t1 - t0 <= 16;  // the two half-warps take alternate halves of the sources
     const int half = split ? lane >> 4 : 0;
@@ -728,7 +727,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? 7 : 5)
 // zero-density ones far away.  The near pairs of a particle are ordered by source, so a pointer walks them beside
 // the tiles.
 __global__ void __launch_bounds__(128, 5)
-    k_far32_both(int nunits, int* __restrict__ counter, const longlong4* __restrict__ work,
+    k_far32_both(unit_t nunits, unit_t* __restrict__ counter, const longlong4* __restrict__ work,
                  const long long* __restrict__ offset, const int* __restrict__ near_first, const int2* __restrict__ near,
                  const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
                  const float4* __restrict__ wmu, double* __restrict__ y, double* __restrict__ y2) {
@@ -737,12 +736,11 @@ __global__ void __launch_bounds__(128, 5)
   const int lane = threadIdx.x & 31;
   float* const ssx = tiles[threadIdx.x >> 5];
   while (true) {
-    int unit = 0;
-    if (lane == 0) unit = atomicAdd(counter, 1);
-    unit = __shfl_sync(0xffffffffu, unit, 0);
+    const unit_t unit = take_unit(counter);
     if (unit >= nunits) return;
-    const longlong4 w = work[unit >> 2];
-    const int ub = (int)w.x + 32 * (unit & 3), ue = min(ub + 32, (int)w.y);
+    const UnitPart u = unit_part(unit, 4);
+    const longlong4 w = work[u.item];
+    const int ub = (int)w.x + 32 * u.part, ue = min(ub + 32, (int)w.y);
     for (int t0 = ub; t0 < ue;) {
       const float4 oh = xhi[t0], ol = xlo[t0];
       const int i = __float_as_int(oh.w);
@@ -830,7 +828,7 @@ __global__ void __launch_bounds__(128, 5)
 // Weighted density as double-float pairs for the double-float kernels: (w mu) rounded to float32 and
 // the rounded remainder, with the bound of their biased sums.
 __global__ void k_weight_df(long long N, const double4* __restrict__ x, const double* __restrict__ dens,
-                            float4* __restrict__ wh, float4* __restrict__ wl, int* __restrict__ units) {
+                            float4* __restrict__ wh, float4* __restrict__ wl, unit_t* __restrict__ units) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t < 2) units[t] = 0;
   if (t >= N) return;
@@ -848,7 +846,7 @@ __global__ void k_weight_df(long long N, const double4* __restrict__ x, const do
 // busy: both sums 126 to 153 Gpair/s (101 particles of 220 nodes), the traction alone 195 to 219 (500 of 220),
 // against two-sum arithmetic throughout in blocks of whole items.
 template <int KIND>
-__global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restrict__ counter,
+__global__ void __launch_bounds__(128, 4) k_pairs_df2(unit_t nunits, unit_t* __restrict__ counter,
                                                       const longlong4* __restrict__ work, DfSkip skip,
                                                       const float4* __restrict__ x3h, const float4* __restrict__ x3m,
                                                       const float4* __restrict__ x3l, const float4* __restrict__ nh,
@@ -861,12 +859,11 @@ __global__ void __launch_bounds__(128, 4) k_pairs_df2(int nunits, int* __restric
   float* const wsm = tiles + (threadIdx.x >> 5) * kTileDfFloats;
   const int lane = threadIdx.x & 31;
   while (true) {
-    int unit = 0;
-    if (lane == 0) unit = atomicAdd(counter, 1);
-    unit = __shfl_sync(0xffffffffu, unit, 0);
+    const unit_t unit = take_unit(counter);
     if (unit >= nunits) return;
-    const longlong4 w = work[unit >> 2];
-    const int t0 = (int)w.x + 32 * (unit & 3), t1 = (int)w.y;
+    const UnitPart u = unit_part(unit, 4);
+    const longlong4 w = work[u.item];
+    const int t0 = (int)w.x + 32 * u.part, t1 = (int)w.y;
     if (t0 >= t1) continue;
     const bool split = t1 - t0 <= 16;
     const int half = split ? lane >> 4 : 0;
@@ -1250,14 +1247,15 @@ static void launch_pairs32(Context& c, double* y) {
   const int items = (int)c.work.size();
   const auto kernel = k_pairs32x2<KIND, NT>;
   kernel<<<resident_grid(c, (const void*)kernel, 128, items), 128, 0, c.stream>>>(
-      4 / NT * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y);
+      (unit_t)(4 / NT) * items, c.d_unit.ptr, c.d_work.ptr, c.d_xhi.ptr, c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, y);
 }
 
 template <int KIND>
 static void launch_pairs_df(Context& c, double* y, double* y2) {
   const int items = (int)c.work.size();
   k_pairs_df2<KIND><<<resident_grid(c, (const void*)k_pairs_df2<KIND>, 128, items), 128, 0, c.stream>>>(
-      4 * items, c.d_unit.ptr, c.d_work.ptr, DfSkip{c.d_near_first.ptr, c.d_near.ptr}, c.d_x3h.ptr, c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
+      (unit_t)4 * items, c.d_unit.ptr, c.d_work.ptr, DfSkip{c.d_near_first.ptr, c.d_near.ptr}, c.d_x3h.ptr, c.d_x3m.ptr,
+      c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr,
       c.d_wmuh.ptr, c.d_wmul.ptr, y, y2);
 }
 
@@ -1413,7 +1411,7 @@ static Status near_sums(Context& c, int kind, int prec, const double* x, double*
   NearArgs A;
   int blocks = 0;
   RBS_TRY(near_args(c, prec != RBS_PREC_DF, A, blocks));
-  if (prec == RBS_PREC_FP64) RBS_CUDA_TRY(cudaMemsetAsync(A.counter, 0, sizeof(int), c.stream));
+  if (prec == RBS_PREC_FP64) RBS_CUDA_TRY(cudaMemsetAsync(A.counter, 0, sizeof(unit_t), c.stream));
 #define RBS_NEAR_LAUNCH(KERNEL, ...) \
   KERNEL<<<resident_grid(c, (const void*)KERNEL, 128, blocks), 128, 0, c.stream>>>(A, __VA_ARGS__)
   if (prec == RBS_PREC_DF) {
@@ -1557,7 +1555,7 @@ Status apply_correction(Context& c, const double* d, double* w, double* v) {
     KernelTimer timer(c, RBS_KC_PAIR_K32);
     const int items = (int)c.work.size();
     k_far32_both<<<resident_grid(c, (const void*)k_far32_both, 128, items), 128, 0, c.stream>>>(
-        4 * items, c.d_unit.ptr, c.d_work.ptr, c.d_offset.ptr, c.d_near_first.ptr, c.d_near.ptr, c.d_xhi.ptr, c.d_xlo.ptr,
+        (unit_t)4 * items, c.d_unit.ptr, c.d_work.ptr, c.d_offset.ptr, c.d_near_first.ptr, c.d_near.ptr, c.d_xhi.ptr, c.d_xlo.ptr,
         c.d_nrm32.ptr, c.d_wmu32.ptr, w, v);
     RBS_CUDA_TRY(cudaGetLastError());
     timer.done(2.0 * ((double)c.stats.far_pairs - c.near_base_nodes));

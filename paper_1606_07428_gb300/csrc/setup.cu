@@ -1448,6 +1448,7 @@ Status build_geometry(Context& c) {
         }
     }
   }
+  if (!units_fit(4 * (long long)c.work.size())) return Status::Err(RBS_ENOMEM, "pair sums: more than 2^32 work units");
   RBS_TRY(upload(c.d_work, c.work, s));
   RBS_TRY(c.d_unit.alloc(2));
   if (!c.near_pairs.empty() && c.N <= kBesideNodes) RBS_TRY(c.side_stream());

@@ -319,16 +319,11 @@ __global__ void k_tree_q64_split(long long rows, int ncp, const double* __restri
   dst[6 * ncp] = bias_bound(h[0], h[1], h[2]);
 }
 
-// Next unit of a warp: units are (work item, run of 32 NT of its targets) in item order, taken from a
+// Units of the pair sums: (work item, run of 32 NT of its targets) in item order, taken by warps from a
 // counter that the launch starts at zero.  Warps never wait for one another, and no warp is tied to a
 // fixed share: with whole-particle blocks striding over the items, the warp that held a particle's
 // last few targets finished early and blocks of an odd warp count loaded the SM's four schedulers
 // unevenly (10 of 15 resident warps active on average).
-__device__ __forceinline__ int next_unit(int* counter) {
-  int u = 0;
-  if ((threadIdx.x & 31) == 0) u = atomicAdd(counter, 1);
-  return __shfl_sync(0xffffffffu, u, 0);
-}
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -360,7 +355,7 @@ constexpr int kRing32 = 4;
 
 template <int KIND, int NT, int NQ2>
 __global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 : 5)) : 4)
-    k_tree32x2(int nunits, int per_item, int* __restrict__ counter, const TreeItem* __restrict__ items,
+    k_tree32x2(unit_t nunits, int per_item, unit_t* __restrict__ counter, const TreeItem* __restrict__ items,
                const int2* __restrict__ segs, long long N, int npx, int nq, int nbp, int ncp,
                const float4* __restrict__ xhi, const float4* __restrict__ xlo, const float4* __restrict__ nrm32,
                const float4* __restrict__ sq, const float4* __restrict__ axis, const float* __restrict__ pq,
@@ -381,10 +376,10 @@ __global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 
   float* const ring = wsm;                   // kRing32 slabs
   float* const sax = wsm + kRing32 * slab;   // 3 nq (+ 3 pad) origin-relative proxy coordinates, negated
   const uint32_t ring_s = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
-  for (int unit = next_unit(counter); unit < nunits; unit = next_unit(counter)) {
-    const int item = unit / per_item;
-    const TreeItem w = items[item];
-    const int tb = w.t0 + (unit - item * per_item) * 32 * NT;
+  for (unit_t unit = take_unit(counter); unit < nunits; unit = take_unit(counter)) {
+    const UnitPart u = unit_part(unit, per_item);
+    const TreeItem w = items[u.item];
+    const int tb = w.t0 + u.part * 32 * NT;
     if (tb >= w.t1) continue;
     const int nu = min(NT, (w.t1 - tb + 31) / 32);      // target slots that hold a target
     const bool split = w.t1 - tb <= 16;
@@ -652,7 +647,7 @@ __global__ void __launch_bounds__(128, NT == 1 ? (KIND == 2 ? 4 : (NQ2 <= 4 ? 6 
 // on 1,500 particles of 144 nodes, 128 to 154 on 700 of 312 (fewer of whose pairs are with proxies).
 template <int KIND>
 __global__ void __launch_bounds__(128, 4)
-    k_tree_df2(int nunits, int per_item, int* __restrict__ counter, const TreeItem* __restrict__ items,
+    k_tree_df2(unit_t nunits, int per_item, unit_t* __restrict__ counter, const TreeItem* __restrict__ items,
                const int2* __restrict__ segs, long long N, int npx, int nq, int nbp, int ncp,
                const float4* __restrict__ x3h, const float4* __restrict__ x3m, const float4* __restrict__ x3l,
                const float4* __restrict__ nh, const float4* __restrict__ nl, const float4* __restrict__ sqh,
@@ -666,10 +661,10 @@ __global__ void __launch_bounds__(128, 4)
   // origin-relative proxy coordinates
   float2* const sz = reinterpret_cast<float2*>(wsm) + lane;
   float2* const sax = reinterpret_cast<float2*>(wsm + nq2 * 6 * 64);
-  for (int unit = next_unit(counter); unit < nunits; unit = next_unit(counter)) {
-    const int item = unit / per_item;
-    const TreeItem w = items[item];
-    const int tb = w.t0 + (unit - item * per_item) * 32;
+  for (unit_t unit = take_unit(counter); unit < nunits; unit = take_unit(counter)) {
+    const UnitPart u = unit_part(unit, per_item);
+    const TreeItem w = items[u.item];
+    const int tb = w.t0 + u.part * 32;
     if (tb >= w.t1) continue;
     const bool split = w.t1 - tb <= 16;
     const int half = split ? lane >> 4 : 0;
@@ -1288,10 +1283,10 @@ static Status launch_tree(Context& c, const TreeState& T, double* y, double* y2 
   const size_t smem = 4 * (size_t)warp_floats * sizeof(float);
   const int per_item = (T.tmax + 32 * NT - 1) / (32 * NT);
   const long long units = (long long)T.items.size() * per_item;
-  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "treecode: more than 2^31 work units");
+  if (!units_fit(units)) return Status::Err(RBS_ENOMEM, "treecode: more than 2^32 work units");
   const auto kernel = k_tree32x2<KIND, NT, NQ2>;
   kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
-      (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_xhi.ptr,
+      (unit_t)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_xhi.ptr,
       c.d_xlo.ptr, c.d_nrm32.ptr, c.d_wmu32.ptr, T.d_axis.ptr, T.d_pq.ptr, warp_floats, y, y2);
   RBS_CUDA_TRY(cudaGetLastError());
   return Status::Ok();
@@ -1398,10 +1393,10 @@ static Status launch_tree_df(Context& c, double* y, double* y2) {
   const size_t smem = 4 * (size_t)warp_floats * sizeof(float);
   const int per_item = (T.tmax + 31) / 32;
   const long long units = (long long)T.items.size() * per_item;
-  if (units > INT_MAX) return Status::Err(RBS_ENOMEM, "treecode: more than 2^31 work units");
+  if (!units_fit(units)) return Status::Err(RBS_ENOMEM, "treecode: more than 2^32 work units");
   const auto kernel = k_tree_df2<KIND>;
   kernel<<<tree_grid(c, (const void*)kernel, smem, units), 128, smem, c.stream>>>(
-      (int)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_x3h.ptr,
+      (unit_t)units, per_item, c.d_unit.ptr, T.d_items.ptr, T.d_segs.ptr, c.N, T.npx, nq, T.nbp, T.ncp, c.d_x3h.ptr,
       c.d_x3m.ptr, c.d_x3l.ptr, c.d_nrmh.ptr, c.d_nrml.ptr, c.d_wmuh.ptr, c.d_wmul.ptr, T.d_axis.ptr, T.d_pq.ptr,
       warp_floats, y, y2);
   RBS_CUDA_TRY(cudaGetLastError());
