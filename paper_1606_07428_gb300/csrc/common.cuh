@@ -340,6 +340,7 @@ struct Context {
   bool near_multi = false;        // some target particle has several near sources
   DevBuf<int2> d_near;
   DevBuf<int> d_near_first;       // n + 1: first near pair of each target particle
+  DevBuf<NearUnitItem> d_near_units;  // work units of the near corrections
   std::vector<int> up_index;      // per particle: index into upsampled-source list or -1
   std::vector<long long> up_offset;  // per upsampled source particle: first upsampled node
   std::vector<int> up_particle;

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(128, 5) k_lap_near(NearArgs A, const float4* _
   const int lane = threadIdx.x & 31;
   NearUnit n;
   while (next_near_unit(A, n)) {
-    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    if (n.s0 >= n.s1) continue;
     const bool split = n.t1 - n.t0 <= 16;
     const int half = split ? lane >> 4 : 0;
     const int t = n.t0 + (split ? lane & 15 : lane);

@@ -8,17 +8,16 @@
 namespace rbs {
 
 // Near correction.  For a near pair (target particle i, source particle j) the contribution of j's
-// upsampled nodes is added and that of its base nodes (already in the smooth sum) removed.  A unit is
-// (pair, 32 targets of i, one of `parts` equal runs of the N_up + N_j sources), taken by warps from a
-// counter; parts grows until small near lists fill the GPU.  A pair of 144-node particles is 688 sources
-// against five units of targets, so one block per pair left most of the SMs idle on lists of a few hundred
-// pairs and most of its threads idle where orders mix.
+// upsampled nodes is added and that of its base nodes (already in the smooth sum) removed.  Warps take the units
+// of list_near_units from a counter.  A pair of 144-node particles is 688 sources against five units of
+// targets, so one block per pair left most of the SMs idle on lists of a few hundred pairs and most of its threads idle
+// where orders mix.
 // base: with the base nodes; else the upsampled nodes alone (for sums that leave near sources out).
 struct NearArgs {
   unit_t nunits;
-  int chunks, parts;
   bool base;
   unit_t* counter;
+  const NearUnitItem* units;
   const int2* near;
   const long long* offset;
   const int* nodes;
@@ -26,49 +25,38 @@ struct NearArgs {
   const long long* up_off;
 };
 struct NearUnit {
-  int t0, t1;           // targets [t0, t1) of particle i that the unit holds, 32 at most (t0 >= t1: none)
+  int t0, t1;           // targets [t0, t1) of particle i that the unit holds, 32 at most
   long long ub, oj;     // first upsampled node and first base node of j
   int s0, s1, nup;      // sources [s0, s1): below nup upsampled nodes, then base nodes
 };
 __device__ __forceinline__ bool next_near_unit(const NearArgs& A, NearUnit& n) {
   const unit_t unit = take_unit(A.counter);
   if (unit >= A.nunits) return false;
-  const UnitPart u1 = unit_part(unit, A.parts), u2 = unit_part(u1.item, A.chunks);
-  const int part = u1.part, chunk = u2.part;
-  const int2 pr = A.near[u2.item];
+  const NearUnitItem it = A.units[unit];
+  const int2 pr = A.near[it.pair];
   const long long oi = A.offset[pr.x];
-  n.t0 = (int)oi + 32 * chunk;
+  n.t0 = (int)oi + it.t;
   n.t1 = min(n.t0 + 32, (int)oi + A.nodes[pr.x]);
   const int u = A.up_index[pr.y];
   n.ub = A.up_off[u];
   n.nup = (int)(A.up_off[u + 1] - n.ub);
   n.oj = A.offset[pr.y];
   const int total = n.nup + (A.base ? A.nodes[pr.y] : 0);
-  const int step = ((total + A.parts - 1) / A.parts + 3) & ~3;
-  n.s0 = min(total, part * step);
+  const int step = ((total + it.parts - 1) / it.parts + 3) & ~3;
+  n.s0 = min(total, it.part * step);
   n.s1 = min(total, n.s0 + step);
   return true;
 }
-
 
 // The units of the context's near list (its counter, d_unit[1], is zeroed by the caller or the weight kernels);
 // blocks: as many 128-thread blocks as have a unit per warp.
 inline Status near_args(Context& c, bool base, NearArgs& A, int& blocks) {
   A.base = base;
-  const long long nn = (long long)c.near_pairs.size();
-  A.chunks = (c.max_np + 31) / 32;
-  // source runs: about 16 units per SM, of at least 128 sources and at most about 512 (a unit of one p = 16
-  // source particle, 2,656 sources, would outlast a list of mixed orders)
-  int most = 1;
-  for (Grid* g : c.grids) most = std::max(most, g->nup + g->np);
-  const long long units1 = std::max(1LL, nn * A.chunks);
-  A.parts = (int)std::max((most + 511LL) / 512, std::min<long long>((16LL * c.sm_count + units1 - 1) / units1, most / 128));
-  // a float64 context's targets with one near source each keep one addition, the same bits on every run
-  if (!prec_f32(c.opt.precision) && !c.near_multi) A.parts = 1;
-  const long long units = units1 * A.parts;
+  const long long units = (long long)c.d_near_units.n;
   if (!units_fit(units)) return Status::Err(RBS_ENOMEM, "near correction: more than 2^32 work units");
   A.nunits = (unit_t)units;
   A.counter = c.d_unit.ptr + 1;
+  A.units = c.d_near_units.ptr;
   A.near = c.d_near.ptr;
   A.offset = c.d_offset.ptr;
   A.nodes = c.d_nodes.ptr;

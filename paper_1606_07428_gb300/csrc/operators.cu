@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(128, 6) k_near32(NearArgs A, const float4* __r
   float* const ssx = tiles[threadIdx.x >> 5];
   NearUnit n;
   while (next_near_unit(A, n)) {
-    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    if (n.s0 >= n.s1) continue;
     const bool split = n.t1 - n.t0 <= 16;
     const int half = split ? lane >> 4 : 0;
     const int t = n.t0 + (split ? lane & 15 : lane);
@@ -1092,7 +1092,7 @@ __global__ void __launch_bounds__(128, 4) k_near_df(NearArgs A, const float4* __
   const int lane = threadIdx.x & 31;
   NearUnit n;
   while (next_near_unit(A, n)) {
-    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    if (n.s0 >= n.s1) continue;
     const bool split = n.t1 - n.t0 <= 16;
     const int half = split ? lane >> 4 : 0;
     const int t = n.t0 + (split ? lane & 15 : lane);
@@ -1140,7 +1140,7 @@ __global__ void __launch_bounds__(128) k_near64(NearArgs A, const double4* __res
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   NearUnit n;
   while (next_near_unit(A, n)) {
-    if (n.t0 >= n.t1 || n.s0 >= n.s1) continue;
+    if (n.s0 >= n.s1) continue;
     const bool split = n.t1 - n.t0 <= 16;  // the half-warps take alternate halves of the sources
     const int half = split ? lane >> 4 : 0;
     const int t = n.t0 + (split ? lane & 15 : lane);

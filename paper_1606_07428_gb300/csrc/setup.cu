@@ -1103,6 +1103,17 @@ Status build_near(Context& c) {
     c.near_base_nodes += base;
     c.near_pair_nodes += base + (double)(c.offset[pr.x + 1] - c.offset[pr.x]) * c.grids[c.grid_of[pr.y]]->nup;
   }
+  {
+    std::vector<int> targets, sources;
+    for (const int2& pr : c.near_pairs) {
+      targets.push_back((int)(c.offset[pr.x + 1] - c.offset[pr.x]));
+      sources.push_back(c.grids[c.grid_of[pr.y]]->nup + (int)(c.offset[pr.y + 1] - c.offset[pr.y]));
+    }
+    // a float64 context's targets with one near source each keep one addition, the same bits on every run
+    const std::vector<NearUnitItem> units =
+        list_near_units(targets, sources, c.sm_count, !prec_f32(c.opt.precision) && !c.near_multi);
+    RBS_TRY(upload(c.d_near_units, units, s));
+  }
   c.stats.near_pairs = (long long)c.near_pairs.size();
   return build_far_field(c);
 }

@@ -40,3 +40,30 @@ def test_counter_at_the_largest_launches(tmp_path, per_item):
   }}
   std::printf("%d\\n", (int)ok);""")
     assert out == ["1"]
+
+
+def near_units(tmp_path, pairs, sm_count, one_part=0):
+    targets, sources = (", ".join(str(p[k]) for p in pairs) for k in (0, 1))
+    out = run(tmp_path, f"""
+  for (const NearUnitItem& u : list_near_units({{{targets}}}, {{{sources}}}, {sm_count}, {one_part}))
+    std::printf("%d %d %d %d ", u.pair, u.t, u.part, u.parts);""")
+    v = [int(w) for w in out]
+    return [tuple(v[k:k + 4]) for k in range(0, len(v), 4)]
+
+
+@pytest.mark.parametrize("one_part", [0, 1])
+@pytest.mark.parametrize("pairs,sm_count", [
+    ([(144, 688)] * 12, 152),                                # a short list: runs of 128 sources
+    ([(144, 688)] * 2000, 152),                              # a long one: as few runs as 512 sources allow
+    ([(2112, 260)] + [(40, 20680)] + [(40, 260)] * 400, 152),  # one p = 32 particle among small ones
+    ([(12, 52), (33, 127), (32, 128), (1, 1)], 4)])
+def test_near_units_cover_each_pair_once(tmp_path, pairs, sm_count, one_part):
+    units = near_units(tmp_path, pairs, sm_count, one_part)
+    want = []
+    for k, (nt, ns) in enumerate(pairs):
+        parts = {u[3] for u in units if u[0] == k}
+        assert len(parts) == 1
+        p = parts.pop()
+        assert p == 1 if one_part else (ns + 511) // 512 <= p <= max(ns // 128, (ns + 511) // 512)
+        want += [(k, t, q, p) for t in range(0, nt, 32) for q in range(p)]
+    assert units == want  # in order, none empty and none twice
