@@ -1230,14 +1230,15 @@ static int resident_grid(Context& c, const void* kernel, int threads, int items)
   return std::max(1, std::min(items, per_sm * std::max(1, c.sm_count)));
 }
 
-// Targets per lane of the direct float32 sums: two, which share each source's loads, once that still makes
-// 48 units per SM (two rounds of its warps); one below, and where rbs_options.pair_variant asks for it.  Traction
-// Gpair/s with one and two: 117 and 97 at one unit per SM (8 particles of 144 nodes), 1,227 and 1,261 at 64 (40 of
-// 220), 1,405 and 1,438 above (101 of 220).
+// Targets per lane of the direct float32 sums: two, which share each source's loads, once that still makes 24
+// units per SM (a round of its warps); one below, and where rbs_options.pair_variant asks for it.  Traction, us an
+// apply with one and two on p = 8 (p = 10): at 1 unit of two targets per SM 9.8 and 12.8, at 7 (16.0 and 22.0), at 10
+// 18.0 and 24.8, at 17 24.2 and 26.1, at 19 (26.1 and 26.2), at 27 33.4 and 32.3, at 38 44.1 and 41.5, at 43 (46.7
+// and 44.6), at 68 69.2 and 65.7; above, two is 2 to 8% faster.  The Stokeslet sums cross at the same place.
 static int pairs32_targets(const Context& c) {
   const int v = c.opt.pair_variant;
   if (v > 0) return v == 1 || v == kPacked + 1 ? 1 : 2;
-  return 2 * (long long)c.work.size() >= 48LL * c.sm_count ? 2 : 1;
+  return 2 * (long long)c.work.size() >= 24LL * c.sm_count ? 2 : 1;
 }
 
 int direct_variant(const Context& c) { return kPacked + pairs32_targets(c); }
@@ -1259,8 +1260,9 @@ static void launch_pairs_df(Context& c, double* y, double* y2) {
       c.d_wmuh.ptr, c.d_wmul.ptr, y, y2);
 }
 
-// Launch of the direct smooth pair sum; kind 2 (traction into y and Stokeslet into y2 in one pass) exists in
-// double-float only.  The float32 and double-float sums read the weighted densities of this x.
+// Launch of the direct smooth pair sum; kind 2 (traction into y and Stokeslet into y2 in one pass) is for
+// double-float (k_far32_both is float32's, without near sources).  The float32 and double-float sums read the weighted
+// densities of this x.
 static Status launch_pairs(Context& c, int kind, int prec, const double* x, double* y, double* y2 = nullptr) {
   const int items = (int)c.work.size();
   if (prec == RBS_PREC_DF) {
@@ -1456,9 +1458,10 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y) {
     RBS_TRY(weight_df(c, x));
   }
   // The float32 near correction of a small system runs beside the smooth sum (both add into y atomically): each
-  // alone leaves SMs idle at its end.  Solves after one another and beside: 50.7 and 49.2 ms (a step of 101
-  // particles, 22,000 nodes), 49.9 and 49.4 (57,600 nodes), 403.3 and 402.6 (216,000), where the line is drawn: the
-  // gain is within the runs' spread.  Not while kernel classes are timed.
+  // alone leaves SMs idle at its end.  Solves to 1e-6 after one another and beside, ms: 1.51 and 1.44 at 3,456 nodes,
+  // 2.95 and 2.83 at 8,640, 5.73 and 5.50 at 14,544, 16.95 and 16.63 at 28,800, 49.2 and 48.7 at 57,600, 86.2 and 85.8
+  // at 79,200, 165.8 and 165.4 at 115,200, 210.3 and 209.7 at 129,600: a saving of 0.1 to 0.5 ms at every size, 0.3%
+  // where the line is drawn.  Not while kernel classes are timed.
   const bool beside = f32 && c.side && !c.near_pairs.empty() && c.N <= kBesideNodes && c.opt.timing == 0;
   if (beside) {
     RBS_CUDA_TRY(cudaEventRecord(c.fork_ev, c.stream));
