@@ -51,11 +51,11 @@ FP32_LANES_PER_SM = 128
 # float64 operations per pair (the float64 reciprocal square root counted as 7): traction 27, Stokeslet 25
 FLOPS_PER_PAIR = {"traction": 29.0, "stokeslet": 28.0, "both": 57.0}
 FP64_OPS_PER_PAIR = {"traction": 27.0, "stokeslet": 25.0}
-# DRAM bytes per launch from ncu captures of the direct kernels on the 400-ellipsoid profiling case
-# (57,600 nodes), scaled by node count to the benchmarked case: the pair kernels read their inputs
+# DRAM bytes per launch (read and written) from ncu captures of the direct kernels on the 400-ellipsoid profiling
+# case (57,600 nodes), scaled by node count to the benchmarked case: the pair kernels read their inputs
 # once (sources are re-read from L2), so traffic grows with N, not with the N^2 pairs
-NCU_TRAFFIC = {"pair_traction_df": (6.404864e6, 57600), "pair_traction_f32": (4.872192e6, 57600),
-               "pair_both_df": (8.511744e6, 57600)}
+NCU_TRAFFIC = {"pair_traction_df": (8.30e6, 57600), "pair_traction_f32": (5.52e6, 57600),
+               "pair_both_df": (1.016e7, 57600)}
 # float32-pipe operations of a double-float pair with every sum and product error-free on its own (separation
 # 24, r^2 28, reciprocal square root 8, r . density 28, powers 8, then the traction tail 76, the Stokeslet
 # tail 76, or both tails sharing 1/r^5 and r . n: 152)
@@ -67,9 +67,9 @@ DF_INSTR_PER_PAIR = {"traction": 172.0, "stokeslet": 172.0, "both": 248.0}
 DF_INSTR_NODE = {"traction": 154.0, "stokeslet": 139.0, "both": 221.0}
 DF_INSTR_PROXY = {"traction": 82.0, "stokeslet": 105.0, "both": 144.0}
 # DRAM bytes per launch of the fused double-float treecode kernel from an ncu capture on the
-# 2,000-ellipsoid profiling case (288,000 nodes; 83.27 MB read + 6.95 MB written, theta 0.45, degree 11,
-# one target per thread), scaled by node count like the direct kernels' figures
-TREE_DF_TRAFFIC = (9.0224640e7, 288000)
+# 2,000-ellipsoid profiling case (288,000 nodes; 61.61 MB read + 1.22 MB written, theta 0.45, degree 11),
+# scaled by node count like the direct kernels' figures
+TREE_DF_TRAFFIC = (6.283e7, 288000)
 
 
 def parse_args():
@@ -599,7 +599,10 @@ def run_ours(args):
     if plain and "traction_f64_gpair_s" in plain:
         gpairs["traction_f64_plain"] = plain["traction_f64_gpair_s"]
         gpairs["stokeslet_f64_plain"] = plain["stokeslet_f64_gpair_s"]
-    proxy_share = stats["tree_df_proxy_pairs"] / stats["tree_df_pairs"] if stats.get("tree_df_pairs") else 0.0
+    # of the pairs that a double-float treecode pass evaluates (its lists less the own and near particles')
+    both = kernels.get("pair_both_df")
+    evaluated = both["units"] / both["launches"] if both and both["launches"] else stats.get("tree_df_pairs", 0)
+    proxy_share = stats.get("tree_df_proxy_pairs", 0) / evaluated if evaluated else 0.0
     timed = {k: v for k, v in kernels.items() if k != "gmres_graph"}
     dom = max(timed.items(), key=lambda kv: kv[1]["ms"])
     name, e = dom

@@ -197,7 +197,8 @@ typedef struct {
                             proxy pairs; 0 without a treecode */
   long long tree_proxy_pairs; /* of these, the (target node, cluster proxy point) pairs */
   int tree_cells;        /* clusters that carry proxy points */
-  long long tree_df_pairs;       /* the same for the double-float passes' treecode (RBS_FAR_TREECODE_DF) */
+  long long tree_df_pairs;       /* the same for the double-float passes' treecode (RBS_FAR_TREECODE_DF), whose
+                                    sums skip the lists' pairs with the target's own and near particles */
   long long tree_df_proxy_pairs;
   int tree_df_cells;
 } rbs_stats;

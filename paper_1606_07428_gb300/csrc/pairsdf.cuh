@@ -70,8 +70,9 @@ __device__ __forceinline__ df2 bdot2(df2 a0, df2 b0, df2 a1, df2 b1, df2 a2, df2
 }
 
 // Odd powers of 1 / r from r^2 = h + l and the hardware estimate y0 = (1 / r)(1 + O(2^-22)): with
-// t = r^2 y0^2 - 1, (1 / r)^k = y0^k (1 - k t / 2 + k (k + 2) t^2 / 8) to 2^-64.  The powers of y0 are
-// exact to a float32 pair, and the series multiplies a product once, at its end.
+// t = r^2 y0^2 - 1, below 2^-21, (1 / r)^k = y0^k (1 - k t / 2 + k (k + 2) t^2 / 8) but for k (k + 2) (k + 4) t^3 / 48,
+// 2^-64 for k = 1, 2^-62 for k = 3 and 2^-60 for k = 5.  What limits the powers is their evaluation: those of y0 are
+// float32 pairs, and the series, in float32, multiplies a product once, at its end (2^-24 of t: 44 bits and more).
 struct inv_powers {
   float2 y0, q, qe, t;  // q + qe = y0^2
   __device__ __forceinline__ inv_powers(float2 r2h, float2 r2l, float2 y) : y0(y) {

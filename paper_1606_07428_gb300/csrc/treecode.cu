@@ -11,15 +11,16 @@
 // else descends, and evaluates the particles of unaccepted leaves directly.  An accepted cell
 // carries (n + 1)^3 proxy points on the tensor Chebyshev grid of its box and charges
 //   q_abc = sum_s L_a(y_s,x) L_b(y_s,y) L_c(y_s,z) w_s mu_s     (barycentric Lagrange basis L),
-// recomputed for every apply; the pair kernels then treat proxy points as ordinary sources.
+// recomputed for every apply.  The pair kernels use the grid's tensor form: separations, and what depends on one axis of
+// them alone, are formed per axis and row, not per proxy point.
 //
-// Layout: one source array holds the N nodes followed by the proxy points of every accepted cell
-// (float32: hi + lo positions and weighted density; double-float: three-float positions and float32
-// pairs of weighted density, with float64 cluster charges); each target particle has a list of
-// (first, count) segments into it: its own particle first (masked by particle id), then the particles near
-// it, then the other directly evaluated ones, then its accepted cells.  Work items pair the targets of one particle (or a
-// near-equal part of it, at most 512) with a run of those segments.  The host plan (plan_treecode)
-// does no device work, so it also serves the host-only entry point rbs_treecode_plan.
+// Layout: a cluster keeps the n + 1 coordinates of each axis of its grid and its charges by rows of the last axis
+// (float32, or float32 pairs split from float64 charges); nodes are read from the context's own arrays.
+// Each target particle has a list of (first, count) segments over N node indexes followed by (n + 1)^3 per accepted cell:
+// its own particle first (masked by particle id in the inner solve's float32 sums, skipped in the others), then the
+// particles near it (skipped in the others too), then the other directly evaluated ones, then its accepted cells.  Work
+// items pair the targets of one particle (or a near-equal part of it, at most 512) with a run of those segments.  The
+// host plan (plan_treecode) does no device work, so it also serves the host-only entry point rbs_treecode_plan.
 #include <algorithm>
 #include <climits>
 #include <cmath>
