@@ -51,7 +51,7 @@ extern "C" {
                             block-diagonal preconditioner of Section 3.2 and the K self blocks of its
                             restarts) stored in float16 and applied with float32 accumulation: on the
                             tensor cores for particles sharing a shape (a batched GEMM), on CUDA cores
-                            otherwise.  Refinement residuals and float32 corrections keep float32
+                            otherwise.  Refinement residuals and corrections keep float64
                             blocks, so only the inner operator's accuracy changes (about 5e-4) */
 #define RBS_PREC_DF 3    /* float64-class operator: pair sums in double-float arithmetic (unevaluated
                             sums of two float32 numbers, ~1e-12 relative), blocks and vectors in
@@ -116,12 +116,13 @@ typedef struct {
                           with mu_ratio != 1 and a non-zero field, every rbs_advance stage adds the
                           magnetic forces and torques of rbs_magnetic_forces to F and T */
   int far_field;       /* RBS_FAR_DIRECT (default): every smooth pair sum runs over all node pairs.
-                          RBS_FAR_TREECODE: the float32 applies of the mixed solve (inner GMRES and
-                          float32 corrections) approximate the smooth sums over well-separated
+                          RBS_FAR_TREECODE: the float32 applies of the mixed solve (inner GMRES)
+                          approximate the smooth sums over well-separated
                           clusters of particles with a barycentric Lagrange treecode, the
                           hierarchical far field in place of Section 3.1's fast multipole method;
-                          the double-float and float64 passes, and so the converged result, stay
-                          direct.  RBS_FAR_TREECODE_DF: the double-float passes use a treecode too,
+                          the double-float and float64 passes, the corrections between them, and so
+                          the converged result, stay direct.  RBS_FAR_TREECODE_DF: the
+                          double-float passes and corrections use a treecode too,
                           at tree_df_theta and tree_df_degree (relative error about 5e-11 at the
                           defaults); float64 passes stay direct.  Only with precision
                           RBS_PREC_MIXED */

@@ -497,6 +497,10 @@ Status apply_tree_df(Context& c, int kind, const double* x, double* y, double* y
 // y += traction and y2 += Stokeslet sum over the double-float passes' lists in float32 arithmetic (d_wmu32; the
 // charges formed in float64), without the sources on particles near the target's.
 Status apply_tree_df_f32(Context& c, const double* x, double* y, double* y2);
+// The same over the float32 lists.
+Status apply_tree_both(Context& c, double* y, double* y2);
+// Relative error assumed for the float32 lists' approximation; infinite without a treecode.
+double tree_error(const Context& c);
 
 // ---- setup (setup.cu)
 Status build_geometry(Context& c);
@@ -550,8 +554,9 @@ Status apply_pairs(Context& c, int kind, int prec, const double* x, double* y); 
 Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, double* yS);
 Status apply_operator(Context& c, int op, int prec, const double* x, double* y);
 // w = A d and v = S d for a correction d: float64 blocks, the near pairs' upsampled sums in double-float, and the
-// smooth sums between particles that are not near in float32, over the same lists as the double-float passes.
-Status apply_correction(Context& c, const double* d, double* w, double* v);
+// smooth sums between particles that are not near in float32, over the same lists as the double-float passes (cheap:
+// over the float32 treecode's).
+Status apply_correction(Context& c, const double* d, double* w, double* v, bool cheap);
 
 // ---- solver (solver.cu)
 Status mobility_solve(Context& c, const double* F, const double* T, double tol, double* v, double* om,

@@ -1546,13 +1546,15 @@ Status apply_pairs_both(Context& c, int prec, const double* x, double* yK, doubl
   return Status::Ok();
 }
 
-Status apply_correction(Context& c, const double* d, double* w, double* v) {
+Status apply_correction(Context& c, const double* d, double* w, double* v, bool cheap) {
   RBS_TRY(apply_blocks(c, kModeSelfK, RBS_PREC_DF, d, w, nullptr, 1.0));
   RBS_TRY(apply_blocks(c, kModeSelfS, RBS_PREC_DF, d, v, nullptr, 1.0));
   c.stats.launches += 2;
   RBS_TRY(weight_f32(c, d));
   RBS_TRY(weight_df(c, d));
-  if (c.tree_df.active) {
+  if (cheap) {
+    RBS_TRY(apply_tree_both(c, w, v));
+  } else if (c.tree_df.active) {
     RBS_TRY(apply_tree_df_f32(c, d, w, v));
   } else if (!c.work.empty()) {
     KernelTimer timer(c, RBS_KC_PAIR_K32);

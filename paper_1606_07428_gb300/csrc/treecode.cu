@@ -954,6 +954,15 @@ void TreeState::release() {
   direct_pairs = proxy_pairs = charge_work = lead_pairs = 0;
 }
 
+double tree_error(const Context& c) {
+  if (!c.tree.active) return INFINITY;
+  // empirical model of the treecode's relative error: C(theta) rho^-n with rho the Bernstein ellipse
+  // parameter 1/theta + sqrt(1/theta^2 - 1) and C = 0.25 max(1, (theta / 0.5)^2)
+  const double th = c.tree.theta, a = 1.0 / th;
+  const double C = 0.25 * std::max(1.0, (th / 0.5) * (th / 0.5));
+  return C * std::pow(a + std::sqrt(a * a - 1.0), -c.tree.degree);
+}
+
 Status plan_treecode(const PlanInput& c, double theta, int degree, TreePlan& T) {
   const int n = c.n;
   const int nq = degree + 1, npx = nq * nq * nq;
@@ -1318,32 +1327,58 @@ int tree_variant(const Context& c) {
   return c.tree.degree > 7 || c.opt.pair_variant == 1 || c.opt.pair_variant == kPacked + 1 ? 1 : 2;
 }
 
-Status apply_tree(Context& c, int kind, double* y) {
+// Cluster charges of the float32 lists from the weighted densities in d_wmu32.
+static Status charges32(Context& c) {
   TreeState& T = c.tree;
-  {
-    KernelTimer timer(c, RBS_KC_TREE);
-    int launches = 0;
-    if (T.n_cells > 0) {
-      RBS_CUDA_TRY(cudaMemsetAsync(T.d_pq.ptr, 0, sizeof(float) * T.d_pq.n, c.stream));
-      const int nq = T.degree + 1;
+  KernelTimer timer(c, RBS_KC_TREE);
+  int launches = 0;
+  if (T.n_cells > 0) {
+    RBS_CUDA_TRY(cudaMemsetAsync(T.d_pq.ptr, 0, sizeof(float) * T.d_pq.n, c.stream));
+    const int nq = T.degree + 1;
 #define RBS_CHARGE_ARGS                                                                                            \
   T.d_charge_items.ptr, T.d_order.ptr, c.d_offset.ptr, c.d_x.ptr, c.d_wmu32.ptr, T.d_box.ptr, T.d_cheb.ptr, nq, T.nbp, \
       T.ncp, T.d_pq.ptr
-      if (nq <= 8)
-        k_tree_charges32<8><<<(unsigned)T.charge_items.size(), kChargeThreads32, 0, c.stream>>>(RBS_CHARGE_ARGS);
-      else
-        k_tree_charges32<12><<<(unsigned)T.charge_items.size(), kChargeThreads32, 0, c.stream>>>(RBS_CHARGE_ARGS);
+    if (nq <= 8)
+      k_tree_charges32<8><<<(unsigned)T.charge_items.size(), kChargeThreads32, 0, c.stream>>>(RBS_CHARGE_ARGS);
+    else
+      k_tree_charges32<12><<<(unsigned)T.charge_items.size(), kChargeThreads32, 0, c.stream>>>(RBS_CHARGE_ARGS);
 #undef RBS_CHARGE_ARGS
-      launches = 1;
-    }
-    RBS_CUDA_TRY(cudaGetLastError());
-    timer.done((double)T.charge_work, launches);
+    launches = 1;
   }
+  RBS_CUDA_TRY(cudaGetLastError());
+  timer.done((double)T.charge_work, launches);
+  return Status::Ok();
+}
+
+Status apply_tree(Context& c, int kind, double* y) {
+  TreeState& T = c.tree;
+  RBS_TRY(charges32(c));
   if (T.items.empty()) return Status::Ok();
   KernelTimer timer(c, kind == 0 ? RBS_KC_PAIR_K32 : RBS_KC_PAIR_S32);
   RBS_TRY(kind == 0 ? launch_tree<0>(c, y) : launch_tree<1>(c, y));
   timer.done((double)(T.direct_pairs + T.proxy_pairs));
   return Status::Ok();
+}
+
+// y += traction and y2 += Stokeslet sum over the lists of T in float32, without the own and near particles.
+static Status launch_both(Context& c, const TreeState& T, double* y, double* y2) {
+  if (T.items.empty()) return Status::Ok();
+  KernelTimer timer(c, RBS_KC_PAIR_K32);
+  switch ((T.degree + 2) / 2) {  // degree 2 to 12
+    case 2: RBS_TRY((launch_tree<2, 1, 2>(c, T, y, y2))); break;
+    case 3: RBS_TRY((launch_tree<2, 1, 3>(c, T, y, y2))); break;
+    case 4: RBS_TRY((launch_tree<2, 1, 4>(c, T, y, y2))); break;
+    case 5: RBS_TRY((launch_tree<2, 1, 5>(c, T, y, y2))); break;
+    case 6: RBS_TRY((launch_tree<2, 1, 6>(c, T, y, y2))); break;
+    default: RBS_TRY((launch_tree<2, 1, 7>(c, T, y, y2)));
+  }
+  timer.done(2.0 * (double)(T.direct_pairs - T.lead_pairs + T.proxy_pairs));
+  return Status::Ok();
+}
+
+Status apply_tree_both(Context& c, double* y, double* y2) {
+  RBS_TRY(charges32(c));
+  return launch_both(c, c.tree, y, y2);
 }
 
 // Float64 cluster charges of the double-float lists, as the float32 kernel reads them.
@@ -1372,18 +1407,7 @@ Status apply_tree_df_f32(Context& c, const double* x, double* y, double* y2) {
     RBS_CUDA_TRY(cudaGetLastError());
     timer.done((double)T.charge_work, 2);
   }
-  if (T.items.empty()) return Status::Ok();
-  KernelTimer timer(c, RBS_KC_PAIR_K32);
-  switch ((T.degree + 2) / 2) {  // degree 2 to 12
-    case 2: RBS_TRY((launch_tree<2, 1, 2>(c, T, y, y2))); break;
-    case 3: RBS_TRY((launch_tree<2, 1, 3>(c, T, y, y2))); break;
-    case 4: RBS_TRY((launch_tree<2, 1, 4>(c, T, y, y2))); break;
-    case 5: RBS_TRY((launch_tree<2, 1, 5>(c, T, y, y2))); break;
-    case 6: RBS_TRY((launch_tree<2, 1, 6>(c, T, y, y2))); break;
-    default: RBS_TRY((launch_tree<2, 1, 7>(c, T, y, y2)));
-  }
-  timer.done(2.0 * (double)(T.direct_pairs - T.lead_pairs + T.proxy_pairs));
-  return Status::Ok();
+  return launch_both(c, T, y, y2);
 }
 
 template <int KIND>

@@ -116,6 +116,23 @@ def test_updates_over_clusters(rbs, degree):
         check(rbs, ctx, s, out, rbs.RBS_PREC_DF)
 
 
+@pytest.mark.parametrize("degree", [4, 7, 8, 10])
+@pytest.mark.parametrize("gap", [0.2, 0.02])
+def test_small_updates_over_the_float32_treecode(rbs, degree, gap):
+    # 16-bit blocks: several refinements, the last ones small enough for the float32 lists; passes are direct
+    m = 18  # particles of 84 nodes: more nodes in a chain than the 1,331 proxy points of degree 10
+    x = np.concatenate([np.arange(m) * (2 + gap), np.arange(m) * (2 + gap) + 6.0 * m])
+    s = bodies(np.stack([x, 0 * x, 0 * x], 1), 6, seed=4)
+    with rbs.Context(device=0, precision=rbs.RBS_PREC_MIXED_BF16, far_field=rbs.RBS_FAR_TREECODE, tree_theta=0.6,
+                     tree_degree=degree) as ctx, rbs.Context(device=0) as exact:
+        ctx.set_suspension(s)
+        exact.set_suspension(s)
+        assert rbs.rbs_get_stats(ctx.ctx)["tree_proxy_pairs"] > 0
+        out = solve(rbs, ctx, s)
+        assert out[4] >= 1 and out[5] >= 1
+        check(rbs, exact, s, out, rbs.RBS_PREC_FP64)
+
+
 def test_no_update_without_a_near_margin(rbs):
     # near_delta 0: particles that are not near may be as close as they like
     s = geometry("turned", 0.3)
