@@ -150,7 +150,7 @@ __global__ void k_weight_df1(long long N, const double4* __restrict__ x, const d
 // The smooth scalar pair sums in double-float arithmetic on the float32 pipes: two sources per packed
 // instruction, tiles and work units as the mobility operators' (pairsdf.cuh).  One pair takes 97 float32
 // operations (K^L) or 71 (S^L), 9 fewer where the tile is on a grid.  Bound by the float32 pipe: the forces on 216
-// particles of 144 nodes went from 49.4 to 27.4 ms with these sums and the near corrections below.
+// particles of 144 nodes went from 49.4 to 26.9 ms with these sums and the near corrections below.
 template <int KIND, int MODE>
 __device__ __forceinline__ void lap_tile_pairs(const float (*sa)[kTileDf], const int* smask, int l0, int l1,
                                                const df2 (&xt)[3], const df2 (&nt)[3], int bit, df2& acc) {

@@ -843,8 +843,9 @@ __global__ void k_weight_df(long long N, const double4* __restrict__ x, const do
 // y2 += Stokeslet sum.  A unit is 32 targets of a work item against its sources; warps take units from
 // a counter, stage their own source tiles and never wait for one another (df_tile, shared with the
 // treecode).  No float64 arithmetic runs but the final accumulation per target.  Bound by the float32 pipe, 84%
-// busy: both sums 126 to 153 Gpair/s (101 particles of 220 nodes), the traction alone 195 to 219 (500 of 220),
-// against two-sum arithmetic throughout in blocks of whole items.
+// busy: both sums 126 to 153 Gpair/s (101 particles of 220 nodes; 150 since near sources are left out, on as many
+// instructions), the traction alone 195 to 219 (500 of 220), against two-sum arithmetic throughout in blocks of whole
+// items.
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_pairs_df2(unit_t nunits, unit_t* __restrict__ counter,
                                                       const longlong4* __restrict__ work, DfSkip skip,
